@@ -277,7 +277,7 @@ int dat_lamb_step(dat_plan_t *plan, float *theta, float *mom, float *var, const 
  *   num_layers      h, 1 <= h <= DAT_STATIC_MAX_LAYERS.
  *   layer_offsets   HOST array of h+1 element offsets (as for dat_plan_create); copied during
  *                   the call.  The layers may span at most DAT_STATIC_MAX_TILES tiles of 4096
- *                   elements (each layer occupies ceil((n_l + 3)/4096) or fewer); larger
+ *                   elements (each layer occupies ceil((n_l + 7)/4096) or fewer); larger
  *                   problems are refused with DAT_ERR_TOO_LARGE before anything is launched.
  *   theta, mom      device fp32[d], updated in place.      g_hat  device fp32[d], read-only.
  *   hp              host pointer, read during the call.
@@ -379,8 +379,7 @@ int dat_step_lamb_two_sided(dat_plan_t *plan, float *theta, float *mom, float *v
  * bit up to the norms' last place, computed by three streaming passes in separate launches: quantizer
  * norms; then levels, signed sum over the workers, g_hat, m' and the layer sums in one pass that keeps
  * codes, sums and g_hat in registers; then the theta update.  The gradients are read twice by
- * construction.  For plans with b < 32 and the shared scale (DAT_ERR_UNSUPPORTED otherwise).  Its first
- * call on a plan allocates two small tables (synchronous: not for use under stream capture). */
+ * construction.  For plans with b < 32 and the shared scale (DAT_ERR_UNSUPPORTED otherwise). */
 int dat_step_passes(dat_plan_t *plan, float *theta, float *mom, const float *const *grads,
                     uint64_t seed, uint64_t step, const dat_hparams_t *hp, int32_t *code_sum_out,
                     float *layer_norms_out, float *scales_out, void *stream);

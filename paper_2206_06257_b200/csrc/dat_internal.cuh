@@ -8,10 +8,12 @@
 
 #include "dat.h"
 
-// Elements per tile of the per-layer tiling (tiles never cross a layer boundary; they start
-// on 4-element boundaries of the flat vector so that float4 accesses stay 16-byte aligned).
+// Elements per tile of the per-layer tiling (tiles never cross a layer boundary; they start on 8-element boundaries
+// of the flat vector: 32-byte accesses, and whole Philox blocks).
 #define DAT_TILE 4096
 #define DAT_THREADS 256
+// Pieces of the flat vector (they may span layers) of which a warp quantizes one, two or four.
+#define DAT_FLAT 512
 
 struct GradPtrs {
     const float *p[DAT_MAX_WORKERS];
@@ -25,6 +27,12 @@ struct PhiloxKeys {
 };
 
 struct PipeSchedule;    // dat_pipeline.cu
+
+// One per-layer tile of the separate-call kernels (see dat_tile_range): what a CTA needs to know, in one load.
+struct TileDesc {
+    int64_t lo, hi, begin;             // the layer's bounds; first element of the tile (a multiple of 8)
+    int32_t layer, first;              // first: the layer's first tile
+};
 
 // LAMB (Algorithm A2): what the kernels need of the hyper-parameters at iteration t.
 struct LambConst {
@@ -49,6 +57,9 @@ struct dat_plan {
     size_t ws_bytes = 0;
     int64_t *d_offsets = nullptr;      // h+1
     int64_t *d_tile_base = nullptr;    // h+1
+    TileDesc *d_tiles = nullptr;       // n_tiles
+    int32_t *d_flat_layer = nullptr;   // pieces of DAT_FLAT elements + 1: the layer of each piece's first element (last entry: h-1)
+    uint32_t *d_count = nullptr;       // h     tiles of the layer that have been summed (k_sumsq; zero between calls)
     double *d_partials = nullptr;      // n_tiles * max(M,2)
     float *d_worker_norms = nullptr;   // M*h
     float *d_scales = nullptr;         // h     nu_l (fused path / scratch)
@@ -59,11 +70,6 @@ struct dat_plan {
     uint32_t *d_status = nullptr;      // 1
 
     PipeSchedule *pipe = nullptr;      // work items and tables of dat_step_pipelined, built with the plan
-
-    // dat_step_passes: per-layer tiles that start on multiples of 8 elements, and their partial sums
-    int64_t *d_tile_base8 = nullptr;   // h+1
-    double *d_partials8 = nullptr;     // 2 per tile
-    int64_t n_tiles8 = 0;
 
     // staging buffers of dat_step_host
     float *stage = nullptr;
@@ -138,6 +144,75 @@ __device__ __forceinline__ float dat_u1_from_half(uint32_t half)
     return __uint_as_float(0x3F800000u | (half << 7));
 }
 
+// Philox with what does not change along the loops taken out.  Of the counter (q, q_hi, worker, seed_hi) the first
+// two rounds multiply words that depend on the element alone or on the worker alone: with those products kept, the
+// block of one (element group, worker) pair is two XORs and rounds 2..9 -- 16 of the 20 wide multiplies, which cost
+// four issue cycles of the multiply pipe each on sm_100 (measured; LOP3, PRMT and shifts cost two of the ALU pipe,
+// FFMA one, a DP2A two of the multiply pipe).
+struct PhiloxElem { uint32_t a, b, c; };         // from the element group's counter word q
+struct PhiloxWorker { uint32_t x, y, z; };       // from the worker (and q_hi, which is the same for a whole tile)
+
+__device__ __forceinline__ PhiloxElem dat_philox_elem(uint32_t q, const PhiloxKeys &k)
+{
+    const uint64_t p0 = (uint64_t)0xD2511F53u * q;
+    const uint64_t p1 = (uint64_t)0xCD9E8D57u * ((uint32_t)(p0 >> 32) ^ k.seed_hi ^ k.k1[0]);
+    return PhiloxElem{(uint32_t)(p1 >> 32), (uint32_t)p1, (uint32_t)p0};
+}
+__host__ __device__ __forceinline__ PhiloxWorker dat_philox_worker(uint32_t q_hi, uint32_t worker, const PhiloxKeys &k)
+{
+    const uint64_t p1 = (uint64_t)0xCD9E8D57u * worker;
+    const uint64_t p0 = (uint64_t)0xD2511F53u * ((uint32_t)(p1 >> 32) ^ q_hi ^ k.k0[0]);
+    return PhiloxWorker{(uint32_t)p1 ^ k.k0[1], (uint32_t)(p0 >> 32) ^ k.k1[1], (uint32_t)p0};
+}
+__device__ __forceinline__ void dat_philox_block(const PhiloxElem &e, const PhiloxWorker &w, const PhiloxKeys &k, uint32_t out[4])
+{
+    uint32_t c0 = e.a ^ w.x, c1 = e.b, c2 = e.c ^ w.y, c3 = w.z;
+#pragma unroll
+    for (int r = 2; r < 10; ++r) {
+        const uint64_t p0 = (uint64_t)0xD2511F53u * c0;
+        const uint64_t p1 = (uint64_t)0xCD9E8D57u * c2;
+        c0 = (uint32_t)(p1 >> 32) ^ c1 ^ k.k0[r];
+        c2 = (uint32_t)(p0 >> 32) ^ c3 ^ k.k1[r];
+        c1 = (uint32_t)p1;
+        c3 = (uint32_t)p0;
+    }
+    out[0] = c0; out[1] = c1; out[2] = c2; out[3] = c3;
+}
+
+// (1 + u) 2^-b of element j of a group of eight, from the group's random words, in one instruction: the exponent
+// field of 2^-b plus the uniform number in the mantissa -- half * 128 + ubits as a two-way dot product (multiply
+// pipe, no ALU) at 16 bits, low 23 bits OR ubits at 23 bits.  Exact: 1 + u has at most 24 significant bits.
+template <bool RNG16>
+__device__ __forceinline__ float dat_u1_scaled(const uint32_t *w, int j, uint32_t ubits)
+{
+    if (RNG16) return __uint_as_float(__dp2a_lo(w[j >> 1], (j & 1) ? 0x8000u : 0x0080u, ubits));
+    return __uint_as_float(ubits | (w[j] & 0x007FFFFFu));
+}
+
+// The random words of the eight elements of one group: one block at 16 bits, two at 23 bits.
+template <bool RNG16> struct PhiloxGroup { PhiloxElem e[RNG16 ? 1 : 2]; };
+template <bool RNG16>
+__device__ __forceinline__ PhiloxGroup<RNG16> dat_philox_group(uint64_t e0, const PhiloxKeys &k)
+{
+    PhiloxGroup<RNG16> g;
+    g.e[0] = dat_philox_elem((uint32_t)(e0 >> (RNG16 ? 3 : 2)), k);
+    if (!RNG16) g.e[RNG16 ? 0 : 1] = dat_philox_elem((uint32_t)(e0 >> 2) + 1u, k);
+    return g;
+}
+template <bool RNG16>
+__device__ __forceinline__ void dat_group_words(const PhiloxGroup<RNG16> &g, const PhiloxWorker &w, const PhiloxKeys &k, uint32_t out[8])
+{
+    dat_philox_block(g.e[0], w, k, out);
+    if (!RNG16) dat_philox_block(g.e[RNG16 ? 0 : 1], w, k, out + 4);
+}
+// Counter words above 32 bits: the same for every group of [begin, begin + n) unless this says so.
+template <bool RNG16>
+__device__ __forceinline__ bool dat_one_counter_page(uint64_t begin, uint64_t n)
+{
+    constexpr int SH = 32 + (RNG16 ? 3 : 2);
+    return (begin >> SH) == ((begin + n - 1) >> SH);
+}
+
 // u1 of the four elements e0 .. e0+3 (e0 a multiple of 4) of `worker`.  rng16 = false: one
 // Philox block per four elements, word j for element e0+j.  rng16 = true: one block per EIGHT
 // elements (counter e/8); element e takes word (e/2) mod 4, low half if e is even, high if odd.
@@ -192,6 +267,21 @@ __device__ __forceinline__ int dat_find(const int64_t *__restrict__ table, int h
     return lo;
 }
 
+// One thread's release / acquire point at GPU scope.  What the CTA's other threads wrote before a barrier that this
+// thread has passed is released with it (and what it acquires holds for threads behind a later barrier), so one thread
+// per CTA fences, and with the acquire-release fence: __threadfence() is the sequentially consistent one.
+__device__ __forceinline__ void dat_fence() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+
+// One thread, the CTA's part of a count being complete: counts it in; returns whether it was the last of `total`
+// (what the others released before counting is then visible to this CTA's threads after their next barrier).
+__device__ __forceinline__ bool dat_count_in(uint32_t *count, uint32_t total)
+{
+    dat_fence();
+    const bool last = atomicAdd(count, 1u) == total - 1u;
+    if (last) dat_fence();
+    return last;
+}
+
 __device__ __forceinline__ double dat_warp_sum(double v)
 {
 #pragma unroll
@@ -219,25 +309,47 @@ __device__ __forceinline__ double dat_block_sum(double v, double *scratch)
 // ------------------------------------------------------------------------------------------
 // Per-layer tiling shared by the norm kernels: tile t belongs to layer l = find(tile_base, t);
 // it covers the flat elements [a + k*DAT_TILE, a + (k+1)*DAT_TILE) ∩ [lo, hi) where
-// lo/hi are the layer's bounds, a = lo rounded down to a multiple of 4 and k = t - tile_base[l].
+// lo/hi are the layer's bounds, a = lo rounded down to a multiple of 8 and k = t - tile_base[l].
 // ------------------------------------------------------------------------------------------
 struct TileRange {
     int layer;
+    int64_t first;         // the layer's first tile
     int64_t lo, hi;        // layer bounds
-    int64_t begin, end;    // begin is a multiple of 4; elements outside [lo, hi) are masked
+    int64_t begin, end;    // begin is a multiple of 8; elements outside [lo, hi) are masked
 };
 
-__device__ __forceinline__ TileRange dat_tile_range(const int64_t *__restrict__ off,
-                                                    const int64_t *__restrict__ tile_base, int h,
-                                                    int64_t tile)
+// The tiles of a plan come from its table; without a plan (dat_lalr_step_static) they are found in the layer table.
+struct TileSource {
+    const TileDesc *tiles;
+    const int64_t *off, *tile_base;
+    int h;
+};
+
+__device__ __forceinline__ TileRange dat_tile_range(const TileSource &src, int64_t tile)
 {
     TileRange r;
-    r.layer = dat_find(tile_base, h, tile);
-    r.lo = __ldg(off + r.layer);
-    r.hi = __ldg(off + r.layer + 1);
-    r.begin = (r.lo & ~(int64_t)3) + (tile - __ldg(tile_base + r.layer)) * DAT_TILE;
+    if (src.tiles) {
+        const longlong2 a = __ldg(reinterpret_cast<const longlong2 *>(src.tiles + tile)), b = __ldg(reinterpret_cast<const longlong2 *>(src.tiles + tile) + 1);
+        r.lo = a.x;
+        r.hi = a.y;
+        r.begin = b.x;
+        r.layer = (int)(uint32_t)b.y;
+        r.first = (int64_t)(b.y >> 32);
+    } else {
+        r.layer = dat_find(src.tile_base, src.h, tile);
+        r.first = __ldg(src.tile_base + r.layer);
+        r.lo = __ldg(src.off + r.layer);
+        r.hi = __ldg(src.off + r.layer + 1);
+        r.begin = (r.lo & ~(int64_t)7) + (tile - r.first) * DAT_TILE;
+    }
     r.end = min(r.begin + (int64_t)DAT_TILE, r.hi);
     return r;
+}
+
+// Tiles of the layer.
+__device__ __forceinline__ int64_t dat_layer_tiles(const TileRange &r)
+{
+    return (r.hi - (r.lo & ~(int64_t)7) + DAT_TILE - 1) / DAT_TILE;
 }
 
 // Loads the four elements e0..e0+3 (e0 a multiple of 4) that lie in [lo, hi); others read 0.
@@ -302,6 +414,19 @@ __device__ __forceinline__ float4 dat_ld4_hint(const float *p, uint64_t pol)
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p), "l"(pol));
     return v;
 }
+// Eight consecutive floats of a stream that is read once.  sm_100 has 32-byte loads; they want a 32-byte boundary, which
+// a 16-byte aligned buffer may not have (wide: the buffer does; e0 is a multiple of 8).
+__device__ __forceinline__ void dat_ld8_stream(const float *p, bool wide, float v[8])
+{
+    if (wide) {
+        asm volatile("ld.global.L1::no_allocate.L2::evict_first.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "l"(p));
+    } else {
+        const float4 a = __ldcs(reinterpret_cast<const float4 *>(p)), b = __ldcs(reinterpret_cast<const float4 *>(p) + 1);
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    }
+}
+__device__ __forceinline__ bool dat_aligned32(const void *p) { return ((uintptr_t)p & 31u) == 0; }
 __device__ __forceinline__ void dat_st4_hint(float *p, float4 v, uint64_t pol)
 {
     asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1,%2,%3,%4}, %5;"

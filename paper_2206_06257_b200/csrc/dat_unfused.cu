@@ -6,55 +6,33 @@
 #include "dat_internal.cuh"
 
 // ------------------------------------------------------------------------------------------
-// S1: quantizer norms.  Pass A: one fp64 partial sum of squares per (tile, worker).
-// Pass B: per layer, fixed-order sum of the partials, nu_l = max_i sqrt(.), S/nu_l.
-// Squares of fp32 values are exact in fp64, so the result does not depend on the tiling
-// beyond the last bits of an fp64 sum.
+// S1: quantizer norms.  One fp64 partial sum of squares per (tile, worker); the CTA that finishes a layer's last
+// tile adds the layer's partials in a fixed order: nu_{i,l}, nu_l = max_i, S/nu.  Squares of fp32 values are exact
+// in fp64, so the result does not depend on the tiling beyond the last bits of an fp64 sum.
+// HBM-bound (129 us for the 818 MB of ResNet-50, M = 8: 6.3 TB/s); finishing in the same launch instead of a second
+// one takes 8.7 us off (a launch of one CTA per layer, nearly all of it latency).
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(DAT_THREADS)
-k_sumsq_partial(GradPtrs gp, const int64_t *__restrict__ off, const int64_t *__restrict__ tile_base,
-                int h, int M, double *__restrict__ partials)
-{
-    __shared__ double scratch[DAT_THREADS / 32];
-    const int64_t tile = blockIdx.x;
-    const int worker = blockIdx.y;
-    const TileRange r = dat_tile_range(off, tile_base, h, tile);
-    const float *__restrict__ g = gp.p[worker];
-    double acc = 0.0;
-    constexpr int ITERS = DAT_TILE / 4 / DAT_THREADS;
-    float v[ITERS][4];
-#pragma unroll
-    for (int it = 0; it < ITERS; ++it) {          // every load of the thread is in flight before the first is used
-        const int64_t e0 = r.begin + 4 * (int64_t)(it * DAT_THREADS + threadIdx.x);
-        if (e0 < r.end) dat_load4(g, e0, r.lo, r.hi, v[it]);
-        else v[it][0] = v[it][1] = v[it][2] = v[it][3] = 0.0f;
-    }
-#pragma unroll
-    for (int it = 0; it < ITERS; ++it) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc = fma((double)v[it][j], (double)v[it][j], acc);
-    }
-    const double s = dat_block_sum(acc, scratch);
-    if (threadIdx.x == 0) partials[tile * M + worker] = s;
-}
+#define SUMSQ_WORKERS 8                           // workers of a tile that one CTA sums, at most (a warp's partials: <= 32)
 
-__global__ void __launch_bounds__(DAT_THREADS)
-k_scales_finalize(const int64_t *__restrict__ tile_base, int h, int M, float S_f,
-                  const double *__restrict__ partials, float *__restrict__ worker_norms,
-                  float *__restrict__ scales, float *__restrict__ qmul, uint32_t *status, bool per_worker)
+struct NormOut {
+    float S_f;
+    float *worker_norms, *scales, *qmul;
+    uint32_t *count, *status;
+    bool per_worker;
+};
+
+__device__ __forceinline__ void sumsq_finish(int l, int64_t t0, int64_t t1, int h, int M, const double *partials, const NormOut &o)
 {
     __shared__ float s_norm[DAT_MAX_WORKERS];
-    const int l = blockIdx.x;
-    const int64_t t0 = tile_base[l], t1 = tile_base[l + 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = warp; i < M; i += DAT_THREADS / 32) {
         double acc = 0.0;
-        for (int64_t t = t0 + lane; t < t1; t += 32) acc += partials[t * M + i];
+        for (int64_t t = t0 + lane; t < t1; t += 32) acc += __ldcg(partials + t * M + i);
         acc = dat_warp_sum(acc);
         if (lane == 0) {
             const float nrm = (float)sqrt(acc);
             s_norm[i] = nrm;
-            worker_norms[(int64_t)i * h + l] = nrm;
+            o.worker_norms[(int64_t)i * h + l] = nrm;
         }
     }
     __syncthreads();
@@ -65,120 +43,309 @@ k_scales_finalize(const int64_t *__restrict__ tile_base, int h, int M, float S_f
             bad |= !isfinite(s_norm[i]);
             nu = (s_norm[i] > nu) ? s_norm[i] : nu;
         }
-        if (per_worker) {
+        if (o.per_worker) {
             // every worker keeps its own norm (Eq. rand_q as written): index i*h + l
             for (int i = 0; i < M; ++i) {
-                scales[(int64_t)i * h + l] = s_norm[i];
-                qmul[(int64_t)i * h + l] = (s_norm[i] == 0.0f) ? 0.0f : S_f / s_norm[i];
+                o.scales[(int64_t)i * h + l] = s_norm[i];
+                o.qmul[(int64_t)i * h + l] = (s_norm[i] == 0.0f) ? 0.0f : o.S_f / s_norm[i];
             }
         } else {
-            scales[l] = nu;
-            qmul[l] = (nu == 0.0f) ? 0.0f : S_f / nu;
+            o.scales[l] = nu;
+            o.qmul[l] = (nu == 0.0f) ? 0.0f : o.S_f / nu;
         }
-        if (bad) atomicOr(status, DAT_STATUS_NONFINITE);
+        if (bad) atomicOr(o.status, DAT_STATUS_NONFINITE);
+        o.count[l] = 0u;                          // ready for the next call
     }
 }
 
-// qmul from caller-supplied norms.
-__global__ void k_qmul_from_scales(int h, float S_f, const float *__restrict__ scales,
-                                   float *__restrict__ qmul, uint32_t *status)
+// NW workers' loads in flight per thread.
+template <int NW>
+__global__ void __launch_bounds__(DAT_THREADS, NW == 1 ? 6 : 4)
+k_sumsq(const __grid_constant__ GradPtrs gp, const TileSource tiles, int M, int per_cta, double *partials, const __grid_constant__ NormOut out)
 {
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= h) return;
-    const float nu = scales[l];
-    qmul[l] = (nu == 0.0f) ? 0.0f : S_f / nu;
-    if (!isfinite(nu)) atomicOr(status, DAT_STATUS_NONFINITE);
+    constexpr int W = DAT_THREADS / 32, ITERS = DAT_TILE / 8 / DAT_THREADS;
+    __shared__ double s_sum[SUMSQ_WORKERS][W];
+    __shared__ bool s_last;
+    const int64_t tile = blockIdx.x;
+    const int w0 = blockIdx.y * per_cta, w1 = min(w0 + per_cta, M);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const TileRange r = dat_tile_range(tiles, tile);
+    const bool inside = r.begin >= r.lo && r.begin + DAT_TILE <= r.hi;
+    for (int i = w0; i < w1; i += NW) {           // every load of NW workers is in flight before the first is used
+        float v[NW][ITERS][8];
+#pragma unroll
+        for (int p = 0; p < NW; ++p) {
+            const float *__restrict__ g = gp.p[min(i + p, w1 - 1)];
+            const bool wide = dat_aligned32(g);
+#pragma unroll
+            for (int it = 0; it < ITERS; ++it) {
+                const int64_t e0 = r.begin + 8 * (int64_t)(it * DAT_THREADS + threadIdx.x);
+                if (inside && i + p < w1) dat_ld8_stream(g + e0, wide, v[p][it]);
+                else {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) v[p][it][j] = (i + p < w1 && e0 + j >= r.lo && e0 + j < r.end) ? g[e0 + j] : 0.0f;
+                }
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < NW; ++p) {
+            double acc = 0.0;
+#pragma unroll
+            for (int it = 0; it < ITERS; ++it)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc = fma((double)v[p][it][j], (double)v[p][it][j], acc);
+            acc = dat_warp_sum(acc);
+            if (lane == 0 && i + p < w1) s_sum[i + p - w0][warp] = acc;
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < w1 - w0; i += DAT_THREADS) {
+        double s = 0.0;
+#pragma unroll
+        for (int w = 0; w < W; ++w) s += s_sum[i][w];
+        partials[tile * M + w0 + i] = s;
+    }
+    const int64_t T = dat_layer_tiles(r);
+    if (warp == 0) {                              // (at most 32 workers: the partials are warp 0's)
+        __syncwarp();
+        if (lane == 0) s_last = dat_count_in(out.count + r.layer, (uint32_t)(T * gridDim.y));
+    }
+    __syncthreads();
+    if (s_last) sumsq_finish(r.layer, r.first, r.first + T, tiles.h, M, partials, out);
+}
+
+static TileSource plan_tiles(const dat_plan_t *plan) { return TileSource{plan->d_tiles, plan->d_offsets, plan->d_tile_base, (int)plan->h}; }
+
+static int sumsq_launch(dat_plan_t *plan, const GradPtrs &gp, int M, float *scales, bool per_worker, cudaStream_t s)
+{
+    const NormOut o = {(float)plan->S, plan->d_worker_norms, scales, plan->d_qmul, plan->d_count, plan->d_status, per_worker};
+    // several workers in a CTA (fewer arrivals at the layer's counter, a longer stream per CTA) as long as the CTAs
+    // still fill the GPU
+    int per_cta = 1;
+    while (per_cta < SUMSQ_WORKERS && per_cta < M && plan->n_tiles * ((M + 2 * per_cta - 1) / (2 * per_cta)) >= 8 * plan->sm_count) per_cta *= 2;
+    dim3 grid((unsigned)plan->n_tiles, (unsigned)((M + per_cta - 1) / per_cta));
+    if (per_cta == 1) k_sumsq<1><<<grid, DAT_THREADS, 0, s>>>(gp, plan_tiles(plan), M, per_cta, plan->d_partials, o);
+    else k_sumsq<2><<<grid, DAT_THREADS, 0, s>>>(gp, plan_tiles(plan), M, per_cta, plan->d_partials, o);
+    DAT_LAUNCHED(plan);
+    return DAT_OK;
 }
 
 // ------------------------------------------------------------------------------------------
-// S2 + S3: stochastic levels and the packed planes.  Tiles are DAT_TILE consecutive elements of
-// the FLAT vector (they may span layers); thread t of iteration k owns the aligned group of four
-// elements 4*(k*256+t).., which is exactly one Philox block.  The packed bits of a tile are
-// assembled in shared memory and written out with 128-bit stores.
+// S2 + S3: stochastic levels and the packed planes.  A warp takes 256 * `groups` consecutive elements of the flat
+// vector (they may span layers) of one worker, a lane a group of eight of every 256 -- one Philox block at 16 bits,
+// two at 23.  The packed bits are assembled in the warp's own shared memory and written out with 128-bit stores.
+// HBM-bound once the arithmetic is short (4 bytes read and (b+1)/8 written per element; see dat_u1_scaled): 187 us for
+// ResNet-50, M = 8, b = 8, 5.6 TB/s.  It was 390 us with four elements per thread (each block of eight drawn twice), the
+// plain form of the level and no loads in flight while levels are drawn.
 // ------------------------------------------------------------------------------------------
-template <int BITS>
-__global__ void __launch_bounds__(DAT_THREADS)
-k_quantize(GradPtrs gp, PhiloxKeys keys, const int64_t *__restrict__ off, int h, int64_t d,
-           const float *__restrict__ qmul_all, uint8_t *__restrict__ levels, uint8_t *__restrict__ signs,
-           int64_t level_bytes, int64_t sign_bytes, bool rng16, bool per_worker, uint32_t stream_base, int64_t elem_base)
+#define QUANT_GROUPS 8                           // groups of eight per lane, at most (a multiple of 2)
+#define QUANT_CTAS 4                             // resident CTAs per SM (3: 199 us, 5 with spills: 232 us instead of 187)
+
+struct QuantScale {                              // where a layer's S/nu comes from
+    const float *qmul;                           // computed before (scales_in == nullptr), or
+    const float *scales_in;                      // the caller's norms, from which it is formed here; they are copied to scales
+    float *scales;
+    int n_scales;
+    float S_f;
+    uint32_t *status;
+};
+__device__ __forceinline__ float quant_mul(const QuantScale &q, int64_t k)
 {
-    constexpr int GROUPS = DAT_TILE / 4;                     // aligned groups per tile
-    constexpr int LEVEL_TILE_BYTES = DAT_TILE * BITS / 8;
-    constexpr int SIGN_TILE_BYTES = DAT_TILE / 8;
-    __shared__ uint4 s_level[LEVEL_TILE_BYTES / 16];
-    __shared__ uint4 s_sign[SIGN_TILE_BYTES / 16];
-    __shared__ int s_first;
+    if (!q.scales_in) return __ldg(q.qmul + k);
+    const float nu = __ldg(q.scales_in + k);
+    return (nu == 0.0f) ? 0.0f : q.S_f / nu;
+}
 
-    const int64_t tile = blockIdx.x;
-    const int worker = blockIdx.y;
-    const int64_t e_tile = tile * DAT_TILE;
-    const float *__restrict__ g = gp.p[worker];
-    const float *__restrict__ qmul = qmul_all + (per_worker ? (int64_t)worker * h : 0);
-    const float S1_f = (float)(1u << BITS);                  // S + 1
-
-    if (threadIdx.x == 0) s_first = dat_find(off, h, e_tile);
-    __syncthreads();
-    int l = s_first;
-    int64_t l_hi = __ldg(off + l + 1);
-    float t = __ldg(qmul + l);
-
-    float gall[GROUPS / DAT_THREADS][4];
-#pragma unroll
-    for (int it = 0; it < GROUPS / DAT_THREADS; ++it)      // every load of the thread is in flight before the first is used
-        dat_load4(g, e_tile + 4 * (int64_t)(it * DAT_THREADS + threadIdx.x), 0, d, gall[it]);
-#pragma unroll
-    for (int it = 0; it < GROUPS / DAT_THREADS; ++it) {
-        const int v = it * DAT_THREADS + threadIdx.x;
-        const int64_t e0 = e_tile + 4 * (int64_t)v;
-        const float *gv = gall[it];
+// A group at the vector's end, across layers, or whose layer's scale is outside the range of the scaled form: the
+// plain form of Eq. xi, element by element.  Leaves the group's packed levels and signs in shared memory.
+template <int BITS>
+__device__ __noinline__ void quantize_slow8(const float *__restrict__ g, int64_t e0, const int64_t *__restrict__ off, int l0, int nl, int64_t d,
+                                            const QuantScale &qs, int64_t q0, uint64_t elem, uint32_t stream, const PhiloxKeys &keys, bool rng16,
+                                            uint8_t *s_level, uint8_t *s_sign)
+{
+    uint32_t neg = 0;
+    int64_t l_hi = 0;
+    float t = 0.0f;
+#pragma unroll 1
+    for (int p = 0; p < 2; ++p) {
         float u1[4];
-        dat_u1x4((uint64_t)(e0 + elem_base), stream_base + (uint32_t)worker, keys, rng16, u1);     // the worker's random stream
-        uint32_t lev[4], neg = 0;
+        uint64_t packed = 0;
+        dat_u1x4(elem + 4 * p, stream, keys, rng16, u1);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int64_t e = e0 + j;
-            while (e >= l_hi && l + 1 < h) {     // advance to the element's layer
-                ++l;
-                l_hi = __ldg(off + l + 1);
-                t = __ldg(qmul + l);
+            const int64_t e = e0 + 4 * p + j;
+            if (e < d) {
+                if (e >= l_hi) {                  // (also the first element: l_hi = 0)
+                    const int l = l0 + dat_find(off + l0, nl, e);
+                    l_hi = __ldg(off + l + 1);
+                    t = quant_mul(qs, q0 + l);
+                }
+                const float x = g[e];
+                packed |= (uint64_t)dat_level_u1(x, t, (float)(1u << BITS), u1[j]) << (BITS * j);
+                neg |= (uint32_t)(x < 0.0f) << (4 * p + j);
             }
-            lev[j] = (e < d) ? dat_level_u1(gv[j], t, S1_f, u1[j]) : 0u;
-            neg |= (uint32_t)(gv[j] < 0.0f) << j;
         }
-        // pack the group's level bits
-        if (BITS == 16) {
-            reinterpret_cast<uint2 *>(s_level)[v] = make_uint2(lev[0] | (lev[1] << 16), lev[2] | (lev[3] << 16));
-        } else if (BITS == 8) {
-            reinterpret_cast<uint32_t *>(s_level)[v] = lev[0] | (lev[1] << 8) | (lev[2] << 16) | (lev[3] << 24);
-        } else if (BITS == 4) {
-            reinterpret_cast<uint16_t *>(s_level)[v] = (uint16_t)(lev[0] | (lev[1] << 4) | (lev[2] << 8) | (lev[3] << 12));
-        } else if (BITS == 2) {
-            reinterpret_cast<uint8_t *>(s_level)[v] = (uint8_t)(lev[0] | (lev[1] << 2) | (lev[2] << 4) | (lev[3] << 6));
-        } else {   // BITS == 1: two neighbouring groups share a byte
-            const uint32_t nib = lev[0] | (lev[1] << 1) | (lev[2] << 2) | (lev[3] << 3);
-            const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, nib, 1);
-            if ((threadIdx.x & 1) == 0) reinterpret_cast<uint8_t *>(s_level)[v >> 1] = (uint8_t)(nib | (other << 4));
-        }
-        const uint32_t other_neg = __shfl_xor_sync(0xFFFFFFFFu, neg, 1);
-        if ((threadIdx.x & 1) == 0) reinterpret_cast<uint8_t *>(s_sign)[v >> 1] = (uint8_t)(neg | (other_neg << 4));
+        if (BITS == 16) reinterpret_cast<uint64_t *>(s_level)[p] = packed;
+        else if (BITS == 8) reinterpret_cast<uint32_t *>(s_level)[p] = (uint32_t)packed;
+        else if (BITS == 4) reinterpret_cast<uint16_t *>(s_level)[p] = (uint16_t)packed;
+        else if (BITS == 2) s_level[p] = (uint8_t)packed;
+        else s_level[0] = (uint8_t)((p ? s_level[0] : 0u) | (uint32_t)packed << (4 * p));
     }
-    __syncthreads();
+    *s_sign = (uint8_t)neg;
+}
 
-    // 128-bit stores of the finished tile (planes are padded to 16 bytes, so whole uint4 fit)
+// Packed levels and signs of one group from its eight elements (lowest first) and random words, by the scaled form:
+// saturation is the clamp to S, min(y, S + 1) 2^-b.
+template <int BITS, bool RNG16>
+__device__ __forceinline__ void quantize8(const float v[8], float ts, const uint32_t w[8], uint8_t *s_level, uint8_t *s_sign)
+{
+    constexpr float TWO_B = (float)(1u << BITS);
+    constexpr uint32_t UBITS = (uint32_t)(127 - BITS) << 23;
+    constexpr int PER = (BITS == 16) ? 2 : (BITS == 8) ? 4 : 8;        // levels in a 32-bit word (b <= 4: all eight)
+    uint32_t word[8 / PER], neg = 0;
+#pragma unroll
+    for (int a = 8 / PER - 1; a >= 0; --a) {
+        uint32_t bias = 0;                        // the float bits carry 0x4B000000 each: a constant modulo 2^32
+        word[a] = 0;
+#pragma unroll
+        for (int j = PER - 1; j >= 0; --j) {
+            const float x = v[a * PER + j] + 0.0f;           // -0 becomes +0: its sign bit is 0
+            const float ys = __saturatef(__fmaf_rn(fabsf(x), ts, dat_u1_scaled<RNG16>(w, a * PER + j, UBITS)));
+            word[a] += __float_as_uint(__fmaf_rz(ys, TWO_B, 8388607.0f)) * (1u << (BITS * j));
+            bias += 0x4B000000u * (1u << (BITS * j));
+            neg = __funnelshift_l(__float_as_uint(x), neg, 1);
+        }
+        word[a] -= bias;
+    }
+    if (BITS == 16) *reinterpret_cast<uint4 *>(s_level) = make_uint4(word[0], word[1 % (8 / PER)], word[2 % (8 / PER)], word[3 % (8 / PER)]);
+    else if (BITS == 8) *reinterpret_cast<uint2 *>(s_level) = make_uint2(word[0], word[1 % (8 / PER)]);
+    else if (BITS == 4) *reinterpret_cast<uint32_t *>(s_level) = word[0];
+    else if (BITS == 2) *reinterpret_cast<uint16_t *>(s_level) = (uint16_t)word[0];
+    else *s_level = (uint8_t)word[0];
+    *s_sign = (uint8_t)neg;
+}
+
+template <int BITS, bool RNG16>
+__global__ void __launch_bounds__(DAT_THREADS, QUANT_CTAS)
+k_quantize(const __grid_constant__ GradPtrs gp, const __grid_constant__ PhiloxKeys keys, const int64_t *__restrict__ off,
+           const int32_t *__restrict__ flat_layer, int h, int64_t d, const __grid_constant__ QuantScale qs, uint8_t *__restrict__ levels,
+           uint8_t *__restrict__ signs, int64_t level_bytes, int64_t sign_bytes, int groups, bool per_worker, uint32_t stream_base, int64_t elem_base)
+{
+    constexpr int MOST = 256 * QUANT_GROUPS;                 // elements of a warp, at most
+    __shared__ uint4 s_level[DAT_THREADS / 32][MOST * BITS / 8 / 16];
+    __shared__ uint4 s_sign[DAT_THREADS / 32][MOST / 8 / 16];
+    const int n_warp = 256 * groups;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int worker = blockIdx.y;
+    const uint32_t stream = stream_base + (uint32_t)worker;  // the worker's random stream
+    if (qs.scales_in) {                                      // copy of the caller's norms, and their check
+        const int64_t n = (int64_t)gridDim.x * gridDim.y * DAT_THREADS;
+        for (int64_t k = ((int64_t)worker * gridDim.x + blockIdx.x) * DAT_THREADS + threadIdx.x; k < qs.n_scales; k += n) {
+            const float nu = qs.scales_in[k];
+            if (qs.scales != qs.scales_in) qs.scales[k] = nu;
+            if (!isfinite(nu)) atomicOr(qs.status, DAT_STATUS_NONFINITE);
+        }
+    }
+    const int64_t part = (int64_t)blockIdx.x * (DAT_THREADS / 32) + warp;
+    const int64_t e_piece = part * n_warp, piece = e_piece / DAT_FLAT, last = min(e_piece + n_warp, d - 1) / DAT_FLAT;
+    if (e_piece >= d) return;
+    const float *__restrict__ g = gp.p[worker] + e_piece + 8 * lane;
+    const uint64_t elem = (uint64_t)(e_piece + elem_base) + 8u * lane;
+    const bool wide = dat_aligned32(gp.p[worker]);
+    const bool whole = e_piece + n_warp <= d;
+    float v[2][8];
+    if (whole) {                                             // two groups per lane are always in flight
+        dat_ld8_stream(g, wide, v[0]);
+        dat_ld8_stream(g + 256, wide, v[1]);
+    }
+    const int l0 = __ldg(flat_layer + piece), nl = __ldg(flat_layer + last + 1) - l0 + 1;   // the warp's layers are among [l0, l0 + nl)
+    const int64_t q0 = per_worker ? (int64_t)worker * h : 0;
+    const int64_t hi = __ldg(off + l0 + 1);                  // end of the first layer
+    const float t0 = quant_mul(qs, q0 + l0);
+    constexpr float TWO_B = (float)(1u << BITS);
+    const bool page = dat_one_counter_page<RNG16>(elem - 8u * lane, n_warp);
+    const PhiloxWorker pw = dat_philox_worker((uint32_t)((elem - 8u * lane) >> (RNG16 ? 35 : 34)), stream, keys);
+    uint8_t *const my_level = reinterpret_cast<uint8_t *>(s_level[warp]) + lane * BITS, *const my_sign = reinterpret_cast<uint8_t *>(s_sign[warp]) + lane;
+    auto scaled = [](float t) { return (t == 0.0f) || (t >= 1.17549435e-38f * TWO_B && t <= 3.402823466e38f); };
+    if (whole && page && hi >= e_piece + n_warp && scaled(t0)) {
+        const float ts = t0 * (1.0f / TWO_B);
+#pragma unroll 1
+        for (int k = 0; k < groups; k += 2) {
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                uint32_t w[8];
+                dat_group_words<RNG16>(dat_philox_group<RNG16>(elem + 256u * (k + p), keys), pw, keys, w);
+                quantize8<BITS, RNG16>(v[p], ts, w, my_level + (k + p) * 32 * BITS, my_sign + (k + p) * 32);
+                if (k + 2 < groups) dat_ld8_stream(g + 256 * (k + p + 2), wide, v[p]);
+            }
+        }
+    } else {
+#pragma unroll 1
+        for (int k = 0; k < groups; ++k) {
+            const int64_t e0 = e_piece + 8 * lane + 256 * k;
+            float t = t0;                                    // the group's layer
+            int64_t l_hi = hi;
+            if (e0 >= hi && e0 < d) {
+                const int l = l0 + dat_find(off + l0, nl, e0);
+                l_hi = __ldg(off + l + 1);
+                t = quant_mul(qs, q0 + l);
+            }
+            if (page && scaled(t) && e0 + 8 <= l_hi) {
+                float x[8];
+                uint32_t w[8];
+                dat_ld8_stream(g + 256 * k, wide, x);
+                dat_group_words<RNG16>(dat_philox_group<RNG16>(elem + 256u * k, keys), pw, keys, w);
+                quantize8<BITS, RNG16>(x, t * (1.0f / TWO_B), w, my_level + k * 32 * BITS, my_sign + k * 32);
+            } else {
+                quantize_slow8<BITS>(g - e_piece - 8 * lane, e0, off, l0, nl, d, qs, q0, elem + 256u * k, stream, keys, RNG16,
+                                     my_level + k * 32 * BITS, my_sign + k * 32);
+            }
+        }
+    }
+    __syncwarp();
+
+    // 128-bit stores of the finished part (planes are padded to 16 bytes, so whole uint4 fit)
     {
-        const int64_t base = tile * LEVEL_TILE_BYTES;
-        const int64_t left = level_bytes - base;
-        const int n16 = (int)((left < LEVEL_TILE_BYTES ? left : LEVEL_TILE_BYTES) / 16);
+        const int64_t bytes = n_warp * BITS / 8, base = part * bytes, left = level_bytes - base;
+        const int n16 = (int)((left < bytes ? left : bytes) / 16);
         uint4 *dst = reinterpret_cast<uint4 *>(levels + (int64_t)worker * level_bytes + base);
-        for (int k = threadIdx.x; k < n16; k += DAT_THREADS) dst[k] = s_level[k];
+        for (int k = lane; k < n16; k += 32) dst[k] = s_level[warp][k];
     }
     {
-        const int64_t base = tile * SIGN_TILE_BYTES;
-        const int64_t left = sign_bytes - base;
-        const int n16 = (int)((left < SIGN_TILE_BYTES ? left : SIGN_TILE_BYTES) / 16);
+        const int64_t bytes = n_warp / 8, base = part * bytes, left = sign_bytes - base;
+        const int n16 = (int)((left < bytes ? left : bytes) / 16);
         uint4 *dst = reinterpret_cast<uint4 *>(signs + (int64_t)worker * sign_bytes + base);
-        for (int k = threadIdx.x; k < n16; k += DAT_THREADS) dst[k] = s_sign[k];
+        for (int k = lane; k < n16; k += 32) dst[k] = s_sign[warp][k];
     }
+}
+
+// Levels of `n` vectors (workers of the plan's streams from `stream_base` on); scales_in as in dat_quantize.
+static int quantize_launch(dat_plan_t *plan, const GradPtrs &gp, int n, uint64_t seed, uint64_t step, uint8_t *levels, uint8_t *signs,
+                           float *scales, const float *scales_in, int n_scales, bool per_worker, uint32_t stream_base, cudaStream_t s)
+{
+    const PhiloxKeys keys = dat_make_keys(seed, step);
+    const int h = (int)plan->h;
+    const QuantScale qs = {plan->d_qmul, scales_in, scales, n_scales, (float)plan->S, plan->d_status};
+    // long runs per warp (the set-up is paid once) while there are four waves of CTAs; shorter ones for small problems
+    int groups = QUANT_GROUPS;
+    auto ctas = [&](int g) { return (plan->d + g * (int64_t)(8 * DAT_THREADS) - 1) / (g * (int64_t)(8 * DAT_THREADS)); };
+    while (groups > 2 && ctas(groups) * n < 4ll * QUANT_CTAS * plan->sm_count) groups /= 2;
+    dim3 grid((unsigned)ctas(groups), (unsigned)n);
+#define DAT_Q(B, R)                                                                                                              \
+    k_quantize<B, R><<<grid, DAT_THREADS, 0, s>>>(gp, keys, plan->d_offsets, plan->d_flat_layer, h, plan->d, qs, levels, signs, \
+                                                  plan->level_bytes, plan->sign_bytes, groups, per_worker, stream_base, plan->elem_base)
+#define DAT_QR(B) do { if (plan->rng_bits == 16) DAT_Q(B, true); else DAT_Q(B, false); } while (0)
+    switch (plan->bits) {
+    case 1: DAT_QR(1); break;
+    case 2: DAT_QR(2); break;
+    case 4: DAT_QR(4); break;
+    case 8: DAT_QR(8); break;
+    default: DAT_QR(16); break;
+    }
+#undef DAT_QR
+#undef DAT_Q
+    DAT_LAUNCHED(plan);
+    return DAT_OK;
 }
 
 extern "C" int dat_quantize(dat_plan_t *plan, const float *const *grads, uint64_t seed, uint64_t step,
@@ -197,40 +364,13 @@ extern "C" int dat_quantize(dat_plan_t *plan, const float *const *grads, uint64_
     if (rc != DAT_OK) return rc;
 
     cudaStream_t s = (cudaStream_t)stream;
-    const int h = (int)plan->h;
-    const float S_f = (float)plan->S;
     const bool per_worker = (plan->scale_mode == DAT_SCALE_PER_WORKER);
-    const int n_scales = per_worker ? h * plan->M : h;
-    if (scales_in) {
-        if (scales_in != scales)
-            DAT_CUDA(plan, cudaMemcpyAsync(scales, scales_in, (size_t)n_scales * 4, cudaMemcpyDeviceToDevice, s));
-        k_qmul_from_scales<<<(n_scales + 255) / 256, 256, 0, s>>>(n_scales, S_f, scales, plan->d_qmul, plan->d_status);
-        DAT_LAUNCHED(plan);
-    } else {
-        dim3 grid((unsigned)plan->n_tiles, (unsigned)plan->M);
-        k_sumsq_partial<<<grid, DAT_THREADS, 0, s>>>(gp, plan->d_offsets, plan->d_tile_base, h, plan->M,
-                                                     plan->d_partials);
-        DAT_LAUNCHED(plan);
-        k_scales_finalize<<<h, DAT_THREADS, 0, s>>>(plan->d_tile_base, h, plan->M, S_f, plan->d_partials,
-                                                    plan->d_worker_norms, scales, plan->d_qmul, plan->d_status, per_worker);
-        DAT_LAUNCHED(plan);
+    if (!scales_in) {
+        rc = sumsq_launch(plan, gp, plan->M, scales, per_worker, s);
+        if (rc != DAT_OK) return rc;
     }
-    const PhiloxKeys keys = dat_make_keys(seed, step);
-    const int64_t flat_tiles = (plan->d + DAT_TILE - 1) / DAT_TILE;
-    dim3 grid((unsigned)flat_tiles, (unsigned)plan->M);
-#define DAT_Q(B)                                                                                           \
-    k_quantize<B><<<grid, DAT_THREADS, 0, s>>>(gp, keys, plan->d_offsets, h, plan->d, plan->d_qmul, levels, \
-                                               signs, plan->level_bytes, plan->sign_bytes, plan->rng_bits == 16, per_worker, plan->worker_base, plan->elem_base)
-    switch (plan->bits) {
-    case 1: DAT_Q(1); break;
-    case 2: DAT_Q(2); break;
-    case 4: DAT_Q(4); break;
-    case 8: DAT_Q(8); break;
-    default: DAT_Q(16); break;
-    }
-#undef DAT_Q
-    DAT_LAUNCHED(plan);
-    return DAT_OK;
+    return quantize_launch(plan, gp, plan->M, seed, step, levels, signs, scales, scales_in, (int)(per_worker ? plan->h * plan->M : plan->h),
+                           per_worker, plan->worker_base, s);
 }
 
 // S1 by itself: the quantizer norm of every (worker, layer), nu_{i,l} = ||g_l^(i)||_2 (Eq. rand_q).
@@ -244,14 +384,9 @@ extern "C" int dat_worker_norms(dat_plan_t *plan, const float *const *grads, flo
     rc = dat_check_grads(plan, grads, &gp);
     if (rc != DAT_OK) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    const int h = (int)plan->h;
-    dim3 grid((unsigned)plan->n_tiles, (unsigned)plan->M);
-    k_sumsq_partial<<<grid, DAT_THREADS, 0, s>>>(gp, plan->d_offsets, plan->d_tile_base, h, plan->M, plan->d_partials);
-    DAT_LAUNCHED(plan);
-    k_scales_finalize<<<h, DAT_THREADS, 0, s>>>(plan->d_tile_base, h, plan->M, (float)plan->S, plan->d_partials,
-                                                plan->d_worker_norms, plan->d_scales, plan->d_qmul, plan->d_status, false);
-    DAT_LAUNCHED(plan);
-    DAT_CUDA(plan, cudaMemcpyAsync(norms_out, plan->d_worker_norms, (size_t)plan->M * h * 4, cudaMemcpyDeviceToDevice, s));
+    rc = sumsq_launch(plan, gp, plan->M, plan->d_scales, false, s);
+    if (rc != DAT_OK) return rc;
+    DAT_CUDA(plan, cudaMemcpyAsync(norms_out, plan->d_worker_norms, (size_t)plan->M * (size_t)plan->h * 4, cudaMemcpyDeviceToDevice, s));
     return DAT_OK;
 }
 
@@ -437,34 +572,18 @@ extern "C" int dat_requantize(dat_plan_t *plan, float *g_hat, uint64_t seed, uin
     cudaStream_t s = (cudaStream_t)stream;
     const int h = (int)plan->h;
     const float S_f = (float)plan->S;
-    if (scales_in) {
-        if (scales_in != scales)
-            DAT_CUDA(plan, cudaMemcpyAsync(scales, scales_in, (size_t)h * 4, cudaMemcpyDeviceToDevice, s));
-        k_qmul_from_scales<<<(h + 255) / 256, 256, 0, s>>>(h, S_f, scales, plan->d_qmul, plan->d_status);
-        DAT_LAUNCHED(plan);
-    } else {
-        dim3 grid((unsigned)plan->n_tiles, 1u);
-        k_sumsq_partial<<<grid, DAT_THREADS, 0, s>>>(gp, plan->d_offsets, plan->d_tile_base, h, 1, plan->d_partials);
-        DAT_LAUNCHED(plan);
-        k_scales_finalize<<<h, DAT_THREADS, 0, s>>>(plan->d_tile_base, h, 1, S_f, plan->d_partials,
-                                                    plan->d_worker_norms, scales, plan->d_qmul, plan->d_status, false);
-        DAT_LAUNCHED(plan);
+    if (!scales_in) {
+        rc = sumsq_launch(plan, gp, 1, scales, false, s);
+        if (rc != DAT_OK) return rc;
     }
-    const PhiloxKeys keys = dat_make_keys(seed, step);
-    const int64_t flat_tiles = (plan->d + DAT_TILE - 1) / DAT_TILE;
-    dim3 qgrid((unsigned)flat_tiles, 1u);
+    rc = quantize_launch(plan, gp, 1, seed, step, levels, signs, scales, scales_in, h, false, plan->worker_base + (uint32_t)plan->M, s);
+    if (rc != DAT_OK) return rc;
     const unsigned agrid = (unsigned)((plan->d + DAT_THREADS * 8 - 1) / (DAT_THREADS * 8));
     k_dq_from_scales<<<(h + 255) / 256, 256, 0, s>>>(h, S_f, scales, plan->d_dq);      // nu / (S * 1)
     DAT_LAUNCHED(plan);
 #define DAT_RQ(B)                                                                                                   \
-    do {                                                                                                            \
-        k_quantize<B><<<qgrid, DAT_THREADS, 0, s>>>(gp, keys, plan->d_offsets, h, plan->d, plan->d_qmul, levels,    \
-                                                    signs, plan->level_bytes, plan->sign_bytes,                     \
-                                                    plan->rng_bits == 16, false, plan->worker_base + (uint32_t)plan->M, plan->elem_base); \
-        DAT_LAUNCHED(plan);                                                                                         \
-        k_aggregate<B, PlanesFlat><<<agrid, DAT_THREADS, 0, s>>>(PlanesFlat{levels, signs, plan->level_bytes, plan->sign_bytes}, 1, \
-                                                                 plan->d_offsets, h, plan->d, plan->d_dq, nullptr, g_hat); \
-    } while (0)
+    k_aggregate<B, PlanesFlat><<<agrid, DAT_THREADS, 0, s>>>(PlanesFlat{levels, signs, plan->level_bytes, plan->sign_bytes}, 1, \
+                                                             plan->d_offsets, h, plan->d, plan->d_dq, nullptr, g_hat)
     switch (plan->bits) {
     case 1: DAT_RQ(1); break;
     case 2: DAT_RQ(2); break;
@@ -587,12 +706,11 @@ extern "C" int dat_average(dat_plan_t *plan, const float *const *grads, float *g
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(DAT_THREADS)
 k_lalr_pass1(const float *__restrict__ theta, float *__restrict__ mom, const float *__restrict__ g_hat,
-             const int64_t *__restrict__ off, const int64_t *__restrict__ tile_base, int h, float mu, float wd,
-             double *__restrict__ partials)
+             const TileSource tiles, float mu, float wd, double *__restrict__ partials)
 {
     __shared__ double scratch[DAT_THREADS / 32];
     const int64_t tile = blockIdx.x;
-    const TileRange r = dat_tile_range(off, tile_base, h, tile);
+    const TileRange r = dat_tile_range(tiles, tile);
     double ss_theta = 0.0, ss_u = 0.0;
 #pragma unroll
     for (int it = 0; it < DAT_TILE / 4 / DAT_THREADS; ++it) {
@@ -639,11 +757,10 @@ k_lalr_finalize(const int64_t *__restrict__ tile_base, const double *__restrict_
 }
 
 __global__ void __launch_bounds__(DAT_THREADS)
-k_lalr_pass2(float *__restrict__ theta, const float *__restrict__ mom, const int64_t *__restrict__ off,
-             const int64_t *__restrict__ tile_base, int h, const float *__restrict__ step_a)
+k_lalr_pass2(float *__restrict__ theta, const float *__restrict__ mom, const TileSource tiles, const float *__restrict__ step_a)
 {
     const int64_t tile = blockIdx.x;
-    const TileRange r = dat_tile_range(off, tile_base, h, tile);
+    const TileRange r = dat_tile_range(tiles, tile);
     const float na = -__ldg(step_a + r.layer);
 #pragma unroll
     for (int it = 0; it < DAT_TILE / 4 / DAT_THREADS; ++it) {
@@ -670,15 +787,13 @@ extern "C" int dat_lalr_step(dat_plan_t *plan, float *theta, float *mom, const f
         return DAT_ERR_ALIGN;
     cudaStream_t s = (cudaStream_t)stream;
     const int h = (int)plan->h;
-    k_lalr_pass1<<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(theta, mom, g_hat, plan->d_offsets,
-                                                                 plan->d_tile_base, h, hp->momentum,
+    k_lalr_pass1<<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(theta, mom, g_hat, plan_tiles(plan), hp->momentum,
                                                                  hp->weight_decay, plan->d_partials);
     DAT_LAUNCHED(plan);
     k_lalr_finalize<<<h, DAT_THREADS, 0, s>>>(plan->d_tile_base, plan->d_partials, hp->lr, hp->c_l, hp->c_u,
                                               plan->d_step_a, layer_norms_out, plan->d_status);
     DAT_LAUNCHED(plan);
-    k_lalr_pass2<<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(theta, mom, plan->d_offsets, plan->d_tile_base,
-                                                                 h, plan->d_step_a);
+    k_lalr_pass2<<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(theta, mom, plan_tiles(plan), plan->d_step_a);
     DAT_LAUNCHED(plan);
     return DAT_OK;
 }
@@ -691,12 +806,11 @@ extern "C" int dat_lalr_step(dat_plan_t *plan, float *theta, float *mom, const f
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(DAT_THREADS)
 k_lamb_pass1(const float *__restrict__ theta, float *__restrict__ mom, float *__restrict__ var,
-             const float *__restrict__ g_hat, const int64_t *__restrict__ off,
-             const int64_t *__restrict__ tile_base, int h, LambConst c, double *__restrict__ partials)
+             const float *__restrict__ g_hat, const TileSource tiles, LambConst c, double *__restrict__ partials)
 {
     __shared__ double scratch[DAT_THREADS / 32];
     const int64_t tile = blockIdx.x;
-    const TileRange r = dat_tile_range(off, tile_base, h, tile);
+    const TileRange r = dat_tile_range(tiles, tile);
     double ss_theta = 0.0, ss_u = 0.0;
 #pragma unroll
     for (int it = 0; it < DAT_TILE / 4 / DAT_THREADS; ++it) {
@@ -727,11 +841,10 @@ k_lamb_pass1(const float *__restrict__ theta, float *__restrict__ mom, float *__
 
 __global__ void __launch_bounds__(DAT_THREADS)
 k_lamb_pass2(float *__restrict__ theta, const float *__restrict__ mom, const float *__restrict__ var,
-             const int64_t *__restrict__ off, const int64_t *__restrict__ tile_base, int h, LambConst c,
-             const float *__restrict__ step_a)
+             const TileSource tiles, LambConst c, const float *__restrict__ step_a)
 {
     const int64_t tile = blockIdx.x;
-    const TileRange r = dat_tile_range(off, tile_base, h, tile);
+    const TileRange r = dat_tile_range(tiles, tile);
     const float na = -__ldg(step_a + r.layer);
 #pragma unroll
     for (int it = 0; it < DAT_TILE / 4 / DAT_THREADS; ++it) {
@@ -765,14 +878,12 @@ extern "C" int dat_lamb_step(dat_plan_t *plan, float *theta, float *mom, float *
     cudaStream_t s = (cudaStream_t)stream;
     const int h = (int)plan->h;
     const LambConst c = dat_lamb_const(hp, t);
-    k_lamb_pass1<<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(theta, mom, var, g_hat, plan->d_offsets,
-                                                                 plan->d_tile_base, h, c, plan->d_partials);
+    k_lamb_pass1<<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(theta, mom, var, g_hat, plan_tiles(plan), c, plan->d_partials);
     DAT_LAUNCHED(plan);
     k_lalr_finalize<<<h, DAT_THREADS, 0, s>>>(plan->d_tile_base, plan->d_partials, hp->lr, hp->c_l, hp->c_u,
                                               plan->d_step_a, layer_norms_out, plan->d_status);
     DAT_LAUNCHED(plan);
-    k_lamb_pass2<<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(theta, mom, var, plan->d_offsets,
-                                                                 plan->d_tile_base, h, c, plan->d_step_a);
+    k_lamb_pass2<<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(theta, mom, var, plan_tiles(plan), c, plan->d_step_a);
     DAT_LAUNCHED(plan);
     return DAT_OK;
 }
@@ -813,7 +924,7 @@ extern "C" int dat_lalr_step_static(int64_t num_layers, const int64_t *layer_off
     for (int64_t l = 0; l < num_layers; ++l) {
         if (layer_offsets[l + 1] <= layer_offsets[l]) return DAT_ERR_LAYOUT;
         tile_base[l] = nt;
-        const int64_t a = layer_offsets[l] & ~(int64_t)3;
+        const int64_t a = layer_offsets[l] & ~(int64_t)7;
         nt += (layer_offsets[l + 1] - a + DAT_TILE - 1) / DAT_TILE;
         if (nt > DAT_STATIC_MAX_TILES) return DAT_ERR_TOO_LARGE;
     }
@@ -843,11 +954,11 @@ extern "C" int dat_lalr_step_static(int64_t num_layers, const int64_t *layer_off
     if (e == cudaSuccess) e = cudaMemsetAsync(&sc->status, 0, sizeof(uint32_t), s);   // the one word that must start at zero
     if (e != cudaSuccess) { (void)cudaGetLastError(); return DAT_ERR_CUDA; }
     const int h = (int)num_layers;
-    k_lalr_pass1<<<(unsigned)nt, DAT_THREADS, 0, s>>>(theta, mom, g_hat, sc->off, sc->tile_base, h, hp->momentum,
-                                                      hp->weight_decay, sc->partials);
+    const TileSource tiles = {nullptr, sc->off, sc->tile_base, h};
+    k_lalr_pass1<<<(unsigned)nt, DAT_THREADS, 0, s>>>(theta, mom, g_hat, tiles, hp->momentum, hp->weight_decay, sc->partials);
     k_lalr_finalize<<<h, DAT_THREADS, 0, s>>>(sc->tile_base, sc->partials, hp->lr, hp->c_l, hp->c_u, sc->step_a,
                                               layer_norms_out, &sc->status);
-    k_lalr_pass2<<<(unsigned)nt, DAT_THREADS, 0, s>>>(theta, mom, sc->off, sc->tile_base, h, sc->step_a);
+    k_lalr_pass2<<<(unsigned)nt, DAT_THREADS, 0, s>>>(theta, mom, tiles, sc->step_a);
     if (cudaGetLastError() != cudaSuccess) return DAT_ERR_CUDA;
     return DAT_OK;
 }
@@ -861,16 +972,17 @@ extern "C" int dat_lalr_step_static(int64_t num_layers, const int64_t *layer_off
 // ------------------------------------------------------------------------------------------
 template <bool RNG16>
 __global__ void __launch_bounds__(DAT_QU_THREADS, DAT_QU_MINB)
-k_quant_update(const __grid_constant__ GradPtrs gp, const __grid_constant__ PhiloxKeys keys, const int64_t *__restrict__ off, const int64_t *__restrict__ tile_base8,
-               int h, int M, const float *__restrict__ qmul, const float *__restrict__ dq, const float *__restrict__ theta,
+k_quant_update(const __grid_constant__ GradPtrs gp, const __grid_constant__ PhiloxKeys keys, const TileSource tiles, int M,
+               const float *__restrict__ qmul, const float *__restrict__ dq, const float *__restrict__ theta,
                float *__restrict__ mom, float S_f, float mu, float wd, double *__restrict__ partials,
                int32_t *__restrict__ code_sum)
 {
+    static_assert(DAT_QU_TILE == DAT_TILE, "the plan's tiles");
     __shared__ double scratch[DAT_THREADS / 32];
     const int64_t tile = blockIdx.x;
-    const int layer = dat_find(tile_base8, h, tile);
-    const int64_t lo = __ldg(off + layer), hi = __ldg(off + layer + 1);
-    const int64_t begin = (lo & ~(int64_t)7) + (tile - __ldg(tile_base8 + layer)) * DAT_QU_TILE;
+    const TileRange r = dat_tile_range(tiles, tile);
+    const int layer = r.layer;
+    const int64_t lo = r.lo, hi = r.hi, begin = r.begin;
     const float t = __ldg(qmul + layer), f = __ldg(dq + layer);
     const float two_b = S_f + 1.0f, inv_two_b = 1.0f / two_b;
     // scaled form of Eq. xi (see dat_step.cu): valid while t 2^-b is a normal number
@@ -940,54 +1052,26 @@ extern "C" int dat_step_passes(dat_plan_t *plan, float *theta, float *mom, const
     rc = dat_check_grads(plan, grads, &gp);
     if (rc != DAT_OK) return rc;
     const int h = (int)plan->h;
-    if (!plan->d_tile_base8) {      // first call: the tiling of the second pass (synchronous)
-        std::vector<int64_t> tb((size_t)h + 1);
-        int64_t nt = 0;
-        for (int l = 0; l < h; ++l) {
-            tb[l] = nt;
-            nt += (plan->offsets[l + 1] - (plan->offsets[l] & ~(int64_t)7) + DAT_QU_TILE - 1) / DAT_QU_TILE;
-        }
-        tb[h] = nt;
-        cudaError_t e = cudaMalloc((void **)&plan->d_tile_base8, ((size_t)h + 1) * 8);
-        if (e == cudaSuccess) e = cudaMalloc((void **)&plan->d_partials8, (size_t)nt * 16);
-        if (e == cudaSuccess) e = cudaMemcpy(plan->d_tile_base8, tb.data(), ((size_t)h + 1) * 8, cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) {
-            if (plan->d_tile_base8) cudaFree(plan->d_tile_base8);
-            if (plan->d_partials8) cudaFree(plan->d_partials8);
-            plan->d_tile_base8 = nullptr;
-            plan->d_partials8 = nullptr;
-            plan->last_cuda = (int)e;
-            (void)cudaGetLastError();
-            return DAT_ERR_NOMEM;
-        }
-        plan->n_tiles8 = nt;
-    }
     cudaStream_t s = (cudaStream_t)stream;
     const float S_f = (float)plan->S;
     const float SM_f = (float)((uint64_t)plan->S * (uint64_t)plan->M);
-    dim3 ngrid((unsigned)plan->n_tiles, (unsigned)plan->M);
-    k_sumsq_partial<<<ngrid, DAT_THREADS, 0, s>>>(gp, plan->d_offsets, plan->d_tile_base, h, plan->M, plan->d_partials);
-    DAT_LAUNCHED(plan);
-    k_scales_finalize<<<h, DAT_THREADS, 0, s>>>(plan->d_tile_base, h, plan->M, S_f, plan->d_partials, plan->d_worker_norms,
-                                                plan->d_scales, plan->d_qmul, plan->d_status, false);
-    DAT_LAUNCHED(plan);
+    rc = sumsq_launch(plan, gp, plan->M, plan->d_scales, false, s);
+    if (rc != DAT_OK) return rc;
     k_dq_from_scales<<<(h + 255) / 256, 256, 0, s>>>(h, SM_f, plan->d_scales, plan->d_dq);
     DAT_LAUNCHED(plan);
     if (scales_out) DAT_CUDA(plan, cudaMemcpyAsync(scales_out, plan->d_scales, (size_t)h * 4, cudaMemcpyDeviceToDevice, s));
     const PhiloxKeys keys = dat_make_keys(seed, step);
     if (plan->rng_bits == 16)
-        k_quant_update<true><<<(unsigned)plan->n_tiles8, DAT_QU_THREADS, 0, s>>>(gp, keys, plan->d_offsets, plan->d_tile_base8, h, plan->M,
-                                                                                 plan->d_qmul, plan->d_dq, theta, mom, S_f, hp->momentum,
-                                                                                 hp->weight_decay, plan->d_partials8, code_sum_out);
+        k_quant_update<true><<<(unsigned)plan->n_tiles, DAT_QU_THREADS, 0, s>>>(gp, keys, plan_tiles(plan), plan->M, plan->d_qmul, plan->d_dq, theta, mom, S_f, hp->momentum,
+                                                                                 hp->weight_decay, plan->d_partials, code_sum_out);
     else
-        k_quant_update<false><<<(unsigned)plan->n_tiles8, DAT_QU_THREADS, 0, s>>>(gp, keys, plan->d_offsets, plan->d_tile_base8, h, plan->M,
-                                                                                  plan->d_qmul, plan->d_dq, theta, mom, S_f, hp->momentum,
-                                                                                  hp->weight_decay, plan->d_partials8, code_sum_out);
+        k_quant_update<false><<<(unsigned)plan->n_tiles, DAT_QU_THREADS, 0, s>>>(gp, keys, plan_tiles(plan), plan->M, plan->d_qmul, plan->d_dq, theta, mom, S_f, hp->momentum,
+                                                                                  hp->weight_decay, plan->d_partials, code_sum_out);
     DAT_LAUNCHED(plan);
-    k_lalr_finalize<<<h, DAT_THREADS, 0, s>>>(plan->d_tile_base8, plan->d_partials8, hp->lr, hp->c_l, hp->c_u, plan->d_step_a,
+    k_lalr_finalize<<<h, DAT_THREADS, 0, s>>>(plan->d_tile_base, plan->d_partials, hp->lr, hp->c_l, hp->c_u, plan->d_step_a,
                                               layer_norms_out, plan->d_status);
     DAT_LAUNCHED(plan);
-    k_lalr_pass2<<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(theta, mom, plan->d_offsets, plan->d_tile_base, h, plan->d_step_a);
+    k_lalr_pass2<<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(theta, mom, plan_tiles(plan), plan->d_step_a);
     DAT_LAUNCHED(plan);
     return DAT_OK;
 }
