@@ -84,7 +84,10 @@ int dat_check_plan(dat_plan_t *plan);                       // device current, n
 int dat_cuda_fail(dat_plan_t *plan, cudaError_t e);          // records e, returns DAT_ERR_CUDA
 bool dat_aligned16(const void *p);
 int dat_check_grads(const dat_plan_t *plan, const float *const *grads, GradPtrs *out);
+bool dat_grads_wide(const dat_plan_t *plan, const float *const *grads);   // every buffer on a 32-byte boundary
 PhiloxKeys dat_make_keys(uint64_t seed, uint64_t step);
+struct PhiloxWorkers;
+void dat_make_worker_table(const PhiloxKeys &keys, int M, PhiloxWorkers *out);
 int dat_pipe_build(dat_plan_t *plan);                        // dat_pipeline.cu (device current)
 void dat_pipe_destroy(dat_plan_t *plan);
 cudaError_t dat_pipe_reset(dat_plan_t *plan, cudaStream_t s);
@@ -414,24 +417,51 @@ __device__ __forceinline__ float4 dat_ld4_hint(const float *p, uint64_t pol)
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p), "l"(pol));
     return v;
 }
-// Eight consecutive floats of a stream that is read once.  sm_100 has 32-byte loads; they want a 32-byte boundary, which
-// a 16-byte aligned buffer may not have (wide: the buffer does; e0 is a multiple of 8).
-__device__ __forceinline__ void dat_ld8_stream(const float *p, bool wide, float v[8])
-{
-    if (wide) {
-        asm volatile("ld.global.L1::no_allocate.L2::evict_first.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "l"(p));
-    } else {
-        const float4 a = __ldcs(reinterpret_cast<const float4 *>(p)), b = __ldcs(reinterpret_cast<const float4 *>(p) + 1);
-        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-    }
-}
-__device__ __forceinline__ bool dat_aligned32(const void *p) { return ((uintptr_t)p & 31u) == 0; }
 __device__ __forceinline__ void dat_st4_hint(float *p, float4 v, uint64_t pol)
 {
     asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1,%2,%3,%4}, %5;"
                  :: "l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "l"(pol) : "memory");
 }
+
+// Eight consecutive floats past L1 with an L2 eviction priority.  sm_100 has 32-byte loads and stores: half the
+// instructions of two 16-byte ones, and no sector is asked for twice.  They want a 32-byte boundary, which a 16-byte
+// aligned buffer may not have (wide: the buffers do; element indices are multiples of 8).
+enum { EV_NORMAL = 0, EV_FIRST = 1, EV_LAST = 2 };
+template <int EV> __device__ __forceinline__ uint64_t dat_policy()
+{
+    return EV == EV_FIRST ? dat_policy_evict_first() : EV == EV_LAST ? dat_policy_evict_last() : dat_policy_evict_normal();
+}
+#define DAT_LD8(Q)                                                                                                          \
+    asm volatile("ld.global.L1::no_allocate" Q ".v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"                                   \
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "l"(p))
+#define DAT_ST8(Q)                                                                                                          \
+    asm volatile("st.global" Q ".v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"                                                   \
+                 :: "l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory")
+template <int EV> __device__ __forceinline__ void dat_ld8(const float *p, bool wide, float v[8])
+{
+    if (wide) {
+        if (EV == EV_FIRST) DAT_LD8(".L2::evict_first");
+        else if (EV == EV_LAST) DAT_LD8(".L2::evict_last");
+        else DAT_LD8("");
+    } else {
+        const float4 a = dat_ld4_hint(p, dat_policy<EV>()), b = dat_ld4_hint(p + 4, dat_policy<EV>());
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    }
+}
+template <int EV> __device__ __forceinline__ void dat_st8(float *p, bool wide, const float v[8])
+{
+    if (wide) {
+        if (EV == EV_FIRST) DAT_ST8(".L2::evict_first");
+        else if (EV == EV_LAST) DAT_ST8(".L2::evict_last");
+        else DAT_ST8("");
+    } else {
+        dat_st4_hint(p, make_float4(v[0], v[1], v[2], v[3]), dat_policy<EV>());
+        dat_st4_hint(p + 4, make_float4(v[4], v[5], v[6], v[7]), dat_policy<EV>());
+    }
+}
+#undef DAT_LD8
+#undef DAT_ST8
+__device__ __forceinline__ bool dat_aligned32(const void *p) { return ((uintptr_t)p & 31u) == 0; }
 
 // ------------------------------------------------------------------------------------------
 // Levels and signed sum over the workers for one thread's group of eight consecutive elements
@@ -452,68 +482,80 @@ __device__ __forceinline__ void dat_st4_hint(float *p, float4 v, uint64_t pol)
 #define DAT_QU_UNROLL_N(n) DAT_QU_PRAGMA(unroll n)
 
 struct QuConst {
-    float t, ts, two_b, c0, c1;
-    uint32_t ubits;
+    float t, ts, two_b, inv_two_b, den_b;         // S/nu_l, S/nu_l 2^-b, 2^b, 2^-b, 2^(b-149)
+    uint32_t ubits;                               // the bits of 2^-b
+    bool wide;
+};
+__device__ __forceinline__ QuConst dat_qu_const(float t, float S_f, bool wide)
+{
+    const float two_b = S_f + 1.0f, inv_two_b = 1.0f / two_b;
+    return QuConst{t, t * inv_two_b, two_b, inv_two_b, two_b * __uint_as_float(1u), __float_as_uint(inv_two_b), wide};
+}
+// Outside the scaled form's range (valid while t 2^-b is a normal number), or beyond the counters of the worker table.
+template <bool RNG16>
+__device__ __forceinline__ bool dat_qu_plain(const QuConst &q, int64_t begin, int64_t n)
+{
+    return (q.t != 0.0f && !(q.t >= 1.17549435e-38f * q.two_b && q.t <= 3.402823466e38f)) || ((begin + n) >> (RNG16 ? 35 : 34)) != 0;
+}
+
+// The worker-dependent products of the Philox blocks (counter word q_hi = 0), formed on the host per call.
+struct PhiloxWorkers {
+    PhiloxWorker w[DAT_MAX_WORKERS + 1];          // the last: the server's stream (index M) of the two-sided step
 };
 
-// The M gradient rows of one group of eight elements: levels and signed sum.  FULL: the group lies
-// inside the layer (16-byte loads); PLAIN: the layer's scale is outside the range of the scaled
-// form.  The common case (FULL, not PLAIN) is inlined, the others are calls.
-template <bool RNG16, bool FULL, bool PLAIN>
-__device__ __forceinline__ void qu_rows_body(const GradPtrs &gp, const PhiloxKeys &keys, const QuConst &qc, int M, int64_t e0,
-                                             int64_t lo, int64_t hi, float acc[8])
+// The M gradient rows of one group of eight elements: levels and signed sum.
+//
+// Scaled form (S + 1 = 2^b): y = sat(fma(|g|, t 2^-b, (1 + u) 2^-b)) is min(fma(|g|, t, 1 + u), S + 1) 2^-b exactly, and
+// one fma towards zero onto the grid of the denormal numbers, y 2^(b-149) - 2^-149, truncates to level 2^-149: the sums
+// are then exact sums of denormal numbers (|sum| < 2^23 units), brought back by an exact scaling at the end.  Per
+// element: one DP2A for (1 + u) 2^-b, three fused multiply-adds and one LOP3 for the sign.  The issue-limited time of
+// this loop per group and worker went from 165 to about 115 cycles per scheduler (both multiply pipe and ALU full).
+template <bool RNG16>
+__device__ __forceinline__ void qu_rows(const GradPtrs &gp, const PhiloxKeys &keys, const PhiloxWorkers &pw, const QuConst &qc, int M, int64_t e0, float acc[8])
 {
-#ifndef DAT_QU_POLICY
-#define DAT_QU_POLICY dat_policy_evict_first
-#endif
-    const uint64_t pol = DAT_QU_POLICY();             // a gradient is dead once its level is drawn
+    const PhiloxGroup<RNG16> pg = dat_philox_group<RNG16>((uint64_t)e0, keys);
     DAT_QU_UNROLL_N(DAT_QU_UNROLL)
     for (int i = 0; i < M; ++i) {
         float v[8];
-        if (FULL) {
-            const float4 a0 = dat_ld4_hint(gp.p[i] + e0, pol), a1 = dat_ld4_hint(gp.p[i] + e0 + 4, pol);
-            v[0] = a0.x; v[1] = a0.y; v[2] = a0.z; v[3] = a0.w; v[4] = a1.x; v[5] = a1.y; v[6] = a1.z; v[7] = a1.w;
-        } else {
-            dat_load4(gp.p[i], e0, lo, hi, v);
-            dat_load4(gp.p[i], e0 + 4, lo, hi, v + 4);
-        }
+        dat_ld8<EV_FIRST>(gp.p[i] + e0, qc.wide, v);         // a gradient is dead once its level is drawn
         uint32_t w[8];
-        if (RNG16) {
-            dat_random_words((uint64_t)e0 >> 3, (uint32_t)i, keys, w);
-        } else {
-            dat_random_words((uint64_t)e0 >> 2, (uint32_t)i, keys, w);
-            dat_random_words(((uint64_t)e0 >> 2) + 1, (uint32_t)i, keys, w + 4);
-        }
+        dat_group_words<RNG16>(pg, pw.w[i], keys, w);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            if (!PLAIN) {
-                float u1s;
-                if (RNG16) u1s = __fmaf_rn(__uint_as_float(__byte_perm(w[j >> 1], 0x4B000000u, (j & 1) ? 0x7632 : 0x7610)), qc.c0, qc.c1);
-                else u1s = __uint_as_float(qc.ubits | (w[j] & 0x007FFFFFu));
-                const float ys = __saturatef(__fmaf_rn(fabsf(v[j]), qc.ts, u1s));
-                const float lf = __fmaf_rz(ys, qc.two_b, 8388607.0f) - 8388608.0f;
-                const float sg = __uint_as_float((__float_as_uint(v[j]) & 0x80000000u) | 0x3F800000u);
-                acc[j] = __fmaf_rn(lf, sg, acc[j]);
-            } else {
-                const float u1 = RNG16 ? dat_u1_from_half((j & 1) ? (w[j >> 1] >> 16) : (w[j >> 1] & 0xFFFFu)) : dat_u1_from_word(w[j]);
-                const float lf = (float)dat_level_u1(v[j], qc.t, qc.two_b, u1);
-                acc[j] += (v[j] < 0.0f) ? -lf : lf;
-            }
+            const float ys = __saturatef(__fmaf_rn(fabsf(v[j]), qc.ts, dat_u1_scaled<RNG16>(w, j, qc.ubits)));
+            const float lev = __fmaf_rz(ys, qc.den_b, __uint_as_float(0x80000001u));
+            const float sg = __uint_as_float((__float_as_uint(v[j]) & 0x80000000u) | 0x3F800000u);
+            acc[j] = __fmaf_rn(lev, sg, acc[j]);
         }
     }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[j] = (acc[j] * 0x1p100f) * 0x1p49f;
 }
-template <bool RNG16, bool FULL, bool PLAIN>
-__device__ __noinline__ void qu_rows_call(const GradPtrs &gp, const PhiloxKeys &keys, const QuConst &qc, int M, int64_t e0,
-                                          int64_t lo, int64_t hi, float acc[8])
+
+// The same by the plain form of Eq. xi with whole Philox blocks, for a group at a layer's ragged ends or outside the
+// scaled form's range (same integers).  Sums in units of one level, four at a time (the call passes no array).
+template <bool RNG16>
+__device__ __noinline__ float4 qu_rows_slow4(const GradPtrs &gp, const PhiloxKeys &keys, float t, float two_b, int M, int64_t e0, int64_t lo, int64_t hi)
 {
-    qu_rows_body<RNG16, FULL, PLAIN>(gp, keys, qc, M, e0, lo, hi, acc);
+    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 1
+    for (int i = 0; i < M; ++i) {
+        float v[4], u1[4];
+        dat_load4(gp.p[i], e0, lo, hi, v);
+        dat_u1x4((uint64_t)e0, (uint32_t)i, keys, RNG16, u1);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float lf = (float)dat_level_u1(v[j], t, two_b, u1[j]);
+            acc[j] += (v[j] < 0.0f) ? -lf : lf;
+        }
+    }
+    return make_float4(acc[0], acc[1], acc[2], acc[3]);
 }
-template <bool RNG16, bool FULL, bool PLAIN>
-__device__ __forceinline__ void qu_rows(const GradPtrs &gp, const PhiloxKeys &keys, const QuConst &qc, int M, int64_t e0,
-                                        int64_t lo, int64_t hi, float acc[8])
+template <bool RNG16>
+__device__ __forceinline__ void qu_rows_slow(const GradPtrs &gp, const PhiloxKeys &keys, const QuConst &qc, int M, int64_t e0, int64_t lo, int64_t hi, float acc[8])
 {
-    if (FULL && !PLAIN) qu_rows_body<RNG16, FULL, PLAIN>(gp, keys, qc, M, e0, lo, hi, acc);
-    else qu_rows_call<RNG16, FULL, PLAIN>(gp, keys, qc, M, e0, lo, hi, acc);
+    const float4 a = qu_rows_slow4<RNG16>(gp, keys, qc.t, qc.two_b, M, e0, lo, hi), b = qu_rows_slow4<RNG16>(gp, keys, qc.t, qc.two_b, M, e0 + 4, lo, hi);
+    acc[0] = a.x; acc[1] = a.y; acc[2] = a.z; acc[3] = a.w; acc[4] = b.x; acc[5] = b.y; acc[6] = b.z; acc[7] = b.w;
 }
 
 #endif  // __CUDACC__

@@ -89,6 +89,7 @@ struct PipeSchedule {
 struct PArgs {
     GradPtrs gp;
     PhiloxKeys keys;
+    PhiloxWorkers workers;
     const PipeItem *items;
     const int64_t *off, *tile_base;
     float *theta, *mom, *var;                     // var: second moment (LAMB only)
@@ -103,6 +104,7 @@ struct PArgs {
     float S_f, SM_f, M_f, mu, wd, lr, c_l, c_u;
     uint32_t epoch, n_items;
     int M, h;
+    bool wide;                                    // every bulk buffer starts on a 32-byte boundary
     int64_t d, n_tiles;
 };
 
@@ -130,23 +132,23 @@ __device__ __forceinline__ void p_load4_cg(const float *__restrict__ p, int64_t 
     }
 }
 
-// Eight consecutive elements with an L2 eviction hint: two 16-byte accesses where the group lies inside the
-// layer, element accesses (no hint) at a layer's ragged ends.
-__device__ __forceinline__ void p_ld8(const float *p, int64_t e0, int64_t lo, int64_t hi, float v[8], uint64_t pol)
+// Eight consecutive elements with an L2 eviction priority where the group lies inside the layer, element accesses
+// (no priority) at a layer's ragged ends.
+template <int EV>
+__device__ __forceinline__ void p_ld8(const float *p, bool wide, int64_t e0, int64_t lo, int64_t hi, float v[8])
 {
     if (e0 >= lo && e0 + 8 <= hi) {
-        const float4 x = dat_ld4_hint(p + e0, pol), y = dat_ld4_hint(p + e0 + 4, pol);
-        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w; v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+        dat_ld8<EV>(p + e0, wide, v);
     } else {
         p_load4_cg(p, e0, lo, hi, v);
         p_load4_cg(p, e0 + 4, lo, hi, v + 4);
     }
 }
-__device__ __forceinline__ void p_st8(float *p, int64_t e0, int64_t lo, int64_t hi, const float v[8], uint64_t pol)
+template <int EV>
+__device__ __forceinline__ void p_st8(float *p, bool wide, int64_t e0, int64_t lo, int64_t hi, const float v[8])
 {
     if (e0 >= lo && e0 + 8 <= hi) {
-        dat_st4_hint(p + e0, make_float4(v[0], v[1], v[2], v[3]), pol);
-        dat_st4_hint(p + e0 + 4, make_float4(v[4], v[5], v[6], v[7]), pol);
+        dat_st8<EV>(p + e0, wide, v);
     } else {
         dat_store4(p, e0, lo, hi, v);
         dat_store4(p, e0 + 4, lo, hi, v + 4);
@@ -192,13 +194,49 @@ __device__ __forceinline__ bool p_tile_inside(const PipePart &pt)
 
 // ---- N: sums of squares of one tile, every worker ------------------------------------------------
 // A tile is cut into 4M units (worker, quarter tile); warp w of W takes the units [w*4M/W, (w+1)*4M/W),
-// lane j the 16-byte pieces j, j+32, ... of a unit, eight pieces in flight.  Units of the same worker
+// lane j the 32-byte pieces j, j+32, ... of a unit, four pieces in flight.  Units of the same worker
 // are summed per lane before the warp reduction; the structure depends on M only, so the sums are the
 // same from run to run.  Leaves one sum per run of units in s_unit (zero elsewhere).
+template <int EV>
+__device__ __forceinline__ void p_norm_units(const PArgs &a, int64_t begin, int u0, int u1, int &run, double &acc, double *s_unit)
+{
+    constexpr int QUARTER = DAT_P_TILE / 4, LPU = QUARTER / 256, UPB = 4 / LPU;   // units per batch of 4 loads
+    static_assert(LPU >= 1 && LPU <= 4 && UPB * LPU == 4, "quarter tiles of 256 .. 1024 elements");
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int ub = u0; ub < u1; ub += UPB) {
+        float v[4][8];
+#pragma unroll
+        for (int k = 0; k < UPB; ++k) {
+            const int u = ub + k;
+            if (u < u1) {
+                const float *g = a.gp.p[u >> 2] + begin + (u & 3) * QUARTER + 8 * lane;
+#pragma unroll
+                for (int b = 0; b < LPU; ++b) dat_ld8<EV>(g + 256 * b, a.wide, v[k * LPU + b]);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < UPB; ++k) {
+            const int u = ub + k;
+            if (u < u1) {
+                if ((u >> 2) != (run >> 2)) {
+                    acc = dat_warp_sum(acc);
+                    if (lane == 0) s_unit[run] = acc;
+                    acc = 0.0;
+                    run = u;
+                }
+#pragma unroll
+                for (int b = 0; b < LPU; ++b)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) acc = fma((double)v[k * LPU + b][j], (double)v[k * LPU + b][j], acc);
+            }
+        }
+    }
+}
+
 __device__ __forceinline__ void p_norm_sums(const PArgs &a, const PipePart &pt, double *s_unit)
 {
-    constexpr int W = DAT_P_THREADS / 32, QUARTER = DAT_P_TILE / 4, LPU = QUARTER / 128, UPB = 8 / LPU;   // units per batch of 8 loads
-    static_assert(LPU >= 1 && LPU <= 8 && UPB * LPU == 8, "quarter tiles of 128 .. 1024 elements");
+    constexpr int W = DAT_P_THREADS / 32, QUARTER = DAT_P_TILE / 4;
     const int M = a.M;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int U = 4 * M;
@@ -207,46 +245,11 @@ __device__ __forceinline__ void p_norm_sums(const PArgs &a, const PipePart &pt, 
     double acc = 0.0;
     int run = u0;
     if (p_tile_inside(pt)) {
-#ifndef DAT_P_N_POLICY
-#define DAT_P_N_POLICY dat_policy_evict_first
-#endif
         // A small layer's lines are still in L2 when the Q part of a later item reads them again, and so are those of
         // a larger layer's last tiles, which the Q stream (walking back from the last tile) reads first; the rest of a
         // large layer is gone by then anyway: better it leaves first than push out those lines, theta and m'.
-        const uint64_t pol = (pt.T <= DAT_P_KEEP_T || pt.tile >= pt.T - DAT_P_KEEP_TAIL) ? dat_policy_evict_normal() : DAT_P_N_POLICY();
-#pragma unroll 1
-        for (int ub = u0; ub < u1; ub += UPB) {
-            float4 v[8];
-#pragma unroll
-            for (int k = 0; k < UPB; ++k) {
-                const int u = ub + k;
-                if (u < u1) {
-                    const float *g = a.gp.p[u >> 2] + begin + (u & 3) * QUARTER + 4 * lane;
-#pragma unroll
-                    for (int b = 0; b < LPU; ++b) v[k * LPU + b] = dat_ld4_hint(g + 128 * b, pol);
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < UPB; ++k) {
-                const int u = ub + k;
-                if (u < u1) {
-                    if ((u >> 2) != (run >> 2)) {
-                        acc = dat_warp_sum(acc);
-                        if (lane == 0) s_unit[run] = acc;
-                        acc = 0.0;
-                        run = u;
-                    }
-#pragma unroll
-                    for (int b = 0; b < LPU; ++b) {
-                        const float4 x = v[k * LPU + b];
-                        acc = fma((double)x.x, (double)x.x, acc);
-                        acc = fma((double)x.y, (double)x.y, acc);
-                        acc = fma((double)x.z, (double)x.z, acc);
-                        acc = fma((double)x.w, (double)x.w, acc);
-                    }
-                }
-            }
-        }
+        if (pt.T <= DAT_P_KEEP_T || pt.tile >= pt.T - DAT_P_KEEP_TAIL) p_norm_units<EV_NORMAL>(a, begin, u0, u1, run, acc, s_unit);
+        else p_norm_units<EV_FIRST>(a, begin, u0, u1, run, acc, s_unit);
     } else {
 #pragma unroll 1
         for (int u = u0; u < u1; ++u) {
@@ -257,11 +260,11 @@ __device__ __forceinline__ void p_norm_sums(const PArgs &a, const PipePart &pt, 
                 run = u;
             }
             const float *__restrict__ g = a.gp.p[u >> 2];
-            const int64_t e = begin + (u & 3) * QUARTER + 4 * lane;
 #pragma unroll
-            for (int b = 0; b < LPU; ++b) {
+            for (int b = 0; b < QUARTER / 128; ++b) {
+                const int64_t e = begin + (u & 3) * QUARTER + 4 * lane + 128 * b;
                 float t[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-                if (e + 128 * b < pt.hi) dat_load4(g, e + 128 * b, pt.lo, pt.hi, t);
+                if (e < pt.hi) dat_load4(g, e, pt.lo, pt.hi, t);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) acc = fma((double)t[k], (double)t[k], acc);
             }
@@ -282,14 +285,8 @@ __device__ __forceinline__ bool p_norm_publish(const PArgs &a, const PipePart &p
         const double *s = s_unit + 4 * i;
         a.partN[((int64_t)pt.tb + pt.tile) * M + i] = ((s[0] + s[1]) + s[2]) + s[3];
     }
-    __threadfence();
     __syncwarp();
-    bool last = false;
-    if (lane == 0) {
-        __threadfence();
-        last = (atomicAdd(a.cntN + pt.layer, 1u) == (uint32_t)pt.T - 1u);
-    }
-    return last;
+    return lane == 0 && dat_count_in(a.cntN + pt.layer, (uint32_t)pt.T);
 }
 
 // The CTA that counted in the layer's last N tile (every thread): nu_{i,l} = sqrt(sum over the tiles),
@@ -301,7 +298,6 @@ __device__ __forceinline__ void p_norm_finish(const PArgs &a, const PipePart &pt
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t tb = pt.tb;
     const uint32_t T = (uint32_t)pt.T;
-    __threadfence();
     for (int i = warp; i < M; i += DAT_P_THREADS / 32) {
         double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
         uint32_t t = lane;
@@ -340,7 +336,6 @@ __device__ __forceinline__ void p_norm_finish(const PArgs &a, const PipePart &pt
         }
         if (bad) atomicOr(a.status, DAT_STATUS_NONFINITE);
         a.cntN[layer] = 0u;
-        __threadfence();
         p_st_release(a.readyN + layer, a.epoch);
     }
 }
@@ -352,7 +347,6 @@ __device__ __forceinline__ void p_quant_finish(const PArgs &a, const PipePart &p
     const int layer = pt.layer;
     const int64_t tb = pt.tb;
     const uint32_t T = (uint32_t)pt.T;
-    __threadfence();
     double x = 0.0, y = 0.0;
     for (uint32_t t = threadIdx.x; t < T; t += DAT_P_THREADS) {
         x += __ldcg(a.partQ + 2 * (tb + t));
@@ -374,43 +368,54 @@ __device__ __forceinline__ void p_quant_finish(const PArgs &a, const PipePart &p
         if (a.norms_out) { a.norms_out[2 * layer] = n_theta; a.norms_out[2 * layer + 1] = n_u; }
         if (!isfinite(n_theta) || !isfinite(n_u)) atomicOr(a.status, DAT_STATUS_NONFINITE);
         a.cntQ[layer] = 0u;
-        __threadfence();
         p_st_release(a.readyQ + layer, a.epoch);
     }
 }
 
 // Eq. grad_agg as written, every worker on its own grid: acc = sum_i nu_{i,l} * (signed level_i), in fp32
-// with one fused multiply-add per worker, ascending; the caller divides by S*M.  Levels by the plain form
-// of Eq. xi with the worker's own S/nu_{i,l}.
+// with one fused multiply-add per worker, ascending; the caller divides by S*M.  Levels by the scaled form (see
+// qu_rows) with the worker's own S/nu_{i,l}; by the plain form of Eq. xi at a layer's ragged ends and where the scaled
+// form does not apply to some worker (one path for all workers of a group: the sum is ordered).
 template <bool RNG16>
-__device__ __forceinline__ void p_rows_per_worker(const PArgs &a, int layer, int64_t e0, int64_t lo, int64_t hi, float acc[8])
+__device__ __noinline__ float4 p_rows_per_worker_slow4(const PArgs &a, const float2 *s_fac, int64_t e0, int64_t lo, int64_t hi)
 {
-    const bool full = (e0 >= lo && e0 + 8 <= hi);
-    const uint64_t pol = dat_policy_evict_first();
-    const float two_b = a.S_f + 1.0f;
+    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll 1
     for (int i = 0; i < a.M; ++i) {
+        float v[4], u1[4];
+        dat_load4(a.gp.p[i], e0, lo, hi, v);
+        dat_u1x4((uint64_t)e0, (uint32_t)i, a.keys, RNG16, u1);
+        const float2 fac = s_fac[i];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float lf = (float)dat_level_u1(v[j], fac.x, a.S_f + 1.0f, u1[j]);
+            acc[j] = __fmaf_rn(fac.y, (v[j] < 0.0f) ? -lf : lf, acc[j]);
+        }
+    }
+    return make_float4(acc[0], acc[1], acc[2], acc[3]);
+}
+template <bool RNG16>
+__device__ __forceinline__ void p_rows_per_worker(const PArgs &a, const QuConst &qc, const float2 *s_fac, bool fast, int64_t e0, int64_t lo, int64_t hi, float acc[8])
+{
+    if (!fast) {
+        const float4 x = p_rows_per_worker_slow4<RNG16>(a, s_fac, e0, lo, hi), y = p_rows_per_worker_slow4<RNG16>(a, s_fac, e0 + 4, lo, hi);
+        acc[0] = x.x; acc[1] = x.y; acc[2] = x.z; acc[3] = x.w; acc[4] = y.x; acc[5] = y.y; acc[6] = y.z; acc[7] = y.w;
+        return;
+    }
+    const PhiloxGroup<RNG16> pg = dat_philox_group<RNG16>((uint64_t)e0, a.keys);
+#pragma unroll 2
+    for (int i = 0; i < a.M; ++i) {
         float v[8];
-        if (full) {
-            const float4 a0 = dat_ld4_hint(a.gp.p[i] + e0, pol), a1 = dat_ld4_hint(a.gp.p[i] + e0 + 4, pol);
-            v[0] = a0.x; v[1] = a0.y; v[2] = a0.z; v[3] = a0.w; v[4] = a1.x; v[5] = a1.y; v[6] = a1.z; v[7] = a1.w;
-        } else {
-            dat_load4(a.gp.p[i], e0, lo, hi, v);
-            dat_load4(a.gp.p[i], e0 + 4, lo, hi, v + 4);
-        }
-        const float t = __ldcg(a.qmul + (int64_t)i * a.h + layer), nu = __ldcg(a.worker_norms + (int64_t)i * a.h + layer);
+        dat_ld8<EV_FIRST>(a.gp.p[i] + e0, a.wide, v);
+        const float2 fac = s_fac[i];                // S/nu_{i,l} and nu_{i,l}
+        const float ts = fac.x * qc.inv_two_b;
         uint32_t w[8];
-        if (RNG16) {
-            dat_random_words((uint64_t)e0 >> 3, (uint32_t)i, a.keys, w);
-        } else {
-            dat_random_words((uint64_t)e0 >> 2, (uint32_t)i, a.keys, w);
-            dat_random_words(((uint64_t)e0 >> 2) + 1, (uint32_t)i, a.keys, w + 4);
-        }
+        dat_group_words<RNG16>(pg, a.workers.w[i], a.keys, w);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const float u1 = RNG16 ? dat_u1_from_half((j & 1) ? (w[j >> 1] >> 16) : (w[j >> 1] & 0xFFFFu)) : dat_u1_from_word(w[j]);
-            const float lf = (float)dat_level_u1(v[j], t, two_b, u1);
-            acc[j] = __fmaf_rn(nu, (v[j] < 0.0f) ? -lf : lf, acc[j]);
+            const float ys = __saturatef(__fmaf_rn(fabsf(v[j]), ts, dat_u1_scaled<RNG16>(w, j, qc.ubits)));
+            const float lf = __fmaf_rz(ys, qc.two_b, 8388607.0f) - 8388608.0f;
+            acc[j] = __fmaf_rn(__uint_as_float((__float_as_uint(v[j]) & 0x80000000u) | __float_as_uint(fac.y)), lf, acc[j]);
         }
     }
 }
@@ -422,14 +427,13 @@ __device__ __forceinline__ void p_direction(const PArgs &a, int64_t e0, int64_t 
                                             double &ss_theta, double &ss_u)
 {
     // what the U part reads again (theta, m', v') is kept in L2 (evict-last); the old m is dead (evict-first)
-    const uint64_t keep = dat_policy_evict_last();
     float th[8], m[8];
-    p_ld8(a.theta, e0, lo, hi, th, keep);
-    p_ld8(a.mom, e0, lo, hi, m, dat_policy_evict_first());
+    p_ld8<EV_LAST>(a.theta, a.wide, e0, lo, hi, th);
+    p_ld8<EV_FIRST>(a.mom, a.wide, e0, lo, hi, m);
     if (OPT == P_OPT_LAMB) {
         // Algorithm A2: both moments are stored, the direction is formed on the fly for the layer sums
         float v[8];
-        p_ld8(a.var, e0, lo, hi, v, keep);
+        p_ld8<EV_LAST>(a.var, a.wide, e0, lo, hi, v);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             m[j] = __fmaf_rn(a.lamb.beta1, m[j], __fmul_rn(a.lamb.om1, ghat[j]));
@@ -439,7 +443,7 @@ __device__ __forceinline__ void p_direction(const PArgs &a, int64_t e0, int64_t 
             ss_theta = fma((double)th[j], (double)th[j], ss_theta);
             ss_u = fma((double)u, (double)u, ss_u);
         }
-        p_st8(a.var, e0, lo, hi, v, keep);
+        p_st8<EV_LAST>(a.var, a.wide, e0, lo, hi, v);
     } else {
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
@@ -448,7 +452,7 @@ __device__ __forceinline__ void p_direction(const PArgs &a, int64_t e0, int64_t 
             ss_u = fma((double)m[j], (double)m[j], ss_u);
         }
     }
-    p_st8(a.mom, e0, lo, hi, m, keep);
+    p_st8<EV_LAST>(a.mom, a.wide, e0, lo, hi, m);
 }
 
 // ---- Q: levels (Eq. xi), signed sum over the workers and g_hat (Eq. grad_agg), m' and the layer sums
@@ -456,16 +460,23 @@ __device__ __forceinline__ void p_direction(const PArgs &a, int64_t e0, int64_t 
 // warp in scratch[2w], scratch[2w + 1].  TWO (Algorithm A1 Step 10 follows): stops at g_hat, which is
 // stored, and leaves the tile's sum of g_hat^2 per warp in scratch[2w]. ----------------------------
 template <bool RNG16, int MODE, int OPT, bool TWO>
-__device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt, double *scratch)
+__device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt, double *scratch, float2 *s_fac)
 {
     const int M = a.M, layer = pt.layer;
     const int64_t lo = pt.lo, hi = pt.hi;
     float t = 0.0f, f = 0.0f;
     if (MODE == P_MODE_SHARED) { t = __ldcg(a.qmul + layer); f = __ldcg(a.dq + layer); }
-    const float two_b = a.S_f + 1.0f, inv_two_b = 1.0f / two_b;
-    // scaled form of Eq. xi: valid while t 2^-b is a normal number
-    const bool plain = (t != 0.0f) && !(t >= 1.17549435e-38f * two_b && t <= 3.402823466e38f);
-    const QuConst qc = {t, t * inv_two_b, two_b, inv_two_b * (1.0f / 65536.0f), -127.0f * inv_two_b, __float_as_uint(inv_two_b)};
+    const QuConst qc = dat_qu_const(t, a.S_f, a.wide);
+    bool plain = dat_qu_plain<RNG16>(qc, p_tile_begin(pt), DAT_P_TILE);
+    if (MODE == P_MODE_PER_WORKER) {               // S/nu and nu of every worker: the layer's, for the whole tile
+        bool out = false;
+        for (int i = threadIdx.x; i < M; i += DAT_P_THREADS) {
+            const float ti = __ldcg(a.qmul + (int64_t)i * a.h + layer);
+            s_fac[i] = make_float2(ti, __ldcg(a.worker_norms + (int64_t)i * a.h + layer));
+            out |= dat_qu_plain<RNG16>(dat_qu_const(ti, a.S_f, a.wide), 0, 8);
+        }
+        plain |= __syncthreads_or(out);
+    }
     double ss_theta = 0.0, ss_u = 0.0;
     const int64_t begin = p_tile_begin(pt);
 #pragma unroll 1
@@ -477,19 +488,16 @@ __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt,
 #pragma unroll
         for (int j = 0; j < 8; ++j) acc[j] = 0.0f;
         if (MODE == P_MODE_IDENTITY) {
-#pragma unroll 2
+#pragma unroll 4
             for (int i = 0; i < M; ++i) {           // Q is the identity: the ordered fp32 sum of the workers' gradients
                 float v[8];
-                dat_load4(a.gp.p[i], e0, lo, hi, v);
-                dat_load4(a.gp.p[i], e0 + 4, lo, hi, v + 4);
+                p_ld8<EV_FIRST>(a.gp.p[i], a.wide, e0, lo, hi, v);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) acc[j] += v[j];
             }
-        } else if (MODE == P_MODE_PER_WORKER) p_rows_per_worker<RNG16>(a, layer, e0, lo, hi, acc);
-        else if (full && !plain) qu_rows<RNG16, true, false>(a.gp, a.keys, qc, M, e0, lo, hi, acc);       // nearly always
-        else if (full) qu_rows<RNG16, true, true>(a.gp, a.keys, qc, M, e0, lo, hi, acc);
-        else if (!plain) qu_rows<RNG16, false, false>(a.gp, a.keys, qc, M, e0, lo, hi, acc);
-        else qu_rows<RNG16, false, true>(a.gp, a.keys, qc, M, e0, lo, hi, acc);
+        } else if (MODE == P_MODE_PER_WORKER) p_rows_per_worker<RNG16>(a, qc, s_fac, full && !plain, e0, lo, hi, acc);
+        else if (full && !plain) qu_rows<RNG16>(a.gp, a.keys, a.workers, qc, M, e0, acc);       // nearly always
+        else qu_rows_slow<RNG16>(a.gp, a.keys, qc, M, e0, lo, hi, acc);
         if (TWO) {
             if (MODE == P_MODE_SHARED && a.code_sum) {
 #pragma unroll
@@ -499,7 +507,7 @@ __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt,
 #pragma unroll
             for (int j = 0; j < 8; ++j)
                 acc[j] = (MODE == P_MODE_IDENTITY) ? acc[j] / a.M_f : (MODE == P_MODE_PER_WORKER) ? acc[j] / a.SM_f : acc[j] * f;
-            p_st8(a.ghat, e0, lo, hi, acc, dat_policy_evict_last());   // the R part of a later item reads it again
+            p_st8<EV_LAST>(a.ghat, a.wide, e0, lo, hi, acc);   // the R part of a later item reads it again
 #pragma unroll
             for (int j = 0; j < 8; ++j) ss_theta = fma((double)acc[j], (double)acc[j], ss_theta);
             continue;
@@ -508,18 +516,8 @@ __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt,
         // arithmetic as p_direction, spelled out so that the loads are issued before g_hat is scaled: the step
         // is 3 % slower with the call.)
         float th[8], m[8];
-        if (full) {                                 // theta is read again by the U part (evict-last), m is dead (evict-first)
-            const uint64_t pf = dat_policy_evict_first(), pth = dat_policy_evict_last();
-            const float4 t0 = dat_ld4_hint(a.theta + e0, pth), t1 = dat_ld4_hint(a.theta + e0 + 4, pth);
-            const float4 m0 = dat_ld4_hint(a.mom + e0, pf), m1 = dat_ld4_hint(a.mom + e0 + 4, pf);
-            th[0] = t0.x; th[1] = t0.y; th[2] = t0.z; th[3] = t0.w; th[4] = t1.x; th[5] = t1.y; th[6] = t1.z; th[7] = t1.w;
-            m[0] = m0.x; m[1] = m0.y; m[2] = m0.z; m[3] = m0.w; m[4] = m1.x; m[5] = m1.y; m[6] = m1.z; m[7] = m1.w;
-        } else {
-            p_load4_cg(a.theta, e0, lo, hi, th);
-            p_load4_cg(a.theta, e0 + 4, lo, hi, th + 4);
-            p_load4_cg(a.mom, e0, lo, hi, m);
-            p_load4_cg(a.mom, e0 + 4, lo, hi, m + 4);
-        }
+        p_ld8<EV_LAST>(a.theta, a.wide, e0, lo, hi, th);       // read again by the U part
+        p_ld8<EV_FIRST>(a.mom, a.wide, e0, lo, hi, m);         // dead
         if (MODE == P_MODE_SHARED && a.code_sum) {
 #pragma unroll
             for (int j = 0; j < 8; ++j)
@@ -528,7 +526,7 @@ __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt,
         if (OPT == P_OPT_LAMB) {
             // Algorithm A2: both moments are stored, the direction is formed on the fly for the layer sums
             float v[8];
-            p_ld8(a.var, e0, lo, hi, v, dat_policy_evict_last());
+            p_ld8<EV_LAST>(a.var, a.wide, e0, lo, hi, v);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const float ghat = (MODE == P_MODE_IDENTITY) ? acc[j] / a.M_f : (MODE == P_MODE_PER_WORKER) ? acc[j] / a.SM_f : acc[j] * f;
@@ -539,7 +537,7 @@ __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt,
                 ss_theta = fma((double)th[j], (double)th[j], ss_theta);
                 ss_u = fma((double)u, (double)u, ss_u);
             }
-            p_st8(a.var, e0, lo, hi, v, dat_policy_evict_last());
+            p_st8<EV_LAST>(a.var, a.wide, e0, lo, hi, v);
         } else {
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
@@ -549,16 +547,8 @@ __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt,
                 ss_u = fma((double)m[j], (double)m[j], ss_u);
             }
         }
-        if (full) {
-            const uint64_t pf = dat_policy_evict_last();   // the U part of a later item reads m' again
-            dat_st4_hint(a.mom + e0, make_float4(m[0], m[1], m[2], m[3]), pf);
-            dat_st4_hint(a.mom + e0 + 4, make_float4(m[4], m[5], m[6], m[7]), pf);
-        } else {
-            dat_store4(a.mom, e0, lo, hi, m);
-            dat_store4(a.mom, e0 + 4, lo, hi, m + 4);
-        }
+        p_st8<EV_LAST>(a.mom, a.wide, e0, lo, hi, m);          // the U part of a later item reads m' again
     }
-    __threadfence();                               // m' (and v'), or g_hat, are read by a later part of another CTA
     ss_theta = dat_warp_sum(ss_theta);
     ss_u = dat_warp_sum(ss_u);
     if ((threadIdx.x & 31) == 0) {
@@ -583,7 +573,7 @@ __device__ __forceinline__ void p_part_requant(const PArgs &a, const PipePart &p
         const int64_t e0 = begin + 8 * (int64_t)(k * DAT_P_THREADS + threadIdx.x);
         if (e0 >= hi) continue;
         float v[8];
-        p_ld8(a.ghat, e0, lo, hi, v, dat_policy_evict_first());
+        p_ld8<EV_FIRST>(a.ghat, a.wide, e0, lo, hi, v);
         uint32_t w[8];
         if (RNG16) {
             dat_random_words((uint64_t)e0 >> 3, (uint32_t)a.M, a.keys, w);
@@ -597,10 +587,9 @@ __device__ __forceinline__ void p_part_requant(const PArgs &a, const PipePart &p
             const int lev = (int)dat_level_u1(v[j], t, two_b, u1);
             v[j] = (float)((v[j] < 0.0f) ? -lev : lev) * f;
         }
-        p_st8(a.ghat, e0, lo, hi, v, dat_policy_evict_first());   // the receiver's value
+        p_st8<EV_FIRST>(a.ghat, a.wide, e0, lo, hi, v);        // the receiver's value
         p_direction<OPT>(a, e0, lo, hi, v, ss_theta, ss_u);
     }
-    __threadfence();
     ss_theta = dat_warp_sum(ss_theta);
     ss_u = dat_warp_sum(ss_u);
     if ((threadIdx.x & 31) == 0) {
@@ -617,8 +606,7 @@ __device__ __forceinline__ bool p_server_publish(const PArgs &a, const PipePart 
 #pragma unroll
     for (int w = 0; w < DAT_P_THREADS / 32; ++w) x += scratch[2 * w];
     a.partR[(int64_t)pt.tb + pt.tile] = x;
-    __threadfence();
-    return atomicAdd(a.cntR + pt.layer, 1u) == (uint32_t)pt.T - 1u;
+    return dat_count_in(a.cntR + pt.layer, (uint32_t)pt.T);
 }
 
 // The CTA that counted in the layer's last Q tile of a two-sided step (every thread): the server's norm
@@ -628,7 +616,6 @@ __device__ __forceinline__ void p_server_finish(const PArgs &a, const PipePart &
     const int layer = pt.layer;
     const int64_t tb = pt.tb;
     const uint32_t T = (uint32_t)pt.T;
-    __threadfence();
     double x = 0.0;
     for (uint32_t t = threadIdx.x; t < T; t += DAT_P_THREADS) x += __ldcg(a.partR + tb + t);
     x = dat_warp_sum(x);
@@ -645,7 +632,6 @@ __device__ __forceinline__ void p_server_finish(const PArgs &a, const PipePart &
         if (a.server_scales_out) a.server_scales_out[layer] = nu;
         if (!isfinite(nu)) atomicOr(a.status, DAT_STATUS_NONFINITE);
         a.cntR[layer] = 0u;
-        __threadfence();
         p_st_release(a.readyR + layer, a.epoch);
     }
 }
@@ -659,8 +645,7 @@ __device__ __forceinline__ bool p_quant_publish(const PArgs &a, const PipePart &
     for (int w = 0; w < DAT_P_THREADS / 32; ++w) { x += scratch[2 * w]; y += scratch[2 * w + 1]; }
     a.partQ[2 * ((int64_t)pt.tb + pt.tile)] = x;
     a.partQ[2 * ((int64_t)pt.tb + pt.tile) + 1] = y;
-    __threadfence();
-    return atomicAdd(a.cntQ + pt.layer, 1u) == (uint32_t)pt.T - 1u;
+    return dat_count_in(a.cntQ + pt.layer, (uint32_t)pt.T);      // releases m' (and v', or g_hat) of the whole CTA too
 }
 
 // ---- U: theta' = theta - a_l m' (Eq. 3, pass 2) of one tile ---------------------------------------
@@ -669,43 +654,31 @@ __device__ __forceinline__ void p_part_update(const PArgs &a, const PipePart &pt
 {
     const int64_t lo = pt.lo, hi = pt.hi;
     const float na = -__ldcg(a.step_a + pt.layer);
-    const uint64_t pol_first = dat_policy_evict_first();
     const int64_t begin = p_tile_begin(pt);
 #pragma unroll
     for (int k = 0; k < DAT_P_GROUPS; ++k) {
         const int64_t e0 = begin + 8 * (int64_t)(k * DAT_P_THREADS + threadIdx.x);
         if (e0 >= hi) continue;
+        float th[8], m[8];
         if (OPT == P_OPT_LAMB) {
             // the direction once more from the stored moments: the same fp32 operations give the same bits
-            float th[8], m[8], v[8];
-            p_ld8(a.theta, e0, lo, hi, th, pol_first);
-            p_ld8(a.mom, e0, lo, hi, m, pol_first);
-            p_ld8(a.var, e0, lo, hi, v, pol_first);
+            float v[8];
+            p_ld8<EV_FIRST>(a.theta, a.wide, e0, lo, hi, th);
+            p_ld8<EV_FIRST>(a.mom, a.wide, e0, lo, hi, m);
+            p_ld8<EV_FIRST>(a.var, a.wide, e0, lo, hi, v);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const bool inside = (e0 + j >= lo && e0 + j < hi);
                 const float u = inside ? dat_lamb_direction(a.lamb, m[j], v[j], th[j]) : 0.0f;
                 th[j] = __fmaf_rn(na, u, th[j]);
             }
-            p_st8(a.theta, e0, lo, hi, th, pol_first);
-        } else if (e0 >= lo && e0 + 8 <= hi) {
-            float4 t0 = dat_ld4_hint(a.theta + e0, pol_first), t1 = dat_ld4_hint(a.theta + e0 + 4, pol_first);
-            const float4 m0 = dat_ld4_hint(a.mom + e0, pol_first), m1 = dat_ld4_hint(a.mom + e0 + 4, pol_first);
-            t0.x = __fmaf_rn(na, m0.x, t0.x); t0.y = __fmaf_rn(na, m0.y, t0.y); t0.z = __fmaf_rn(na, m0.z, t0.z); t0.w = __fmaf_rn(na, m0.w, t0.w);
-            t1.x = __fmaf_rn(na, m1.x, t1.x); t1.y = __fmaf_rn(na, m1.y, t1.y); t1.z = __fmaf_rn(na, m1.z, t1.z); t1.w = __fmaf_rn(na, m1.w, t1.w);
-            dat_st4_hint(a.theta + e0, t0, pol_first);
-            dat_st4_hint(a.theta + e0 + 4, t1, pol_first);
         } else {
-            float th[8], m[8];
-            p_load4_cg(a.theta, e0, lo, hi, th);
-            p_load4_cg(a.theta, e0 + 4, lo, hi, th + 4);
-            p_load4_cg(a.mom, e0, lo, hi, m);
-            p_load4_cg(a.mom, e0 + 4, lo, hi, m + 4);
+            p_ld8<EV_FIRST>(a.theta, a.wide, e0, lo, hi, th);
+            p_ld8<EV_FIRST>(a.mom, a.wide, e0, lo, hi, m);
 #pragma unroll
             for (int j = 0; j < 8; ++j) th[j] = __fmaf_rn(na, m[j], th[j]);
-            dat_store4(a.theta, e0, lo, hi, th);
-            dat_store4(a.theta, e0 + 4, lo, hi, th + 4);
         }
+        p_st8<EV_FIRST>(a.theta, a.wide, e0, lo, hi, th);
     }
 }
 
@@ -715,6 +688,7 @@ k_step_pipelined(const __grid_constant__ PArgs a)
 {
     __shared__ double s_unit[4 * DAT_MAX_WORKERS];
     __shared__ float s_norm[DAT_MAX_WORKERS];
+    __shared__ float2 s_fac[MODE == P_MODE_PER_WORKER ? DAT_MAX_WORKERS : 1];
     __shared__ __align__(16) PipeItem s_item;
     __shared__ int s_ctl[4];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -764,7 +738,7 @@ k_step_pipelined(const __grid_constant__ PArgs a)
     __syncthreads();                               // (A)
     if (s_ctl[0]) p_norm_finish<MODE>(a, pn, s_norm);
     bool alive = (s_ctl[1] != 0);
-    if (alive && pq.layer >= 0) p_part_quant<RNG16, MODE, OPT, TWO>(a, pq, s_unit);
+    if (alive && pq.layer >= 0) p_part_quant<RNG16, MODE, OPT, TWO>(a, pq, s_unit, s_fac);
     __syncthreads();
     if (TWO) {
         // Step 10: the tile's sum of g_hat^2 counted in; the layer's last tile publishes the server's norm;
@@ -948,6 +922,8 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
     const bool per_worker = !identity && plan->scale_mode == DAT_SCALE_PER_WORKER;
     const size_t h = (size_t)plan->h;
     a.keys = dat_make_keys(seed, step);
+    dat_make_worker_table(a.keys, plan->M, &a.workers);
+    a.wide = dat_grads_wide(plan, grads) && (((uintptr_t)theta | (uintptr_t)mom | (uintptr_t)var | (uintptr_t)g_hat) & 31u) == 0;
     a.items = two ? g->d_items2 : g->d_items;
     a.off = plan->d_offsets;
     a.tile_base = g->d_tile_base;

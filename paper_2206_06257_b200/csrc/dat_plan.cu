@@ -37,6 +37,13 @@ int dat_check_grads(const dat_plan_t *plan, const float *const *grads, GradPtrs 
     return DAT_OK;
 }
 
+bool dat_grads_wide(const dat_plan_t *plan, const float *const *grads)
+{
+    uintptr_t all = 0;
+    for (int i = 0; i < plan->M; ++i) all |= (uintptr_t)grads[i];
+    return (all & 31u) == 0;
+}
+
 LambConst dat_lamb_const(const dat_lamb_hparams_t *hp, int64_t t)
 {
     LambConst c;
@@ -63,6 +70,11 @@ PhiloxKeys dat_make_keys(uint64_t seed, uint64_t step)
     }
     k.seed_hi = (uint32_t)(seed >> 32);
     return k;
+}
+
+void dat_make_worker_table(const PhiloxKeys &keys, int M, PhiloxWorkers *out)
+{
+    for (int i = 0; i <= M; ++i) out->w[i] = dat_philox_worker(0u, (uint32_t)i, keys);
 }
 
 extern "C" int dat_plan_create(dat_plan_t **out, int64_t num_layers, const int64_t *layer_offsets,

@@ -80,7 +80,7 @@ k_sumsq(const __grid_constant__ GradPtrs gp, const TileSource tiles, int M, int 
 #pragma unroll
             for (int it = 0; it < ITERS; ++it) {
                 const int64_t e0 = r.begin + 8 * (int64_t)(it * DAT_THREADS + threadIdx.x);
-                if (inside && i + p < w1) dat_ld8_stream(g + e0, wide, v[p][it]);
+                if (inside && i + p < w1) dat_ld8<EV_FIRST>(g + e0, wide, v[p][it]);
                 else {
 #pragma unroll
                     for (int j = 0; j < 8; ++j) v[p][it][j] = (i + p < w1 && e0 + j >= r.lo && e0 + j < r.end) ? g[e0 + j] : 0.0f;
@@ -255,8 +255,8 @@ k_quantize(const __grid_constant__ GradPtrs gp, const __grid_constant__ PhiloxKe
     const bool whole = e_piece + n_warp <= d;
     float v[2][8];
     if (whole) {                                             // two groups per lane are always in flight
-        dat_ld8_stream(g, wide, v[0]);
-        dat_ld8_stream(g + 256, wide, v[1]);
+        dat_ld8<EV_FIRST>(g, wide, v[0]);
+        dat_ld8<EV_FIRST>(g + 256, wide, v[1]);
     }
     const int l0 = __ldg(flat_layer + piece), nl = __ldg(flat_layer + last + 1) - l0 + 1;   // the warp's layers are among [l0, l0 + nl)
     const int64_t q0 = per_worker ? (int64_t)worker * h : 0;
@@ -276,7 +276,7 @@ k_quantize(const __grid_constant__ GradPtrs gp, const __grid_constant__ PhiloxKe
                 uint32_t w[8];
                 dat_group_words<RNG16>(dat_philox_group<RNG16>(elem + 256u * (k + p), keys), pw, keys, w);
                 quantize8<BITS, RNG16>(v[p], ts, w, my_level + (k + p) * 32 * BITS, my_sign + (k + p) * 32);
-                if (k + 2 < groups) dat_ld8_stream(g + 256 * (k + p + 2), wide, v[p]);
+                if (k + 2 < groups) dat_ld8<EV_FIRST>(g + 256 * (k + p + 2), wide, v[p]);
             }
         }
     } else {
@@ -293,7 +293,7 @@ k_quantize(const __grid_constant__ GradPtrs gp, const __grid_constant__ PhiloxKe
             if (page && scaled(t) && e0 + 8 <= l_hi) {
                 float x[8];
                 uint32_t w[8];
-                dat_ld8_stream(g + 256 * k, wide, x);
+                dat_ld8<EV_FIRST>(g + 256 * k, wide, x);
                 dat_group_words<RNG16>(dat_philox_group<RNG16>(elem + 256u * k, keys), pw, keys, w);
                 quantize8<BITS, RNG16>(x, t * (1.0f / TWO_B), w, my_level + k * 32 * BITS, my_sign + k * 32);
             } else {
@@ -972,7 +972,8 @@ extern "C" int dat_lalr_step_static(int64_t num_layers, const int64_t *layer_off
 // ------------------------------------------------------------------------------------------
 template <bool RNG16>
 __global__ void __launch_bounds__(DAT_QU_THREADS, DAT_QU_MINB)
-k_quant_update(const __grid_constant__ GradPtrs gp, const __grid_constant__ PhiloxKeys keys, const TileSource tiles, int M,
+k_quant_update(const __grid_constant__ GradPtrs gp, const __grid_constant__ PhiloxKeys keys, const __grid_constant__ PhiloxWorkers pw,
+               const TileSource tiles, int M, bool wide,
                const float *__restrict__ qmul, const float *__restrict__ dq, const float *__restrict__ theta,
                float *__restrict__ mom, float S_f, float mu, float wd, double *__restrict__ partials,
                int32_t *__restrict__ code_sum)
@@ -984,12 +985,8 @@ k_quant_update(const __grid_constant__ GradPtrs gp, const __grid_constant__ Phil
     const int layer = r.layer;
     const int64_t lo = r.lo, hi = r.hi, begin = r.begin;
     const float t = __ldg(qmul + layer), f = __ldg(dq + layer);
-    const float two_b = S_f + 1.0f, inv_two_b = 1.0f / two_b;
-    // scaled form of Eq. xi (see dat_step.cu): valid while t 2^-b is a normal number
-    const bool plain = (t != 0.0f) && !(t >= 1.17549435e-38f * two_b && t <= 3.402823466e38f);
-    const float ts = t * inv_two_b;
-    const float c0 = inv_two_b * (1.0f / 65536.0f), c1 = -127.0f * inv_two_b;
-    const uint32_t ubits = __float_as_uint(inv_two_b);
+    const QuConst qc = dat_qu_const(t, S_f, wide);
+    const bool plain = dat_qu_plain<RNG16>(qc, begin, DAT_TILE);
     double ss_theta = 0.0, ss_u = 0.0;
 #pragma unroll 1
     for (int k = 0; k < DAT_QU_GROUPS; ++k) {
@@ -999,11 +996,8 @@ k_quant_update(const __grid_constant__ GradPtrs gp, const __grid_constant__ Phil
         float acc[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) acc[j] = 0.0f;
-        const QuConst qc = {t, ts, two_b, c0, c1, ubits};
-        if (full && !plain) qu_rows<RNG16, true, false>(gp, keys, qc, M, e0, lo, hi, acc);       // nearly always
-        else if (full) qu_rows<RNG16, true, true>(gp, keys, qc, M, e0, lo, hi, acc);
-        else if (!plain) qu_rows<RNG16, false, false>(gp, keys, qc, M, e0, lo, hi, acc);
-        else qu_rows<RNG16, false, true>(gp, keys, qc, M, e0, lo, hi, acc);
+        if (full && !plain) qu_rows<RNG16>(gp, keys, pw, qc, M, e0, acc);       // nearly always
+        else qu_rows_slow<RNG16>(gp, keys, qc, M, e0, lo, hi, acc);
         // theta and m only now: registers are what limits the number of resident warps here
         float th[8], m[8];
         if (full) {
@@ -1061,11 +1055,14 @@ extern "C" int dat_step_passes(dat_plan_t *plan, float *theta, float *mom, const
     DAT_LAUNCHED(plan);
     if (scales_out) DAT_CUDA(plan, cudaMemcpyAsync(scales_out, plan->d_scales, (size_t)h * 4, cudaMemcpyDeviceToDevice, s));
     const PhiloxKeys keys = dat_make_keys(seed, step);
+    PhiloxWorkers pw;
+    dat_make_worker_table(keys, plan->M, &pw);
+    const bool wide = dat_grads_wide(plan, grads);
     if (plan->rng_bits == 16)
-        k_quant_update<true><<<(unsigned)plan->n_tiles, DAT_QU_THREADS, 0, s>>>(gp, keys, plan_tiles(plan), plan->M, plan->d_qmul, plan->d_dq, theta, mom, S_f, hp->momentum,
+        k_quant_update<true><<<(unsigned)plan->n_tiles, DAT_QU_THREADS, 0, s>>>(gp, keys, pw, plan_tiles(plan), plan->M, wide, plan->d_qmul, plan->d_dq, theta, mom, S_f, hp->momentum,
                                                                                  hp->weight_decay, plan->d_partials, code_sum_out);
     else
-        k_quant_update<false><<<(unsigned)plan->n_tiles, DAT_QU_THREADS, 0, s>>>(gp, keys, plan_tiles(plan), plan->M, plan->d_qmul, plan->d_dq, theta, mom, S_f, hp->momentum,
+        k_quant_update<false><<<(unsigned)plan->n_tiles, DAT_QU_THREADS, 0, s>>>(gp, keys, pw, plan_tiles(plan), plan->M, wide, plan->d_qmul, plan->d_dq, theta, mom, S_f, hp->momentum,
                                                                                   hp->weight_decay, plan->d_partials, code_sum_out);
     DAT_LAUNCHED(plan);
     k_lalr_finalize<<<h, DAT_THREADS, 0, s>>>(plan->d_tile_base, plan->d_partials, hp->lr, hp->c_l, hp->c_u, plan->d_step_a,
