@@ -35,9 +35,16 @@ struct TileDesc {
 };
 
 // LAMB (Algorithm A2): what the kernels need of the hyper-parameters at iteration t.
-struct LambConst {
-    float beta1, beta2, om1, om2, bc1, bc2, zeta, wd;
+// Division by a constant y as x*hi + x*lo, hi + lo = 1/y to 2^-48: see dat_const_div (dat_plan.cu).
+struct ConstDiv {
+    float y, hi, lo;
+    bool exact;                        // the two-operation form rounds correctly for every x (else: the division itself)
 };
+struct LambConst {
+    float beta1, beta2, om1, om2, zeta, wd;
+    ConstDiv bc1, bc2;                 // 1 - beta1^t, 1 - beta2^t
+};
+ConstDiv dat_const_div(float y);                             // dat_plan.cu
 LambConst dat_lamb_const(const dat_lamb_hparams_t *hp, int64_t t);   // dat_plan.cu
 
 struct dat_plan {
@@ -380,12 +387,18 @@ __device__ __forceinline__ void dat_store4(float *__restrict__ p, int64_t e0, in
     }
 }
 
+// x / c.y, correctly rounded (for |x| < 2^-98 possibly off by the last denormal place).
+__device__ __forceinline__ float dat_div(float x, const ConstDiv &c)
+{
+    return c.exact ? __fmaf_rn(x, c.hi, __fmul_rn(x, c.lo)) : x / c.y;
+}
+
 // The LAMB direction of one element from the stored moments: u = m^/(sqrt(v^) + zeta) + wd*theta with the
 // bias-corrected m^ = m'/(1 - beta1^t), v^ = v'/(1 - beta2^t) (Algorithm A2; one rounding per operation).
 __device__ __forceinline__ float dat_lamb_direction(const LambConst &c, float m_new, float v_new, float theta)
 {
-    const float m_hat = m_new / c.bc1;
-    const float v_hat = v_new / c.bc2;
+    const float m_hat = dat_div(m_new, c.bc1);
+    const float v_hat = dat_div(v_new, c.bc2);
     return __fmaf_rn(c.wd, theta, m_hat / (sqrtf(v_hat) + c.zeta));
 }
 

@@ -931,7 +931,7 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
     a.mom = mom;
     a.var = var;
     if (lamb) a.lamb = *lamb;
-    else a.lamb = LambConst{0.0f, 0.0f, 0.0f, 0.0f, 1.0f, 1.0f, 1.0f, 0.0f};
+    else a.lamb = LambConst{};
     a.partN = g->d_partN;
     a.partQ = g->d_partQ;
     a.partR = g->d_partR;

@@ -44,6 +44,44 @@ bool dat_grads_wide(const dat_plan_t *plan, const float *const *grads)
     return (all & 31u) == 0;
 }
 
+// Correctly rounded division by a number that is known in advance, after Brisebarre, Muller and Raina, "Accelerating
+// correctly rounded floating-point division when the divisor is known in advance" (IEEE Trans. Computers 53(8), 2004):
+// with hi = RN(1/y) and lo = RN(1/y - hi), RN(x*hi + RN(x*lo)) differs from x/y by less than 2^-47 of it before the last
+// rounding, so it can only be wrong for an x whose quotient lies that close to the middle of two floats.  With the
+// 24-bit integers X, Y of the operands' significands, such a quotient has |X 2^s - (2k+1) Y| = e <= 4 for s = 24 or 25;
+// the few X that satisfy one of these congruences are found and tried here.  If one of them fails (none has been seen
+// for 1 - beta^t), the kernels divide.
+ConstDiv dat_const_div(float y)
+{
+    ConstDiv c = {y, 1.0f / y, 0.0f, true};
+    c.lo = fmaf(-y, c.hi, 1.0f) / y;
+    int ex;
+    const uint64_t Y = (uint64_t)(frexpf(y, &ex) * 16777216.0f);         // 2^23 <= Y < 2^24
+    if (!(y > 1e-30f && y < 1e30f)) { c.exact = false; return c; }
+    uint64_t odd = Y;
+    int tz = 0;
+    while (!(odd & 1)) { odd >>= 1; ++tz; }
+    uint64_t inv = odd;                                                  // inverse of `odd` modulo 2^64 (Newton)
+    for (int i = 0; i < 6; ++i) inv *= 2 - odd * inv;
+    for (int s = 24; s <= 25; ++s)
+        for (int e = -4; e <= 4; ++e) {
+            if (e == 0 || (e & ((1 << tz) - 1))) continue;              // 2^tz divides X 2^s and (2k+1) Y, so it divides e
+            if (tz > 2) continue;
+            const uint64_t mod = 1ull << (s - tz);
+            const uint64_t q0 = (uint64_t)(int64_t)(e >> tz) * inv & (mod - 1);     // (2k+1) = e/2^tz * odd^-1 (mod 2^(s-tz))
+            for (uint64_t q = q0; q < (1ull << 25); q += mod) {
+                if (!(q & 1) || q < (1ull << 24)) continue;             // midpoints have 25 significant bits
+                const uint64_t num = q * Y - (uint64_t)(int64_t)e;      // = X 2^s
+                if (num & ((1ull << s) - 1)) continue;
+                const uint64_t X = num >> s;
+                if (X < (1ull << 23) || X >= (1ull << 24)) continue;
+                const float x = (float)X;
+                if (fmaf(x, c.hi, x * c.lo) != x / y) c.exact = false;
+            }
+        }
+    return c;
+}
+
 LambConst dat_lamb_const(const dat_lamb_hparams_t *hp, int64_t t)
 {
     LambConst c;
@@ -51,8 +89,8 @@ LambConst dat_lamb_const(const dat_lamb_hparams_t *hp, int64_t t)
     c.beta2 = hp->beta2;
     c.om1 = 1.0f - hp->beta1;
     c.om2 = 1.0f - hp->beta2;
-    c.bc1 = (float)(1.0 - pow((double)hp->beta1, (double)t));      // 1 - beta^t in double, rounded once
-    c.bc2 = (float)(1.0 - pow((double)hp->beta2, (double)t));
+    c.bc1 = dat_const_div((float)(1.0 - pow((double)hp->beta1, (double)t)));      // 1 - beta^t in double, rounded once
+    c.bc2 = dat_const_div((float)(1.0 - pow((double)hp->beta2, (double)t)));
     c.zeta = hp->zeta;
     c.wd = hp->weight_decay;
     return c;

@@ -701,79 +701,180 @@ extern "C" int dat_average(dat_plan_t *plan, const float *const *grads, float *g
 }
 
 // ------------------------------------------------------------------------------------------
-// S6-S8: LALR (Eq. 3).  Pass 1 (per-layer tiles): m' and the fp64 partial sums of theta^2 and
-// m'^2.  Finalize: per layer, a_l = lr * tau(||theta_l||)/||u_l||.  Pass 2: theta -= a_l * m'.
+// S6-S8: LALR (Eq. 3), and LAMB (Algorithm A2) with the same update.  Pass 1 (per-layer tiles): m' -- for LAMB m' and
+// v', with the direction u = m^/(sqrt(v^) + zeta) + wd*theta formed on the fly -- and the fp64 partial sums of theta^2
+// and u^2; the CTA that finishes a layer's last tile forms a_l = lr * tau(||theta_l||)/||u_l||.  Pass 2:
+// theta -= a_l * u (LAMB: u once more from the stored moments; the same fp32 operations give the same bits).
+// HBM-bound.  Pass 1 walks the tiles back from the last, pass 2 forward from the first: what pass 1 touched last
+// (theta and the moments, kept in L2 with evict-last) is what pass 2 reads first.
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(DAT_THREADS)
-k_lalr_pass1(const float *__restrict__ theta, float *__restrict__ mom, const float *__restrict__ g_hat,
-             const TileSource tiles, float mu, float wd, double *__restrict__ partials)
+enum { OPT_MOMENTUM = 0, OPT_LAMB = 1 };
+#define UPDATE_CTAS 5                            // resident CTAs per SM (4: 71.6 + 39.4 us, 6: 72.3 + 41.0, 5: 67.8 + 40.2 for ResNet-50)
+
+struct UpdateArgs {
+    TileSource tiles;
+    float *theta, *mom, *var;
+    const float *g_hat;
+    LambConst lamb;
+    float mu, wd, lr, c_l, c_u;
+    bool wide;
+    double *partials;
+    float *step_a, *norms_out;
+    uint32_t *count, *status;
+};
+
+template <int EV>
+__device__ __forceinline__ void update_ld8(const float *p, bool full, bool wide, int64_t e0, int64_t lo, int64_t hi, float v[8])
+{
+    if (full) {
+        dat_ld8<EV>(p + e0, wide, v);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = (e0 + j >= lo && e0 + j < hi) ? p[e0 + j] : 0.0f;
+    }
+}
+template <int EV>
+__device__ __forceinline__ void update_st8(float *p, bool full, bool wide, int64_t e0, int64_t lo, int64_t hi, const float v[8])
+{
+    if (full) {
+        dat_st8<EV>(p + e0, wide, v);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (e0 + j >= lo && e0 + j < hi) p[e0 + j] = v[j];
+    }
+}
+
+// Per layer, from the partial sums of its tiles: a_l (every thread of the CTA).
+__device__ __forceinline__ void update_finish(const UpdateArgs &a, int l, int64_t t0, int64_t t1, double *scratch)
+{
+    double x = 0.0, y = 0.0;
+    for (int64_t t = t0 + threadIdx.x; t < t1; t += DAT_THREADS) { x += __ldcg(a.partials + 2 * t); y += __ldcg(a.partials + 2 * t + 1); }
+    x = dat_block_sum(x, scratch);
+    y = dat_block_sum(y, scratch);
+    if (threadIdx.x == 0) {
+        const float n_theta = (float)sqrt(x), n_u = (float)sqrt(y);
+        const float tau = fminf(fmaxf(n_theta, a.c_l), a.c_u);
+        const float ratio = (n_u == 0.0f) ? 0.0f : tau / n_u;
+        a.step_a[l] = a.lr * ratio;
+        if (a.norms_out) { a.norms_out[2 * l] = n_theta; a.norms_out[2 * l + 1] = n_u; }
+        if (!isfinite(n_theta) || !isfinite(n_u)) atomicOr(a.status, DAT_STATUS_NONFINITE);
+        a.count[l] = 0u;                          // ready for the next call
+    }
+}
+
+// The tile's two sums (every thread), counted in; the layer's last tile finishes the layer.
+__device__ __forceinline__ void update_count_in(const UpdateArgs &a, const TileRange &r, int64_t tile, double ss_theta, double ss_u, double *scratch, bool *s_last)
+{
+    const double x = dat_block_sum(ss_theta, scratch);
+    const double y = dat_block_sum(ss_u, scratch);
+    const int64_t T = dat_layer_tiles(r);
+    if (threadIdx.x == 0) {
+        a.partials[2 * tile] = x;
+        a.partials[2 * tile + 1] = y;
+        *s_last = dat_count_in(a.count + r.layer, (uint32_t)T);
+    }
+    __syncthreads();
+    if (*s_last) update_finish(a, r.layer, r.first, r.first + T, scratch);
+}
+
+template <int OPT>
+__global__ void __launch_bounds__(DAT_THREADS, UPDATE_CTAS)
+k_update_pass1(const __grid_constant__ UpdateArgs a)
 {
     __shared__ double scratch[DAT_THREADS / 32];
-    const int64_t tile = blockIdx.x;
-    const TileRange r = dat_tile_range(tiles, tile);
+    __shared__ bool s_last;
+    const int64_t tile = (int64_t)gridDim.x - 1 - blockIdx.x;
+    const TileRange r = dat_tile_range(a.tiles, tile);
     double ss_theta = 0.0, ss_u = 0.0;
+#pragma unroll 1
+    for (int it = 0; it < DAT_TILE / 8 / DAT_THREADS; ++it) {
+        const int64_t e0 = r.begin + 8 * (int64_t)(it * DAT_THREADS + threadIdx.x);
+        if (e0 >= r.end) continue;
+        const bool full = e0 >= r.lo && e0 + 8 <= r.hi;
+        float th[8], m[8], g[8];
+        update_ld8<EV_LAST>(a.theta, full, a.wide, e0, r.lo, r.hi, th);
+        update_ld8<EV_FIRST>(a.mom, full, a.wide, e0, r.lo, r.hi, m);
+        update_ld8<EV_FIRST>(a.g_hat, full, a.wide, e0, r.lo, r.hi, g);
+        if (OPT == OPT_LAMB) {
+            float v[8];
+            update_ld8<EV_FIRST>(a.var, full, a.wide, e0, r.lo, r.hi, v);
 #pragma unroll
-    for (int it = 0; it < DAT_TILE / 4 / DAT_THREADS; ++it) {
-        const int64_t e0 = r.begin + 4 * (int64_t)(it * DAT_THREADS + threadIdx.x);
-        if (e0 < r.end) {
-            float th[4], m[4], g[4];
-            dat_load4(theta, e0, r.lo, r.hi, th);
-            dat_load4(mom, e0, r.lo, r.hi, m);
-            dat_load4(g_hat, e0, r.lo, r.hi, g);
+            for (int j = 0; j < 8; ++j) {
+                m[j] = __fmaf_rn(a.lamb.beta1, m[j], __fmul_rn(a.lamb.om1, g[j]));
+                v[j] = __fmaf_rn(a.lamb.beta2, v[j], __fmul_rn(a.lamb.om2, __fmul_rn(g[j], g[j])));
+                const float u = (full || (e0 + j >= r.lo && e0 + j < r.hi)) ? dat_lamb_direction(a.lamb, m[j], v[j], th[j]) : 0.0f;
+                ss_theta = fma((double)th[j], (double)th[j], ss_theta);
+                ss_u = fma((double)u, (double)u, ss_u);
+            }
+            update_st8<EV_LAST>(a.var, full, a.wide, e0, r.lo, r.hi, v);
+        } else {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                m[j] = __fmaf_rn(mu, m[j], __fmaf_rn(wd, th[j], g[j]));
+            for (int j = 0; j < 8; ++j) {
+                m[j] = __fmaf_rn(a.mu, m[j], __fmaf_rn(a.wd, th[j], g[j]));
                 ss_theta = fma((double)th[j], (double)th[j], ss_theta);
                 ss_u = fma((double)m[j], (double)m[j], ss_u);
             }
-            dat_store4(mom, e0, r.lo, r.hi, m);
         }
+        update_st8<EV_LAST>(a.mom, full, a.wide, e0, r.lo, r.hi, m);
     }
-    const double a = dat_block_sum(ss_theta, scratch);
-    const double b = dat_block_sum(ss_u, scratch);
-    if (threadIdx.x == 0) { partials[2 * tile] = a; partials[2 * tile + 1] = b; }
+    update_count_in(a, r, tile, ss_theta, ss_u, scratch, &s_last);
 }
 
-__global__ void __launch_bounds__(DAT_THREADS)
-k_lalr_finalize(const int64_t *__restrict__ tile_base, const double *__restrict__ partials,
-                float lr, float c_l, float c_u, float *__restrict__ step_a,
-                float *__restrict__ norms_out, uint32_t *status)
+template <int OPT>
+__global__ void __launch_bounds__(DAT_THREADS, UPDATE_CTAS)
+k_update_pass2(const __grid_constant__ UpdateArgs a)
 {
-    __shared__ double scratch[DAT_THREADS / 32];
-    const int l = blockIdx.x;
-    const int64_t t0 = tile_base[l], t1 = tile_base[l + 1];
-    double a = 0.0, b = 0.0;
-    for (int64_t t = t0 + threadIdx.x; t < t1; t += DAT_THREADS) { a += partials[2 * t]; b += partials[2 * t + 1]; }
-    a = dat_block_sum(a, scratch);
-    b = dat_block_sum(b, scratch);
-    if (threadIdx.x == 0) {
-        const float n_theta = (float)sqrt(a), n_u = (float)sqrt(b);
-        const float tau = fminf(fmaxf(n_theta, c_l), c_u);
-        const float ratio = (n_u == 0.0f) ? 0.0f : tau / n_u;
-        step_a[l] = lr * ratio;
-        if (norms_out) { norms_out[2 * l] = n_theta; norms_out[2 * l + 1] = n_u; }
-        if (!isfinite(n_theta) || !isfinite(n_u)) atomicOr(status, DAT_STATUS_NONFINITE);
+    const TileRange r = dat_tile_range(a.tiles, blockIdx.x);
+    const float na = -__ldg(a.step_a + r.layer);
+#pragma unroll
+    for (int it = 0; it < DAT_TILE / 8 / DAT_THREADS; ++it) {
+        const int64_t e0 = r.begin + 8 * (int64_t)(it * DAT_THREADS + threadIdx.x);
+        if (e0 >= r.end) continue;
+        const bool full = e0 >= r.lo && e0 + 8 <= r.hi;
+        float th[8], m[8];
+        update_ld8<EV_FIRST>(a.theta, full, a.wide, e0, r.lo, r.hi, th);
+        update_ld8<EV_FIRST>(a.mom, full, a.wide, e0, r.lo, r.hi, m);
+        if (OPT == OPT_LAMB) {
+            float v[8];
+            update_ld8<EV_FIRST>(a.var, full, a.wide, e0, r.lo, r.hi, v);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float u = (full || (e0 + j >= r.lo && e0 + j < r.hi)) ? dat_lamb_direction(a.lamb, m[j], v[j], th[j]) : 0.0f;
+                th[j] = __fmaf_rn(na, u, th[j]);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) th[j] = __fmaf_rn(na, m[j], th[j]);
+        }
+        update_st8<EV_FIRST>(a.theta, full, a.wide, e0, r.lo, r.hi, th);
     }
 }
 
-__global__ void __launch_bounds__(DAT_THREADS)
-k_lalr_pass2(float *__restrict__ theta, const float *__restrict__ mom, const TileSource tiles, const float *__restrict__ step_a)
+static bool update_wide(const void *a, const void *b, const void *c, const void *d)
 {
-    const int64_t tile = blockIdx.x;
-    const TileRange r = dat_tile_range(tiles, tile);
-    const float na = -__ldg(step_a + r.layer);
-#pragma unroll
-    for (int it = 0; it < DAT_TILE / 4 / DAT_THREADS; ++it) {
-        const int64_t e0 = r.begin + 4 * (int64_t)(it * DAT_THREADS + threadIdx.x);
-        if (e0 < r.end) {
-            float th[4], m[4];
-            dat_load4(theta, e0, r.lo, r.hi, th);
-            dat_load4(mom, e0, r.lo, r.hi, m);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) th[j] = __fmaf_rn(na, m[j], th[j]);
-            dat_store4(theta, e0, r.lo, r.hi, th);
-        }
-    }
+    return (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c | (uintptr_t)d) & 31u) == 0;
+}
+
+// The arguments of a plan's two passes.
+static UpdateArgs update_args(const dat_plan_t *plan, float *theta, float *mom, float *var, const float *g_hat, float lr, float c_l, float c_u, float *norms_out)
+{
+    UpdateArgs a = {};
+    a.tiles = plan_tiles(plan);
+    a.theta = theta;
+    a.mom = mom;
+    a.var = var;
+    a.g_hat = g_hat;
+    a.lr = lr;
+    a.c_l = c_l;
+    a.c_u = c_u;
+    a.wide = update_wide(theta, mom, var, g_hat);
+    a.partials = plan->d_partials;
+    a.step_a = plan->d_step_a;
+    a.norms_out = norms_out;
+    a.count = plan->d_count;
+    a.status = plan->d_status;
+    return a;
 }
 
 extern "C" int dat_lalr_step(dat_plan_t *plan, float *theta, float *mom, const float *g_hat,
@@ -786,83 +887,14 @@ extern "C" int dat_lalr_step(dat_plan_t *plan, float *theta, float *mom, const f
         (layer_norms_out && !dat_aligned16(layer_norms_out)))
         return DAT_ERR_ALIGN;
     cudaStream_t s = (cudaStream_t)stream;
-    const int h = (int)plan->h;
-    k_lalr_pass1<<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(theta, mom, g_hat, plan_tiles(plan), hp->momentum,
-                                                                 hp->weight_decay, plan->d_partials);
+    UpdateArgs a = update_args(plan, theta, mom, nullptr, g_hat, hp->lr, hp->c_l, hp->c_u, layer_norms_out);
+    a.mu = hp->momentum;
+    a.wd = hp->weight_decay;
+    k_update_pass1<OPT_MOMENTUM><<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(a);
     DAT_LAUNCHED(plan);
-    k_lalr_finalize<<<h, DAT_THREADS, 0, s>>>(plan->d_tile_base, plan->d_partials, hp->lr, hp->c_l, hp->c_u,
-                                              plan->d_step_a, layer_norms_out, plan->d_status);
-    DAT_LAUNCHED(plan);
-    k_lalr_pass2<<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(theta, mom, plan_tiles(plan), plan->d_step_a);
+    k_update_pass2<OPT_MOMENTUM><<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(a);
     DAT_LAUNCHED(plan);
     return DAT_OK;
-}
-
-// ------------------------------------------------------------------------------------------
-// LAMB (Algorithm A2) with the update of Eq. upth = Eq. 3.  Pass 1: the moments m', v' are stored,
-// the direction u = m^/(sqrt(v^) + zeta) + wd*theta is formed on the fly for the fp64 partial sums
-// of theta^2 and u^2.  Finalize as for LALR.  Pass 2 forms u again from the stored moments (the same
-// fp32 operations give the same bits) and moves theta.
-// ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(DAT_THREADS)
-k_lamb_pass1(const float *__restrict__ theta, float *__restrict__ mom, float *__restrict__ var,
-             const float *__restrict__ g_hat, const TileSource tiles, LambConst c, double *__restrict__ partials)
-{
-    __shared__ double scratch[DAT_THREADS / 32];
-    const int64_t tile = blockIdx.x;
-    const TileRange r = dat_tile_range(tiles, tile);
-    double ss_theta = 0.0, ss_u = 0.0;
-#pragma unroll
-    for (int it = 0; it < DAT_TILE / 4 / DAT_THREADS; ++it) {
-        const int64_t e0 = r.begin + 4 * (int64_t)(it * DAT_THREADS + threadIdx.x);
-        if (e0 < r.end) {
-            float th[4], m[4], v[4], g[4];
-            dat_load4(theta, e0, r.lo, r.hi, th);
-            dat_load4(mom, e0, r.lo, r.hi, m);
-            dat_load4(var, e0, r.lo, r.hi, v);
-            dat_load4(g_hat, e0, r.lo, r.hi, g);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                m[j] = __fmaf_rn(c.beta1, m[j], __fmul_rn(c.om1, g[j]));
-                v[j] = __fmaf_rn(c.beta2, v[j], __fmul_rn(c.om2, __fmul_rn(g[j], g[j])));
-                const bool inside = (e0 + j >= r.lo && e0 + j < r.hi);
-                const float u = inside ? dat_lamb_direction(c, m[j], v[j], th[j]) : 0.0f;
-                ss_theta = fma((double)th[j], (double)th[j], ss_theta);
-                ss_u = fma((double)u, (double)u, ss_u);
-            }
-            dat_store4(mom, e0, r.lo, r.hi, m);
-            dat_store4(var, e0, r.lo, r.hi, v);
-        }
-    }
-    const double a = dat_block_sum(ss_theta, scratch);
-    const double b = dat_block_sum(ss_u, scratch);
-    if (threadIdx.x == 0) { partials[2 * tile] = a; partials[2 * tile + 1] = b; }
-}
-
-__global__ void __launch_bounds__(DAT_THREADS)
-k_lamb_pass2(float *__restrict__ theta, const float *__restrict__ mom, const float *__restrict__ var,
-             const TileSource tiles, LambConst c, const float *__restrict__ step_a)
-{
-    const int64_t tile = blockIdx.x;
-    const TileRange r = dat_tile_range(tiles, tile);
-    const float na = -__ldg(step_a + r.layer);
-#pragma unroll
-    for (int it = 0; it < DAT_TILE / 4 / DAT_THREADS; ++it) {
-        const int64_t e0 = r.begin + 4 * (int64_t)(it * DAT_THREADS + threadIdx.x);
-        if (e0 < r.end) {
-            float th[4], m[4], v[4];
-            dat_load4(theta, e0, r.lo, r.hi, th);
-            dat_load4(mom, e0, r.lo, r.hi, m);
-            dat_load4(var, e0, r.lo, r.hi, v);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const bool inside = (e0 + j >= r.lo && e0 + j < r.hi);
-                const float u = inside ? dat_lamb_direction(c, m[j], v[j], th[j]) : 0.0f;
-                th[j] = __fmaf_rn(na, u, th[j]);
-            }
-            dat_store4(theta, e0, r.lo, r.hi, th);
-        }
-    }
 }
 
 extern "C" int dat_lamb_step(dat_plan_t *plan, float *theta, float *mom, float *var, const float *g_hat,
@@ -876,14 +908,11 @@ extern "C" int dat_lamb_step(dat_plan_t *plan, float *theta, float *mom, float *
         (layer_norms_out && !dat_aligned16(layer_norms_out)))
         return DAT_ERR_ALIGN;
     cudaStream_t s = (cudaStream_t)stream;
-    const int h = (int)plan->h;
-    const LambConst c = dat_lamb_const(hp, t);
-    k_lamb_pass1<<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(theta, mom, var, g_hat, plan_tiles(plan), c, plan->d_partials);
+    UpdateArgs a = update_args(plan, theta, mom, var, g_hat, hp->lr, hp->c_l, hp->c_u, layer_norms_out);
+    a.lamb = dat_lamb_const(hp, t);
+    k_update_pass1<OPT_LAMB><<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(a);
     DAT_LAUNCHED(plan);
-    k_lalr_finalize<<<h, DAT_THREADS, 0, s>>>(plan->d_tile_base, plan->d_partials, hp->lr, hp->c_l, hp->c_u,
-                                              plan->d_step_a, layer_norms_out, plan->d_status);
-    DAT_LAUNCHED(plan);
-    k_lamb_pass2<<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(theta, mom, var, plan_tiles(plan), c, plan->d_step_a);
+    k_update_pass2<OPT_LAMB><<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(a);
     DAT_LAUNCHED(plan);
     return DAT_OK;
 }
@@ -898,7 +927,7 @@ struct StaticScratch {
     int64_t tile_base[DAT_STATIC_MAX_LAYERS + 1];
     double partials[2 * DAT_STATIC_MAX_TILES];
     float step_a[DAT_STATIC_MAX_LAYERS];
-    uint32_t status;
+    uint32_t status, count[DAT_STATIC_MAX_LAYERS];
 };
 
 static __device__ __align__(256) unsigned char g_static_scratch[sizeof(StaticScratch)];
@@ -951,14 +980,26 @@ extern "C" int dat_lalr_step_static(int64_t num_layers, const int64_t *layer_off
     const size_t table = (size_t)(num_layers + 1) * sizeof(int64_t);
     cudaError_t e = cudaMemcpyAsync(sc->off, layer_offsets, table, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(sc->tile_base, tile_base, table, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(&sc->status, 0, sizeof(uint32_t), s);   // the one word that must start at zero
+    if (e == cudaSuccess) e = cudaMemsetAsync(&sc->status, 0, sizeof(uint32_t) * (size_t)(1 + num_layers), s);   // status and counters start at zero
     if (e != cudaSuccess) { (void)cudaGetLastError(); return DAT_ERR_CUDA; }
-    const int h = (int)num_layers;
-    const TileSource tiles = {nullptr, sc->off, sc->tile_base, h};
-    k_lalr_pass1<<<(unsigned)nt, DAT_THREADS, 0, s>>>(theta, mom, g_hat, tiles, hp->momentum, hp->weight_decay, sc->partials);
-    k_lalr_finalize<<<h, DAT_THREADS, 0, s>>>(sc->tile_base, sc->partials, hp->lr, hp->c_l, hp->c_u, sc->step_a,
-                                              layer_norms_out, &sc->status);
-    k_lalr_pass2<<<(unsigned)nt, DAT_THREADS, 0, s>>>(theta, mom, tiles, sc->step_a);
+    UpdateArgs a = {};
+    a.tiles = TileSource{nullptr, sc->off, sc->tile_base, (int)num_layers};
+    a.theta = theta;
+    a.mom = mom;
+    a.g_hat = g_hat;
+    a.mu = hp->momentum;
+    a.wd = hp->weight_decay;
+    a.lr = hp->lr;
+    a.c_l = hp->c_l;
+    a.c_u = hp->c_u;
+    a.wide = update_wide(theta, mom, nullptr, g_hat);
+    a.partials = sc->partials;
+    a.step_a = sc->step_a;
+    a.norms_out = layer_norms_out;
+    a.count = sc->count;
+    a.status = &sc->status;
+    k_update_pass1<OPT_MOMENTUM><<<(unsigned)nt, DAT_THREADS, 0, s>>>(a);
+    k_update_pass2<OPT_MOMENTUM><<<(unsigned)nt, DAT_THREADS, 0, s>>>(a);
     if (cudaGetLastError() != cudaSuccess) return DAT_ERR_CUDA;
     return DAT_OK;
 }
@@ -973,24 +1014,22 @@ extern "C" int dat_lalr_step_static(int64_t num_layers, const int64_t *layer_off
 template <bool RNG16>
 __global__ void __launch_bounds__(DAT_QU_THREADS, DAT_QU_MINB)
 k_quant_update(const __grid_constant__ GradPtrs gp, const __grid_constant__ PhiloxKeys keys, const __grid_constant__ PhiloxWorkers pw,
-               const TileSource tiles, int M, bool wide,
-               const float *__restrict__ qmul, const float *__restrict__ dq, const float *__restrict__ theta,
-               float *__restrict__ mom, float S_f, float mu, float wd, double *__restrict__ partials,
+               const __grid_constant__ UpdateArgs a, int M, const float *__restrict__ qmul, const float *__restrict__ scales, float S_f, float SM_f,
                int32_t *__restrict__ code_sum)
 {
-    static_assert(DAT_QU_TILE == DAT_TILE, "the plan's tiles");
+    static_assert(DAT_QU_TILE == DAT_TILE && DAT_QU_THREADS == DAT_THREADS, "the plan's tiles");
     __shared__ double scratch[DAT_THREADS / 32];
-    const int64_t tile = blockIdx.x;
-    const TileRange r = dat_tile_range(tiles, tile);
-    const int layer = r.layer;
-    const int64_t lo = r.lo, hi = r.hi, begin = r.begin;
-    const float t = __ldg(qmul + layer), f = __ldg(dq + layer);
-    const QuConst qc = dat_qu_const(t, S_f, wide);
-    const bool plain = dat_qu_plain<RNG16>(qc, begin, DAT_TILE);
+    __shared__ bool s_last;
+    const int64_t tile = (int64_t)gridDim.x - 1 - blockIdx.x;     // back from the last tile: what k_sumsq read last is in L2
+    const TileRange r = dat_tile_range(a.tiles, tile);
+    const int64_t lo = r.lo, hi = r.hi;
+    const float nu = __ldg(scales + r.layer), f = (nu == 0.0f) ? 0.0f : nu / SM_f;
+    const QuConst qc = dat_qu_const(__ldg(qmul + r.layer), S_f, a.wide);
+    const bool plain = dat_qu_plain<RNG16>(qc, r.begin, DAT_TILE);
     double ss_theta = 0.0, ss_u = 0.0;
 #pragma unroll 1
     for (int k = 0; k < DAT_QU_GROUPS; ++k) {
-        const int64_t e0 = begin + 8 * (int64_t)(k * DAT_QU_THREADS + threadIdx.x);
+        const int64_t e0 = r.begin + 8 * (int64_t)(k * DAT_QU_THREADS + threadIdx.x);
         if (e0 >= hi) continue;
         const bool full = (e0 >= lo && e0 + 8 <= hi);
         float acc[8];
@@ -1000,17 +1039,8 @@ k_quant_update(const __grid_constant__ GradPtrs gp, const __grid_constant__ Phil
         else qu_rows_slow<RNG16>(gp, keys, qc, M, e0, lo, hi, acc);
         // theta and m only now: registers are what limits the number of resident warps here
         float th[8], m[8];
-        if (full) {
-            const float4 t0 = __ldcg(reinterpret_cast<const float4 *>(theta + e0)), t1 = __ldcg(reinterpret_cast<const float4 *>(theta + e0) + 1);
-            const float4 m0 = __ldcs(reinterpret_cast<const float4 *>(mom + e0)), m1 = __ldcs(reinterpret_cast<const float4 *>(mom + e0) + 1);
-            th[0] = t0.x; th[1] = t0.y; th[2] = t0.z; th[3] = t0.w; th[4] = t1.x; th[5] = t1.y; th[6] = t1.z; th[7] = t1.w;
-            m[0] = m0.x; m[1] = m0.y; m[2] = m0.z; m[3] = m0.w; m[4] = m1.x; m[5] = m1.y; m[6] = m1.z; m[7] = m1.w;
-        } else {
-            dat_load4(theta, e0, lo, hi, th);
-            dat_load4(theta, e0 + 4, lo, hi, th + 4);
-            dat_load4(mom, e0, lo, hi, m);
-            dat_load4(mom, e0 + 4, lo, hi, m + 4);
-        }
+        update_ld8<EV_LAST>(a.theta, full, a.wide, e0, lo, hi, th);
+        update_ld8<EV_FIRST>(a.mom, full, a.wide, e0, lo, hi, m);
         if (code_sum) {
 #pragma unroll
             for (int j = 0; j < 8; ++j)
@@ -1018,16 +1048,13 @@ k_quant_update(const __grid_constant__ GradPtrs gp, const __grid_constant__ Phil
         }
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            m[j] = __fmaf_rn(mu, m[j], __fmaf_rn(wd, th[j], acc[j] * f));
+            m[j] = __fmaf_rn(a.mu, m[j], __fmaf_rn(a.wd, th[j], acc[j] * f));
             ss_theta = fma((double)th[j], (double)th[j], ss_theta);
             ss_u = fma((double)m[j], (double)m[j], ss_u);
         }
-        dat_store4(mom, e0, lo, hi, m);
-        dat_store4(mom, e0 + 4, lo, hi, m + 4);
+        update_st8<EV_LAST>(a.mom, full, a.wide, e0, lo, hi, m);
     }
-    const double a = dat_block_sum(ss_theta, scratch);
-    const double b = dat_block_sum(ss_u, scratch);
-    if (threadIdx.x == 0) { partials[2 * tile] = a; partials[2 * tile + 1] = b; }
+    update_count_in(a, r, tile, ss_theta, ss_u, scratch, &s_last);
 }
 
 extern "C" int dat_step_passes(dat_plan_t *plan, float *theta, float *mom, const float *const *grads,
@@ -1045,30 +1072,26 @@ extern "C" int dat_step_passes(dat_plan_t *plan, float *theta, float *mom, const
     GradPtrs gp;
     rc = dat_check_grads(plan, grads, &gp);
     if (rc != DAT_OK) return rc;
-    const int h = (int)plan->h;
     cudaStream_t s = (cudaStream_t)stream;
     const float S_f = (float)plan->S;
     const float SM_f = (float)((uint64_t)plan->S * (uint64_t)plan->M);
     rc = sumsq_launch(plan, gp, plan->M, plan->d_scales, false, s);
     if (rc != DAT_OK) return rc;
-    k_dq_from_scales<<<(h + 255) / 256, 256, 0, s>>>(h, SM_f, plan->d_scales, plan->d_dq);
-    DAT_LAUNCHED(plan);
-    if (scales_out) DAT_CUDA(plan, cudaMemcpyAsync(scales_out, plan->d_scales, (size_t)h * 4, cudaMemcpyDeviceToDevice, s));
+    if (scales_out) DAT_CUDA(plan, cudaMemcpyAsync(scales_out, plan->d_scales, (size_t)plan->h * 4, cudaMemcpyDeviceToDevice, s));
     const PhiloxKeys keys = dat_make_keys(seed, step);
     PhiloxWorkers pw;
     dat_make_worker_table(keys, plan->M, &pw);
-    const bool wide = dat_grads_wide(plan, grads);
+    UpdateArgs ua = update_args(plan, theta, mom, nullptr, nullptr, hp->lr, hp->c_l, hp->c_u, layer_norms_out);
+    ua.mu = hp->momentum;
+    ua.wd = hp->weight_decay;
+    ua.wide = ua.wide && dat_grads_wide(plan, grads);
+    const unsigned grid = (unsigned)plan->n_tiles;
     if (plan->rng_bits == 16)
-        k_quant_update<true><<<(unsigned)plan->n_tiles, DAT_QU_THREADS, 0, s>>>(gp, keys, pw, plan_tiles(plan), plan->M, wide, plan->d_qmul, plan->d_dq, theta, mom, S_f, hp->momentum,
-                                                                                 hp->weight_decay, plan->d_partials, code_sum_out);
+        k_quant_update<true><<<grid, DAT_QU_THREADS, 0, s>>>(gp, keys, pw, ua, plan->M, plan->d_qmul, plan->d_scales, S_f, SM_f, code_sum_out);
     else
-        k_quant_update<false><<<(unsigned)plan->n_tiles, DAT_QU_THREADS, 0, s>>>(gp, keys, pw, plan_tiles(plan), plan->M, wide, plan->d_qmul, plan->d_dq, theta, mom, S_f, hp->momentum,
-                                                                                  hp->weight_decay, plan->d_partials, code_sum_out);
+        k_quant_update<false><<<grid, DAT_QU_THREADS, 0, s>>>(gp, keys, pw, ua, plan->M, plan->d_qmul, plan->d_scales, S_f, SM_f, code_sum_out);
     DAT_LAUNCHED(plan);
-    k_lalr_finalize<<<h, DAT_THREADS, 0, s>>>(plan->d_tile_base, plan->d_partials, hp->lr, hp->c_l, hp->c_u, plan->d_step_a,
-                                              layer_norms_out, plan->d_status);
-    DAT_LAUNCHED(plan);
-    k_lalr_pass2<<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(theta, mom, plan_tiles(plan), plan->d_step_a);
+    k_update_pass2<OPT_MOMENTUM><<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(ua);
     DAT_LAUNCHED(plan);
     return DAT_OK;
 }
