@@ -53,11 +53,13 @@ bool dat_grads_wide(const dat_plan_t *plan, const float *const *grads)
 // for 1 - beta^t), the kernels divide.
 ConstDiv dat_const_div(float y)
 {
-    ConstDiv c = {y, 1.0f / y, 0.0f, true};
+    ConstDiv c = {y, 0.0f, 0.0f, false};
+    if (!(y > 1e-30f && y < 1e30f)) return c;
+    c.exact = true;
+    c.hi = 1.0f / y;
     c.lo = fmaf(-y, c.hi, 1.0f) / y;
     int ex;
     const uint64_t Y = (uint64_t)(frexpf(y, &ex) * 16777216.0f);         // 2^23 <= Y < 2^24
-    if (!(y > 1e-30f && y < 1e30f)) { c.exact = false; return c; }
     uint64_t odd = Y;
     int tz = 0;
     while (!(odd & 1)) { odd >>= 1; ++tz; }

@@ -12,6 +12,9 @@
 // HBM-bound (129 us for the 818 MB of ResNet-50, M = 8: 6.3 TB/s); finishing in the same launch instead of a second
 // one takes 8.7 us off (a launch of one CTA per layer, nearly all of it latency).
 // ------------------------------------------------------------------------------------------
+#ifndef SUMSQ_KEEP_BYTES
+#define SUMSQ_KEEP_BYTES (64ll << 20)             // of the last tiles' gradients, that stay in L2
+#endif
 #define SUMSQ_WORKERS 8                           // workers of a tile that one CTA sums, at most (a warp's partials: <= 32)
 
 struct NormOut {
@@ -61,7 +64,7 @@ __device__ __forceinline__ void sumsq_finish(int l, int64_t t0, int64_t t1, int 
 // NW workers' loads in flight per thread.
 template <int NW>
 __global__ void __launch_bounds__(DAT_THREADS, NW == 1 ? 6 : 4)
-k_sumsq(const __grid_constant__ GradPtrs gp, const TileSource tiles, int M, int per_cta, double *partials, const __grid_constant__ NormOut out)
+k_sumsq(const __grid_constant__ GradPtrs gp, const TileSource tiles, int M, int per_cta, int64_t keep_from, double *partials, const __grid_constant__ NormOut out)
 {
     constexpr int W = DAT_THREADS / 32, ITERS = DAT_TILE / 8 / DAT_THREADS;
     __shared__ double s_sum[SUMSQ_WORKERS][W];
@@ -71,6 +74,7 @@ k_sumsq(const __grid_constant__ GradPtrs gp, const TileSource tiles, int M, int 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const TileRange r = dat_tile_range(tiles, tile);
     const bool inside = r.begin >= r.lo && r.begin + DAT_TILE <= r.hi;
+    const bool keep = tile >= keep_from;          // read again first thing by the call that follows (which walks back)
     for (int i = w0; i < w1; i += NW) {           // every load of NW workers is in flight before the first is used
         float v[NW][ITERS][8];
 #pragma unroll
@@ -80,7 +84,10 @@ k_sumsq(const __grid_constant__ GradPtrs gp, const TileSource tiles, int M, int 
 #pragma unroll
             for (int it = 0; it < ITERS; ++it) {
                 const int64_t e0 = r.begin + 8 * (int64_t)(it * DAT_THREADS + threadIdx.x);
-                if (inside && i + p < w1) dat_ld8<EV_FIRST>(g + e0, wide, v[p][it]);
+                if (inside && i + p < w1) {
+                    if (keep) dat_ld8<EV_NORMAL>(g + e0, wide, v[p][it]);
+                    else dat_ld8<EV_FIRST>(g + e0, wide, v[p][it]);
+                }
                 else {
 #pragma unroll
                     for (int j = 0; j < 8; ++j) v[p][it][j] = (i + p < w1 && e0 + j >= r.lo && e0 + j < r.end) ? g[e0 + j] : 0.0f;
@@ -124,8 +131,9 @@ static int sumsq_launch(dat_plan_t *plan, const GradPtrs &gp, int M, float *scal
     int per_cta = 1;
     while (per_cta < SUMSQ_WORKERS && per_cta < M && plan->n_tiles * ((M + 2 * per_cta - 1) / (2 * per_cta)) >= 8 * plan->sm_count) per_cta *= 2;
     dim3 grid((unsigned)plan->n_tiles, (unsigned)((M + per_cta - 1) / per_cta));
-    if (per_cta == 1) k_sumsq<1><<<grid, DAT_THREADS, 0, s>>>(gp, plan_tiles(plan), M, per_cta, plan->d_partials, o);
-    else k_sumsq<2><<<grid, DAT_THREADS, 0, s>>>(gp, plan_tiles(plan), M, per_cta, plan->d_partials, o);
+    const int64_t keep_from = plan->n_tiles - SUMSQ_KEEP_BYTES / (4 * DAT_TILE * M);
+    if (per_cta == 1) k_sumsq<1><<<grid, DAT_THREADS, 0, s>>>(gp, plan_tiles(plan), M, per_cta, keep_from, plan->d_partials, o);
+    else k_sumsq<2><<<grid, DAT_THREADS, 0, s>>>(gp, plan_tiles(plan), M, per_cta, keep_from, plan->d_partials, o);
     DAT_LAUNCHED(plan);
     return DAT_OK;
 }
@@ -155,17 +163,23 @@ __device__ __forceinline__ float quant_mul(const QuantScale &q, int64_t k)
     const float nu = __ldg(q.scales_in + k);
     return (nu == 0.0f) ? 0.0f : q.S_f / nu;
 }
+// The receiver's factor nu/S (one vector, one norm per layer).
+__device__ __forceinline__ float quant_back(const QuantScale &q, int64_t k)
+{
+    const float nu = __ldg((q.scales_in ? q.scales_in : q.scales) + k);
+    return (nu == 0.0f) ? 0.0f : nu / q.S_f;
+}
 
 // A group at the vector's end, across layers, or whose layer's scale is outside the range of the scaled form: the
 // plain form of Eq. xi, element by element.  Leaves the group's packed levels and signs in shared memory.
-template <int BITS>
-__device__ __noinline__ void quantize_slow8(const float *__restrict__ g, int64_t e0, const int64_t *__restrict__ off, int l0, int nl, int64_t d,
+template <int BITS, bool BACK>
+__device__ __noinline__ void quantize_slow8(const float *g, int64_t e0, const int64_t *__restrict__ off, int l0, int nl, int64_t d,
                                             const QuantScale &qs, int64_t q0, uint64_t elem, uint32_t stream, const PhiloxKeys &keys, bool rng16,
-                                            uint8_t *s_level, uint8_t *s_sign)
+                                            uint8_t *s_level, uint8_t *s_sign, float *back)
 {
     uint32_t neg = 0;
     int64_t l_hi = 0;
-    float t = 0.0f;
+    float t = 0.0f, f = 0.0f;
 #pragma unroll 1
     for (int p = 0; p < 2; ++p) {
         float u1[4];
@@ -179,10 +193,13 @@ __device__ __noinline__ void quantize_slow8(const float *__restrict__ g, int64_t
                     const int l = l0 + dat_find(off + l0, nl, e);
                     l_hi = __ldg(off + l + 1);
                     t = quant_mul(qs, q0 + l);
+                    if (BACK) f = quant_back(qs, l);
                 }
                 const float x = g[e];
-                packed |= (uint64_t)dat_level_u1(x, t, (float)(1u << BITS), u1[j]) << (BITS * j);
+                const uint32_t lev = dat_level_u1(x, t, (float)(1u << BITS), u1[j]);
+                packed |= (uint64_t)lev << (BITS * j);
                 neg |= (uint32_t)(x < 0.0f) << (4 * p + j);
+                if (BACK) back[e] = (float)((x < 0.0f) ? -(int)lev : (int)lev) * f;
             }
         }
         if (BITS == 16) reinterpret_cast<uint64_t *>(s_level)[p] = packed;
@@ -196,8 +213,9 @@ __device__ __noinline__ void quantize_slow8(const float *__restrict__ g, int64_t
 
 // Packed levels and signs of one group from its eight elements (lowest first) and random words, by the scaled form:
 // saturation is the clamp to S, min(y, S + 1) 2^-b.
-template <int BITS, bool RNG16>
-__device__ __forceinline__ void quantize8(const float v[8], float ts, const uint32_t w[8], uint8_t *s_level, uint8_t *s_sign)
+// BACK: v becomes the receiver's value, sign * level * f.
+template <int BITS, bool RNG16, bool BACK>
+__device__ __forceinline__ void quantize8(float v[8], float ts, float f, const uint32_t w[8], uint8_t *s_level, uint8_t *s_sign)
 {
     constexpr float TWO_B = (float)(1u << BITS);
     constexpr uint32_t UBITS = (uint32_t)(127 - BITS) << 23;
@@ -211,7 +229,10 @@ __device__ __forceinline__ void quantize8(const float v[8], float ts, const uint
         for (int j = PER - 1; j >= 0; --j) {
             const float x = v[a * PER + j] + 0.0f;           // -0 becomes +0: its sign bit is 0
             const float ys = __saturatef(__fmaf_rn(fabsf(x), ts, dat_u1_scaled<RNG16>(w, a * PER + j, UBITS)));
-            word[a] += __float_as_uint(__fmaf_rz(ys, TWO_B, 8388607.0f)) * (1u << (BITS * j));
+            const float q = __fmaf_rz(ys, TWO_B, 8388607.0f);
+            word[a] += __float_as_uint(q) * (1u << (BITS * j));
+            if (BACK)                             // (a level of 0 gives +0, whatever the sign)
+                v[a * PER + j] = __fmaf_rn(q - 8388608.0f, __uint_as_float((__float_as_uint(x) & 0x80000000u) | 0x3F800000u), 0.0f) * f;
             bias += 0x4B000000u * (1u << (BITS * j));
             neg = __funnelshift_l(__float_as_uint(x), neg, 1);
         }
@@ -225,31 +246,35 @@ __device__ __forceinline__ void quantize8(const float v[8], float ts, const uint
     *s_sign = (uint8_t)neg;
 }
 
-template <int BITS, bool RNG16>
+template <int BITS, bool RNG16, bool BACK>
 __global__ void __launch_bounds__(DAT_THREADS, QUANT_CTAS)
 k_quantize(const __grid_constant__ GradPtrs gp, const __grid_constant__ PhiloxKeys keys, const int64_t *__restrict__ off,
            const int32_t *__restrict__ flat_layer, int h, int64_t d, const __grid_constant__ QuantScale qs, uint8_t *__restrict__ levels,
-           uint8_t *__restrict__ signs, int64_t level_bytes, int64_t sign_bytes, int groups, bool per_worker, uint32_t stream_base, int64_t elem_base)
+           uint8_t *__restrict__ signs, int64_t level_bytes, int64_t sign_bytes, int groups, int n, bool per_worker, uint32_t stream_base,
+           int64_t elem_base, float *back)
 {
     constexpr int MOST = 256 * QUANT_GROUPS;                 // elements of a warp, at most
     __shared__ uint4 s_level[DAT_THREADS / 32][MOST * BITS / 8 / 16];
     __shared__ uint4 s_sign[DAT_THREADS / 32][MOST / 8 / 16];
     const int n_warp = 256 * groups;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int worker = blockIdx.y;
+    // back from the vector's end, the workers side by side: k_sumsq walked forward, tile by tile over the workers, and
+    // what it read last is still in L2
+    const unsigned cta = gridDim.x - 1u - blockIdx.x;
+    const int worker = (int)(cta % (unsigned)n);
     const uint32_t stream = stream_base + (uint32_t)worker;  // the worker's random stream
     if (qs.scales_in) {                                      // copy of the caller's norms, and their check
-        const int64_t n = (int64_t)gridDim.x * gridDim.y * DAT_THREADS;
-        for (int64_t k = ((int64_t)worker * gridDim.x + blockIdx.x) * DAT_THREADS + threadIdx.x; k < qs.n_scales; k += n) {
+        const int64_t step = (int64_t)gridDim.x * DAT_THREADS;
+        for (int64_t k = (int64_t)blockIdx.x * DAT_THREADS + threadIdx.x; k < qs.n_scales; k += step) {
             const float nu = qs.scales_in[k];
             if (qs.scales != qs.scales_in) qs.scales[k] = nu;
             if (!isfinite(nu)) atomicOr(qs.status, DAT_STATUS_NONFINITE);
         }
     }
-    const int64_t part = (int64_t)blockIdx.x * (DAT_THREADS / 32) + warp;
+    const int64_t part = (int64_t)(cta / (unsigned)n) * (DAT_THREADS / 32) + warp;
     const int64_t e_piece = part * n_warp, piece = e_piece / DAT_FLAT, last = min(e_piece + n_warp, d - 1) / DAT_FLAT;
     if (e_piece >= d) return;
-    const float *__restrict__ g = gp.p[worker] + e_piece + 8 * lane;
+    const float *const g = gp.p[worker] + e_piece + 8 * lane;
     const uint64_t elem = (uint64_t)(e_piece + elem_base) + 8u * lane;
     const bool wide = dat_aligned32(gp.p[worker]);
     const bool whole = e_piece + n_warp <= d;
@@ -268,14 +293,15 @@ k_quantize(const __grid_constant__ GradPtrs gp, const __grid_constant__ PhiloxKe
     uint8_t *const my_level = reinterpret_cast<uint8_t *>(s_level[warp]) + lane * BITS, *const my_sign = reinterpret_cast<uint8_t *>(s_sign[warp]) + lane;
     auto scaled = [](float t) { return (t == 0.0f) || (t >= 1.17549435e-38f * TWO_B && t <= 3.402823466e38f); };
     if (whole && page && hi >= e_piece + n_warp && scaled(t0)) {
-        const float ts = t0 * (1.0f / TWO_B);
+        const float ts = t0 * (1.0f / TWO_B), f = BACK ? quant_back(qs, l0) : 0.0f;
 #pragma unroll 1
         for (int k = 0; k < groups; k += 2) {
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
                 uint32_t w[8];
                 dat_group_words<RNG16>(dat_philox_group<RNG16>(elem + 256u * (k + p), keys), pw, keys, w);
-                quantize8<BITS, RNG16>(v[p], ts, w, my_level + (k + p) * 32 * BITS, my_sign + (k + p) * 32);
+                quantize8<BITS, RNG16, BACK>(v[p], ts, f, w, my_level + (k + p) * 32 * BITS, my_sign + (k + p) * 32);
+                if (BACK) dat_st8<EV_LAST>(back + e_piece + 8 * lane + 256 * (k + p), wide, v[p]);
                 if (k + 2 < groups) dat_ld8<EV_FIRST>(g + 256 * (k + p + 2), wide, v[p]);
             }
         }
@@ -285,8 +311,9 @@ k_quantize(const __grid_constant__ GradPtrs gp, const __grid_constant__ PhiloxKe
             const int64_t e0 = e_piece + 8 * lane + 256 * k;
             float t = t0;                                    // the group's layer
             int64_t l_hi = hi;
+            int l = l0;
             if (e0 >= hi && e0 < d) {
-                const int l = l0 + dat_find(off + l0, nl, e0);
+                l = l0 + dat_find(off + l0, nl, e0);
                 l_hi = __ldg(off + l + 1);
                 t = quant_mul(qs, q0 + l);
             }
@@ -295,10 +322,11 @@ k_quantize(const __grid_constant__ GradPtrs gp, const __grid_constant__ PhiloxKe
                 uint32_t w[8];
                 dat_ld8<EV_FIRST>(g + 256 * k, wide, x);
                 dat_group_words<RNG16>(dat_philox_group<RNG16>(elem + 256u * k, keys), pw, keys, w);
-                quantize8<BITS, RNG16>(x, t * (1.0f / TWO_B), w, my_level + k * 32 * BITS, my_sign + k * 32);
+                quantize8<BITS, RNG16, BACK>(x, t * (1.0f / TWO_B), BACK ? quant_back(qs, l) : 0.0f, w, my_level + k * 32 * BITS, my_sign + k * 32);
+                if (BACK) dat_st8<EV_LAST>(back + e0, wide, x);
             } else {
-                quantize_slow8<BITS>(g - e_piece - 8 * lane, e0, off, l0, nl, d, qs, q0, elem + 256u * k, stream, keys, RNG16,
-                                     my_level + k * 32 * BITS, my_sign + k * 32);
+                quantize_slow8<BITS, BACK>(g - e_piece - 8 * lane, e0, off, l0, nl, d, qs, q0, elem + 256u * k, stream, keys, RNG16,
+                                     my_level + k * 32 * BITS, my_sign + k * 32, back);
             }
         }
     }
@@ -319,9 +347,10 @@ k_quantize(const __grid_constant__ GradPtrs gp, const __grid_constant__ PhiloxKe
     }
 }
 
-// Levels of `n` vectors (workers of the plan's streams from `stream_base` on); scales_in as in dat_quantize.
+// Levels of `n` vectors (workers of the plan's streams from `stream_base` on); scales_in as in dat_quantize.  back: the
+// one vector's receiver's value overwrites it (Algorithm A1 Step 10).
 static int quantize_launch(dat_plan_t *plan, const GradPtrs &gp, int n, uint64_t seed, uint64_t step, uint8_t *levels, uint8_t *signs,
-                           float *scales, const float *scales_in, int n_scales, bool per_worker, uint32_t stream_base, cudaStream_t s)
+                           float *scales, const float *scales_in, int n_scales, bool per_worker, uint32_t stream_base, cudaStream_t s, float *back = nullptr)
 {
     const PhiloxKeys keys = dat_make_keys(seed, step);
     const int h = (int)plan->h;
@@ -330,11 +359,12 @@ static int quantize_launch(dat_plan_t *plan, const GradPtrs &gp, int n, uint64_t
     int groups = QUANT_GROUPS;
     auto ctas = [&](int g) { return (plan->d + g * (int64_t)(8 * DAT_THREADS) - 1) / (g * (int64_t)(8 * DAT_THREADS)); };
     while (groups > 2 && ctas(groups) * n < 4ll * QUANT_CTAS * plan->sm_count) groups /= 2;
-    dim3 grid((unsigned)ctas(groups), (unsigned)n);
-#define DAT_Q(B, R)                                                                                                              \
-    k_quantize<B, R><<<grid, DAT_THREADS, 0, s>>>(gp, keys, plan->d_offsets, plan->d_flat_layer, h, plan->d, qs, levels, signs, \
-                                                  plan->level_bytes, plan->sign_bytes, groups, per_worker, stream_base, plan->elem_base)
-#define DAT_QR(B) do { if (plan->rng_bits == 16) DAT_Q(B, true); else DAT_Q(B, false); } while (0)
+    const unsigned grid = (unsigned)(ctas(groups) * n);
+#define DAT_Q(B, R, K)                                                                                                          \
+    k_quantize<B, R, K><<<grid, DAT_THREADS, 0, s>>>(gp, keys, plan->d_offsets, plan->d_flat_layer, h, plan->d, qs, levels, signs, \
+                                                     plan->level_bytes, plan->sign_bytes, groups, n, per_worker, stream_base, plan->elem_base, back)
+#define DAT_QK(B, R) do { if (back) DAT_Q(B, R, true); else DAT_Q(B, R, false); } while (0)
+#define DAT_QR(B) do { if (plan->rng_bits == 16) DAT_QK(B, true); else DAT_QK(B, false); } while (0)
     switch (plan->bits) {
     case 1: DAT_QR(1); break;
     case 2: DAT_QR(2); break;
@@ -343,6 +373,7 @@ static int quantize_launch(dat_plan_t *plan, const GradPtrs &gp, int n, uint64_t
     default: DAT_QR(16); break;
     }
 #undef DAT_QR
+#undef DAT_QK
 #undef DAT_Q
     DAT_LAUNCHED(plan);
     return DAT_OK;
@@ -391,17 +422,8 @@ extern "C" int dat_worker_norms(dat_plan_t *plan, const float *const *grads, flo
 }
 
 // ------------------------------------------------------------------------------------------
-// S4 + S5: unpack, integer sum over workers, one scaling.  Each thread owns 8 consecutive
-// elements (b bytes of levels and one sign byte per worker).
+// S4 + S5: unpack, integer sum over workers, one scaling.
 // ------------------------------------------------------------------------------------------
-__global__ void k_dq_from_scales(int h, float SM_f, const float *__restrict__ scales, float *__restrict__ dq)
-{
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= h) return;
-    const float nu = scales[l];
-    dq[l] = (nu == 0.0f) ? 0.0f : nu / SM_f;
-}
-
 template <int BITS>
 __device__ __forceinline__ void dat_unpack8(const uint8_t *__restrict__ plane, int64_t e0, uint32_t lev[8])
 {
@@ -439,53 +461,141 @@ struct PlanesTable {
     __device__ __forceinline__ const uint8_t *sg(int i) const { return signs[i]; }
 };
 
+// A thread owns 16 consecutive elements and takes four workers at a time: their bytes are transposed, so that one
+// four-way dot product (DP4A, two at 16 bits) adds the four workers' signed levels of an element -- per element and
+// worker about one issue slot instead of five for unpacking, negating and adding one level at a time, which limited
+// this kernel (75 us for 332 MB at M = 8, b = 8; 50 us for 157 MB at M = 16, b = 4).
+// The words of one worker: 16 levels, two sign bytes.
+template <int BITS> struct AggWords { uint32_t lv[BITS / 2 > 0 ? BITS / 2 : 1]; uint32_t sg; };
+
 template <int BITS, class SRC>
-__global__ void __launch_bounds__(DAT_THREADS)
-k_aggregate(const __grid_constant__ SRC src, int M, const int64_t *__restrict__ off, int h, int64_t d,
-            const float *__restrict__ dq, int32_t *__restrict__ code_sum, float *__restrict__ g_hat)
+__device__ __forceinline__ AggWords<BITS> agg_load(const SRC &src, int i, int M, int64_t e0, bool tail)
 {
-    __shared__ int s_first;
-    const int64_t e_blk = (int64_t)blockIdx.x * (DAT_THREADS * 8);
-    if (threadIdx.x == 0) s_first = dat_find(off, h, e_blk);
-    __syncthreads();
-    const int64_t e0 = e_blk + 8 * (int64_t)threadIdx.x;
-    if (e0 >= d) return;
-    int sum[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) sum[j] = 0;
-#pragma unroll 4
-    for (int i = 0; i < M; ++i) {                // four workers' loads in flight at a time
-        uint32_t lev[8];
-        dat_unpack8<BITS>(src.lv(i), e0, lev);
-        const uint32_t sg = src.sg(i)[e0 >> 3];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) sum[j] += ((sg >> j) & 1u) ? -(int)lev[j] : (int)lev[j];
-    }
-    int l = s_first;
-    int64_t l_hi = __ldg(off + l + 1);
-    float f = __ldg(dq + l);
-    float out[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const int64_t e = e0 + j;
-        while (e >= l_hi && l + 1 < h) {
-            ++l;
-            l_hi = __ldg(off + l + 1);
-            f = __ldg(dq + l);
+    AggWords<BITS> w = {};
+    if (i >= M) return w;                        // absent workers add level 0
+    const uint8_t *p = src.lv(i) + e0 * BITS / 8;
+    const uint8_t *q = src.sg(i) + (e0 >> 3);
+    if (BITS == 16) {
+        const uint4 a = __ldcs(reinterpret_cast<const uint4 *>(p));
+        w.lv[0] = a.x; w.lv[1 % (BITS / 2 + 1)] = a.y; w.lv[2 % (BITS / 2 + 1)] = a.z; w.lv[3 % (BITS / 2 + 1)] = a.w;
+        if (!tail) {                             // (the plane's padding ends with the first eight elements)
+            const uint4 b = __ldcs(reinterpret_cast<const uint4 *>(p) + 1);
+            w.lv[4 % (BITS / 2 + 1)] = b.x; w.lv[5 % (BITS / 2 + 1)] = b.y; w.lv[6 % (BITS / 2 + 1)] = b.z; w.lv[7 % (BITS / 2 + 1)] = b.w;
         }
-        out[j] = (float)sum[j] * f;
-    }
-    if (e0 + 8 <= d) {
-        reinterpret_cast<float4 *>(g_hat + e0)[0] = make_float4(out[0], out[1], out[2], out[3]);
-        reinterpret_cast<float4 *>(g_hat + e0)[1] = make_float4(out[4], out[5], out[6], out[7]);
-        if (code_sum) {
-            reinterpret_cast<int4 *>(code_sum + e0)[0] = make_int4(sum[0], sum[1], sum[2], sum[3]);
-            reinterpret_cast<int4 *>(code_sum + e0)[1] = make_int4(sum[4], sum[5], sum[6], sum[7]);
-        }
+    } else if (BITS == 8) {                      // planes are padded to 16 bytes: whatever the group holds, its words exist
+        const uint4 a = __ldcs(reinterpret_cast<const uint4 *>(p));
+        w.lv[0] = a.x; w.lv[1 % (BITS / 2 + 1)] = a.y; w.lv[2 % (BITS / 2 + 1)] = a.z; w.lv[3 % (BITS / 2 + 1)] = a.w;
+    } else if (BITS == 4) {
+        const uint2 a = __ldcs(reinterpret_cast<const uint2 *>(p));
+        w.lv[0] = a.x; w.lv[1 % (BITS / 2 + 1)] = a.y;
+    } else if (BITS == 2) {
+        w.lv[0] = __ldcs(reinterpret_cast<const uint32_t *>(p));
     } else {
-        for (int j = 0; j < 8 && e0 + j < d; ++j) {
-            g_hat[e0 + j] = out[j];
-            if (code_sum) code_sum[e0 + j] = sum[j];
+        w.lv[0] = __ldcs(reinterpret_cast<const uint16_t *>(p));
+    }
+    w.sg = __ldcs(reinterpret_cast<const uint16_t *>(q));
+    return w;
+}
+
+// out[k] = byte k of the four words, one byte per word: a 4x4 transpose.
+__device__ __forceinline__ void agg_transpose(uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t out[4])
+{
+    const uint32_t ab0 = __byte_perm(a, b, 0x5140), ab1 = __byte_perm(a, b, 0x7362);
+    const uint32_t cd0 = __byte_perm(c, d, 0x5140), cd1 = __byte_perm(c, d, 0x7362);
+    out[0] = __byte_perm(ab0, cd0, 0x5410);
+    out[1] = __byte_perm(ab0, cd0, 0x7632);
+    out[2] = __byte_perm(ab1, cd1, 0x5410);
+    out[3] = __byte_perm(ab1, cd1, 0x7632);
+}
+
+__device__ __forceinline__ int agg_dp4(uint32_t u, uint32_t s, int c)      // c + sum of unsigned bytes times signed bytes
+{
+    int r;
+    asm("dp4a.u32.s32 %0, %1, %2, %3;" : "=r"(r) : "r"(u), "r"(s), "r"(c));
+    return r;
+}
+__device__ __forceinline__ int agg_dp2(uint32_t u, uint32_t s, int c)      // c + sum of unsigned halves times the low signed bytes
+{
+    int r;
+    asm("dp2a.lo.u32.s32 %0, %1, %2, %3;" : "=r"(r) : "r"(u), "r"(s), "r"(c));
+    return r;
+}
+
+template <int BITS>
+__device__ __forceinline__ void agg_add4(const AggWords<BITS> w[4], int sum[16])
+{
+    uint32_t sg[4];
+    agg_transpose(w[0].sg, w[1].sg, w[2].sg, w[3].sg, sg);                  // sg[0], sg[1]: the sign bytes of elements 0-7, 8-15
+    constexpr int PER = (BITS < 8) ? 8 / BITS : 1;                          // levels in a byte
+    constexpr uint32_t MASK = (BITS >= 8) ? 0xFFFFFFFFu : ((1u << BITS) - 1u) * 0x01010101u;
+    uint32_t by[4];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        // the workers' signs as bytes +1 / -1
+        const uint32_t s = ((sg[j >> 3] >> (j & 7)) & 0x01010101u) * 0xFEu + 0x01010101u;
+        if (BITS == 16) {
+            const uint32_t a = __byte_perm(w[0].lv[(j >> 1) % (BITS / 2 + 1)], w[1].lv[(j >> 1) % (BITS / 2 + 1)], (j & 1) ? 0x7632 : 0x5410);
+            const uint32_t b = __byte_perm(w[2].lv[(j >> 1) % (BITS / 2 + 1)], w[3].lv[(j >> 1) % (BITS / 2 + 1)], (j & 1) ? 0x7632 : 0x5410);
+            sum[j] = agg_dp2(b, s >> 16, agg_dp2(a, s, sum[j]));
+        } else {
+            const int byte = j / PER;                                       // of the worker's 2 * BITS level bytes
+            if (byte % 4 == 0 && j % PER == 0) agg_transpose(w[0].lv[byte / 4], w[1].lv[byte / 4], w[2].lv[byte / 4], w[3].lv[byte / 4], by);
+            sum[j] = agg_dp4((by[byte % 4] >> (BITS * (j % PER) % 8)) & MASK, s, sum[j]);
+        }
+    }
+}
+
+template <int BITS, class SRC>
+__global__ void __launch_bounds__(DAT_THREADS, 4)
+k_aggregate(const __grid_constant__ SRC src, int M, const int64_t *__restrict__ off, const int32_t *__restrict__ flat_layer, int64_t d,
+            const float *__restrict__ scales, float SM_f, bool wide, int32_t *__restrict__ code_sum, float *__restrict__ g_hat)
+{
+    const int64_t e0 = 16 * ((int64_t)blockIdx.x * DAT_THREADS + threadIdx.x);
+    if (e0 >= d) return;
+    const bool tail = BITS == 16 && e0 + 8 >= d;
+    int sum[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) sum[j] = 0;
+#pragma unroll 1
+    for (int i = 0; i < M; i += 4) {
+        AggWords<BITS> w[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[k] = agg_load<BITS>(src, i + k, M, e0, tail);
+        agg_add4<BITS>(w, sum);
+    }
+    const int64_t piece = e0 / DAT_FLAT;
+    const int l0 = __ldg(flat_layer + piece), nl = __ldg(flat_layer + piece + 1) - l0 + 1;
+    int l = l0 + ((nl > 1) ? dat_find(off + l0, nl, e0) : 0);
+    int64_t l_hi = __ldg(off + l + 1);
+    float nu = __ldg(scales + l), f = (nu == 0.0f) ? 0.0f : nu / SM_f;
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        const int64_t e = e0 + 8 * p;
+        if (e >= d) break;
+        float out[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            while (e + j >= l_hi && e + j < d) {
+                ++l;
+                l_hi = __ldg(off + l + 1);
+                nu = __ldg(scales + l);
+                f = (nu == 0.0f) ? 0.0f : nu / SM_f;
+            }
+            out[j] = (float)sum[8 * p + j] * f;
+        }
+        if (e + 8 <= d) {
+            dat_st8<EV_LAST>(g_hat + e, wide, out);          // the update that follows reads it
+            if (code_sum) {
+                reinterpret_cast<int4 *>(code_sum + e)[0] = make_int4(sum[8 * p], sum[8 * p + 1], sum[8 * p + 2], sum[8 * p + 3]);
+                reinterpret_cast<int4 *>(code_sum + e)[1] = make_int4(sum[8 * p + 4], sum[8 * p + 5], sum[8 * p + 6], sum[8 * p + 7]);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (e + j < d) {
+                    g_hat[e + j] = out[j];
+                    if (code_sum) code_sum[e + j] = sum[8 * p + j];
+                }
         }
     }
 }
@@ -495,18 +605,16 @@ k_aggregate(const __grid_constant__ SRC src, int M, const int64_t *__restrict__ 
 // multiply-add per worker, in ascending worker order.
 template <int BITS, class SRC>
 __global__ void __launch_bounds__(DAT_THREADS)
-k_aggregate_per_worker(const __grid_constant__ SRC src, int M, const int64_t *__restrict__ off, int h, int64_t d,
-                       const float *__restrict__ scales, float SM_f, float *__restrict__ g_hat)
+k_aggregate_per_worker(const __grid_constant__ SRC src, int M, const int64_t *__restrict__ off, const int32_t *__restrict__ flat_layer, int h,
+                       int64_t d, const float *__restrict__ scales, float SM_f, float *__restrict__ g_hat)
 {
-    __shared__ int s_first;
-    const int64_t e_blk = (int64_t)blockIdx.x * (DAT_THREADS * 8);
-    if (threadIdx.x == 0) s_first = dat_find(off, h, e_blk);
-    __syncthreads();
-    const int64_t e0 = e_blk + 8 * (int64_t)threadIdx.x;
+    const int64_t e0 = 8 * ((int64_t)blockIdx.x * DAT_THREADS + threadIdx.x);
     if (e0 >= d) return;
     int lidx[8];
     {
-        int l = s_first;
+        const int64_t piece = e0 / DAT_FLAT;
+        const int l0 = __ldg(flat_layer + piece), nl = __ldg(flat_layer + piece + 1) - l0 + 1;
+        int l = l0 + ((nl > 1) ? dat_find(off + l0, nl, e0) : 0);
         int64_t l_hi = __ldg(off + l + 1);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
@@ -549,9 +657,9 @@ k_aggregate_per_worker(const __grid_constant__ SRC src, int M, const int64_t *__
 }
 
 // ------------------------------------------------------------------------------------------
-// Algorithm A1 Step 10 (two-sided quantisation): g_hat <- Q(g_hat) at the server.  The same
-// kernels as Steps 7 and 9 on ONE vector: norm per layer, levels on the random stream of index M
-// (the first one no worker uses), packed message, and the receiver's value nu_l * sign * level / S.
+// Algorithm A1 Step 10 (two-sided quantisation): g_hat <- Q(g_hat) at the server.  The kernels of Step 7 on ONE
+// vector: norm per layer, levels on the random stream of index M (the first one no worker uses), packed message; the
+// receiver's value nu_l * sign * level / S is written back by the kernel that draws the level.
 // ------------------------------------------------------------------------------------------
 extern "C" int dat_requantize(dat_plan_t *plan, float *g_hat, uint64_t seed, uint64_t step,
                               uint8_t *levels, uint8_t *signs, float *scales, const float *scales_in,
@@ -570,31 +678,15 @@ extern "C" int dat_requantize(dat_plan_t *plan, float *g_hat, uint64_t seed, uin
     gp.p[0] = g_hat;
 
     cudaStream_t s = (cudaStream_t)stream;
-    const int h = (int)plan->h;
-    const float S_f = (float)plan->S;
     if (!scales_in) {
         rc = sumsq_launch(plan, gp, 1, scales, false, s);
         if (rc != DAT_OK) return rc;
     }
-    rc = quantize_launch(plan, gp, 1, seed, step, levels, signs, scales, scales_in, h, false, plan->worker_base + (uint32_t)plan->M, s);
-    if (rc != DAT_OK) return rc;
-    const unsigned agrid = (unsigned)((plan->d + DAT_THREADS * 8 - 1) / (DAT_THREADS * 8));
-    k_dq_from_scales<<<(h + 255) / 256, 256, 0, s>>>(h, S_f, scales, plan->d_dq);      // nu / (S * 1)
-    DAT_LAUNCHED(plan);
-#define DAT_RQ(B)                                                                                                   \
-    k_aggregate<B, PlanesFlat><<<agrid, DAT_THREADS, 0, s>>>(PlanesFlat{levels, signs, plan->level_bytes, plan->sign_bytes}, 1, \
-                                                             plan->d_offsets, h, plan->d, plan->d_dq, nullptr, g_hat)
-    switch (plan->bits) {
-    case 1: DAT_RQ(1); break;
-    case 2: DAT_RQ(2); break;
-    case 4: DAT_RQ(4); break;
-    case 8: DAT_RQ(8); break;
-    default: DAT_RQ(16); break;
-    }
-#undef DAT_RQ
-    DAT_LAUNCHED(plan);
-    return DAT_OK;
+    return quantize_launch(plan, gp, 1, seed, step, levels, signs, scales, scales_in, (int)plan->h, false,
+                           plan->worker_base + (uint32_t)plan->M, s, g_hat);
 }
+
+static bool dat_aligned32_host(const void *p) { return ((uintptr_t)p & 31u) == 0; }
 
 template <class SRC>
 static int aggregate_launch(dat_plan_t *plan, const SRC &src, const float *scales, int32_t *code_sum, float *g_hat, void *stream)
@@ -606,7 +698,7 @@ static int aggregate_launch(dat_plan_t *plan, const SRC &src, const float *scale
     if (plan->scale_mode == DAT_SCALE_PER_WORKER) {
         if (code_sum) return DAT_ERR_ARG;        // differently scaled codes have no integer sum
 #define DAT_APW(B)                                                                                                  \
-    k_aggregate_per_worker<B, SRC><<<grid, DAT_THREADS, 0, s>>>(src, plan->M, plan->d_offsets, h, plan->d, scales, SM_f, g_hat)
+    k_aggregate_per_worker<B, SRC><<<grid, DAT_THREADS, 0, s>>>(src, plan->M, plan->d_offsets, plan->d_flat_layer, h, plan->d, scales, SM_f, g_hat)
         switch (plan->bits) {
         case 1: DAT_APW(1); break;
         case 2: DAT_APW(2); break;
@@ -618,10 +710,10 @@ static int aggregate_launch(dat_plan_t *plan, const SRC &src, const float *scale
         DAT_LAUNCHED(plan);
         return DAT_OK;
     }
-    k_dq_from_scales<<<(h + 255) / 256, 256, 0, s>>>(h, SM_f, scales, plan->d_dq);
-    DAT_LAUNCHED(plan);
-#define DAT_A(B)                                                                                         \
-    k_aggregate<B, SRC><<<grid, DAT_THREADS, 0, s>>>(src, plan->M, plan->d_offsets, h, plan->d, plan->d_dq, code_sum, g_hat)
+    const unsigned grid16 = (unsigned)((plan->d + DAT_THREADS * 16 - 1) / (DAT_THREADS * 16));
+#define DAT_A(B)                                                                                                                 \
+    k_aggregate<B, SRC><<<grid16, DAT_THREADS, 0, s>>>(src, plan->M, plan->d_offsets, plan->d_flat_layer, plan->d, scales, SM_f, \
+                                                       dat_aligned32_host(g_hat), code_sum, g_hat)
     switch (plan->bits) {
     case 1: DAT_A(1); break;
     case 2: DAT_A(2); break;
