@@ -12,9 +12,7 @@
 // HBM-bound (129 us for the 818 MB of ResNet-50, M = 8: 6.3 TB/s); finishing in the same launch instead of a second
 // one takes 8.7 us off (a launch of one CTA per layer, nearly all of it latency).
 // ------------------------------------------------------------------------------------------
-#ifndef SUMSQ_KEEP_BYTES
 #define SUMSQ_KEEP_BYTES (64ll << 20)             // of the last tiles' gradients, that stay in L2
-#endif
 #define SUMSQ_WORKERS 8                           // workers of a tile that one CTA sums, at most (a warp's partials: <= 32)
 
 struct NormOut {
@@ -170,13 +168,27 @@ __device__ __forceinline__ float quant_back(const QuantScale &q, int64_t k)
     return (nu == 0.0f) ? 0.0f : nu / q.S_f;
 }
 
+struct QuantArgs {
+    GradPtrs gp;
+    PhiloxKeys keys;
+    QuantScale qs;
+    const int64_t *off;
+    const int32_t *flat_layer;
+    uint8_t *levels, *signs;
+    float *back;                                 // the receiver's value, if it is wanted
+    int64_t d, level_bytes, sign_bytes, elem_base;
+    uint32_t stream_base;
+    int h, n, groups;
+    bool per_worker;
+};
+
 // A group at the vector's end, across layers, or whose layer's scale is outside the range of the scaled form: the
 // plain form of Eq. xi, element by element.  Leaves the group's packed levels and signs in shared memory.
-template <int BITS, bool BACK>
-__device__ __noinline__ void quantize_slow8(const float *g, int64_t e0, const int64_t *__restrict__ off, int l0, int nl, int64_t d,
-                                            const QuantScale &qs, int64_t q0, uint64_t elem, uint32_t stream, const PhiloxKeys &keys, bool rng16,
-                                            uint8_t *s_level, uint8_t *s_sign, float *back)
+template <int BITS, bool RNG16, bool BACK>
+__device__ __forceinline__ void quantize_slow8(const QuantArgs &a, int worker, int64_t e0, int l0, int nl, uint8_t *s_level, uint8_t *s_sign)
 {
+    const float *g = a.gp.p[worker];
+    const int64_t q0 = a.per_worker ? (int64_t)worker * a.h : 0;
     uint32_t neg = 0;
     int64_t l_hi = 0;
     float t = 0.0f, f = 0.0f;
@@ -184,22 +196,22 @@ __device__ __noinline__ void quantize_slow8(const float *g, int64_t e0, const in
     for (int p = 0; p < 2; ++p) {
         float u1[4];
         uint64_t packed = 0;
-        dat_u1x4(elem + 4 * p, stream, keys, rng16, u1);
+        dat_u1x4((uint64_t)(e0 + a.elem_base) + 4 * p, a.stream_base + (uint32_t)worker, a.keys, RNG16, u1);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int64_t e = e0 + 4 * p + j;
-            if (e < d) {
+            if (e < a.d) {
                 if (e >= l_hi) {                  // (also the first element: l_hi = 0)
-                    const int l = l0 + dat_find(off + l0, nl, e);
-                    l_hi = __ldg(off + l + 1);
-                    t = quant_mul(qs, q0 + l);
-                    if (BACK) f = quant_back(qs, l);
+                    const int l = l0 + dat_find(a.off + l0, nl, e);
+                    l_hi = __ldg(a.off + l + 1);
+                    t = quant_mul(a.qs, q0 + l);
+                    if (BACK) f = quant_back(a.qs, l);
                 }
                 const float x = g[e];
                 const uint32_t lev = dat_level_u1(x, t, (float)(1u << BITS), u1[j]);
                 packed |= (uint64_t)lev << (BITS * j);
                 neg |= (uint32_t)(x < 0.0f) << (4 * p + j);
-                if (BACK) back[e] = (float)((x < 0.0f) ? -(int)lev : (int)lev) * f;
+                if (BACK) a.back[e] = (float)((x < 0.0f) ? -(int)lev : (int)lev) * f;
             }
         }
         if (BITS == 16) reinterpret_cast<uint64_t *>(s_level)[p] = packed;
@@ -246,103 +258,124 @@ __device__ __forceinline__ void quantize8(float v[8], float ts, float f, const u
     *s_sign = (uint8_t)neg;
 }
 
+template <int BITS>
+__device__ __forceinline__ bool quant_scaled(float t)        // the scaled form's range: t 2^-b a normal number
+{
+    constexpr float TWO_B = (float)(1u << BITS);
+    return (t == 0.0f) || (t >= 1.17549435e-38f * TWO_B && t <= 3.402823466e38f);
+}
+
+// A warp's part that is not the plain case of the kernel below: several layers, the vector's end, a 16-byte aligned
+// buffer.  (A call, so that what it keeps in registers is its own.)
+template <int BITS, bool RNG16, bool BACK>
+__device__ __noinline__ void quantize_mixed(const QuantArgs &a, int worker, int64_t e_piece, uint8_t *s_level, uint8_t *s_sign)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t piece = e_piece / DAT_FLAT, last = min(e_piece + 256 * a.groups, a.d - 1) / DAT_FLAT;
+    const int l0 = __ldg(a.flat_layer + piece), nl = __ldg(a.flat_layer + last + 1) - l0 + 1;   // the layers are among [l0, l0 + nl)
+    const int64_t q0 = a.per_worker ? (int64_t)worker * a.h : 0;
+    const float *const g = a.gp.p[worker];
+    const bool wide = dat_aligned32(g);
+    const bool page = dat_one_counter_page<RNG16>((uint64_t)(e_piece + a.elem_base), 256 * a.groups);
+    const PhiloxWorker pw = dat_philox_worker((uint32_t)((uint64_t)(e_piece + a.elem_base) >> (RNG16 ? 35 : 34)), a.stream_base + (uint32_t)worker, a.keys);
+    int64_t l_hi = 0;
+    int l = l0;
+    float t = 0.0f;
+#pragma unroll 1
+    for (int k = 0; k < a.groups; ++k) {
+        const int64_t e0 = e_piece + 8 * lane + 256 * k;
+        uint8_t *const my_level = s_level + (lane + 32 * k) * BITS, *const my_sign = s_sign + lane + 32 * k;
+        if (e0 < a.d && e0 >= l_hi) {                        // the group's layer
+            l = l0 + dat_find(a.off + l0, nl, e0);
+            l_hi = __ldg(a.off + l + 1);
+            t = quant_mul(a.qs, q0 + l);
+        }
+        if (page && quant_scaled<BITS>(t) && e0 + 8 <= l_hi) {
+            float x[8];
+            uint32_t w[8];
+            dat_ld8<EV_FIRST>(g + e0, wide, x);
+            dat_group_words<RNG16>(dat_philox_group<RNG16>((uint64_t)(e0 + a.elem_base), a.keys), pw, a.keys, w);
+            quantize8<BITS, RNG16, BACK>(x, t * (1.0f / (float)(1u << BITS)), BACK ? quant_back(a.qs, l) : 0.0f, w, my_level, my_sign);
+            if (BACK) dat_st8<EV_LAST>(a.back + e0, wide, x);
+        } else {
+            quantize_slow8<BITS, RNG16, BACK>(a, worker, e0, l0, nl, my_level, my_sign);
+        }
+    }
+}
+
 template <int BITS, bool RNG16, bool BACK>
 __global__ void __launch_bounds__(DAT_THREADS, QUANT_CTAS)
-k_quantize(const __grid_constant__ GradPtrs gp, const __grid_constant__ PhiloxKeys keys, const int64_t *__restrict__ off,
-           const int32_t *__restrict__ flat_layer, int h, int64_t d, const __grid_constant__ QuantScale qs, uint8_t *__restrict__ levels,
-           uint8_t *__restrict__ signs, int64_t level_bytes, int64_t sign_bytes, int groups, int n, bool per_worker, uint32_t stream_base,
-           int64_t elem_base, float *back)
+k_quantize(const __grid_constant__ QuantArgs a)
 {
     constexpr int MOST = 256 * QUANT_GROUPS;                 // elements of a warp, at most
     __shared__ uint4 s_level[DAT_THREADS / 32][MOST * BITS / 8 / 16];
     __shared__ uint4 s_sign[DAT_THREADS / 32][MOST / 8 / 16];
-    const int n_warp = 256 * groups;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // back from the vector's end, the workers side by side: k_sumsq walked forward, tile by tile over the workers, and
     // what it read last is still in L2
     const unsigned cta = gridDim.x - 1u - blockIdx.x;
-    const int worker = (int)(cta % (unsigned)n);
-    const uint32_t stream = stream_base + (uint32_t)worker;  // the worker's random stream
-    if (qs.scales_in) {                                      // copy of the caller's norms, and their check
-        const int64_t step = (int64_t)gridDim.x * DAT_THREADS;
-        for (int64_t k = (int64_t)blockIdx.x * DAT_THREADS + threadIdx.x; k < qs.n_scales; k += step) {
-            const float nu = qs.scales_in[k];
-            if (qs.scales != qs.scales_in) qs.scales[k] = nu;
-            if (!isfinite(nu)) atomicOr(qs.status, DAT_STATUS_NONFINITE);
+    const int worker = (int)(cta % (unsigned)a.n);
+    if (a.qs.scales_in) {                                    // copy of the caller's norms, and their check
+        for (int64_t k = (int64_t)blockIdx.x * DAT_THREADS + threadIdx.x; k < a.qs.n_scales; k += (int64_t)gridDim.x * DAT_THREADS) {
+            const float nu = a.qs.scales_in[k];
+            if (a.qs.scales != a.qs.scales_in) a.qs.scales[k] = nu;
+            if (!isfinite(nu)) atomicOr(a.qs.status, DAT_STATUS_NONFINITE);
         }
     }
-    const int64_t part = (int64_t)(cta / (unsigned)n) * (DAT_THREADS / 32) + warp;
-    const int64_t e_piece = part * n_warp, piece = e_piece / DAT_FLAT, last = min(e_piece + n_warp, d - 1) / DAT_FLAT;
-    if (e_piece >= d) return;
-    const float *const g = gp.p[worker] + e_piece + 8 * lane;
-    const uint64_t elem = (uint64_t)(e_piece + elem_base) + 8u * lane;
-    const bool wide = dat_aligned32(gp.p[worker]);
-    const bool whole = e_piece + n_warp <= d;
+    const int64_t part = (int64_t)(cta / (unsigned)a.n) * (DAT_THREADS / 32) + warp, e_piece = part * (256 * a.groups);
+    if (e_piece >= a.d) return;
+    const float *ahead = a.gp.p[worker] + e_piece + 8 * lane;
+    const bool whole = dat_aligned32(a.gp.p[worker]) && e_piece + 256 * a.groups <= a.d;
     float v[2][8];
     if (whole) {                                             // two groups per lane are always in flight
-        dat_ld8<EV_FIRST>(g, wide, v[0]);
-        dat_ld8<EV_FIRST>(g + 256, wide, v[1]);
+        dat_ld8<EV_FIRST>(ahead, true, v[0]);
+        dat_ld8<EV_FIRST>(ahead + 256, true, v[1]);
     }
-    const int l0 = __ldg(flat_layer + piece), nl = __ldg(flat_layer + last + 1) - l0 + 1;   // the warp's layers are among [l0, l0 + nl)
-    const int64_t q0 = per_worker ? (int64_t)worker * h : 0;
-    const int64_t hi = __ldg(off + l0 + 1);                  // end of the first layer
-    const float t0 = quant_mul(qs, q0 + l0);
-    constexpr float TWO_B = (float)(1u << BITS);
-    const bool page = dat_one_counter_page<RNG16>(elem - 8u * lane, n_warp);
-    const PhiloxWorker pw = dat_philox_worker((uint32_t)((elem - 8u * lane) >> (RNG16 ? 35 : 34)), stream, keys);
-    uint8_t *const my_level = reinterpret_cast<uint8_t *>(s_level[warp]) + lane * BITS, *const my_sign = reinterpret_cast<uint8_t *>(s_sign[warp]) + lane;
-    auto scaled = [](float t) { return (t == 0.0f) || (t >= 1.17549435e-38f * TWO_B && t <= 3.402823466e38f); };
-    if (whole && page && hi >= e_piece + n_warp && scaled(t0)) {
-        const float ts = t0 * (1.0f / TWO_B), f = BACK ? quant_back(qs, l0) : 0.0f;
+    const int l0 = __ldg(a.flat_layer + e_piece / DAT_FLAT);
+    const float t = quant_mul(a.qs, (a.per_worker ? (int64_t)worker * a.h : 0) + l0);
+    if (whole && __ldg(a.off + l0 + 1) >= e_piece + 256 * a.groups && quant_scaled<BITS>(t) &&
+        dat_one_counter_page<RNG16>((uint64_t)(e_piece + a.elem_base), 256 * a.groups)) {
+        const float ts = t * (1.0f / (float)(1u << BITS)), f = BACK ? quant_back(a.qs, l0) : 0.0f;
+        const PhiloxWorker pw = dat_philox_worker((uint32_t)((uint64_t)(e_piece + a.elem_base) >> (RNG16 ? 35 : 34)), a.stream_base + (uint32_t)worker, a.keys);
+        uint32_t counter = (uint32_t)((uint64_t)(e_piece + a.elem_base) >> (RNG16 ? 3 : 2)) + (RNG16 ? 1u : 2u) * lane;
+        uint8_t *to_level = reinterpret_cast<uint8_t *>(s_level[warp]) + lane * BITS, *to_sign = reinterpret_cast<uint8_t *>(s_sign[warp]) + lane;
+        float *back = BACK ? a.back + e_piece + 8 * lane : nullptr;
+        ahead += 512;
 #pragma unroll 1
-        for (int k = 0; k < groups; k += 2) {
+        for (int k = a.groups; k > 0; k -= 2) {
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
                 uint32_t w[8];
-                dat_group_words<RNG16>(dat_philox_group<RNG16>(elem + 256u * (k + p), keys), pw, keys, w);
-                quantize8<BITS, RNG16, BACK>(v[p], ts, f, w, my_level + (k + p) * 32 * BITS, my_sign + (k + p) * 32);
-                if (BACK) dat_st8<EV_LAST>(back + e_piece + 8 * lane + 256 * (k + p), wide, v[p]);
-                if (k + 2 < groups) dat_ld8<EV_FIRST>(g + 256 * (k + p + 2), wide, v[p]);
+                PhiloxGroup<RNG16> pg;
+                pg.e[0] = dat_philox_elem(counter, a.keys);
+                if (!RNG16) pg.e[RNG16 ? 0 : 1] = dat_philox_elem(counter + 1u, a.keys);
+                dat_group_words<RNG16>(pg, pw, a.keys, w);
+                quantize8<BITS, RNG16, BACK>(v[p], ts, f, w, to_level + p * 32 * BITS, to_sign + p * 32);
+                if (BACK) dat_st8<EV_LAST>(back + 256 * p, true, v[p]);
+                if (k > 2) dat_ld8<EV_FIRST>(ahead + 256 * p, true, v[p]);
+                counter += RNG16 ? 32u : 64u;
             }
+            ahead += 512;
+            if (BACK) back += 512;
+            to_level += 64 * BITS;
+            to_sign += 64;
         }
     } else {
-#pragma unroll 1
-        for (int k = 0; k < groups; ++k) {
-            const int64_t e0 = e_piece + 8 * lane + 256 * k;
-            float t = t0;                                    // the group's layer
-            int64_t l_hi = hi;
-            int l = l0;
-            if (e0 >= hi && e0 < d) {
-                l = l0 + dat_find(off + l0, nl, e0);
-                l_hi = __ldg(off + l + 1);
-                t = quant_mul(qs, q0 + l);
-            }
-            if (page && scaled(t) && e0 + 8 <= l_hi) {
-                float x[8];
-                uint32_t w[8];
-                dat_ld8<EV_FIRST>(g + 256 * k, wide, x);
-                dat_group_words<RNG16>(dat_philox_group<RNG16>(elem + 256u * k, keys), pw, keys, w);
-                quantize8<BITS, RNG16, BACK>(x, t * (1.0f / TWO_B), BACK ? quant_back(qs, l) : 0.0f, w, my_level + k * 32 * BITS, my_sign + k * 32);
-                if (BACK) dat_st8<EV_LAST>(back + e0, wide, x);
-            } else {
-                quantize_slow8<BITS, BACK>(g - e_piece - 8 * lane, e0, off, l0, nl, d, qs, q0, elem + 256u * k, stream, keys, RNG16,
-                                     my_level + k * 32 * BITS, my_sign + k * 32, back);
-            }
-        }
+        quantize_mixed<BITS, RNG16, BACK>(a, worker, e_piece, reinterpret_cast<uint8_t *>(s_level[warp]), reinterpret_cast<uint8_t *>(s_sign[warp]));
     }
     __syncwarp();
 
     // 128-bit stores of the finished part (planes are padded to 16 bytes, so whole uint4 fit)
     {
-        const int64_t bytes = n_warp * BITS / 8, base = part * bytes, left = level_bytes - base;
+        const int64_t bytes = 32 * BITS * a.groups, base = part * bytes, left = a.level_bytes - base;
         const int n16 = (int)((left < bytes ? left : bytes) / 16);
-        uint4 *dst = reinterpret_cast<uint4 *>(levels + (int64_t)worker * level_bytes + base);
+        uint4 *dst = reinterpret_cast<uint4 *>(a.levels + (int64_t)worker * a.level_bytes + base);
         for (int k = lane; k < n16; k += 32) dst[k] = s_level[warp][k];
     }
     {
-        const int64_t bytes = n_warp / 8, base = part * bytes, left = sign_bytes - base;
+        const int64_t bytes = 32 * a.groups, base = part * bytes, left = a.sign_bytes - base;
         const int n16 = (int)((left < bytes ? left : bytes) / 16);
-        uint4 *dst = reinterpret_cast<uint4 *>(signs + (int64_t)worker * sign_bytes + base);
+        uint4 *dst = reinterpret_cast<uint4 *>(a.signs + (int64_t)worker * a.sign_bytes + base);
         for (int k = lane; k < n16; k += 32) dst[k] = s_sign[warp][k];
     }
 }
@@ -352,17 +385,30 @@ k_quantize(const __grid_constant__ GradPtrs gp, const __grid_constant__ PhiloxKe
 static int quantize_launch(dat_plan_t *plan, const GradPtrs &gp, int n, uint64_t seed, uint64_t step, uint8_t *levels, uint8_t *signs,
                            float *scales, const float *scales_in, int n_scales, bool per_worker, uint32_t stream_base, cudaStream_t s, float *back = nullptr)
 {
-    const PhiloxKeys keys = dat_make_keys(seed, step);
-    const int h = (int)plan->h;
-    const QuantScale qs = {plan->d_qmul, scales_in, scales, n_scales, (float)plan->S, plan->d_status};
     // long runs per warp (the set-up is paid once) while there are four waves of CTAs; shorter ones for small problems
     int groups = QUANT_GROUPS;
     auto ctas = [&](int g) { return (plan->d + g * (int64_t)(8 * DAT_THREADS) - 1) / (g * (int64_t)(8 * DAT_THREADS)); };
     while (groups > 2 && ctas(groups) * n < 4ll * QUANT_CTAS * plan->sm_count) groups /= 2;
     const unsigned grid = (unsigned)(ctas(groups) * n);
-#define DAT_Q(B, R, K)                                                                                                          \
-    k_quantize<B, R, K><<<grid, DAT_THREADS, 0, s>>>(gp, keys, plan->d_offsets, plan->d_flat_layer, h, plan->d, qs, levels, signs, \
-                                                     plan->level_bytes, plan->sign_bytes, groups, n, per_worker, stream_base, plan->elem_base, back)
+    QuantArgs a;
+    a.gp = gp;
+    a.keys = dat_make_keys(seed, step);
+    a.qs = QuantScale{plan->d_qmul, scales_in, scales, n_scales, (float)plan->S, plan->d_status};
+    a.off = plan->d_offsets;
+    a.flat_layer = plan->d_flat_layer;
+    a.levels = levels;
+    a.signs = signs;
+    a.back = back;
+    a.d = plan->d;
+    a.level_bytes = plan->level_bytes;
+    a.sign_bytes = plan->sign_bytes;
+    a.elem_base = plan->elem_base;
+    a.stream_base = stream_base;
+    a.h = (int)plan->h;
+    a.n = n;
+    a.groups = groups;
+    a.per_worker = per_worker;
+#define DAT_Q(B, R, K) k_quantize<B, R, K><<<grid, DAT_THREADS, 0, s>>>(a)
 #define DAT_QK(B, R) do { if (back) DAT_Q(B, R, true); else DAT_Q(B, R, false); } while (0)
 #define DAT_QR(B) do { if (plan->rng_bits == 16) DAT_QK(B, true); else DAT_QK(B, false); } while (0)
     switch (plan->bits) {
