@@ -178,6 +178,21 @@ int dat_quantize(dat_plan_t *plan, const float *const *grads, uint64_t seed, uin
                  uint8_t *levels, uint8_t *signs, float *scales, const float *scales_in,
                  void *stream);
 
+/* dat_quantize_ranges -- dat_quantize with caller-supplied norms for several ranges of the SAME M vectors, in one launch:
+ * what one rank of a sharded step sends to the owners of the ranges.
+ *   plans        host array of num_ranges plans, one per range, with the origin of their range set
+ *                (dat_plan_set_origin); all with the same M, bits, rng_bits, worker origin and the shared scale.
+ *   first_layer  host array: global index of the range's first layer (its norm is norms[first_layer]).
+ *   padded       host array: non-zero if the plan's layer 0 only fills the range up to a multiple of 8 elements
+ *                (its codes are drawn with norm 1); first_layer then belongs to the plan's layer 1.
+ *   grads        host array of M device pointers to the WHOLE vectors; range k starts at its plan's element origin.
+ *   norms        device fp32, the norms of all layers of the whole vectors.
+ *   levels, signs  host arrays of device pointers: where range k's planes go (sizes and layout as in dat_quantize).
+ * The planes are those of dat_quantize on each range, bit for bit.  Errors: ARG, ALIGN, BITS, CUDA. */
+int dat_quantize_ranges(int num_ranges, dat_plan_t *const *plans, const int64_t *first_layer, const int32_t *padded,
+                        const float *const *grads, uint64_t seed, uint64_t step, const float *norms,
+                        uint8_t *const *levels, uint8_t *const *signs, void *stream);
+
 /* dat_worker_norms -- the norms of Eq. rand_q by themselves: nu_{i,l} = ||g_l^(i)||_2 for every worker and
  * layer (fp64 sums of exact squares, one rounding), without drawing any level.  A sharded step needs them
  * before it can agree on the shared norm max_i nu_{i,l} across ranks.

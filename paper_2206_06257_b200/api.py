@@ -6,6 +6,7 @@ binding passes their data_ptr().  Importing this module loads the library and fa
 if it has not been built (python -m paper_2206_06257_b200.build); there is no CPU fallback.
 """
 import ctypes as C
+import functools
 import os
 
 import numpy as np
@@ -30,7 +31,7 @@ DAT_STATIC_MAX_LAYERS, DAT_STATIC_MAX_TILES = 4096, 32768
 DAT_STATUS_NONFINITE, DAT_STATUS_TIMEOUT, DAT_STATUS_BOUNDS = 1, 2, 4
 
 # every symbol include/dat.h declares
-EXPORTS = ["dat_plan_create", "dat_plan_set_origin", "dat_plan_destroy", "dat_plan_sizes", "dat_worker_norms", "dat_quantize", "dat_aggregate", "dat_aggregate_gather", "dat_requantize",
+EXPORTS = ["dat_plan_create", "dat_plan_set_origin", "dat_plan_destroy", "dat_plan_sizes", "dat_worker_norms", "dat_quantize", "dat_quantize_ranges", "dat_aggregate", "dat_aggregate_gather", "dat_requantize",
            "dat_average", "dat_lalr_step", "dat_lamb_step", "dat_lalr_step_static", "dat_step", "dat_step_lamb", "dat_step_two_sided", "dat_step_lamb_two_sided", "dat_step_passes", "dat_step_pipelined", "dat_plan_test_stall", "dat_step_host", "dat_get_status",
            "dat_plan_launch_count", "dat_strerror", "dat_last_cuda_error"]
 
@@ -52,6 +53,7 @@ _lib.dat_plan_set_origin.argtypes = [_p, _i64, _i64]
 _lib.dat_worker_norms.argtypes = [_p, _p, _p, _p]
 _lib.dat_plan_sizes.argtypes = [_p, C.POINTER(_i64), C.POINTER(_i64), C.POINTER(_i64), C.POINTER(_i64)]
 _lib.dat_quantize.argtypes = [_p, _p, _u64, _u64, _p, _p, _p, _p, _p]
+_lib.dat_quantize_ranges.argtypes = [_int, _p, _p, _p, _p, _u64, _u64, _p, _p, _p, _p]
 _lib.dat_aggregate.argtypes = [_p, _p, _p, _p, _p, _p, _p]
 _lib.dat_aggregate_gather.argtypes = [_p, _p, _p, _p, _p, _p, _p]
 _lib.dat_requantize.argtypes = [_p, _p, _u64, _u64, _p, _p, _p, _p, _p]
@@ -90,35 +92,42 @@ def _ok(code, where):
 
 
 def _ptr(x):
-    """Address of a tensor / array / int / None, as c_void_p."""
+    """Address of a tensor / array / int / None."""
     if x is None:
         return None
     if isinstance(x, torch.Tensor):
-        return _p(x.data_ptr())
+        return x.data_ptr()
     if isinstance(x, np.ndarray):
-        return _p(x.ctypes.data)
-    return _p(int(x))
+        return x.ctypes.data
+    return int(x)
+
+
+@functools.lru_cache(maxsize=None)
+def _array_type(ctype, n):
+    return ctype * n
 
 
 def _ptr_array(xs):
-    arr = (C.c_void_p * len(xs))()
-    for k, x in enumerate(xs):
-        arr[k] = _ptr(x).value if x is not None else None
-    return arr
+    return _array_type(C.c_void_p, len(xs))(*[_ptr(x) for x in xs])
 
 
 def _stream(stream):
     if stream is None:
-        return _p(torch.cuda.current_stream().cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     if isinstance(stream, torch.cuda.Stream):
-        return _p(stream.cuda_stream)
-    return _p(int(stream))
+        return stream.cuda_stream
+    return int(stream)
+
+
+@functools.lru_cache(maxsize=64)
+def _hp_struct(hp):
+    return dat_hparams_t(*hp)
 
 
 def _hp(hp):
     if isinstance(hp, dat_hparams_t):
         return hp
-    return dat_hparams_t(*[float(v) for v in hp])
+    return _hp_struct(tuple([float(v) for v in hp]))
 
 
 def dat_strerror(code):
@@ -135,59 +144,66 @@ def dat_plan_create(layer_offsets, num_workers, bits, scale_mode=DAT_SCALE_SHARE
 
 
 def dat_plan_set_origin(plan, elem_base, worker_base):
-    _ok(_lib.dat_plan_set_origin(_p(plan), int(elem_base), int(worker_base)), "dat_plan_set_origin")
+    _ok(_lib.dat_plan_set_origin(plan, int(elem_base), int(worker_base)), "dat_plan_set_origin")
 
 
 def dat_worker_norms(plan, grads, norms_out, stream=None):
-    _ok(_lib.dat_worker_norms(_p(plan), _ptr_array(grads), _ptr(norms_out), _stream(stream)), "dat_worker_norms")
+    _ok(_lib.dat_worker_norms(plan, _ptr_array(grads), _ptr(norms_out), _stream(stream)), "dat_worker_norms")
 
 
 def dat_plan_destroy(plan):
-    _ok(_lib.dat_plan_destroy(_p(plan)), "dat_plan_destroy")
+    _ok(_lib.dat_plan_destroy(plan), "dat_plan_destroy")
 
 
 def dat_plan_sizes(plan):
     """(level_bytes_per_worker, sign_bytes_per_worker, num_scales, workspace_bytes)"""
     a, b, c, d = _i64(), _i64(), _i64(), _i64()
-    _ok(_lib.dat_plan_sizes(_p(plan), C.byref(a), C.byref(b), C.byref(c), C.byref(d)), "dat_plan_sizes")
+    _ok(_lib.dat_plan_sizes(plan, C.byref(a), C.byref(b), C.byref(c), C.byref(d)), "dat_plan_sizes")
     return a.value, b.value, c.value, d.value
 
 
 def dat_quantize(plan, grads, seed, step, levels, signs, scales, scales_in=None, stream=None):
-    _ok(_lib.dat_quantize(_p(plan), _ptr_array(grads), int(seed), int(step), _ptr(levels), _ptr(signs),
+    _ok(_lib.dat_quantize(plan, _ptr_array(grads), int(seed), int(step), _ptr(levels), _ptr(signs),
                           _ptr(scales), _ptr(scales_in), _stream(stream)), "dat_quantize")
 
 
+def dat_quantize_ranges(plans, first_layer, padded, grads, seed, step, norms, levels, signs, stream=None):
+    """One entry per range in plans, first_layer, padded, levels, signs; grads: the M whole vectors."""
+    n = len(plans)
+    _ok(_lib.dat_quantize_ranges(n, _ptr_array(plans), _array_type(_i64, n)(*first_layer), _array_type(C.c_int32, n)(*padded), _ptr_array(grads),
+                                 int(seed), int(step), _ptr(norms), _ptr_array(levels), _ptr_array(signs), _stream(stream)), "dat_quantize_ranges")
+
+
 def dat_aggregate(plan, levels, signs, scales, code_sum, g_hat, stream=None):
-    _ok(_lib.dat_aggregate(_p(plan), _ptr(levels), _ptr(signs), _ptr(scales), _ptr(code_sum), _ptr(g_hat),
+    _ok(_lib.dat_aggregate(plan, _ptr(levels), _ptr(signs), _ptr(scales), _ptr(code_sum), _ptr(g_hat),
                            _stream(stream)), "dat_aggregate")
 
 
 def dat_aggregate_gather(plan, level_planes, sign_planes, scales, code_sum, g_hat, stream=None):
     """level_planes, sign_planes: M tensors (or addresses), worker i's planes each."""
-    _ok(_lib.dat_aggregate_gather(_p(plan), _ptr_array(level_planes), _ptr_array(sign_planes), _ptr(scales),
+    _ok(_lib.dat_aggregate_gather(plan, _ptr_array(level_planes), _ptr_array(sign_planes), _ptr(scales),
                                   _ptr(code_sum), _ptr(g_hat), _stream(stream)), "dat_aggregate_gather")
 
 
 def dat_requantize(plan, g_hat, seed, step, levels, signs, scales, scales_in=None, stream=None):
-    _ok(_lib.dat_requantize(_p(plan), _ptr(g_hat), int(seed), int(step), _ptr(levels), _ptr(signs), _ptr(scales),
+    _ok(_lib.dat_requantize(plan, _ptr(g_hat), int(seed), int(step), _ptr(levels), _ptr(signs), _ptr(scales),
                             _ptr(scales_in), _stream(stream)), "dat_requantize")
 
 
 def dat_average(plan, grads, g_hat, stream=None):
-    _ok(_lib.dat_average(_p(plan), _ptr_array(grads), _ptr(g_hat), _stream(stream)), "dat_average")
+    _ok(_lib.dat_average(plan, _ptr_array(grads), _ptr(g_hat), _stream(stream)), "dat_average")
 
 
 def dat_lalr_step(plan, theta, mom, g_hat, hp, layer_norms_out=None, stream=None):
     h = _hp(hp)
-    _ok(_lib.dat_lalr_step(_p(plan), _ptr(theta), _ptr(mom), _ptr(g_hat), C.byref(h), _ptr(layer_norms_out),
+    _ok(_lib.dat_lalr_step(plan, _ptr(theta), _ptr(mom), _ptr(g_hat), C.byref(h), _ptr(layer_norms_out),
                            _stream(stream)), "dat_lalr_step")
 
 
 def dat_lamb_step(plan, theta, mom, var, g_hat, hp, t, layer_norms_out=None, stream=None):
     """hp: dat_lamb_hparams_t or (lr, beta1, beta2, zeta, weight_decay, c_l, c_u); t >= 1."""
     h = hp if isinstance(hp, dat_lamb_hparams_t) else dat_lamb_hparams_t(*[float(x) for x in hp])
-    _ok(_lib.dat_lamb_step(_p(plan), _ptr(theta), _ptr(mom), _ptr(var), _ptr(g_hat), C.byref(h), int(t),
+    _ok(_lib.dat_lamb_step(plan, _ptr(theta), _ptr(mom), _ptr(var), _ptr(g_hat), C.byref(h), int(t),
                            _ptr(layer_norms_out), _stream(stream)), "dat_lamb_step")
 
 
@@ -203,7 +219,7 @@ def dat_lalr_step_static(layer_offsets, theta, mom, g_hat, hp, layer_norms_out=N
 def dat_step(plan, theta, mom, grads, seed, step, hp, code_sum_out=None, layer_norms_out=None,
              scales_out=None, stream=None):
     h = _hp(hp)
-    _ok(_lib.dat_step(_p(plan), _ptr(theta), _ptr(mom), _ptr_array(grads), int(seed), int(step), C.byref(h),
+    _ok(_lib.dat_step(plan, _ptr(theta), _ptr(mom), _ptr_array(grads), int(seed), int(step), C.byref(h),
                       _ptr(code_sum_out), _ptr(layer_norms_out), _ptr(scales_out), _stream(stream)), "dat_step")
 
 
@@ -211,7 +227,7 @@ def dat_step_lamb(plan, theta, mom, var, grads, seed, step, hp, t, code_sum_out=
                   scales_out=None, stream=None):
     """hp: dat_lamb_hparams_t or (lr, beta1, beta2, zeta, weight_decay, c_l, c_u); t >= 1."""
     h = hp if isinstance(hp, dat_lamb_hparams_t) else dat_lamb_hparams_t(*[float(x) for x in hp])
-    _ok(_lib.dat_step_lamb(_p(plan), _ptr(theta), _ptr(mom), _ptr(var), _ptr_array(grads), int(seed), int(step), C.byref(h),
+    _ok(_lib.dat_step_lamb(plan, _ptr(theta), _ptr(mom), _ptr(var), _ptr_array(grads), int(seed), int(step), C.byref(h),
                            int(t), _ptr(code_sum_out), _ptr(layer_norms_out), _ptr(scales_out), _stream(stream)), "dat_step_lamb")
 
 
@@ -219,7 +235,7 @@ def dat_step_two_sided(plan, theta, mom, grads, seed, step, hp, g_hat, code_sum_
                        scales_out=None, server_scales_out=None, stream=None):
     """g_hat: fp32[d] workspace; on return the receiver's value of Algorithm A1 Step 10."""
     h = _hp(hp)
-    _ok(_lib.dat_step_two_sided(_p(plan), _ptr(theta), _ptr(mom), _ptr_array(grads), int(seed), int(step), C.byref(h),
+    _ok(_lib.dat_step_two_sided(plan, _ptr(theta), _ptr(mom), _ptr_array(grads), int(seed), int(step), C.byref(h),
                                 _ptr(g_hat), _ptr(code_sum_out), _ptr(layer_norms_out), _ptr(scales_out),
                                 _ptr(server_scales_out), _stream(stream)), "dat_step_two_sided")
 
@@ -227,45 +243,45 @@ def dat_step_two_sided(plan, theta, mom, grads, seed, step, hp, g_hat, code_sum_
 def dat_step_lamb_two_sided(plan, theta, mom, var, grads, seed, step, hp, t, g_hat, code_sum_out=None,
                             layer_norms_out=None, scales_out=None, server_scales_out=None, stream=None):
     h = hp if isinstance(hp, dat_lamb_hparams_t) else dat_lamb_hparams_t(*[float(x) for x in hp])
-    _ok(_lib.dat_step_lamb_two_sided(_p(plan), _ptr(theta), _ptr(mom), _ptr(var), _ptr_array(grads), int(seed), int(step),
+    _ok(_lib.dat_step_lamb_two_sided(plan, _ptr(theta), _ptr(mom), _ptr(var), _ptr_array(grads), int(seed), int(step),
                                      C.byref(h), int(t), _ptr(g_hat), _ptr(code_sum_out), _ptr(layer_norms_out),
                                      _ptr(scales_out), _ptr(server_scales_out), _stream(stream)), "dat_step_lamb_two_sided")
 
 
 def dat_plan_test_stall(plan, wait_cycles, layer=-1, stream=None):
     """Test hook: wait limit in SM cycles (0: default) and a layer whose norm never completes next call."""
-    _ok(_lib.dat_plan_test_stall(_p(plan), int(wait_cycles), int(layer), _stream(stream)), "dat_plan_test_stall")
+    _ok(_lib.dat_plan_test_stall(plan, int(wait_cycles), int(layer), _stream(stream)), "dat_plan_test_stall")
 
 
 def dat_step_passes(plan, theta, mom, grads, seed, step, hp, code_sum_out=None, layer_norms_out=None,
                     scales_out=None, stream=None):
     h = _hp(hp)
-    _ok(_lib.dat_step_passes(_p(plan), _ptr(theta), _ptr(mom), _ptr_array(grads), int(seed), int(step), C.byref(h),
+    _ok(_lib.dat_step_passes(plan, _ptr(theta), _ptr(mom), _ptr_array(grads), int(seed), int(step), C.byref(h),
                              _ptr(code_sum_out), _ptr(layer_norms_out), _ptr(scales_out), _stream(stream)), "dat_step_passes")
 
 
 def dat_step_pipelined(plan, theta, mom, grads, seed, step, hp, code_sum_out=None, layer_norms_out=None,
                      scales_out=None, stream=None):
     h = _hp(hp)
-    _ok(_lib.dat_step_pipelined(_p(plan), _ptr(theta), _ptr(mom), _ptr_array(grads), int(seed), int(step), C.byref(h),
+    _ok(_lib.dat_step_pipelined(plan, _ptr(theta), _ptr(mom), _ptr_array(grads), int(seed), int(step), C.byref(h),
                               _ptr(code_sum_out), _ptr(layer_norms_out), _ptr(scales_out), _stream(stream)), "dat_step_pipelined")
 
 
 def dat_step_host(plan, theta_host, mom_host, grads_host, seed, step, hp, stream=None):
     h = _hp(hp)
-    _ok(_lib.dat_step_host(_p(plan), _ptr(theta_host), _ptr(mom_host), _ptr_array(grads_host), int(seed),
+    _ok(_lib.dat_step_host(plan, _ptr(theta_host), _ptr(mom_host), _ptr_array(grads_host), int(seed),
                            int(step), C.byref(h), _stream(stream)), "dat_step_host")
 
 
 def dat_get_status(plan, stream=None):
     v = C.c_uint32()
-    _ok(_lib.dat_get_status(_p(plan), C.byref(v), _stream(stream)), "dat_get_status")
+    _ok(_lib.dat_get_status(plan, C.byref(v), _stream(stream)), "dat_get_status")
     return v.value
 
 
 def dat_plan_launch_count(plan):
-    return int(_lib.dat_plan_launch_count(_p(plan)))
+    return int(_lib.dat_plan_launch_count(plan))
 
 
 def dat_last_cuda_error(plan):
-    return int(_lib.dat_last_cuda_error(_p(plan)))
+    return int(_lib.dat_last_cuda_error(plan))

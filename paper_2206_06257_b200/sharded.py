@@ -66,9 +66,11 @@ class RangeLayout:
         self.h = self.offsets.size - 1
 
     def scales(self, nu):
-        """The sub-problem's norms from the global per-layer norms (the pad layer gets 1)."""
+        """The sub-problem's norms from the global per-layer norms (the pad layer gets 1), on a 16-byte boundary."""
         own = nu[self.l0:self.l1]
-        return torch.cat([torch.ones(1, dtype=own.dtype, device=own.device), own]) if self.pad else own.clone()
+        if self.pad:
+            return torch.cat([torch.ones(1, dtype=own.dtype, device=own.device), own])
+        return own if own.data_ptr() % 16 == 0 else own.clone()
 
 
 class ShardedStep:
@@ -87,10 +89,13 @@ class ShardedStep:
     # by handing the messages over itself; step() below drives them with torch.distributed.
     def local_norms(self, grads_local):
         """Step 7, first half: max over this rank's workers of ||g_l^(i)||_2, per layer."""
-        return self.ops.worker_norms(grads_local).max(dim=0).values.contiguous()
+        norms = self.ops.worker_norms(grads_local)
+        return norms[0] if self.M_loc == 1 else norms.max(dim=0).values.contiguous()
 
     def quantize(self, nu, grads_local, seed, step):
         """Step 7, second half: this rank's workers, range by range.  Returns [(levels, signs)] per owner."""
+        if hasattr(self.ops, "quantize_ranges"):      # all ranges in one launch
+            return self.ops.quantize_ranges(self.ranges, grads_local, nu, seed, step)
         return [self.ops.quantize_range(q, self.ranges[q], grads_local, self.ranges[q].scales(nu), seed, step)
                 for q in range(self.world)]
 
@@ -125,6 +130,9 @@ class ShardedStep:
             sg0 = sg.data_ptr() if isinstance(sg, torch.Tensor) else int(sg)
             lv_ptrs += [lv0 + j * lb for j in range(self.M_loc)]         # global worker order: rank-major
             sg_ptrs += [sg0 + j * sb for j in range(self.M_loc)]
+        if own.pad == 0:             # the range is the owner's from its first element: in place
+            self.ops.aggregate_update_gather(own, lv_ptrs, sg_ptrs, own.scales(nu), theta[own.a:own.b], mom_own, hp)
+            return
         theta_own = theta[own.a8:own.b].clone()
         self.ops.aggregate_update_gather(own, lv_ptrs, sg_ptrs, own.scales(nu), theta_own, mom_own, hp)
         theta[own.a:own.b].copy_(theta_own[own.pad:])
@@ -158,11 +166,8 @@ class ShardedStep:
         nu = self.local_norms(grads_local)
         if multi:
             dist.all_reduce(nu, op=dist.ReduceOp.MAX, group=self.group)
-        for q in range(self.world):
-            lb, sb = self.ops.plane_bytes(self.ranges[q])
-            lo, so = layout[q]
-            self.ops.quantize_range(q, self.ranges[q], grads_local, self.ranges[q].scales(nu), seed, step,
-                                    out=(self._out[lo:lo + self.M_loc * lb], self._out[so:so + self.M_loc * sb]))
+        base = self._out.data_ptr()
+        self.ops.quantize_ranges(self.ranges, grads_local, nu, seed, step, out=[(base + lo, base + so) for lo, so in layout])
         if multi:
             torch.cuda.current_stream().synchronize()
             dist.barrier(group=self.group)                                # every rank's planes are complete
@@ -214,12 +219,12 @@ class CudaOps:
         self.h = self.offsets.size - 1
         self.bits, self.rng_bits = bits, rng_bits
         self.plan_norms = api.dat_plan_create(self.offsets, M_loc, bits, rng_bits=rng_bits)
-        self.plans_q, self.plans_agg = {}, {}
+        self.plans_q, self.plans_agg, self.messages = {}, {}, {}
 
     def close(self):
         for p in [self.plan_norms] + list(self.plans_q.values()) + list(self.plans_agg.values()):
             self.api.dat_plan_destroy(p)
-        self.plans_q, self.plans_agg, self.plan_norms = {}, {}, None
+        self.plans_q, self.plans_agg, self.messages, self.plan_norms = {}, {}, {}, None
 
     def _plan(self, table, rg, workers, worker_base):
         key = (rg.l0, rg.l1)
@@ -247,6 +252,33 @@ class CudaOps:
         sc = torch.empty(ns, dtype=torch.float32, device=dev)
         self.api.dat_quantize(plan, [g[rg.a8:rg.b] for g in grads_local], seed, step, lv, sg, sc, scales_in=scales.contiguous())
         return lv, sg
+
+    def _messages(self, ranges):
+        """Plans, layer origins and plane sizes of a rank's messages to the owners of `ranges`."""
+        key = tuple((rg.l0, rg.l1) for rg in ranges)
+        if key not in self.messages:
+            plans = [self._plan(self.plans_q, rg, self.M_loc, self.rank * self.M_loc) for rg in ranges]
+            sizes = []
+            for p in plans:
+                lb, sb, _, _ = self.api.dat_plan_sizes(p)
+                sizes += [self.M_loc * lb, self.M_loc * sb]             # (multiples of 16 bytes)
+            at = np.concatenate([[0], np.cumsum(sizes)]).tolist()
+            self.messages[key] = (plans, [rg.l0 for rg in ranges], [int(rg.pad > 0) for rg in ranges], sizes, at)
+        return self.messages[key]
+
+    def quantize_ranges(self, ranges, grads_local, nu, seed, step, out=None):
+        """The messages to the owners of all ranges in one launch: [(levels, signs)] per range.  nu: the norms of all
+        layers.  out: where the planes go (tensors or addresses), or None for tensors of their own."""
+        plans, first, padded, sizes, at = self._messages(ranges)
+        if out is None:
+            buf = torch.empty(at[-1], dtype=torch.uint8, device=grads_local[0].device)
+            parts, base = buf.split(sizes), buf.data_ptr()
+            res = list(zip(parts[0::2], parts[1::2]))
+            lv, sg = [base + x for x in at[0:-1:2]], [base + x for x in at[1::2]]
+        else:
+            res, lv, sg = out, [o[0] for o in out], [o[1] for o in out]
+        self.api.dat_quantize_ranges(plans, first, padded, grads_local, seed, step, nu.contiguous(), lv, sg)
+        return res
 
     def aggregate_update_gather(self, rg, lv_ptrs, sg_ptrs, scales, theta_own, mom_own, hp):
         plan = self._plan(self.plans_agg, rg, self.M, 0)
