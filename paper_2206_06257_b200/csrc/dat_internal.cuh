@@ -78,8 +78,10 @@ struct dat_plan {
 
     PipeSchedule *pipe = nullptr;      // work items and tables of dat_step_pipelined, built with the plan
 
-    // staging buffers of dat_step_host
+    // dat_step_host: staging buffers, streams for the copies in and out, events
     float *stage = nullptr;
+    cudaStream_t copy_in = nullptr, copy_out = nullptr;
+    std::vector<cudaEvent_t> events;
 
     int sm_count = 0;
     int64_t launches = 0;
@@ -98,6 +100,12 @@ void dat_make_worker_table(const PhiloxKeys &keys, int M, PhiloxWorkers *out);
 int dat_pipe_build(dat_plan_t *plan);                        // dat_pipeline.cu (device current)
 void dat_pipe_destroy(dat_plan_t *plan);
 cudaError_t dat_pipe_reset(dat_plan_t *plan, cudaStream_t s);
+int dat_pipe_groups(dat_plan_t *plan, int most, size_t *bytes);      // the step group by group (dat_step_host)
+int dat_pipe_groups_upload(dat_plan_t *plan, void *mem);
+int dat_pipe_group_count(const dat_plan_t *plan);
+void dat_pipe_group_range(const dat_plan_t *plan, int k, int64_t *e0, int64_t *e1);
+int dat_pipe_step_group(dat_plan_t *plan, int k, float *theta, float *mom, const float *const *grads, uint64_t seed, uint64_t step,
+                        const dat_hparams_t *hp, cudaStream_t s);
 
 #define DAT_CUDA(plan, call)                                              \
     do {                                                                  \

@@ -67,6 +67,12 @@ struct PipeItem {
     PipePart n, q, u, r;                          // r: the server's quantizer (two-sided schedules only)
 };
 
+// A contiguous range of layers as a list of its own (dat_step_host: the step range by range, as the data arrives).
+struct PipeGroup {
+    int64_t e0, e1;                               // elements
+    int64_t first, n_items;                       // in group_items
+};
+
 struct PipeSchedule {
     char *mem = nullptr;                          // one device allocation, carved up
     size_t mem_bytes = 0;
@@ -82,6 +88,10 @@ struct PipeSchedule {
     uint32_t *d_sync = nullptr;                   // [0] ticket, [1] abort epoch, then cntN[h], cntQ[h], readyN[h], readyQ[h], cntR[h], readyR[h]
     size_t sync_bytes = 0;
     int64_t n_tiles = 0;
+    std::vector<int64_t> tile_base;               // h + 1
+    std::vector<PipeGroup> groups;                // built by the first dat_step_host
+    std::vector<PipeItem> group_items;
+    PipeItem *d_group_items = nullptr;            // in the caller's memory (dat_pipe_groups_upload)
     uint32_t epoch = 0;                           // calls made so far
     long long wait_cycles = DAT_P_WAIT_CYCLES;
 };
@@ -776,6 +786,64 @@ void dat_pipe_destroy(dat_plan_t *plan)
 
 static size_t p_align(size_t x) { return (x + 255) / 256 * 256; }
 
+// The items of the layers [l0, l1).
+static std::vector<PipeItem> p_items(const dat_plan_t *plan, const std::vector<int64_t> &tb, int l0, int l1, bool two)
+{
+    const bool identity = (plan->bits == 32);
+    const int h = l1 - l0;
+    // layers smallest first (ties in index order): the distance between the N and the Q stream is the
+    // size of the layer being worked on, so it grows slowly and the streams stay paired to the end
+    std::vector<int> order((size_t)h);
+    for (int l = 0; l < h; ++l) order[l] = l0 + l;
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+        return plan->offsets[x + 1] - plan->offsets[x] < plan->offsets[y + 1] - plan->offsets[y];
+    });
+    // slot of every tile in each of the three streams (four with the server's quantizer between Q and U)
+    const PipePart nopart = {0, 1, 0, 1, -1, 0};
+    const PipeItem none = {nopart, nopart, nopart, nopart};
+    auto part = [&](int l, int64_t t) {
+        PipePart pp = {plan->offsets[l], plan->offsets[l + 1], (int32_t)tb[l], (int32_t)(tb[l + 1] - tb[l]), l, (int32_t)t};
+        return pp;
+    };
+    std::vector<PipeItem> items;
+    auto at = [&](int64_t slot) -> PipeItem & {
+        if ((int64_t)items.size() <= slot) items.resize((size_t)slot + 1, none);
+        return items[(size_t)slot];
+    };
+    std::vector<int64_t> done_n((size_t)l1, -1 - (int64_t)DAT_P_LAG), done_q((size_t)l1, 0), done_r((size_t)l1, 0);
+    int64_t slot = 0;
+    if (!identity)
+        for (int k = 0; k < h; ++k) {
+            const int l = order[k];
+            for (int64_t t = 0; t < tb[l + 1] - tb[l]; ++t) { at(slot).n = part(l, t); done_n[l] = slot++; }
+        }
+    slot = 0;
+    for (int k = 0; k < h; ++k) {
+        const int l = order[k];
+        const int64_t T = tb[l + 1] - tb[l];
+        slot = std::max(slot, done_n[l] + DAT_P_LAG + 1);
+        // a layer that L2 cannot hold next to what streams in meanwhile is walked back from its last
+        // tile (what N read last, and marked to stay, is read first); the others in N's order
+        const bool reverse = T >= DAT_P_REVERSE_FROM;
+        for (int64_t t = 0; t < T; ++t) { at(slot).q = part(l, reverse ? T - 1 - t : t); done_q[l] = slot++; }
+    }
+    if (two) {
+        slot = 0;
+        for (int k = 0; k < h; ++k) {
+            const int l = order[k];
+            slot = std::max(slot, done_q[l] + DAT_P_LAG_U + 1);
+            for (int64_t t = 0; t < tb[l + 1] - tb[l]; ++t) { at(slot).r = part(l, t); done_r[l] = slot++; }
+        }
+    }
+    slot = 0;
+    for (int k = 0; k < h; ++k) {
+        const int l = order[k];
+        slot = std::max(slot, (two ? done_r[l] : done_q[l]) + DAT_P_LAG_U + 1);
+        for (int64_t t = 0; t < tb[l + 1] - tb[l]; ++t) { at(slot).u = part(l, t); ++slot; }
+    }
+    return items;
+}
+
 // Called by dat_plan_create (device current).  Allocates the schedule's tables (synchronous).
 int dat_pipe_build(dat_plan_t *plan)
 {
@@ -794,61 +862,9 @@ int dat_pipe_build(dat_plan_t *plan)
         tb[h] = nt;
         g->n_tiles = nt;
         if (nt > ((int64_t)1 << 30)) return DAT_ERR_UNSUPPORTED;
-        // layers smallest first (ties in index order): the distance between the N and the Q stream is the
-        // size of the layer being worked on, so it grows slowly and the streams stay paired to the end
-        std::vector<int> order((size_t)h);
-        for (int l = 0; l < h; ++l) order[l] = l;
-        std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
-            return plan->offsets[x + 1] - plan->offsets[x] < plan->offsets[y + 1] - plan->offsets[y];
-        });
-        // slot of every tile in each of the three streams (four with the server's quantizer between Q and U)
-        const PipePart nopart = {0, 1, 0, 1, -1, 0};
-        const PipeItem none = {nopart, nopart, nopart, nopart};
-        auto part = [&](int l, int64_t t) {
-            PipePart pp = {plan->offsets[l], plan->offsets[l + 1], (int32_t)tb[l], (int32_t)(tb[l + 1] - tb[l]), l, (int32_t)t};
-            return pp;
-        };
-        auto build = [&](bool two) {
-            std::vector<PipeItem> items;
-            auto at = [&](int64_t slot) -> PipeItem & {
-                if ((int64_t)items.size() <= slot) items.resize((size_t)slot + 1, none);
-                return items[(size_t)slot];
-            };
-            std::vector<int64_t> done_n((size_t)h, -1 - (int64_t)DAT_P_LAG), done_q((size_t)h, 0), done_r((size_t)h, 0);
-            int64_t slot = 0;
-            if (!identity)
-                for (int k = 0; k < h; ++k) {
-                    const int l = order[k];
-                    for (int64_t t = 0; t < tb[l + 1] - tb[l]; ++t) { at(slot).n = part(l, t); done_n[l] = slot++; }
-                }
-            slot = 0;
-            for (int k = 0; k < h; ++k) {
-                const int l = order[k];
-                const int64_t T = tb[l + 1] - tb[l];
-                slot = std::max(slot, done_n[l] + DAT_P_LAG + 1);
-                // a layer that L2 cannot hold next to what streams in meanwhile is walked back from its last
-                // tile (what N read last, and marked to stay, is read first); the others in N's order
-                const bool reverse = T >= DAT_P_REVERSE_FROM;
-                for (int64_t t = 0; t < T; ++t) { at(slot).q = part(l, reverse ? T - 1 - t : t); done_q[l] = slot++; }
-            }
-            if (two) {
-                slot = 0;
-                for (int k = 0; k < h; ++k) {
-                    const int l = order[k];
-                    slot = std::max(slot, done_q[l] + DAT_P_LAG_U + 1);
-                    for (int64_t t = 0; t < tb[l + 1] - tb[l]; ++t) { at(slot).r = part(l, t); done_r[l] = slot++; }
-                }
-            }
-            slot = 0;
-            for (int k = 0; k < h; ++k) {
-                const int l = order[k];
-                slot = std::max(slot, (two ? done_r[l] : done_q[l]) + DAT_P_LAG_U + 1);
-                for (int64_t t = 0; t < tb[l + 1] - tb[l]; ++t) { at(slot).u = part(l, t); ++slot; }
-            }
-            return items;
-        };
-        const std::vector<PipeItem> items = build(false);
-        const std::vector<PipeItem> items2 = identity ? std::vector<PipeItem>() : build(true);
+        const std::vector<PipeItem> items = p_items(plan, tb, 0, h, false);
+        const std::vector<PipeItem> items2 = identity ? std::vector<PipeItem>() : p_items(plan, tb, 0, h, true);
+        g->tile_base = tb;
         g->n_items2 = (int64_t)items2.size();
         g->n_items = (int64_t)items.size();
 
@@ -884,6 +900,49 @@ int dat_pipe_build(dat_plan_t *plan)
     return DAT_OK;
 }
 
+// The plan's layers cut into at most `most` contiguous groups of about equal size; *bytes: the device memory their
+// lists take, which dat_pipe_groups_upload fills (synchronous).
+int dat_pipe_groups(dat_plan_t *plan, int most, size_t *bytes)
+{
+    PipeSchedule *g = plan->pipe;
+    if (!g || !g->mem) return DAT_ERR_ARG;
+    try {
+        if (g->groups.empty())
+            for (int64_t l0 = 0, l1; l0 < plan->h; l0 = l1) {
+                const int64_t left = most - (int64_t)g->groups.size();
+                const int64_t want = plan->offsets[l0] + (plan->d - plan->offsets[l0] + left - 1) / left;
+                for (l1 = l0 + 1; left > 1 && l1 < plan->h && plan->offsets[l1] < want; ++l1) {}
+                if (left <= 1) l1 = plan->h;
+                const std::vector<PipeItem> list = p_items(plan, g->tile_base, (int)l0, (int)l1, false);
+                g->groups.push_back(PipeGroup{plan->offsets[l0], plan->offsets[l1], (int64_t)g->group_items.size(), (int64_t)list.size()});
+                g->group_items.insert(g->group_items.end(), list.begin(), list.end());
+            }
+    } catch (...) {
+        g->groups.clear();
+        g->group_items.clear();
+        return DAT_ERR_NOMEM;
+    }
+    *bytes = g->group_items.size() * sizeof(PipeItem);
+    return DAT_OK;
+}
+
+int dat_pipe_groups_upload(dat_plan_t *plan, void *mem)
+{
+    PipeSchedule *g = plan->pipe;
+    DAT_CUDA(plan, cudaMemcpy(mem, g->group_items.data(), g->group_items.size() * sizeof(PipeItem), cudaMemcpyHostToDevice));
+    g->d_group_items = (PipeItem *)mem;
+    g->group_items = std::vector<PipeItem>();
+    return DAT_OK;
+}
+
+int dat_pipe_group_count(const dat_plan_t *plan) { return (int)plan->pipe->groups.size(); }
+
+void dat_pipe_group_range(const dat_plan_t *plan, int k, int64_t *e0, int64_t *e1)
+{
+    *e0 = plan->pipe->groups[(size_t)k].e0;
+    *e1 = plan->pipe->groups[(size_t)k].e1;
+}
+
 // After a call that timed out the arrival counters and the ticket are left mid-way: clear them
 // (enqueued on `s`; called by dat_get_status when it finds DAT_STATUS_TIMEOUT).
 cudaError_t dat_pipe_reset(dat_plan_t *plan, cudaStream_t s)
@@ -898,7 +957,7 @@ cudaError_t dat_pipe_reset(dat_plan_t *plan, cudaStream_t s)
 static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, const float *const *grads,
                     uint64_t seed, uint64_t step, const dat_hparams_t *hp, const LambConst *lamb, float lr, float c_l, float c_u,
                     int32_t *code_sum_out, float *layer_norms_out, float *scales_out, void *stream,
-                    float *g_hat = nullptr, float *server_scales_out = nullptr)
+                    float *g_hat = nullptr, float *server_scales_out = nullptr, const PipeGroup *group = nullptr)
 {
     if (step >> 32) return DAT_ERR_ARG;
     if (plan->elem_base || plan->worker_base) return DAT_ERR_UNSUPPORTED;     // a slice of a larger problem: separate calls only
@@ -924,7 +983,7 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
     a.keys = dat_make_keys(seed, step);
     dat_make_worker_table(a.keys, plan->M, &a.workers);
     a.wide = dat_grads_wide(plan, grads) && (((uintptr_t)theta | (uintptr_t)mom | (uintptr_t)var | (uintptr_t)g_hat) & 31u) == 0;
-    a.items = two ? g->d_items2 : g->d_items;
+    a.items = group ? g->d_group_items + group->first : two ? g->d_items2 : g->d_items;
     a.off = plan->d_offsets;
     a.tile_base = g->d_tile_base;
     a.theta = theta;
@@ -967,7 +1026,7 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
     a.c_u = c_u;
     if (++g->epoch == 0u) ++g->epoch;              // 0 is what the words hold before the first call
     a.epoch = g->epoch;
-    a.n_items = (uint32_t)(two ? g->n_items2 : g->n_items);
+    a.n_items = (uint32_t)(group ? group->n_items : two ? g->n_items2 : g->n_items);
     a.M = plan->M;
     a.h = (int)plan->h;
     a.d = plan->d;
@@ -991,6 +1050,14 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
 #undef P_GO
     DAT_LAUNCHED(plan);
     return DAT_OK;
+}
+
+// dat_step on the layers of one group.
+int dat_pipe_step_group(dat_plan_t *plan, int k, float *theta, float *mom, const float *const *grads, uint64_t seed, uint64_t step,
+                        const dat_hparams_t *hp, cudaStream_t s)
+{
+    return p_launch(plan, theta, mom, nullptr, grads, seed, step, hp, nullptr, hp->lr, hp->c_l, hp->c_u, nullptr, nullptr, nullptr, s,
+                    nullptr, nullptr, &plan->pipe->groups[(size_t)k]);
 }
 
 extern "C" int dat_step_pipelined(dat_plan_t *plan, float *theta, float *mom, const float *const *grads,
