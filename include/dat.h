@@ -318,8 +318,9 @@ int dat_lalr_step_static(int64_t num_layers, const int64_t *layer_offsets, float
  * dat_step -- Steps 7, 9 and 12 of Algorithm A1 in one call: the result equals
  * dat_quantize -> dat_aggregate -> dat_lalr_step (or dat_average -> dat_lalr_step when b = 32),
  * but codes, code sums and g_hat are never written to device memory.  One kernel launch
- * (dat_step_pipelined); nothing is allocated and nothing synchronises: every table the launch
- * needs was built by dat_plan_create.
+ * (dat_step_pipelined) for problems that fill the GPU, one launch per phase (dat_step_passes) for smaller ones and
+ * for a single worker; nothing is allocated and nothing synchronises: every table the launches
+ * need was built by dat_plan_create.
  *   theta, mom        device fp32[d], updated in place.
  *   grads             host array of M device pointers, fp32[d] each, read-only.
  *   seed, step        as in dat_quantize.
@@ -344,7 +345,7 @@ int dat_step(dat_plan_t *plan, float *theta, float *mom, const float *const *gra
              uint64_t seed, uint64_t step, const dat_hparams_t *hp,
              int32_t *code_sum_out, float *layer_norms_out, float *scales_out, void *stream);
 
-/* dat_step_pipelined -- what dat_step calls: the step as ONE launch of ordinary thread blocks.  The
+/* dat_step_pipelined -- what dat_step calls for large problems: the step as ONE launch of ordinary thread blocks.  The
  * vector is cut into per-layer tiles; a work item holds one tile for each of three phases -- sums of
  * squares for the quantizer norms (N), levels + signed sum + g_hat + m' + layer sums (Q), parameter
  * update (U) -- with the Q tiles running a fixed distance behind the N tiles and the U tiles behind the
@@ -391,10 +392,10 @@ int dat_step_lamb_two_sided(dat_plan_t *plan, float *theta, float *mom, float *v
                             float *server_scales_out, void *stream);
 
 /* dat_step_passes -- the same step as dat_step, with the same arguments and the same results bit for
- * bit up to the norms' last place, computed by three streaming passes in separate launches: quantizer
- * norms; then levels, signed sum over the workers, g_hat, m' and the layer sums in one pass that keeps
- * codes, sums and g_hat in registers; then the theta update.  The gradients are read twice by
- * construction.  For plans with b < 32 and the shared scale (DAT_ERR_UNSUPPORTED otherwise). */
+ * bit up to the norms' last place, as one launch per phase: quantizer norms; then levels, signed sum over the
+ * workers, g_hat, m' and the layer sums in one pass that keeps codes, sums and g_hat in registers; then the theta
+ * update.  What dat_step does for small problems, whatever the size.  For plans with b < 32 and the shared scale
+ * (DAT_ERR_UNSUPPORTED otherwise). */
 int dat_step_passes(dat_plan_t *plan, float *theta, float *mom, const float *const *grads,
                     uint64_t seed, uint64_t step, const dat_hparams_t *hp, int32_t *code_sum_out,
                     float *layer_norms_out, float *scales_out, void *stream);

@@ -100,6 +100,7 @@ void dat_make_worker_table(const PhiloxKeys &keys, int M, PhiloxWorkers *out);
 int dat_pipe_build(dat_plan_t *plan);                        // dat_pipeline.cu (device current)
 void dat_pipe_destroy(dat_plan_t *plan);
 cudaError_t dat_pipe_reset(dat_plan_t *plan, cudaStream_t s);
+int dat_norm_phase(dat_plan_t *plan, const GradPtrs &gp, float *scales_out, cudaStream_t s);      // dat_unfused.cu
 int dat_pipe_groups(dat_plan_t *plan, int most, size_t *bytes);      // the step group by group (dat_step_host)
 int dat_pipe_groups_upload(dat_plan_t *plan, void *mem);
 int dat_pipe_group_count(const dat_plan_t *plan);
@@ -383,6 +384,17 @@ __device__ __forceinline__ void dat_load4(const float *__restrict__ p, int64_t e
     }
 }
 
+// The same without a branch: reads inside the layer only, what lies outside is 0.  Several of these stay in flight.
+__device__ __forceinline__ void dat_load4_masked(const float *__restrict__ p, int64_t e0, int64_t lo, int64_t hi, float v[4])
+{
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int64_t e = e0 + j;
+        const float x = p[max(lo, min(e, hi - 1))];
+        v[j] = (e >= lo && e < hi) ? x : 0.0f;
+    }
+}
+
 __device__ __forceinline__ void dat_store4(float *__restrict__ p, int64_t e0, int64_t lo,
                                            int64_t hi, const float v[4])
 {
@@ -488,20 +500,6 @@ __device__ __forceinline__ bool dat_aligned32(const void *p) { return ((uintptr_
 // Levels and signed sum over the workers for one thread's group of eight consecutive elements
 // (Eq. xi, Eq. grad_agg), shared by the kernels that keep codes and sums in registers.
 // ------------------------------------------------------------------------------------------
-#define DAT_QU_THREADS 256
-#ifndef DAT_QU_GROUPS
-#define DAT_QU_GROUPS 2                          // groups of 8 elements per thread
-#endif
-#ifndef DAT_QU_UNROLL
-#define DAT_QU_UNROLL 2                          // workers whose loads and Philox blocks are in flight together
-#endif
-#ifndef DAT_QU_MINB
-#define DAT_QU_MINB 4                            // resident CTAs per SM asked for (64 registers per thread): this pass lives on many warps
-#endif
-#define DAT_QU_TILE (DAT_QU_THREADS * 8 * DAT_QU_GROUPS)
-#define DAT_QU_PRAGMA(x) _Pragma(#x)
-#define DAT_QU_UNROLL_N(n) DAT_QU_PRAGMA(unroll n)
-
 struct QuConst {
     float t, ts, two_b, inv_two_b, den_b;         // S/nu_l, S/nu_l 2^-b, 2^b, 2^-b, 2^(b-149)
     uint32_t ubits;                               // the bits of 2^-b
@@ -531,12 +529,12 @@ struct PhiloxWorkers {
 // are then exact sums of denormal numbers (|sum| < 2^23 units), brought back by an exact scaling at the end.  Per
 // element: one DP2A for (1 + u) 2^-b, three fused multiply-adds and one LOP3 for the sign.  The issue-limited time of
 // this loop per group and worker went from 165 to about 115 cycles per scheduler (both multiply pipe and ALU full).
-template <bool RNG16>
+template <bool RNG16, int UNROLL>
 __device__ __forceinline__ void qu_rows(const GradPtrs &gp, const PhiloxKeys &keys, const PhiloxWorkers &pw, const QuConst &qc, int M, int64_t e0, float acc[8])
 {
     const PhiloxGroup<RNG16> pg = dat_philox_group<RNG16>((uint64_t)e0, keys);
-    DAT_QU_UNROLL_N(DAT_QU_UNROLL)
-    for (int i = 0; i < M; ++i) {
+#pragma unroll UNROLL
+    for (int i = 0; i < M; ++i) {          // UNROLL workers' loads and Philox blocks in flight together
         float v[8];
         dat_ld8<EV_FIRST>(gp.p[i] + e0, qc.wide, v);         // a gradient is dead once its level is drawn
         uint32_t w[8];
@@ -555,14 +553,15 @@ __device__ __forceinline__ void qu_rows(const GradPtrs &gp, const PhiloxKeys &ke
 
 // The same by the plain form of Eq. xi with whole Philox blocks, for a group at a layer's ragged ends or outside the
 // scaled form's range (same integers).  Sums in units of one level, four at a time (the call passes no array).
-template <bool RNG16>
+template <bool RNG16, int UNROLL>
 __device__ __noinline__ float4 qu_rows_slow4(const GradPtrs &gp, const PhiloxKeys &keys, float t, float two_b, int M, int64_t e0, int64_t lo, int64_t hi)
 {
     float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll 1
-    for (int i = 0; i < M; ++i) {
+#pragma unroll UNROLL
+    for (int i = 0; i < M; ++i) {              // (one lane here holds up its warp)
         float v[4], u1[4];
-        dat_load4(gp.p[i], e0, lo, hi, v);
+        if (UNROLL > 1) dat_load4_masked(gp.p[i], e0, lo, hi, v);
+        else dat_load4(gp.p[i], e0, lo, hi, v);
         dat_u1x4((uint64_t)e0, (uint32_t)i, keys, RNG16, u1);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -572,10 +571,10 @@ __device__ __noinline__ float4 qu_rows_slow4(const GradPtrs &gp, const PhiloxKey
     }
     return make_float4(acc[0], acc[1], acc[2], acc[3]);
 }
-template <bool RNG16>
+template <bool RNG16, int UNROLL>
 __device__ __forceinline__ void qu_rows_slow(const GradPtrs &gp, const PhiloxKeys &keys, const QuConst &qc, int M, int64_t e0, int64_t lo, int64_t hi, float acc[8])
 {
-    const float4 a = qu_rows_slow4<RNG16>(gp, keys, qc.t, qc.two_b, M, e0, lo, hi), b = qu_rows_slow4<RNG16>(gp, keys, qc.t, qc.two_b, M, e0 + 4, lo, hi);
+    const float4 a = qu_rows_slow4<RNG16, UNROLL>(gp, keys, qc.t, qc.two_b, M, e0, lo, hi), b = qu_rows_slow4<RNG16, UNROLL>(gp, keys, qc.t, qc.two_b, M, e0 + 4, lo, hi);
     acc[0] = a.x; acc[1] = a.y; acc[2] = a.z; acc[3] = a.w; acc[4] = b.x; acc[5] = b.y; acc[6] = b.z; acc[7] = b.w;
 }
 

@@ -1,5 +1,5 @@
 // dat_step_pipelined: Steps 7, 9 and 12 of Algorithm A1 in ONE launch of ordinary (non-persistent)
-// CTAs.  Codes, integer sums and g_hat never reach memory; the gradients are read twice (for the norm, then
+// CTAs (and, further down, the same parts as one launch per phase, which small problems take: see p_phases).  Codes, integer sums and g_hat never reach memory; the gradients are read twice (for the norm, then
 // for the levels), the second time from L2 only where a layer is small enough to still be there.
 //
 // The quantizer norm of a layer (Eq. rand_q) must be known before the first level of that layer
@@ -78,13 +78,13 @@ struct PipeSchedule {
     size_t mem_bytes = 0;
     PipeItem *d_items = nullptr;                  // the three streams N, Q, U
     int64_t n_items = 0;
+    PipePart *d_parts = nullptr;                  // n_tiles: every tile once, in slot order (the phases)
     PipeItem *d_items2 = nullptr;                 // the four streams N, Q, R, U of the two-sided step
     int64_t n_items2 = 0;
-    double *d_partR = nullptr;                    // n_tiles
+    double *d_partR = nullptr;                    // 1 per half tile
     float *d_server = nullptr;                    // 2h: S / nu^_l and nu^_l / S
-    int64_t *d_tile_base = nullptr;               // h + 1
     double *d_partN = nullptr;                    // n_tiles * M
-    double *d_partQ = nullptr;                    // n_tiles * 2
+    double *d_partQ = nullptr;                    // 2 per half tile
     uint32_t *d_sync = nullptr;                   // [0] ticket, [1] abort epoch, then cntN[h], cntQ[h], readyN[h], readyQ[h], cntR[h], readyR[h]
     size_t sync_bytes = 0;
     int64_t n_tiles = 0;
@@ -101,7 +101,7 @@ struct PArgs {
     PhiloxKeys keys;
     PhiloxWorkers workers;
     const PipeItem *items;
-    const int64_t *off, *tile_base;
+    const PipePart *parts;
     float *theta, *mom, *var;                     // var: second moment (LAMB only)
     LambConst lamb;
     double *partN, *partQ, *partR;
@@ -386,14 +386,15 @@ __device__ __forceinline__ void p_quant_finish(const PArgs &a, const PipePart &p
 // with one fused multiply-add per worker, ascending; the caller divides by S*M.  Levels by the scaled form (see
 // qu_rows) with the worker's own S/nu_{i,l}; by the plain form of Eq. xi at a layer's ragged ends and where the scaled
 // form does not apply to some worker (one path for all workers of a group: the sum is ordered).
-template <bool RNG16>
+template <bool RNG16, int UNROLL>
 __device__ __noinline__ float4 p_rows_per_worker_slow4(const PArgs &a, const float2 *s_fac, int64_t e0, int64_t lo, int64_t hi)
 {
     float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll 1
+#pragma unroll UNROLL
     for (int i = 0; i < a.M; ++i) {
         float v[4], u1[4];
-        dat_load4(a.gp.p[i], e0, lo, hi, v);
+        if (UNROLL > 1) dat_load4_masked(a.gp.p[i], e0, lo, hi, v);
+        else dat_load4(a.gp.p[i], e0, lo, hi, v);
         dat_u1x4((uint64_t)e0, (uint32_t)i, a.keys, RNG16, u1);
         const float2 fac = s_fac[i];
 #pragma unroll
@@ -404,11 +405,11 @@ __device__ __noinline__ float4 p_rows_per_worker_slow4(const PArgs &a, const flo
     }
     return make_float4(acc[0], acc[1], acc[2], acc[3]);
 }
-template <bool RNG16>
+template <bool RNG16, int UNROLL>
 __device__ __forceinline__ void p_rows_per_worker(const PArgs &a, const QuConst &qc, const float2 *s_fac, bool fast, int64_t e0, int64_t lo, int64_t hi, float acc[8])
 {
     if (!fast) {
-        const float4 x = p_rows_per_worker_slow4<RNG16>(a, s_fac, e0, lo, hi), y = p_rows_per_worker_slow4<RNG16>(a, s_fac, e0 + 4, lo, hi);
+        const float4 x = p_rows_per_worker_slow4<RNG16, UNROLL>(a, s_fac, e0, lo, hi), y = p_rows_per_worker_slow4<RNG16, UNROLL>(a, s_fac, e0 + 4, lo, hi);
         acc[0] = x.x; acc[1] = x.y; acc[2] = x.z; acc[3] = x.w; acc[4] = y.x; acc[5] = y.y; acc[6] = y.z; acc[7] = y.w;
         return;
     }
@@ -469,8 +470,9 @@ __device__ __forceinline__ void p_direction(const PArgs &a, int64_t e0, int64_t 
 // (Eq. 3, pass 1) of one tile; codes, sums and g_hat stay in registers.  Leaves the tile's two sums per
 // warp in scratch[2w], scratch[2w + 1].  TWO (Algorithm A1 Step 10 follows): stops at g_hat, which is
 // stored, and leaves the tile's sum of g_hat^2 per warp in scratch[2w]. ----------------------------
-template <bool RNG16, int MODE, int OPT, bool TWO>
-__device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt, double *scratch, float2 *s_fac)
+// G: groups of eight per thread, from the tile's piece `piece` on (G = 2: the whole tile, piece 0; G = 1: half a tile).
+template <bool RNG16, int MODE, int OPT, bool TWO, int G>
+__device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt, int piece, double *scratch, float2 *s_fac)
 {
     const int M = a.M, layer = pt.layer;
     const int64_t lo = pt.lo, hi = pt.hi;
@@ -488,9 +490,9 @@ __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt,
         plain |= __syncthreads_or(out);
     }
     double ss_theta = 0.0, ss_u = 0.0;
-    const int64_t begin = p_tile_begin(pt);
+    const int64_t begin = p_tile_begin(pt) + (int64_t)piece * (8 * DAT_P_THREADS);
 #pragma unroll 1
-    for (int k = 0; k < DAT_P_GROUPS; ++k) {
+    for (int k = 0; k < G; ++k) {
         const int64_t e0 = begin + 8 * (int64_t)(k * DAT_P_THREADS + threadIdx.x);
         if (e0 >= hi) continue;
         const bool full = (e0 >= lo && e0 + 8 <= hi);
@@ -505,9 +507,9 @@ __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt,
 #pragma unroll
                 for (int j = 0; j < 8; ++j) acc[j] += v[j];
             }
-        } else if (MODE == P_MODE_PER_WORKER) p_rows_per_worker<RNG16>(a, qc, s_fac, full && !plain, e0, lo, hi, acc);
-        else if (full && !plain) qu_rows<RNG16>(a.gp, a.keys, a.workers, qc, M, e0, acc);       // nearly always
-        else qu_rows_slow<RNG16>(a.gp, a.keys, qc, M, e0, lo, hi, acc);
+        } else if (MODE == P_MODE_PER_WORKER) p_rows_per_worker<RNG16, G == 1 ? 4 : 1>(a, qc, s_fac, full && !plain, e0, lo, hi, acc);
+        else if (full && !plain) qu_rows<RNG16, G == 1 ? 4 : 2>(a.gp, a.keys, a.workers, qc, M, e0, acc);       // nearly always
+        else qu_rows_slow<RNG16, G == 1 ? 4 : 1>(a.gp, a.keys, qc, M, e0, lo, hi, acc);
         if (TWO) {
             if (MODE == P_MODE_SHARED && a.code_sum) {
 #pragma unroll
@@ -570,16 +572,16 @@ __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt,
 // ---- R: Algorithm A1 Step 10 on one tile.  g_hat <- nu^_l * sign * level / S with the level of Eq. xi
 // drawn on the random stream of index M (the first one no worker uses), then m' and the layer sums as in
 // the Q part of the one-sided step. ------------------------------------------------------------------
-template <bool RNG16, int OPT>
-__device__ __forceinline__ void p_part_requant(const PArgs &a, const PipePart &pt, double *scratch)
+template <bool RNG16, int OPT, int G>
+__device__ __forceinline__ void p_part_requant(const PArgs &a, const PipePart &pt, int piece, double *scratch)
 {
     const int64_t lo = pt.lo, hi = pt.hi;
     const float t = __ldcg(a.qmul2 + pt.layer), f = __ldcg(a.dq2 + pt.layer);
     const float two_b = a.S_f + 1.0f;
     double ss_theta = 0.0, ss_u = 0.0;
-    const int64_t begin = p_tile_begin(pt);
+    const int64_t begin = p_tile_begin(pt) + (int64_t)piece * (8 * DAT_P_THREADS);
 #pragma unroll 1
-    for (int k = 0; k < DAT_P_GROUPS; ++k) {
+    for (int k = 0; k < G; ++k) {
         const int64_t e0 = begin + 8 * (int64_t)(k * DAT_P_THREADS + threadIdx.x);
         if (e0 >= hi) continue;
         float v[8];
@@ -659,14 +661,14 @@ __device__ __forceinline__ bool p_quant_publish(const PArgs &a, const PipePart &
 }
 
 // ---- U: theta' = theta - a_l m' (Eq. 3, pass 2) of one tile ---------------------------------------
-template <int OPT>
-__device__ __forceinline__ void p_part_update(const PArgs &a, const PipePart &pt)
+template <int OPT, int G>
+__device__ __forceinline__ void p_part_update(const PArgs &a, const PipePart &pt, int piece)
 {
     const int64_t lo = pt.lo, hi = pt.hi;
     const float na = -__ldcg(a.step_a + pt.layer);
-    const int64_t begin = p_tile_begin(pt);
+    const int64_t begin = p_tile_begin(pt) + (int64_t)piece * (8 * DAT_P_THREADS);
 #pragma unroll
-    for (int k = 0; k < DAT_P_GROUPS; ++k) {
+    for (int k = 0; k < G; ++k) {
         const int64_t e0 = begin + 8 * (int64_t)(k * DAT_P_THREADS + threadIdx.x);
         if (e0 >= hi) continue;
         float th[8], m[8];
@@ -692,8 +694,11 @@ __device__ __forceinline__ void p_part_update(const PArgs &a, const PipePart &pt
     }
 }
 
+// Resident CTAs per SM: four, at 64 registers.  Without a quantizer there are fewer live values than that and only
+// loads to wait for, so five (ResNet-50, M = 8, b = 32: 240 us with four, 222 with five, 218 with six, which costs 8 million
+// elements, M = 16, 131 instead of 124).
 template <bool RNG16, int MODE, int OPT, bool TWO>
-__global__ void __launch_bounds__(DAT_P_THREADS, DAT_P_MINB)
+__global__ void __launch_bounds__(DAT_P_THREADS, MODE == P_MODE_IDENTITY ? 5 : DAT_P_MINB)
 k_step_pipelined(const __grid_constant__ PArgs a)
 {
     __shared__ double s_unit[4 * DAT_MAX_WORKERS];
@@ -748,7 +753,7 @@ k_step_pipelined(const __grid_constant__ PArgs a)
     __syncthreads();                               // (A)
     if (s_ctl[0]) p_norm_finish<MODE>(a, pn, s_norm);
     bool alive = (s_ctl[1] != 0);
-    if (alive && pq.layer >= 0) p_part_quant<RNG16, MODE, OPT, TWO>(a, pq, s_unit, s_fac);
+    if (alive && pq.layer >= 0) p_part_quant<RNG16, MODE, OPT, TWO, DAT_P_GROUPS>(a, pq, 0, s_unit, s_fac);
     __syncthreads();
     if (TWO) {
         // Step 10: the tile's sum of g_hat^2 counted in; the layer's last tile publishes the server's norm;
@@ -760,7 +765,7 @@ k_step_pipelined(const __grid_constant__ PArgs a)
         if (threadIdx.x == 0) s_ctl[1] = (alive && pm.layer >= 0) ? (int)p_poll(a, a.readyR + pm.layer) : (int)alive;
         __syncthreads();
         alive = (s_ctl[1] != 0);
-        if (alive && pm.layer >= 0) p_part_requant<RNG16, OPT>(a, pm, s_unit);
+        if (alive && pm.layer >= 0) p_part_requant<RNG16, OPT, DAT_P_GROUPS>(a, pm, 0, s_unit);
         __syncthreads();
     }
     if (threadIdx.x == 0) {
@@ -772,7 +777,82 @@ k_step_pipelined(const __grid_constant__ PArgs a)
     }
     __syncthreads();                               // (B)
     if (s_ctl[2]) p_quant_finish(a, pm, s_unit);
-    if (s_ctl[3] && pu.layer >= 0) p_part_update<OPT>(a, pu);
+    if (s_ctl[3] && pu.layer >= 0) p_part_update<OPT, DAT_P_GROUPS>(a, pu, 0);
+}
+
+// ---- the step as separate launches, one per phase: N (k_sumsq), Q, R (two-sided), U ---------------------------------
+// The same parts on one tile per CTA, without tickets and polls: a launch ends when the layers' results are there.  The
+// next phase's CTAs are set up under the last ones of the phase before (programmatic dependent launch) and walk the tiles
+// the other way, so that they find in L2 what was touched last.
+__device__ __forceinline__ PipePart p_part_of(const PArgs &a, uint32_t tile)
+{
+    PipePart pt;
+    const uint4 *src = reinterpret_cast<const uint4 *>(a.parts + tile);
+    reinterpret_cast<uint4 *>(&pt)[0] = __ldg(src);
+    reinterpret_cast<uint4 *>(&pt)[1] = __ldg(src + 1);
+    return pt;
+}
+// The part as the partial sums see it: pieces of tiles, each with a slot of its own.
+template <int G>
+__device__ __forceinline__ PipePart p_piece_of(const PipePart &pt, int piece)
+{
+    constexpr int PIECES = DAT_P_GROUPS / G;
+    PipePart x = pt;
+    x.tb *= PIECES;
+    x.T *= PIECES;
+    x.tile = x.tile * PIECES + piece;
+    return x;
+}
+
+// G = 2: a tile per CTA.  G = 1: half a tile (see p_halves): twice the CTAs, and four workers' loads in flight
+// per thread, which then has the registers (300 thousand elements, M = 64: 166 us with G = 2, 121 with G = 1).
+template <bool RNG16, int MODE, int OPT, bool TWO, int G>
+__global__ void __launch_bounds__(DAT_P_THREADS, G == 1 ? 3 : DAT_P_MINB)
+k_phase_quant(const __grid_constant__ PArgs a)
+{
+    constexpr int PIECES = DAT_P_GROUPS / G;
+    __shared__ double s_red[2 * (DAT_P_THREADS / 32)];
+    __shared__ float2 s_fac[MODE == P_MODE_PER_WORKER ? DAT_MAX_WORKERS : 1];
+    __shared__ bool s_last;
+    const uint32_t cta = gridDim.x - 1u - blockIdx.x;
+    const PipePart pt = p_part_of(a, cta / PIECES), pp = p_piece_of<G>(pt, cta % PIECES);
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
+    p_part_quant<RNG16, MODE, OPT, TWO, G>(a, pt, cta % PIECES, s_red, s_fac);
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = TWO ? p_server_publish(a, pp, s_red) : p_quant_publish(a, pp, s_red);
+    __syncthreads();
+    if (!s_last) return;
+    if (TWO) p_server_finish(a, pp, s_red);
+    else p_quant_finish(a, pp, s_red);
+}
+
+template <bool RNG16, int OPT, int G>
+__global__ void __launch_bounds__(DAT_P_THREADS, DAT_P_MINB)
+k_phase_requant(const __grid_constant__ PArgs a)
+{
+    constexpr int PIECES = DAT_P_GROUPS / G;
+    __shared__ double s_red[2 * (DAT_P_THREADS / 32)];
+    __shared__ bool s_last;
+    const PipePart pt = p_part_of(a, blockIdx.x / PIECES), pp = p_piece_of<G>(pt, blockIdx.x % PIECES);
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
+    p_part_requant<RNG16, OPT, G>(a, pt, blockIdx.x % PIECES, s_red);
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = p_quant_publish(a, pp, s_red);
+    __syncthreads();
+    if (s_last) p_quant_finish(a, pp, s_red);
+}
+
+template <int OPT, bool BACK, int G>
+__global__ void __launch_bounds__(DAT_P_THREADS, DAT_P_MINB)
+k_phase_update(const __grid_constant__ PArgs a)
+{
+    constexpr int PIECES = DAT_P_GROUPS / G;
+    const uint32_t cta = BACK ? gridDim.x - 1u - blockIdx.x : blockIdx.x;
+    const PipePart pt = p_part_of(a, cta / PIECES);
+    cudaGridDependencySynchronize();
+    p_part_update<OPT, G>(a, pt, cta % PIECES);
 }
 
 // ---- host: the item list -----------------------------------------------------------------------------
@@ -871,8 +951,12 @@ int dat_pipe_build(dat_plan_t *plan)
         size_t off = 0;
         auto take = [&](size_t bytes) { size_t o = off; off = p_align(off + bytes); return o; };
         const size_t o_items = take(items.size() * sizeof(PipeItem)), o_items2 = take(items2.size() * sizeof(PipeItem));
-        const size_t o_tb = take(((size_t)h + 1) * 8);
-        const size_t o_pn = take((size_t)nt * (size_t)M * 8), o_pq = take((size_t)nt * 16), o_pr = take((size_t)nt * 8);
+        std::vector<PipePart> parts;
+        for (int l = 0; l < h; ++l)
+            for (int64_t t = 0; t < tb[l + 1] - tb[l]; ++t)
+                parts.push_back(PipePart{plan->offsets[l], plan->offsets[l + 1], (int32_t)tb[l], (int32_t)(tb[l + 1] - tb[l]), l, (int32_t)t});
+        const size_t o_parts = take(parts.size() * sizeof(PipePart));
+        const size_t o_pn = take((size_t)nt * (size_t)M * 8), o_pq = take((size_t)nt * 32), o_pr = take((size_t)nt * 16);
         const size_t o_server = take(2 * (size_t)h * 4);
         g->sync_bytes = (2 + 6 * (size_t)h) * 4;
         const size_t o_sync = take(g->sync_bytes);
@@ -884,7 +968,7 @@ int dat_pipe_build(dat_plan_t *plan)
         g->d_items2 = (PipeItem *)(g->mem + o_items2);
         g->d_partR = (double *)(g->mem + o_pr);
         g->d_server = (float *)(g->mem + o_server);
-        g->d_tile_base = (int64_t *)(g->mem + o_tb);
+        g->d_parts = (PipePart *)(g->mem + o_parts);
         g->d_partN = (double *)(g->mem + o_pn);
         g->d_partQ = (double *)(g->mem + o_pq);
         g->d_sync = (uint32_t *)(g->mem + o_sync);
@@ -892,7 +976,7 @@ int dat_pipe_build(dat_plan_t *plan)
         if (e == cudaSuccess) e = cudaMemcpy(g->d_items, items.data(), items.size() * sizeof(PipeItem), cudaMemcpyHostToDevice);
         if (e == cudaSuccess && !items2.empty())
             e = cudaMemcpy(g->d_items2, items2.data(), items2.size() * sizeof(PipeItem), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(g->d_tile_base, tb.data(), ((size_t)h + 1) * 8, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy(g->d_parts, parts.data(), parts.size() * sizeof(PipePart), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) return dat_cuda_fail(plan, e);
     } catch (...) {
         return DAT_ERR_NOMEM;
@@ -952,12 +1036,56 @@ cudaError_t dat_pipe_reset(dat_plan_t *plan, cudaStream_t s)
     return cudaMemsetAsync(g->d_sync, 0, g->sync_bytes, s);
 }
 
+// Which form a step takes.  One launch per phase wins where the GPU is not full: the one launch keeps its streams 256 and
+// 512 items apart, so a small problem runs through waves of nearly empty CTAs (us, one launch / phases, B200):
+//   tiny MLP (61 tiles) M = 4: 22.9 / 18.2    300 thousand elements, M = 8: 38.3 / 24.3, M = 64 in 200 layers: 265 / 121
+//   1 million (290 tiles), M = 8: 50.1 / 37.3, b = 32: 22.1 / 17.5; LAMB 60.3 / 43.4; two-sided 58.7 / 46.0
+// Up to nine tiles per SM it still does, the two-sided step's four launches with few workers excepted:
+//   3 million (800 tiles), M = 16: 119 / 108   4 million, M = 3: 59.1 / 51.1, LAMB M = 8: 107 / 95   5 million, M = 16: 176 / 165
+//   3 million, M = 3, two-sided: 63.9 / 66.1
+// Beyond that the overlap of the streams wins: 8 million (2000 tiles), M = 4: 103 / 102, 60 million, M = 4: 536 / 585, ResNet-50,
+// M = 8: 312 / 381.  With one worker there is little to overlap (a gradient is read twice and the update's vectors four
+// times): 60 million, 413 / 365; LAMB 607 / 531; two-sided 538 / 511.
+#define P_PHASES_WAVE 4                           // tiles per SM: one wave of a phase's CTAs
+#define P_PHASES_MOST 9
+enum { P_BY_RULE = 0, P_ONE_LAUNCH = 1, P_PHASES = 2 };
+static bool p_phases(const dat_plan_t *plan, bool two)
+{
+    const int64_t n = plan->pipe->n_tiles, sm = plan->sm_count;
+    if (n <= P_PHASES_WAVE * sm) return true;
+    if (plan->bits == 32) return false;
+    return plan->M == 1 || (n <= P_PHASES_MOST * sm && (!two || plan->M >= 8));
+}
+// Half a tile per CTA: in one wave, and with many workers (a long loop per CTA, so that a last wave of whole tiles costs
+// much: 2.5 million elements, 617 tiles, M = 32: 185 / 156 us; 4 million, M = 3: 51.1 / 53.5).
+static bool p_halves(const dat_plan_t *plan)
+{
+    const int64_t n = plan->pipe->n_tiles, sm = plan->sm_count;
+    return n <= P_PHASES_WAVE * sm || (n <= P_PHASES_MOST * sm && plan->M >= 8);
+}
+
+// A launch that may be set up while the one before it ends (its kernel waits for that end itself).
+template <class K>
+static cudaError_t p_launch_after(K kernel, unsigned grid, cudaStream_t s, const PArgs &a)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(DAT_P_THREADS);
+    cfg.stream = s;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
 // One launch of the step.  lamb == nullptr: the momentum direction with hp; else Algorithm A2 with *lamb.
 // g_hat != nullptr: the two-sided step (Algorithm A1 Step 10 between the aggregation and the update).
 static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, const float *const *grads,
                     uint64_t seed, uint64_t step, const dat_hparams_t *hp, const LambConst *lamb, float lr, float c_l, float c_u,
                     int32_t *code_sum_out, float *layer_norms_out, float *scales_out, void *stream,
-                    float *g_hat = nullptr, float *server_scales_out = nullptr, const PipeGroup *group = nullptr)
+                    float *g_hat = nullptr, float *server_scales_out = nullptr, const PipeGroup *group = nullptr, int how = P_BY_RULE)
 {
     if (step >> 32) return DAT_ERR_ARG;
     if (plan->elem_base || plan->worker_base) return DAT_ERR_UNSUPPORTED;     // a slice of a larger problem: separate calls only
@@ -984,8 +1112,7 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
     dat_make_worker_table(a.keys, plan->M, &a.workers);
     a.wide = dat_grads_wide(plan, grads) && (((uintptr_t)theta | (uintptr_t)mom | (uintptr_t)var | (uintptr_t)g_hat) & 31u) == 0;
     a.items = group ? g->d_group_items + group->first : two ? g->d_items2 : g->d_items;
-    a.off = plan->d_offsets;
-    a.tile_base = g->d_tile_base;
+    a.parts = g->d_parts;
     a.theta = theta;
     a.mom = mom;
     a.var = var;
@@ -1032,9 +1159,31 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
     a.d = plan->d;
     a.n_tiles = g->n_tiles;
     cudaStream_t s = (cudaStream_t)stream;
-    const unsigned grid = a.n_items;
     const bool rng16 = (plan->rng_bits == 16);
-#define P_GO(R, MODE, OPT, TWO) k_step_pipelined<R, MODE, OPT, TWO><<<grid, DAT_P_THREADS, 0, s>>>(a)
+    const bool phases = !group && how != P_ONE_LAUNCH && (how == P_PHASES || (g->wait_cycles == DAT_P_WAIT_CYCLES && p_phases(plan, two)));
+    const bool halves = phases && p_halves(plan);
+    const unsigned grid = phases ? (unsigned)g->n_tiles * (halves ? 2u : 1u) : a.n_items;
+    if (phases && !identity) {
+        rc = dat_norm_phase(plan, a.gp, a.scales_out, s);
+        if (rc != DAT_OK) return rc;
+    }
+#define P_PHASES_GO(R, MODE, OPT, TWO, G)                                                                           \
+    do {                                                                                                            \
+        if (MODE == P_MODE_IDENTITY) k_phase_quant<R, MODE, OPT, TWO, G><<<grid, DAT_P_THREADS, 0, s>>>(a);         \
+        else DAT_CUDA(plan, p_launch_after(k_phase_quant<R, MODE, OPT, TWO, G>, grid, s, a));                       \
+        DAT_LAUNCHED(plan);                                                                                         \
+        if (TWO) {                                                                                                  \
+            DAT_CUDA(plan, p_launch_after(k_phase_requant<R, OPT, G>, grid, s, a));                                 \
+            DAT_LAUNCHED(plan);                                                                                     \
+        }                                                                                                           \
+        DAT_CUDA(plan, p_launch_after(k_phase_update<OPT, TWO, G>, grid, s, a));                                    \
+    } while (0)
+#define P_GO(R, MODE, OPT, TWO)                                                                                     \
+    do {                                                                                                            \
+        if (!phases) k_step_pipelined<R, MODE, OPT, TWO><<<grid, DAT_P_THREADS, 0, s>>>(a);                         \
+        else if (halves) P_PHASES_GO(R, MODE, OPT, TWO, 1);                                                         \
+        else P_PHASES_GO(R, MODE, OPT, TWO, 2);                                                                     \
+    } while (0)
 #define P_GO_OPT(R, MODE)                                                                                           \
     do {                                                                                                            \
         if (two) { if (lamb) P_GO(R, MODE, P_OPT_LAMB, true); else P_GO(R, MODE, P_OPT_MOMENTUM, true); }           \
@@ -1068,7 +1217,32 @@ extern "C" int dat_step_pipelined(dat_plan_t *plan, float *theta, float *mom, co
     if (rc != DAT_OK) return rc;
     if (!theta || !mom || !hp) return DAT_ERR_ARG;
     return p_launch(plan, theta, mom, nullptr, grads, seed, step, hp, nullptr, hp->lr, hp->c_l, hp->c_u, code_sum_out,
+                    layer_norms_out, scales_out, stream, nullptr, nullptr, nullptr, P_ONE_LAUNCH);
+}
+
+// dat_step: Steps 7, 9 and 12 in the form that p_phases chooses.
+extern "C" int dat_step(dat_plan_t *plan, float *theta, float *mom, const float *const *grads,
+                        uint64_t seed, uint64_t step, const dat_hparams_t *hp,
+                        int32_t *code_sum_out, float *layer_norms_out, float *scales_out, void *stream)
+{
+    int rc = dat_check_plan(plan);
+    if (rc != DAT_OK) return rc;
+    if (!theta || !mom || !hp) return DAT_ERR_ARG;
+    return p_launch(plan, theta, mom, nullptr, grads, seed, step, hp, nullptr, hp->lr, hp->c_l, hp->c_u, code_sum_out,
                     layer_norms_out, scales_out, stream);
+}
+
+// dat_step_passes: the same as one launch per phase.
+extern "C" int dat_step_passes(dat_plan_t *plan, float *theta, float *mom, const float *const *grads,
+                               uint64_t seed, uint64_t step, const dat_hparams_t *hp,
+                               int32_t *code_sum_out, float *layer_norms_out, float *scales_out, void *stream)
+{
+    int rc = dat_check_plan(plan);
+    if (rc != DAT_OK) return rc;
+    if (!theta || !mom || !hp) return DAT_ERR_ARG;
+    if (plan->bits == 32 || plan->scale_mode != DAT_SCALE_SHARED_MAX) return DAT_ERR_UNSUPPORTED;
+    return p_launch(plan, theta, mom, nullptr, grads, seed, step, hp, nullptr, hp->lr, hp->c_l, hp->c_u, code_sum_out,
+                    layer_norms_out, scales_out, stream, nullptr, nullptr, nullptr, P_PHASES);
 }
 
 extern "C" int dat_step_lamb(dat_plan_t *plan, float *theta, float *mom, float *var, const float *const *grads,

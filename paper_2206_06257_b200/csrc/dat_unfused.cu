@@ -18,6 +18,8 @@
 struct NormOut {
     float S_f;
     float *worker_norms, *scales, *qmul;
+    float *dq, *scales_out;                       // nu/(S M) and a copy of the norms, if wanted
+    float SM_f;
     uint32_t *count, *status;
     bool per_worker;
 };
@@ -49,30 +51,48 @@ __device__ __forceinline__ void sumsq_finish(int l, int64_t t0, int64_t t1, int 
             for (int i = 0; i < M; ++i) {
                 o.scales[(int64_t)i * h + l] = s_norm[i];
                 o.qmul[(int64_t)i * h + l] = (s_norm[i] == 0.0f) ? 0.0f : o.S_f / s_norm[i];
+                if (o.scales_out) o.scales_out[(int64_t)i * h + l] = s_norm[i];
             }
         } else {
             o.scales[l] = nu;
             o.qmul[l] = (nu == 0.0f) ? 0.0f : o.S_f / nu;
+            if (o.dq) o.dq[l] = (nu == 0.0f) ? 0.0f : nu / o.SM_f;
+            if (o.scales_out) o.scales_out[l] = nu;
         }
         if (bad) atomicOr(o.status, DAT_STATUS_NONFINITE);
         o.count[l] = 0u;                          // ready for the next call
     }
 }
 
-// NW workers' loads in flight per thread.
-template <int NW>
-__global__ void __launch_bounds__(DAT_THREADS, NW == 1 ? 6 : 4)
-k_sumsq(const __grid_constant__ GradPtrs gp, const TileSource tiles, int M, int per_cta, int64_t keep_from, double *partials, const __grid_constant__ NormOut out)
+// A tile's groups of eight that lie partly outside the layer: the first (thread 0) and the last (thread 1).  Returns the
+// group's first element, or -1.
+__device__ __forceinline__ int64_t sumsq_ragged_at(const TileRange &r)
 {
-    constexpr int W = DAT_THREADS / 32, ITERS = DAT_TILE / 8 / DAT_THREADS;
-    __shared__ double s_sum[SUMSQ_WORKERS][W];
-    __shared__ bool s_last;
-    const int64_t tile = blockIdx.x;
-    const int w0 = blockIdx.y * per_cta, w1 = min(w0 + per_cta, M);
+    const int64_t first = r.begin, last = (r.end - 1) & ~(int64_t)7;
+    if (threadIdx.x == 0) return (first < r.lo || first + 8 > r.hi) ? first : -1;
+    return (last > first && last + 8 > r.hi) ? last : -1;
+}
+__device__ __noinline__ double sumsq_ragged(const float *g, const TileRange &r)
+{
+    const int64_t e0 = sumsq_ragged_at(r);
+    float v[8];
+    dat_load4_masked(g, e0, r.lo, r.hi, v);
+    dat_load4_masked(g, e0 + 4, r.lo, r.hi, v + 4);
+    double acc = 0.0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc = fma((double)v[j], (double)v[j], acc);
+    return acc;
+}
+
+// The tile's sums of workers [w0, w1), one per warp and worker, into s_sum.  NW workers' loads in flight per thread.
+// INSIDE: the tile lies wholly in the layer.
+template <int NW, bool INSIDE>
+__device__ __forceinline__ void sumsq_rows(const GradPtrs &gp, const TileRange &r, int w0, int w1, bool keep, double (*s_sum)[DAT_THREADS / 32])
+{
+    constexpr int ITERS = DAT_TILE / 8 / DAT_THREADS;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const TileRange r = dat_tile_range(tiles, tile);
-    const bool inside = r.begin >= r.lo && r.begin + DAT_TILE <= r.hi;
-    const bool keep = tile >= keep_from;          // read again first thing by the call that follows (which walks back)
+    // a group at one of the layer's ends that is not whole (threads 0 and 1 look after the two)
+    const bool ragged = !INSIDE && threadIdx.x < 2 && sumsq_ragged_at(r) >= 0;
     for (int i = w0; i < w1; i += NW) {           // every load of NW workers is in flight before the first is used
         float v[NW][ITERS][8];
 #pragma unroll
@@ -82,13 +102,12 @@ k_sumsq(const __grid_constant__ GradPtrs gp, const TileSource tiles, int M, int 
 #pragma unroll
             for (int it = 0; it < ITERS; ++it) {
                 const int64_t e0 = r.begin + 8 * (int64_t)(it * DAT_THREADS + threadIdx.x);
-                if (inside && i + p < w1) {
+                if (i + p < w1 && (INSIDE || (e0 >= r.lo && e0 + 8 <= r.hi))) {
                     if (keep) dat_ld8<EV_NORMAL>(g + e0, wide, v[p][it]);
                     else dat_ld8<EV_FIRST>(g + e0, wide, v[p][it]);
-                }
-                else {
+                } else {
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) v[p][it][j] = (i + p < w1 && e0 + j >= r.lo && e0 + j < r.end) ? g[e0 + j] : 0.0f;
+                    for (int j = 0; j < 8; ++j) v[p][it][j] = 0.0f;
                 }
             }
         }
@@ -99,10 +118,28 @@ k_sumsq(const __grid_constant__ GradPtrs gp, const TileSource tiles, int M, int 
             for (int it = 0; it < ITERS; ++it)
 #pragma unroll
                 for (int j = 0; j < 8; ++j) acc = fma((double)v[p][it][j], (double)v[p][it][j], acc);
+            if (ragged && i + p < w1) acc += sumsq_ragged(gp.p[i + p], r);
             acc = dat_warp_sum(acc);
             if (lane == 0 && i + p < w1) s_sum[i + p - w0][warp] = acc;
         }
     }
+}
+
+template <int NW>
+__global__ void __launch_bounds__(DAT_THREADS, NW == 1 ? 6 : 4)
+k_sumsq(const __grid_constant__ GradPtrs gp, const TileSource tiles, int M, int per_cta, int64_t keep_from, double *partials, const __grid_constant__ NormOut out)
+{
+    constexpr int W = DAT_THREADS / 32;
+    __shared__ double s_sum[SUMSQ_WORKERS][W];
+    __shared__ bool s_last;
+    cudaTriggerProgrammaticLaunchCompletion();    // a step's next phase may set itself up; it waits for this one's end
+    const int64_t tile = blockIdx.x;
+    const int w0 = blockIdx.y * per_cta, w1 = min(w0 + per_cta, M);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const TileRange r = dat_tile_range(tiles, tile);
+    const bool keep = tile >= keep_from;          // read again first thing by the call that follows (which walks back)
+    if (r.begin >= r.lo && r.begin + DAT_TILE <= r.hi) sumsq_rows<NW, true>(gp, r, w0, w1, keep, s_sum);
+    else sumsq_rows<NW, false>(gp, r, w0, w1, keep, s_sum);
     __syncthreads();
     for (int i = threadIdx.x; i < w1 - w0; i += DAT_THREADS) {
         double s = 0.0;
@@ -121,9 +158,8 @@ k_sumsq(const __grid_constant__ GradPtrs gp, const TileSource tiles, int M, int 
 
 static TileSource plan_tiles(const dat_plan_t *plan) { return TileSource{plan->d_tiles, plan->d_offsets, plan->d_tile_base, (int)plan->h}; }
 
-static int sumsq_launch(dat_plan_t *plan, const GradPtrs &gp, int M, float *scales, bool per_worker, cudaStream_t s, float *norms_out = nullptr)
+static int sumsq_go(dat_plan_t *plan, const GradPtrs &gp, int M, const NormOut &o, cudaStream_t s)
 {
-    const NormOut o = {(float)plan->S, norms_out ? norms_out : plan->d_worker_norms, scales, plan->d_qmul, plan->d_count, plan->d_status, per_worker};
     // several workers in a CTA (fewer arrivals at the layer's counter, a longer stream per CTA) as long as the CTAs
     // still fill the GPU
     int per_cta = 1;
@@ -134,6 +170,22 @@ static int sumsq_launch(dat_plan_t *plan, const GradPtrs &gp, int M, float *scal
     else k_sumsq<2><<<grid, DAT_THREADS, 0, s>>>(gp, plan_tiles(plan), M, per_cta, keep_from, plan->d_partials, o);
     DAT_LAUNCHED(plan);
     return DAT_OK;
+}
+
+static int sumsq_launch(dat_plan_t *plan, const GradPtrs &gp, int M, float *scales, bool per_worker, cudaStream_t s, float *norms_out = nullptr)
+{
+    const NormOut o = {(float)plan->S, norms_out ? norms_out : plan->d_worker_norms, scales, plan->d_qmul, nullptr, nullptr, 1.0f,
+                       plan->d_count, plan->d_status, per_worker};
+    return sumsq_go(plan, gp, M, o, s);
+}
+
+// The norms as the step's phases want them (dat_pipeline.cu): with the layers' nu/(S M).
+int dat_norm_phase(dat_plan_t *plan, const GradPtrs &gp, float *scales_out, cudaStream_t s)
+{
+    const NormOut o = {(float)plan->S, plan->d_worker_norms, plan->scale_mode == DAT_SCALE_PER_WORKER ? plan->d_worker_norms : plan->d_scales, plan->d_qmul,
+                       plan->d_dq, scales_out, (float)((uint64_t)plan->S * (uint64_t)plan->M), plan->d_count, plan->d_status,
+                       plan->scale_mode == DAT_SCALE_PER_WORKER};
+    return sumsq_go(plan, gp, plan->M, o, s);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1215,106 +1267,4 @@ extern "C" int dat_lalr_step_static(int64_t num_layers, const int64_t *layer_off
     k_update_pass2<OPT_MOMENTUM><<<(unsigned)nt, DAT_THREADS, 0, s>>>(a);
     if (cudaGetLastError() != cudaSuccess) return DAT_ERR_CUDA;
     return DAT_OK;
-}
-
-// ------------------------------------------------------------------------------------------
-// dat_step_passes: Steps 7, 9 and 12 of Algorithm A1 as three streaming passes without the
-// packed message -- norms; levels, signed sum over the workers, g_hat, m' and the layer sums
-// in one kernel (codes, sums and g_hat stay in registers); theta update.  The same arithmetic
-// as dat_step, element by element; what differs is that the gradients are read from memory
-// twice by construction and that the passes are separate launches.
-// ------------------------------------------------------------------------------------------
-template <bool RNG16>
-__global__ void __launch_bounds__(DAT_QU_THREADS, DAT_QU_MINB)
-k_quant_update(const __grid_constant__ GradPtrs gp, const __grid_constant__ PhiloxKeys keys, const __grid_constant__ PhiloxWorkers pw,
-               const __grid_constant__ UpdateArgs a, int M, const float *__restrict__ qmul, const float *__restrict__ scales, float S_f, float SM_f,
-               int32_t *__restrict__ code_sum)
-{
-    static_assert(DAT_QU_TILE == DAT_TILE && DAT_QU_THREADS == DAT_THREADS, "the plan's tiles");
-    __shared__ double scratch[DAT_THREADS / 32];
-    __shared__ bool s_last;
-    const int64_t tile = (int64_t)gridDim.x - 1 - blockIdx.x;     // back from the last tile: what k_sumsq read last is in L2
-    const TileRange r = dat_tile_range(a.tiles, tile);
-    const int64_t lo = r.lo, hi = r.hi;
-    const float nu = __ldg(scales + r.layer), f = (nu == 0.0f) ? 0.0f : nu / SM_f;
-    const QuConst qc = dat_qu_const(__ldg(qmul + r.layer), S_f, a.wide);
-    const bool plain = dat_qu_plain<RNG16>(qc, r.begin, DAT_TILE);
-    double ss_theta = 0.0, ss_u = 0.0;
-#pragma unroll 1
-    for (int k = 0; k < DAT_QU_GROUPS; ++k) {
-        const int64_t e0 = r.begin + 8 * (int64_t)(k * DAT_QU_THREADS + threadIdx.x);
-        if (e0 >= hi) continue;
-        const bool full = (e0 >= lo && e0 + 8 <= hi);
-        float acc[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[j] = 0.0f;
-        if (full && !plain) qu_rows<RNG16>(gp, keys, pw, qc, M, e0, acc);       // nearly always
-        else qu_rows_slow<RNG16>(gp, keys, qc, M, e0, lo, hi, acc);
-        // theta and m only now: registers are what limits the number of resident warps here
-        float th[8], m[8];
-        update_ld8<EV_LAST>(a.theta, full, a.wide, e0, lo, hi, th);
-        update_ld8<EV_FIRST>(a.mom, full, a.wide, e0, lo, hi, m);
-        if (code_sum) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (e0 + j >= lo && e0 + j < hi) code_sum[e0 + j] = (int)acc[j];
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            m[j] = __fmaf_rn(a.mu, m[j], __fmaf_rn(a.wd, th[j], acc[j] * f));
-            ss_theta = fma((double)th[j], (double)th[j], ss_theta);
-            ss_u = fma((double)m[j], (double)m[j], ss_u);
-        }
-        update_st8<EV_LAST>(a.mom, full, a.wide, e0, lo, hi, m);
-    }
-    update_count_in(a, r, tile, ss_theta, ss_u, scratch, &s_last);
-}
-
-extern "C" int dat_step_passes(dat_plan_t *plan, float *theta, float *mom, const float *const *grads,
-                               uint64_t seed, uint64_t step, const dat_hparams_t *hp,
-                               int32_t *code_sum_out, float *layer_norms_out, float *scales_out, void *stream)
-{
-    int rc = dat_check_plan(plan);
-    if (rc != DAT_OK) return rc;
-    if (!theta || !mom || !hp) return DAT_ERR_ARG;
-    if (plan->bits == 32 || plan->scale_mode != DAT_SCALE_SHARED_MAX || plan->elem_base || plan->worker_base) return DAT_ERR_UNSUPPORTED;
-    if (step >> 32) return DAT_ERR_ARG;
-    if (!dat_aligned16(theta) || !dat_aligned16(mom) || (code_sum_out && !dat_aligned16(code_sum_out)) ||
-        (layer_norms_out && !dat_aligned16(layer_norms_out)) || (scales_out && !dat_aligned16(scales_out)))
-        return DAT_ERR_ALIGN;
-    GradPtrs gp;
-    rc = dat_check_grads(plan, grads, &gp);
-    if (rc != DAT_OK) return rc;
-    cudaStream_t s = (cudaStream_t)stream;
-    const float S_f = (float)plan->S;
-    const float SM_f = (float)((uint64_t)plan->S * (uint64_t)plan->M);
-    rc = sumsq_launch(plan, gp, plan->M, plan->d_scales, false, s);
-    if (rc != DAT_OK) return rc;
-    if (scales_out) DAT_CUDA(plan, cudaMemcpyAsync(scales_out, plan->d_scales, (size_t)plan->h * 4, cudaMemcpyDeviceToDevice, s));
-    const PhiloxKeys keys = dat_make_keys(seed, step);
-    PhiloxWorkers pw;
-    dat_make_worker_table(keys, plan->M, &pw);
-    UpdateArgs ua = update_args(plan, theta, mom, nullptr, nullptr, hp->lr, hp->c_l, hp->c_u, layer_norms_out);
-    ua.mu = hp->momentum;
-    ua.wd = hp->weight_decay;
-    ua.wide = ua.wide && dat_grads_wide(plan, grads);
-    const unsigned grid = (unsigned)plan->n_tiles;
-    if (plan->rng_bits == 16)
-        k_quant_update<true><<<grid, DAT_QU_THREADS, 0, s>>>(gp, keys, pw, ua, plan->M, plan->d_qmul, plan->d_scales, S_f, SM_f, code_sum_out);
-    else
-        k_quant_update<false><<<grid, DAT_QU_THREADS, 0, s>>>(gp, keys, pw, ua, plan->M, plan->d_qmul, plan->d_scales, S_f, SM_f, code_sum_out);
-    DAT_LAUNCHED(plan);
-    k_update_pass2<OPT_MOMENTUM><<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(ua);
-    DAT_LAUNCHED(plan);
-    return DAT_OK;
-}
-
-// ------------------------------------------------------------------------------------------
-// dat_step: one call for Steps 7, 9 and 12 -- the single pipelined launch of dat_pipeline.cu.
-// ------------------------------------------------------------------------------------------
-extern "C" int dat_step(dat_plan_t *plan, float *theta, float *mom, const float *const *grads,
-                        uint64_t seed, uint64_t step, const dat_hparams_t *hp,
-                        int32_t *code_sum_out, float *layer_norms_out, float *scales_out, void *stream)
-{
-    return dat_step_pipelined(plan, theta, mom, grads, seed, step, hp, code_sum_out, layer_norms_out, scales_out, stream);
 }
