@@ -38,7 +38,7 @@ struct TileDesc {
 // Division by a constant y as x*hi + x*lo, hi + lo = 1/y to 2^-48: see dat_const_div (dat_plan.cu).
 struct ConstDiv {
     float y, hi, lo;
-    bool exact;                        // the two-operation form rounds correctly for every x (else: the division itself)
+    bool exact;                        // the two-operation form rounds correctly (for which x: dat_div_short)
 };
 struct LambConst {
     float beta1, beta2, om1, om2, zeta, wd;
@@ -407,18 +407,26 @@ __device__ __forceinline__ void dat_store4(float *__restrict__ p, int64_t e0, in
     }
 }
 
-// x / c.y, correctly rounded (for |x| < 2^-98 possibly off by the last denormal place).
-__device__ __forceinline__ float dat_div(float x, const ConstDiv &c)
+// Whether x*hi + RN(x*lo) is x / c.y correctly rounded: x finite and so large that x*lo keeps its bits (2^-98 <= |x|: the
+// denormal grid is then below 2^-52 of the quotient, see dat_const_div).  Infinities (inf*lo is NaN or of the other
+// sign), zeros and what decays towards them are divided.
+__device__ __forceinline__ bool dat_div_short(float x, const ConstDiv &c)
 {
-    return c.exact ? __fmaf_rn(x, c.hi, __fmul_rn(x, c.lo)) : x / c.y;
+    return c.exact && (__float_as_uint(x) & 0x7FFFFFFFu) - (29u << 23) < ((255u - 29u) << 23);
 }
 
 // The LAMB direction of one element from the stored moments: u = m^/(sqrt(v^) + zeta) + wd*theta with the
 // bias-corrected m^ = m'/(1 - beta1^t), v^ = v'/(1 - beta2^t) (Algorithm A2; one rounding per operation).
 __device__ __forceinline__ float dat_lamb_direction(const LambConst &c, float m_new, float v_new, float theta)
 {
-    const float m_hat = dat_div(m_new, c.bc1);
-    const float v_hat = dat_div(v_new, c.bc2);
+    float m_hat, v_hat;
+    if (dat_div_short(m_new, c.bc1) && dat_div_short(v_new, c.bc2)) {
+        m_hat = __fmaf_rn(m_new, c.bc1.hi, __fmul_rn(m_new, c.bc1.lo));
+        v_hat = __fmaf_rn(v_new, c.bc2.hi, __fmul_rn(v_new, c.bc2.lo));
+    } else {
+        m_hat = m_new / c.bc1.y;
+        v_hat = v_new / c.bc2.y;
+    }
     return __fmaf_rn(c.wd, theta, m_hat / (sqrtf(v_hat) + c.zeta));
 }
 
