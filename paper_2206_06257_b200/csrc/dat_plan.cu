@@ -53,11 +53,11 @@ bool dat_grads_wide(const dat_plan_t *plan, const float *const *grads)
 // rounding, so it can only be wrong for an x whose quotient lies that close to the middle of two floats.  With the
 // 24-bit integers X, Y of the operands' significands, such a quotient has |X 2^s - (2k+1) Y| = e <= 4 for s = 24 or 25;
 // the few X that satisfy one of these congruences are found and tried here.  If one of them fails (none has been seen
-// for 1 - beta^t), the kernels divide; they also divide where x*lo would lose bits to the denormal grid and where x is
-// infinite (dat_div_short).
+// for 1 - beta^t), and where x*lo would lose bits to the denormal grid, the kernels form the quotient in double precision
+// (dat_div_any).
 ConstDiv dat_const_div(float y)
 {
-    ConstDiv c = {y, 0.0f, 0.0f, false};
+    ConstDiv c = {1.0 / (double)y, 0.0f, 0.0f, false};
     if (!(y > 1e-30f && y < 1e30f)) return c;
     c.exact = true;
     c.hi = 1.0f / y;
