@@ -256,11 +256,24 @@ __device__ __forceinline__ void dat_u1x4(uint64_t e0, uint32_t worker, const Phi
 // Stochastic level of one element (Eq. xi): level = min(floor(|g|*qmul + u), S) with u uniform
 // on [0,1).  With u1 = 1 + u in [1,2), y = fma(|g|, qmul, u1) is clamped to S+1 and
 // level = floor(y) - 1.  y lies in [1, 65537): adding 2^23 - 1 with rounding toward -inf leaves
-// floor(y) - 1 in the low mantissa bits.  Returns those float bits, 0x4B000000 + level.
+// floor(y) - 1 in the low mantissa bits.  Returns those float bits, 0x4B000000 + level.  (A NaN has level S.)
 __device__ __forceinline__ uint32_t dat_level_bits_u1(float g, float qmul, float S1_f, float u1)
 {
-    const float y = fminf(__fmaf_rn(fabsf(g), qmul, u1), S1_f);
+    const float y = fminf(__fmaf_rn(fabsf(g), fabsf(qmul), u1), S1_f);
     return __float_as_uint(__fadd_rd(y, 8388607.0f));
+}
+
+// The factor S/nu of a layer with norm nu (0 for a zero layer).  Its sign bit set says that some gradient of the layer is
+// not finite: the scaled form of the level, which knows neither NaN nor infinity times 0, is then left alone.
+__device__ __forceinline__ float dat_level_factor(float nu, float S_f, bool finite)
+{
+    const float t = (nu == 0.0f) ? 0.0f : S_f / nu;
+    return finite ? t : __uint_as_float(__float_as_uint(t) | 0x80000000u);
+}
+// Whether the scaled form applies: t 2^-b is 0 or a normal number.
+__device__ __forceinline__ bool dat_scaled_factor(float t, float two_b)
+{
+    return __float_as_uint(t) == 0u || (t >= 1.17549435e-38f * two_b && t <= 3.402823466e38f);
 }
 
 __device__ __forceinline__ uint32_t dat_level_u1(float g, float qmul, float S1_f, float u1)
@@ -527,11 +540,11 @@ __device__ __forceinline__ QuConst dat_qu_const(float t, float S_f, bool wide)
     const float two_b = S_f + 1.0f, inv_two_b = 1.0f / two_b;
     return QuConst{t, t * inv_two_b, two_b, inv_two_b, two_b * __uint_as_float(1u), __float_as_uint(inv_two_b), wide};
 }
-// Outside the scaled form's range (valid while t 2^-b is a normal number), or beyond the counters of the worker table.
+// Outside the scaled form's range, or beyond the counters of the worker table.
 template <bool RNG16>
 __device__ __forceinline__ bool dat_qu_plain(const QuConst &q, int64_t begin, int64_t n)
 {
-    return (q.t != 0.0f && !(q.t >= 1.17549435e-38f * q.two_b && q.t <= 3.402823466e38f)) || ((begin + n) >> (RNG16 ? 35 : 34)) != 0;
+    return !dat_scaled_factor(q.t, q.two_b) || ((begin + n) >> (RNG16 ? 35 : 34)) != 0;
 }
 
 // The worker-dependent products of the Philox blocks (counter word q_hi = 0), formed on the host per call.

@@ -335,12 +335,12 @@ __device__ __forceinline__ void p_norm_finish(const PArgs &a, const PipePart &pt
         if (MODE == P_MODE_PER_WORKER) {
             // every worker keeps its own norm (Eq. rand_q as written): index i*h + l; nu_{i,l} itself is in worker_norms
             for (int i = 0; i < M; ++i) {
-                a.qmul[(int64_t)i * a.h + layer] = (s_norm[i] == 0.0f) ? 0.0f : a.S_f / s_norm[i];
+                a.qmul[(int64_t)i * a.h + layer] = dat_level_factor(s_norm[i], a.S_f, isfinite(s_norm[i]));
                 if (a.scales_out) a.scales_out[(int64_t)i * a.h + layer] = s_norm[i];
             }
         } else {
             a.scales[layer] = nu;
-            a.qmul[layer] = (nu == 0.0f) ? 0.0f : a.S_f / nu;
+            a.qmul[layer] = dat_level_factor(nu, a.S_f, !bad);
             a.dq[layer] = (nu == 0.0f) ? 0.0f : nu / a.SM_f;
             if (a.scales_out) a.scales_out[layer] = nu;
         }

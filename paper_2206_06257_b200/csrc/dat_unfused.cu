@@ -50,12 +50,12 @@ __device__ __forceinline__ void sumsq_finish(int l, int64_t t0, int64_t t1, int 
             // every worker keeps its own norm (Eq. rand_q as written): index i*h + l
             for (int i = 0; i < M; ++i) {
                 o.scales[(int64_t)i * h + l] = s_norm[i];
-                o.qmul[(int64_t)i * h + l] = (s_norm[i] == 0.0f) ? 0.0f : o.S_f / s_norm[i];
+                o.qmul[(int64_t)i * h + l] = dat_level_factor(s_norm[i], o.S_f, isfinite(s_norm[i]));
                 if (o.scales_out) o.scales_out[(int64_t)i * h + l] = s_norm[i];
             }
         } else {
             o.scales[l] = nu;
-            o.qmul[l] = (nu == 0.0f) ? 0.0f : o.S_f / nu;
+            o.qmul[l] = dat_level_factor(nu, o.S_f, !bad);
             if (o.dq) o.dq[l] = (nu == 0.0f) ? 0.0f : nu / o.SM_f;
             if (o.scales_out) o.scales_out[l] = nu;
         }
@@ -212,7 +212,7 @@ __device__ __forceinline__ float quant_mul(const QuantScale &q, int64_t k)
 {
     if (!q.scales_in) return __ldg(q.qmul + k);
     const float nu = (q.pad && k == 0) ? 1.0f : __ldg(q.scales_in + k);
-    return (nu == 0.0f) ? 0.0f : q.S_f / nu;
+    return dat_level_factor(nu, q.S_f, isfinite(nu));
 }
 // The receiver's factor nu/S (one vector, one norm per layer).
 __device__ __forceinline__ float quant_back(const QuantScale &q, int64_t k)
@@ -284,7 +284,8 @@ __device__ __forceinline__ void quantize_slow8(const GradPtrs &gp, const PhiloxK
 }
 
 // Packed levels and signs of one group from its eight elements (lowest first) and random words, by the scaled form:
-// saturation is the clamp to S, min(y, S + 1) 2^-b.
+// min(y, S + 1) 2^-b is the clamp to S.  (A minimum and no saturation, which would make a NaN 0, that is level -1, and
+// take it from the word's other levels: the caller's norms say nothing about single elements.)
 // BACK: v becomes the receiver's value, sign * level * f.
 template <int BITS, bool RNG16, bool BACK>
 __device__ __forceinline__ void quantize8(float v[8], float ts, float f, const uint32_t w[8], uint8_t *s_level, uint8_t *s_sign)
@@ -300,7 +301,7 @@ __device__ __forceinline__ void quantize8(float v[8], float ts, float f, const u
 #pragma unroll
         for (int j = PER - 1; j >= 0; --j) {
             const float x = v[a * PER + j] + 0.0f;           // -0 becomes +0: its sign bit is 0
-            const float ys = __saturatef(__fmaf_rn(fabsf(x), ts, dat_u1_scaled<RNG16>(w, a * PER + j, UBITS)));
+            const float ys = fminf(__fmaf_rn(fabsf(x), ts, dat_u1_scaled<RNG16>(w, a * PER + j, UBITS)), 1.0f);
             const float q = __fmaf_rz(ys, TWO_B, 8388607.0f);
             word[a] += __float_as_uint(q) * (1u << (BITS * j));
             if (BACK)                             // (a level of 0 gives +0, whatever the sign)
@@ -316,13 +317,6 @@ __device__ __forceinline__ void quantize8(float v[8], float ts, float f, const u
     else if (BITS == 2) *reinterpret_cast<uint16_t *>(s_level) = (uint16_t)word[0];
     else *s_level = (uint8_t)word[0];
     *s_sign = (uint8_t)neg;
-}
-
-template <int BITS>
-__device__ __forceinline__ bool quant_scaled(float t)        // the scaled form's range: t 2^-b a normal number
-{
-    constexpr float TWO_B = (float)(1u << BITS);
-    return (t == 0.0f) || (t >= 1.17549435e-38f * TWO_B && t <= 3.402823466e38f);
 }
 
 // A warp's part that is not the plain case of the kernel below: several layers, the vector's end, a 16-byte aligned
@@ -353,7 +347,7 @@ __device__ __noinline__ void quantize_mixed(const QuantArgs<N> &all, int range, 
             l_hi = __ldg(a.off + l + 1);
             t = quant_mul(a.qs, q0 + l);
         }
-        if (page && quant_scaled<BITS>(t) && e0 + 8 <= l_hi) {
+        if (page && dat_scaled_factor(t, (float)(1u << BITS)) && e0 + 8 <= l_hi) {
             float x[8];
             uint32_t w[8];
             dat_ld8<EV_FIRST>(g + e0, wide, x);
@@ -401,7 +395,7 @@ k_quantize(const __grid_constant__ QuantArgs<N> all)
     }
     const int l0 = __ldg(a.flat_layer + e_piece / DAT_FLAT);
     const float t = quant_mul(a.qs, (a.per_worker ? (int64_t)worker * a.h : 0) + l0);
-    if (whole && __ldg(a.off + l0 + 1) >= e_piece + 256 * a.groups && quant_scaled<BITS>(t) &&
+    if (whole && __ldg(a.off + l0 + 1) >= e_piece + 256 * a.groups && dat_scaled_factor(t, (float)(1u << BITS)) &&
         dat_one_counter_page<RNG16>((uint64_t)(e_piece + a.elem_base), 256 * a.groups)) {
         const float ts = t * (1.0f / (float)(1u << BITS)), f = BACK ? quant_back(a.qs, l0) : 0.0f;
         const PhiloxWorker pw = dat_philox_worker((uint32_t)((uint64_t)(e_piece + a.elem_base) >> (RNG16 ? 35 : 34)), a.stream_base + (uint32_t)worker, all.keys);
