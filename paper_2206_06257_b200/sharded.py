@@ -130,12 +130,14 @@ class ShardedStep:
             sg0 = sg.data_ptr() if isinstance(sg, torch.Tensor) else int(sg)
             lv_ptrs += [lv0 + j * lb for j in range(self.M_loc)]         # global worker order: rank-major
             sg_ptrs += [sg0 + j * sb for j in range(self.M_loc)]
-        if own.pad == 0:             # the range is the owner's from its first element: in place
-            self.ops.aggregate_update_gather(own, lv_ptrs, sg_ptrs, own.scales(nu), theta[own.a:own.b], mom_own, hp)
-            return
-        theta_own = theta[own.a8:own.b].clone()
+        theta_own = theta[own.a8:own.b]
+        # in place where the range is the owner's from its first element and theta lies as the calls want it
+        in_place = own.pad == 0 and theta_own.is_contiguous() and theta_own.data_ptr() % 16 == 0
+        if not in_place:
+            theta_own = theta_own.clone(memory_format=torch.contiguous_format)
         self.ops.aggregate_update_gather(own, lv_ptrs, sg_ptrs, own.scales(nu), theta_own, mom_own, hp)
-        theta[own.a:own.b].copy_(theta_own[own.pad:])
+        if not in_place:
+            theta[own.a:own.b].copy_(theta_own[own.pad:])
 
     def _pull_layout(self):
         """Byte offsets, in every rank's outgoing buffer, of the level and sign planes meant for owner q."""
