@@ -92,11 +92,12 @@ class ShardedStep:
         norms = self.ops.worker_norms(grads_local)
         return norms[0] if self.M_loc == 1 else norms.max(dim=0).values.contiguous()
 
-    def quantize(self, nu, grads_local, seed, step):
-        """Step 7, second half: this rank's workers, range by range.  Returns [(levels, signs)] per owner."""
-        if hasattr(self.ops, "quantize_ranges"):      # all ranges in one launch
-            return self.ops.quantize_ranges(self.ranges, grads_local, nu, seed, step)
-        return [self.ops.quantize_range(q, self.ranges[q], grads_local, self.ranges[q].scales(nu), seed, step)
+    def quantize(self, nu, grads_local, seed, step, out=None):
+        """Step 7, second half: this rank's workers, range by range.  Returns [(levels, signs)] per owner; out: such a
+        list, where the planes go.  Operations without quantize_ranges (all ranges in one launch) get a call per range."""
+        if hasattr(self.ops, "quantize_ranges"):
+            return self.ops.quantize_ranges(self.ranges, grads_local, nu, seed, step, out=out)
+        return [self.ops.quantize_range(q, self.ranges[q], grads_local, self.ranges[q].scales(nu), seed, step, **({} if out is None else {"out": out[q]}))
                 for q in range(self.world)]
 
     def receive_buffers(self, device):
@@ -168,8 +169,8 @@ class ShardedStep:
         nu = self.local_norms(grads_local)
         if multi:
             dist.all_reduce(nu, op=dist.ReduceOp.MAX, group=self.group)
-        base = self._out.data_ptr()
-        self.ops.quantize_ranges(self.ranges, grads_local, nu, seed, step, out=[(base + lo, base + so) for lo, so in layout])
+        ends = [lo for lo, _ in layout[1:]] + [total]
+        self.quantize(nu, grads_local, seed, step, out=[(self._out[lo:so], self._out[so:end]) for (lo, so), end in zip(layout, ends)])
         if multi:
             torch.cuda.current_stream().synchronize()
             dist.barrier(group=self.group)                                # every rank's planes are complete
