@@ -119,15 +119,10 @@ def _stream(stream):
     return int(stream)
 
 
-@functools.lru_cache(maxsize=64)
-def _hp_struct(hp):
-    return dat_hparams_t(*hp)
-
-
 def _hp(hp):
     if isinstance(hp, dat_hparams_t):
         return hp
-    return _hp_struct(tuple([float(v) for v in hp]))
+    return dat_hparams_t(*[float(v) for v in hp])
 
 
 def dat_strerror(code):
