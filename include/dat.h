@@ -395,7 +395,8 @@ int dat_step_lamb_two_sided(dat_plan_t *plan, float *theta, float *mom, float *v
  * bit up to the norms' last place, as one launch per phase: quantizer norms; then levels, signed sum over the
  * workers, g_hat, m' and the layer sums in one pass that keeps codes, sums and g_hat in registers; then the theta
  * update.  What dat_step does for small problems, whatever the size.  For plans with b < 32 and the shared scale
- * (DAT_ERR_UNSUPPORTED otherwise). */
+ * (DAT_ERR_UNSUPPORTED otherwise).  The call can be recorded into a CUDA graph; a replay repeats the recorded seed and
+ * step. */
 int dat_step_passes(dat_plan_t *plan, float *theta, float *mom, const float *const *grads,
                     uint64_t seed, uint64_t step, const dat_hparams_t *hp, int32_t *code_sum_out,
                     float *layer_norms_out, float *scales_out, void *stream);

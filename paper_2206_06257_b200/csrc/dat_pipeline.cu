@@ -1094,7 +1094,7 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
         (g_hat && !dat_aligned16(g_hat)) || (server_scales_out && !dat_aligned16(server_scales_out)))
         return DAT_ERR_ALIGN;
     const bool two = (g_hat != nullptr);
-    {   // the call's epoch and the Philox key are launch parameters: a captured graph would replay them unchanged
+    if (how != P_PHASES) {   // the call's epoch and the Philox key are launch parameters: a captured graph would replay them unchanged
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing((cudaStream_t)stream, &cap) != cudaSuccess) { (void)cudaGetLastError(); return DAT_ERR_CUDA; }
         if (cap != cudaStreamCaptureStatusNone) return DAT_ERR_UNSUPPORTED;
@@ -1232,7 +1232,7 @@ extern "C" int dat_step(dat_plan_t *plan, float *theta, float *mom, const float 
                     layer_norms_out, scales_out, stream);
 }
 
-// dat_step_passes: the same as one launch per phase.
+// dat_step_passes: the same as one launch per phase, which wait for no epoch: the call can be recorded into a graph.
 extern "C" int dat_step_passes(dat_plan_t *plan, float *theta, float *mom, const float *const *grads,
                                uint64_t seed, uint64_t step, const dat_hparams_t *hp,
                                int32_t *code_sum_out, float *layer_norms_out, float *scales_out, void *stream)
