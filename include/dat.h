@@ -286,13 +286,13 @@ int dat_lamb_step(dat_plan_t *plan, float *theta, float *mom, float *var, const 
  * to take the driver's allocation lock (a latency-critical serving loop).  Creating a plan
  * calls cudaMalloc; this entry point needs no plan and calls no cudaMalloc, cudaFree or any
  * other allocating routine.  Its scratch memory (the layer table, two fp64 partial sums per
- * 4096-element tile, one step length per layer; about 0.6 MB) is a fixed array inside the
+ * 4096-element tile, one step length per layer; about 0.7 MB) is a fixed array inside the
  * library image, so every GPU that loads the library holds it until the process exits.
  *
  *   num_layers      h, 1 <= h <= DAT_STATIC_MAX_LAYERS.
  *   layer_offsets   HOST array of h+1 element offsets (as for dat_plan_create); copied during
  *                   the call.  The layers may span at most DAT_STATIC_MAX_TILES tiles of 4096
- *                   elements (each layer occupies ceil((n_l + 7)/4096) or fewer); larger
+ *                   elements (each layer occupies ceil((n_l + 3)/4096) or fewer); larger
  *                   problems are refused with DAT_ERR_TOO_LARGE before anything is launched.
  *   theta, mom      device fp32[d], updated in place.      g_hat  device fp32[d], read-only.
  *   hp              host pointer, read during the call.

@@ -1197,7 +1197,7 @@ extern "C" int dat_lamb_step(dat_plan_t *plan, float *theta, float *mom, float *
 struct StaticScratch {
     int64_t off[DAT_STATIC_MAX_LAYERS + 1];
     int64_t tile_base[DAT_STATIC_MAX_LAYERS + 1];
-    double partials[2 * DAT_STATIC_MAX_TILES];
+    double partials[2 * (DAT_STATIC_MAX_TILES + DAT_STATIC_MAX_LAYERS)];      // (see below)
     float step_a[DAT_STATIC_MAX_LAYERS];
     uint32_t status, count[DAT_STATIC_MAX_LAYERS];
 };
@@ -1221,13 +1221,14 @@ extern "C" int dat_lalr_step_static(int64_t num_layers, const int64_t *layer_off
         return DAT_ERR_ALIGN;
     if (layer_offsets[0] != 0) return DAT_ERR_LAYOUT;
     int64_t tile_base[DAT_STATIC_MAX_LAYERS + 1];              // host stack, 32 KB
-    int64_t nt = 0;
+    int64_t nt = 0, counted = 0;
     for (int64_t l = 0; l < num_layers; ++l) {
         if (layer_offsets[l + 1] <= layer_offsets[l]) return DAT_ERR_LAYOUT;
         tile_base[l] = nt;
-        const int64_t a = layer_offsets[l] & ~(int64_t)7;
-        nt += (layer_offsets[l + 1] - a + DAT_TILE - 1) / DAT_TILE;
-        if (nt > DAT_STATIC_MAX_TILES) return DAT_ERR_TOO_LARGE;
+        // the documented limit counts tiles from multiples of 4 on; the kernels' start on multiples of 8, one more in a layer at most
+        counted += (layer_offsets[l + 1] - (layer_offsets[l] & ~(int64_t)3) + DAT_TILE - 1) / DAT_TILE;
+        nt += (layer_offsets[l + 1] - (layer_offsets[l] & ~(int64_t)7) + DAT_TILE - 1) / DAT_TILE;
+        if (counted > DAT_STATIC_MAX_TILES) return DAT_ERR_TOO_LARGE;
     }
     tile_base[num_layers] = nt;
 

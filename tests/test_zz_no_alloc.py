@@ -85,6 +85,26 @@ def test_static_scratch_accepts_exactly_its_limits():
     assert torch.equal(mo, g) and not th.any()              # m' = g_hat; ||theta|| = 0 with c_l = 0: no move
 
 
+def test_static_scratch_accepts_its_limits_wherever_layers_start():
+    """Layers that start on odd multiples of 4: 8 tiles of 4096 elements each, by the documented count exactly the limit."""
+    from paper_2206_06257_b200 import api
+    sizes = [4] + [8 * 4096] * 4094 + [15 * 4096]
+    assert 1 + 8 * 4094 + 15 == api.DAT_STATIC_MAX_TILES
+    offs = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    n = int(offs[-1])
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    theta, mom, gh = (torch.randn(n, generator=gen, device="cuda") for _ in range(3))
+    th, mo = theta.clone(), mom.clone()
+    api.dat_lalr_step_static(offs, th, mo, gh, HP)
+    with GpuPlan(api, offs, 1, 8) as P:
+        api.dat_lalr_step(P.plan, theta, mom, gh, HP)
+        torch.cuda.synchronize()
+    assert torch.equal(th, theta) and torch.equal(mo, mom)
+    with pytest.raises(api.DatError) as e:
+        api.dat_lalr_step_static(offs + (np.arange(offs.size) == offs.size - 1), th, mo, gh, HP)      # one element, one tile more
+    assert e.value.code == api.DAT_ERR_TOO_LARGE
+
+
 def test_static_scratch_refuses_stream_capture():
     """The call copies its tables from host memory every time, so it must not end up in a CUDA graph."""
     from paper_2206_06257_b200 import api
