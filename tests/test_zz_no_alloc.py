@@ -105,6 +105,14 @@ def test_static_scratch_accepts_its_limits_wherever_layers_start():
     assert e.value.code == api.DAT_ERR_TOO_LARGE
 
 
+@pytest.mark.parametrize("h", [1, 2, 31, 32, 33, 1023, 1025])
+def test_static_scratch_finds_every_layer(h):
+    """The search of a tile's layer by a warp, around its powers of 32; layers of one tile, and of several in between."""
+    from paper_2206_06257_b200 import api
+    rng = np.random.RandomState(h)
+    _run_both(api, *_case(h, np.where(rng.rand(h) < 0.2, rng.randint(4000, 13000, h), rng.randint(1, 20, h))))
+
+
 def test_static_scratch_refuses_stream_capture():
     """The call copies its tables from host memory every time, so it must not end up in a CUDA graph."""
     from paper_2206_06257_b200 import api
