@@ -410,13 +410,13 @@ int dat_plan_test_stall(dat_plan_t *plan, int64_t wait_cycles, int64_t layer, vo
 
 /* dat_step_host -- dat_step for callers whose data lives in HOST memory: copies theta, mom and
  * the M gradient buffers to plan-owned device staging buffers, runs the step, copies theta and
- * mom back, and synchronises `stream` before returning.  Large vectors go group of layers by group of
- * layers on streams the plan owns (ordered after what `stream` holds), so that a group's step and its
- * copies back run under the copies in of the next.
+ * mom back, and synchronises `stream` before returning.  Vectors of eight megabytes and more, all of them in pinned memory,
+ * go group of layers by group of layers on streams the plan owns (ordered after what `stream` holds), so that a group's
+ * step (dat_step_pipelined on its layers) and its copies back run under the copies in of the next.
  *   theta_host, mom_host   host fp32[d], updated in place (pinned memory makes the copies fast).
  *   grads_host             host array of M host pointers, fp32[d] each.
- * The first call allocates the staging buffers ((M+2)*d*4 bytes), streams and events, kept until the plan is
- * destroyed.  Errors: ARG, NOMEM, UNSUPPORTED (plan with an origin; capturing stream), CUDA. */
+ * The first call allocates the staging buffers ((M+2)*d*4 bytes), the first in groups also the groups' lists,
+ * streams and events; all are kept until the plan is destroyed.  Errors: ARG, NOMEM, UNSUPPORTED (plan with an origin; capturing stream), CUDA. */
 int dat_step_host(dat_plan_t *plan, float *theta_host, float *mom_host,
                   const float *const *grads_host, uint64_t seed, uint64_t step,
                   const dat_hparams_t *hp, void *stream);

@@ -102,8 +102,7 @@ int dat_pipe_build(dat_plan_t *plan);                        // dat_pipeline.cu 
 void dat_pipe_destroy(dat_plan_t *plan);
 cudaError_t dat_pipe_reset(dat_plan_t *plan, cudaStream_t s);
 int dat_norm_phase(dat_plan_t *plan, const GradPtrs &gp, float *scales_out, cudaStream_t s);      // dat_unfused.cu
-int dat_pipe_groups(dat_plan_t *plan, int most, size_t *bytes);      // the step group by group (dat_step_host)
-int dat_pipe_groups_upload(dat_plan_t *plan, void *mem);
+int dat_pipe_groups(dat_plan_t *plan, int most);             // the step group by group (dat_step_host)
 int dat_pipe_group_count(const dat_plan_t *plan);
 void dat_pipe_group_range(const dat_plan_t *plan, int k, int64_t *e0, int64_t *e1);
 int dat_pipe_step_group(dat_plan_t *plan, int k, float *theta, float *mom, const float *const *grads, uint64_t seed, uint64_t step,

@@ -70,7 +70,7 @@ struct PipeItem {
 // A contiguous range of layers as a list of its own (dat_step_host: the step range by range, as the data arrives).
 struct PipeGroup {
     int64_t e0, e1;                               // elements
-    int64_t first, n_items;                       // in group_items
+    int64_t first, n_items;                       // in d_group_items
 };
 
 struct PipeSchedule {
@@ -89,9 +89,8 @@ struct PipeSchedule {
     size_t sync_bytes = 0;
     int64_t n_tiles = 0;
     std::vector<int64_t> tile_base;               // h + 1
-    std::vector<PipeGroup> groups;                // built by the first dat_step_host
-    std::vector<PipeItem> group_items;
-    PipeItem *d_group_items = nullptr;            // in the caller's memory (dat_pipe_groups_upload)
+    std::vector<PipeGroup> groups;                // built by the first dat_step_host that goes in groups
+    PipeItem *d_group_items = nullptr;
     uint32_t epoch = 0;                           // calls made so far
     long long wait_cycles = DAT_P_WAIT_CYCLES;
 };
@@ -860,6 +859,7 @@ void dat_pipe_destroy(dat_plan_t *plan)
 {
     if (!plan->pipe) return;
     if (plan->pipe->mem) cudaFree(plan->pipe->mem);
+    if (plan->pipe->d_group_items) cudaFree(plan->pipe->d_group_items);
     delete plan->pipe;
     plan->pipe = nullptr;
 }
@@ -984,38 +984,34 @@ int dat_pipe_build(dat_plan_t *plan)
     return DAT_OK;
 }
 
-// The plan's layers cut into at most `most` contiguous groups of about equal size; *bytes: the device memory their
-// lists take, which dat_pipe_groups_upload fills (synchronous).
-int dat_pipe_groups(dat_plan_t *plan, int most, size_t *bytes)
+// The plan's layers cut into at most `most` contiguous groups of about equal size, each with a list of items of its own
+// (built and uploaded by the first call; synchronous).
+int dat_pipe_groups(dat_plan_t *plan, int most)
 {
     PipeSchedule *g = plan->pipe;
     if (!g || !g->mem) return DAT_ERR_ARG;
+    if (g->d_group_items) return DAT_OK;
+    std::vector<PipeItem> all;
     try {
-        if (g->groups.empty())
-            for (int64_t l0 = 0, l1; l0 < plan->h; l0 = l1) {
-                const int64_t left = most - (int64_t)g->groups.size();
-                const int64_t want = plan->offsets[l0] + (plan->d - plan->offsets[l0] + left - 1) / left;
-                for (l1 = l0 + 1; left > 1 && l1 < plan->h && plan->offsets[l1] < want; ++l1) {}
-                if (left <= 1) l1 = plan->h;
-                const std::vector<PipeItem> list = p_items(plan, g->tile_base, (int)l0, (int)l1, false);
-                g->groups.push_back(PipeGroup{plan->offsets[l0], plan->offsets[l1], (int64_t)g->group_items.size(), (int64_t)list.size()});
-                g->group_items.insert(g->group_items.end(), list.begin(), list.end());
-            }
-    } catch (...) {
         g->groups.clear();
-        g->group_items.clear();
+        for (int64_t l0 = 0, l1; l0 < plan->h; l0 = l1) {
+            const int64_t left = most - (int64_t)g->groups.size();
+            const int64_t want = plan->offsets[l0] + (plan->d - plan->offsets[l0] + left - 1) / left;
+            for (l1 = l0 + 1; left > 1 && l1 < plan->h && plan->offsets[l1] < want; ++l1) {}
+            if (left <= 1) l1 = plan->h;
+            const std::vector<PipeItem> list = p_items(plan, g->tile_base, (int)l0, (int)l1, false);
+            g->groups.push_back(PipeGroup{plan->offsets[l0], plan->offsets[l1], (int64_t)all.size(), (int64_t)list.size()});
+            all.insert(all.end(), list.begin(), list.end());
+        }
+    } catch (...) {
         return DAT_ERR_NOMEM;
     }
-    *bytes = g->group_items.size() * sizeof(PipeItem);
-    return DAT_OK;
-}
-
-int dat_pipe_groups_upload(dat_plan_t *plan, void *mem)
-{
-    PipeSchedule *g = plan->pipe;
-    DAT_CUDA(plan, cudaMemcpy(mem, g->group_items.data(), g->group_items.size() * sizeof(PipeItem), cudaMemcpyHostToDevice));
-    g->d_group_items = (PipeItem *)mem;
-    g->group_items = std::vector<PipeItem>();
+    PipeItem *mem = nullptr;
+    cudaError_t e = cudaMalloc((void **)&mem, all.size() * sizeof(PipeItem));
+    if (e != cudaSuccess) { plan->last_cuda = (int)e; (void)cudaGetLastError(); return DAT_ERR_NOMEM; }
+    e = cudaMemcpy(mem, all.data(), all.size() * sizeof(PipeItem), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) { cudaFree(mem); return dat_cuda_fail(plan, e); }
+    g->d_group_items = mem;
     return DAT_OK;
 }
 

@@ -5,7 +5,7 @@
 #include "dat_internal.cuh"
 
 #define HOST_GROUPS 8                            // groups of layers of dat_step_host, at most
-#define HOST_GROUP_BYTES (1ll << 20)             // of a vector, at least
+#define HOST_GROUP_BYTES (4ll << 20)             // of a vector, at least
 
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -310,24 +310,44 @@ extern "C" const char *dat_strerror(int code)
     }
 }
 
-// The staging buffers, streams and events of dat_step_host (first call of a plan).
-static int host_prepare(dat_plan_t *plan, size_t stride)
+// The staging buffers of dat_step_host (first call of a plan).
+static int host_stage(dat_plan_t *plan, size_t stride)
 {
-    cudaError_t e = cudaSuccess;
-    if (!plan->stage) {
-        // Groups of at least a megabyte per vector: below that a copy's fixed cost shows.  What does not overlap is the
-        // last group's step and copies back; 8, 16, 32 groups: 7.37, 7.42, 7.65 ms for ResNet-18, M = 6 (one: 8.2 ms).
-        int64_t most = plan->d * 4 / HOST_GROUP_BYTES;
-        most = most < 1 ? 1 : most > HOST_GROUPS ? HOST_GROUPS : most;
-        size_t lists = 0;
-        int rc = dat_pipe_groups(plan, (int)most, &lists);
-        if (rc != DAT_OK) return rc;
-        const size_t vectors = (size_t)(plan->M + 2) * stride * 4;
-        e = cudaMalloc((void **)&plan->stage, vectors + lists);
-        if (e != cudaSuccess) { plan->stage = nullptr; plan->last_cuda = (int)e; (void)cudaGetLastError(); return DAT_ERR_NOMEM; }
-        rc = dat_pipe_groups_upload(plan, (char *)plan->stage + vectors);
-        if (rc != DAT_OK) { cudaFree(plan->stage); plan->stage = nullptr; return rc; }
+    if (plan->stage) return DAT_OK;
+    const cudaError_t e = cudaMalloc((void **)&plan->stage, (size_t)(plan->M + 2) * stride * 4);
+    if (e == cudaSuccess) return DAT_OK;
+    plan->stage = nullptr;
+    plan->last_cuda = (int)e;
+    (void)cudaGetLastError();
+    return DAT_ERR_NOMEM;
+}
+
+// Groups of layers that the call is cut into: of at least four megabytes per vector, below which the copies' fixed costs
+// show, and at most eight; what does not overlap is the last group's step and copies back (ms, one group / 1 MB / 4 MB /
+// 8 MB and more, pinned memory):
+//   3 million elements, M = 2: 1.39 / 1.35 / 1.28 / 1.36, M = 8: 2.76 / 2.85 / 2.62 / 2.72, M = 32: 8.21 / 8.98 / 8.17 / 8.12
+//   1 million, M = 8: 0.99 / 1.05 / one    ResNet-18, M = 6: 8.21 / 7.37 / 7.37 / 7.30 (16, 32 groups: 7.42, 7.65)
+// One group where some buffer is pageable: those copies block the host one by one, so nothing overlaps, and they are
+// slower in pieces (ResNet-18, M = 3: 25.3 ms in groups, 24.2 in one; 3 million elements, M = 2: 5.5, 4.7).
+static int host_groups(const dat_plan_t *plan, const float *theta, const float *mom, const float *const *grads)
+{
+    const int64_t most = plan->d * 4 / HOST_GROUP_BYTES;
+    if (most < 2) return 1;
+    for (int i = -2; i < plan->M; ++i) {
+        cudaPointerAttributes at;
+        const bool known = cudaPointerGetAttributes(&at, i == -2 ? theta : i == -1 ? mom : grads[i]) == cudaSuccess;
+        if (!known) (void)cudaGetLastError();
+        if (!known || at.type == cudaMemoryTypeUnregistered) return 1;
     }
+    return most > HOST_GROUPS ? HOST_GROUPS : (int)most;
+}
+
+// The groups' lists, the streams and events (first call in groups).
+static int host_prepare(dat_plan_t *plan, int groups)
+{
+    const int rc = dat_pipe_groups(plan, groups);
+    if (rc != DAT_OK) return rc;
+    cudaError_t e = cudaSuccess;
     if (!plan->copy_in) e = cudaStreamCreateWithFlags(&plan->copy_in, cudaStreamNonBlocking);
     if (e == cudaSuccess && !plan->copy_out) e = cudaStreamCreateWithFlags(&plan->copy_out, cudaStreamNonBlocking);
     while (e == cudaSuccess && plan->events.size() < 2 + 2 * (size_t)dat_pipe_group_count(plan)) {
@@ -336,6 +356,27 @@ static int host_prepare(dat_plan_t *plan, size_t stride)
         if (e == cudaSuccess) plan->events.push_back(ev);
     }
     return e == cudaSuccess ? DAT_OK : dat_cuda_fail(plan, e);
+}
+
+// All of it on the caller's stream: copies in, the step, copies back.
+static int host_in_one(dat_plan_t *plan, float *theta_host, float *mom_host, const float *const *grads_host, size_t stride, uint64_t seed, uint64_t step,
+                       const dat_hparams_t *hp, cudaStream_t s)
+{
+    const size_t bytes = (size_t)plan->d * 4;
+    float *d_theta = plan->stage, *d_mom = plan->stage + stride;
+    const float *d_grads[DAT_MAX_WORKERS];
+    DAT_CUDA(plan, cudaMemcpyAsync(d_theta, theta_host, bytes, cudaMemcpyHostToDevice, s));
+    DAT_CUDA(plan, cudaMemcpyAsync(d_mom, mom_host, bytes, cudaMemcpyHostToDevice, s));
+    for (int i = 0; i < plan->M; ++i) {
+        float *g = plan->stage + (size_t)(i + 2) * stride;
+        DAT_CUDA(plan, cudaMemcpyAsync(g, grads_host[i], bytes, cudaMemcpyHostToDevice, s));
+        d_grads[i] = g;
+    }
+    const int rc = dat_step(plan, d_theta, d_mom, d_grads, seed, step, hp, nullptr, nullptr, nullptr, s);
+    if (rc != DAT_OK) return rc;
+    DAT_CUDA(plan, cudaMemcpyAsync(theta_host, d_theta, bytes, cudaMemcpyDeviceToHost, s));
+    DAT_CUDA(plan, cudaMemcpyAsync(mom_host, d_mom, bytes, cudaMemcpyDeviceToHost, s));
+    return DAT_OK;
 }
 
 // The copies are what this call costs (PCIe); they run group of layers by group of layers on streams of their own, so
@@ -389,12 +430,20 @@ extern "C" int dat_step_host(dat_plan_t *plan, float *theta_host, float *mom_hos
     if (cap != cudaStreamCaptureStatusNone) return DAT_ERR_UNSUPPORTED;
     // every staged vector starts on a 256-byte boundary
     const size_t stride = align_up((size_t)plan->d * 4, 256) / 4;
-    rc = host_prepare(plan, stride);
+    rc = host_stage(plan, stride);
     if (rc != DAT_OK) return rc;
-    rc = host_enqueue(plan, theta_host, mom_host, grads_host, stride, seed, step, hp, s);
+    const int groups = host_groups(plan, theta_host, mom_host, grads_host);
+    if (groups > 1) {
+        rc = host_prepare(plan, groups);
+        if (rc != DAT_OK) return rc;
+        rc = host_enqueue(plan, theta_host, mom_host, grads_host, stride, seed, step, hp, s);
+    } else {
+        rc = host_in_one(plan, theta_host, mom_host, grads_host, stride, seed, step, hp, s);
+    }
     if (rc != DAT_OK) {                             // nothing is left in flight on the caller's buffers
-        (void)cudaStreamSynchronize(plan->copy_in);
-        (void)cudaStreamSynchronize(plan->copy_out);
+        if (groups > 1) (void)cudaStreamSynchronize(plan->copy_in);
+        if (groups > 1) (void)cudaStreamSynchronize(plan->copy_out);
+        (void)cudaStreamSynchronize(s);
         return rc;
     }
     DAT_CUDA(plan, cudaStreamSynchronize(s));
