@@ -405,8 +405,13 @@ int dat_step_passes(dat_plan_t *plan, float *theta, float *mom, const float *con
  * `wait_cycles` SM clock cycles (0 restores the default) and, if `layer` >= 0, marks that layer's norm
  * as never completing for the next call (its tile counter is pre-set on the host side of the stream so
  * that the count cannot be reached): work items that need the layer give up after the limit and the
- * call ends with DAT_STATUS_TIMEOUT.  Nothing else uses this.  Errors: ARG, CUDA. */
+ * call ends with DAT_STATUS_TIMEOUT.  Only the one launch waits, so the plan's steps take that form until a call with
+ * (0, -1) gives it back to the rule by size.  Nothing else uses this.  Errors: ARG, CUDA. */
 int dat_plan_test_stall(dat_plan_t *plan, int64_t wait_cycles, int64_t layer, void *stream);
+
+/* dat_plan_test_form -- TEST HOOK: the form of the plan's dat_step, dat_step_lamb and two-sided steps whatever their size:
+ * 1 the one launch, 2 a launch per phase, 0 by the rule again.  Nothing else uses this.  Errors: ARG. */
+int dat_plan_test_form(dat_plan_t *plan, int form);
 
 /* dat_step_host -- dat_step for callers whose data lives in HOST memory: copies theta, mom and
  * the M gradient buffers to plan-owned device staging buffers, runs the step, copies theta and

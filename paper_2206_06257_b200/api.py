@@ -32,7 +32,7 @@ DAT_STATUS_NONFINITE, DAT_STATUS_TIMEOUT, DAT_STATUS_BOUNDS = 1, 2, 4
 
 # every symbol include/dat.h declares
 EXPORTS = ["dat_plan_create", "dat_plan_set_origin", "dat_plan_destroy", "dat_plan_sizes", "dat_worker_norms", "dat_quantize", "dat_quantize_ranges", "dat_aggregate", "dat_aggregate_gather", "dat_requantize",
-           "dat_average", "dat_lalr_step", "dat_lamb_step", "dat_lalr_step_static", "dat_step", "dat_step_lamb", "dat_step_two_sided", "dat_step_lamb_two_sided", "dat_step_passes", "dat_step_pipelined", "dat_plan_test_stall", "dat_step_host", "dat_get_status",
+           "dat_average", "dat_lalr_step", "dat_lamb_step", "dat_lalr_step_static", "dat_step", "dat_step_lamb", "dat_step_two_sided", "dat_step_lamb_two_sided", "dat_step_passes", "dat_step_pipelined", "dat_plan_test_stall", "dat_plan_test_form", "dat_step_host", "dat_get_status",
            "dat_plan_launch_count", "dat_strerror", "dat_last_cuda_error"]
 
 
@@ -63,6 +63,7 @@ _lib.dat_lamb_step.argtypes = [_p, _p, _p, _p, _p, C.POINTER(dat_lamb_hparams_t)
 _lib.dat_lalr_step_static.argtypes = [_i64, _p, _p, _p, _p, C.POINTER(dat_hparams_t), _p, _p]
 _lib.dat_step.argtypes = [_p, _p, _p, _p, _u64, _u64, C.POINTER(dat_hparams_t), _p, _p, _p, _p]
 _lib.dat_plan_test_stall.argtypes = [_p, _i64, _i64, _p]
+_lib.dat_plan_test_form.argtypes = [_p, _int]
 _lib.dat_step_lamb.argtypes = [_p, _p, _p, _p, _p, _u64, _u64, C.POINTER(dat_lamb_hparams_t), _i64, _p, _p, _p, _p]
 _lib.dat_step_two_sided.argtypes = [_p, _p, _p, _p, _u64, _u64, C.POINTER(dat_hparams_t), _p, _p, _p, _p, _p, _p]
 _lib.dat_step_lamb_two_sided.argtypes = [_p, _p, _p, _p, _p, _u64, _u64, C.POINTER(dat_lamb_hparams_t), _i64, _p, _p, _p, _p, _p, _p]
@@ -246,6 +247,11 @@ def dat_step_lamb_two_sided(plan, theta, mom, var, grads, seed, step, hp, t, g_h
 def dat_plan_test_stall(plan, wait_cycles, layer=-1, stream=None):
     """Test hook: wait limit in SM cycles (0: default) and a layer whose norm never completes next call."""
     _ok(_lib.dat_plan_test_stall(plan, int(wait_cycles), int(layer), _stream(stream)), "dat_plan_test_stall")
+
+
+def dat_plan_test_form(plan, form):
+    """Test hook: 1 one launch, 2 a launch per phase, 0 by the rule."""
+    _ok(_lib.dat_plan_test_form(plan, int(form)), "dat_plan_test_form")
 
 
 def dat_step_passes(plan, theta, mom, grads, seed, step, hp, code_sum_out=None, layer_norms_out=None,

@@ -55,6 +55,7 @@
 #endif
 #define DAT_P_WAIT_CYCLES (4000000000ll)          // about two seconds
 
+enum { P_BY_RULE = 0, P_ONE_LAUNCH = 1, P_PHASES = 2 };     // which form a step takes (see p_phases)
 enum { P_MODE_SHARED = 0, P_MODE_PER_WORKER = 1, P_MODE_IDENTITY = 2 };
 enum { P_OPT_MOMENTUM = 0, P_OPT_LAMB = 1 };     // the descent direction u of Eq. 3: heavy-ball momentum, or Algorithm A2
 
@@ -92,6 +93,7 @@ struct PipeSchedule {
     std::vector<PipeGroup> groups;                // built by the first dat_step_host that goes in groups
     PipeItem *d_group_items = nullptr;
     uint32_t epoch = 0;                           // calls made so far
+    int form = P_BY_RULE;                         // of the calls that leave it to the rule (test hooks)
     long long wait_cycles = DAT_P_WAIT_CYCLES;
 };
 
@@ -1044,7 +1046,6 @@ cudaError_t dat_pipe_reset(dat_plan_t *plan, cudaStream_t s)
 // times): 60 million, 413 / 365; LAMB 607 / 531; two-sided 538 / 511.
 #define P_PHASES_WAVE 4                           // tiles per SM: one wave of a phase's CTAs
 #define P_PHASES_MOST 9
-enum { P_BY_RULE = 0, P_ONE_LAUNCH = 1, P_PHASES = 2 };
 static bool p_phases(const dat_plan_t *plan, bool two)
 {
     const int64_t n = plan->pipe->n_tiles, sm = plan->sm_count;
@@ -1156,7 +1157,8 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
     a.n_tiles = g->n_tiles;
     cudaStream_t s = (cudaStream_t)stream;
     const bool rng16 = (plan->rng_bits == 16);
-    const bool phases = !group && how != P_ONE_LAUNCH && (how == P_PHASES || (g->wait_cycles == DAT_P_WAIT_CYCLES && p_phases(plan, two)));
+    const int form = group ? P_ONE_LAUNCH : how == P_BY_RULE ? g->form : how;
+    const bool phases = form == P_PHASES || (form == P_BY_RULE && p_phases(plan, two));
     const bool halves = phases && p_halves(plan);
     const unsigned grid = phases ? (unsigned)g->n_tiles * (halves ? 2u : 1u) : a.n_items;
     if (phases && !identity) {
@@ -1280,6 +1282,16 @@ extern "C" int dat_step_lamb_two_sided(dat_plan_t *plan, float *theta, float *mo
                     layer_norms_out, scales_out, stream, g_hat, server_scales_out);
 }
 
+// Test hook (see dat.h): the form of the plan's steps, whatever the rule says.
+extern "C" int dat_plan_test_form(dat_plan_t *plan, int form)
+{
+    int rc = dat_check_plan(plan);
+    if (rc != DAT_OK) return rc;
+    if (!plan->pipe || (form != P_BY_RULE && form != P_ONE_LAUNCH && form != P_PHASES)) return DAT_ERR_ARG;
+    plan->pipe->form = form;
+    return DAT_OK;
+}
+
 // Test hook (see dat.h): a short wait limit, and a layer whose norm never completes in the next call.
 extern "C" int dat_plan_test_stall(dat_plan_t *plan, int64_t wait_cycles, int64_t layer, void *stream)
 {
@@ -1288,6 +1300,7 @@ extern "C" int dat_plan_test_stall(dat_plan_t *plan, int64_t wait_cycles, int64_
     PipeSchedule *g = plan->pipe;
     if (!g || !g->mem || wait_cycles < 0 || layer >= plan->h) return DAT_ERR_ARG;
     g->wait_cycles = wait_cycles ? (long long)wait_cycles : DAT_P_WAIT_CYCLES;
+    g->form = (wait_cycles || layer >= 0) ? P_ONE_LAUNCH : P_BY_RULE;        // only the one launch waits
     if (layer >= 0) {
         // a count that the layer's tiles cannot bring to T - 1: nobody becomes the layer's last tile
         static const uint32_t far = 0x40000000u;
