@@ -189,6 +189,11 @@ __device__ __forceinline__ bool p_poll(const PArgs &a, const uint32_t *word)
 // a violation sets DAT_STATUS_BOUNDS and the item is skipped, nothing faults.
 #ifdef DAT_SELFCHECK
 #define P_CHECK(a, cond) ((cond) ? true : (atomicOr((a).status, DAT_STATUS_BOUNDS), false))
+__device__ __forceinline__ bool p_part_valid(const PArgs &a, const PipePart &p)
+{
+    return p.layer >= 0 && p.layer < a.h && p.tile >= 0 && p.tile < p.T && p.tb >= 0 && (int64_t)p.tb + p.tile < a.n_tiles &&
+           p.lo >= 0 && p.lo < p.hi && p.hi <= a.d && (p.lo & ~(int64_t)7) + (int64_t)p.tile * DAT_P_TILE < p.hi;
+}
 #else
 #define P_CHECK(a, cond) true
 #endif
@@ -726,14 +731,10 @@ k_step_pipelined(const __grid_constant__ PArgs a)
     PipePart pm = pq;                               // the part that leaves m' and the tile's two sums of Eq. 3
 #ifdef DAT_SELFCHECK
     {
-        bool ok = pn.layer < a.h && pq.layer < a.h && pu.layer < a.h;
         const PipePart pr = TWO ? s_item.r : pq;
-        ok = ok && pr.layer < a.h;
         const PipePart *pp[4] = {&pn, &pq, &pu, &pr};
-        for (int k = 0; k < 4 && ok; ++k)
-            if (pp[k]->layer >= 0)
-                ok = pp[k]->tile >= 0 && pp[k]->tile < pp[k]->T && (int64_t)pp[k]->tb + pp[k]->tile < a.n_tiles &&
-                     pp[k]->lo >= 0 && pp[k]->lo < pp[k]->hi && pp[k]->hi <= a.d;
+        bool ok = true;
+        for (int k = 0; k < 4; ++k) ok = ok && (pp[k]->layer < 0 || p_part_valid(a, *pp[k]));
         if (!P_CHECK(a, ok)) return;
     }
 #endif
@@ -788,6 +789,7 @@ k_step_pipelined(const __grid_constant__ PArgs a)
 __device__ __forceinline__ PipePart p_part_of(const PArgs &a, uint32_t tile)
 {
     PipePart pt;
+    if (!P_CHECK(a, tile < a.n_tiles)) tile = 0;
     const uint4 *src = reinterpret_cast<const uint4 *>(a.parts + tile);
     reinterpret_cast<uint4 *>(&pt)[0] = __ldg(src);
     reinterpret_cast<uint4 *>(&pt)[1] = __ldg(src + 1);
@@ -819,6 +821,7 @@ k_phase_quant(const __grid_constant__ PArgs a)
     const PipePart pt = p_part_of(a, cta / PIECES), pp = p_piece_of<G>(pt, cta % PIECES);
     cudaTriggerProgrammaticLaunchCompletion();
     cudaGridDependencySynchronize();
+    if (!P_CHECK(a, p_part_valid(a, pt))) return;
     p_part_quant<RNG16, MODE, OPT, TWO, G>(a, pt, cta % PIECES, s_red, s_fac);
     __syncthreads();
     if (threadIdx.x == 0) s_last = TWO ? p_server_publish(a, pp, s_red) : p_quant_publish(a, pp, s_red);
@@ -838,6 +841,7 @@ k_phase_requant(const __grid_constant__ PArgs a)
     const PipePart pt = p_part_of(a, blockIdx.x / PIECES), pp = p_piece_of<G>(pt, blockIdx.x % PIECES);
     cudaTriggerProgrammaticLaunchCompletion();
     cudaGridDependencySynchronize();
+    if (!P_CHECK(a, p_part_valid(a, pt))) return;
     p_part_requant<RNG16, OPT, G>(a, pt, blockIdx.x % PIECES, s_red);
     __syncthreads();
     if (threadIdx.x == 0) s_last = p_quant_publish(a, pp, s_red);
@@ -853,6 +857,7 @@ k_phase_update(const __grid_constant__ PArgs a)
     const uint32_t cta = BACK ? gridDim.x - 1u - blockIdx.x : blockIdx.x;
     const PipePart pt = p_part_of(a, cta / PIECES);
     cudaGridDependencySynchronize();
+    if (!P_CHECK(a, p_part_valid(a, pt))) return;
     p_part_update<OPT, G>(a, pt, cta % PIECES);
 }
 

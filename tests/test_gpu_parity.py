@@ -564,7 +564,8 @@ def test_bounded_wait_runs_out_and_plan_recovers(api, oracle):
 
 def test_self_checking_build_runs_the_ragged_cases():
     """The build with -DDAT_SELFCHECK (DAT_DEBUG=1: every tile an item names is checked before use, a
-    violation sets DAT_STATUS_BOUNDS instead of faulting) passes the ragged parity cases with a clean status."""
+    violation sets DAT_STATUS_BOUNDS instead of faulting) passes the ragged parity cases, the steps' in both of their
+    forms, with a clean status."""
     import os
     import subprocess
     import sys
@@ -572,7 +573,8 @@ def test_self_checking_build_runs_the_ragged_cases():
     env = dict(os.environ, DAT_DEBUG="1")
     subprocess.check_call([sys.executable, "-m", "paper_2206_06257_b200.build"], cwd=root, env=env)   # no-op when up to date
     r = subprocess.run([sys.executable, "-m", "pytest", "-q", "-x", "-m", "gpu", os.path.join(root, "tests", "test_gpu_parity.py"),
-                        "-k", "test_fused_parity_ragged and rng16"], env=env,
+                        os.path.join(root, "tests", "test_gpu_both_forms.py"),
+                        "-k", "(test_fused_parity_ragged or test_ragged or test_two_sided) and rng16 or test_lamb"], env=env,
                        cwd=root, capture_output=True, text=True, timeout=600)
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-2000:]
 
