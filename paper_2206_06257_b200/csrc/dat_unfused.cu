@@ -9,11 +9,10 @@
 // S1: quantizer norms.  One fp64 partial sum of squares per (tile, worker); the CTA that finishes a layer's last
 // tile adds the layer's partials in a fixed order: nu_{i,l}, nu_l = max_i, S/nu.  Squares of fp32 values are exact
 // in fp64, so the result does not depend on the tiling beyond the last bits of an fp64 sum.
-// HBM-bound (129 us for the 818 MB of ResNet-50, M = 8: 6.3 TB/s); finishing in the same launch instead of a second
-// one takes 8.7 us off (a launch of one CTA per layer, nearly all of it latency).
+// HBM-bound: 122 us for the 818 MB of ResNet-50, M = 8 (139 as two launches and a copy).
 // ------------------------------------------------------------------------------------------
 #define SUMSQ_KEEP_BYTES (64ll << 20)             // of the last tiles' gradients, that stay in L2
-#define SUMSQ_WORKERS 8                           // workers of a tile that one CTA sums, at most (a warp's partials: <= 32)
+#define SUMSQ_JOBS 8                              // sums (of a tile and a worker) of a CTA, at most (a warp's partials: <= 32)
 
 struct NormOut {
     float S_f;
@@ -125,35 +124,63 @@ __device__ __forceinline__ void sumsq_rows(const GradPtrs &gp, const TileRange &
     }
 }
 
-template <int NW>
+// A CTA sums `per_cta` workers of a tile, or of `tiles_per_cta` consecutive ones (TILES).  What it does once, at its end -- barrier, fence, count,
+// a chain of three round trips -- takes longer than a tile's loads, so with few workers a CTA per tile keeps too few bytes
+// in flight (us for the norms, a tile per CTA / up to eight sums per CTA / the two launches that these were before: 25.6
+// million elements, M = 1: 32.8 / 27.0 / 30.7; 100 million, M = 2: 157 / 133 / 146, M = 3: 216 / 203 / 205; 200 million, M = 1:
+// 197 / 157 / 141).  Sixteen sums: 163 in the last, 126 instead of 122 for ResNet-50, M = 8.
+template <int NW, bool TILES>
 __global__ void __launch_bounds__(DAT_THREADS, NW == 1 ? 6 : 4)
-k_sumsq(const __grid_constant__ GradPtrs gp, const TileSource tiles, int M, int per_cta, int64_t keep_from, double *partials, const __grid_constant__ NormOut out)
+k_sumsq(const __grid_constant__ GradPtrs gp, const TileSource tiles, int M, int per_cta, int tiles_per_cta, int64_t n_tiles, int64_t keep_from,
+        double *partials, const __grid_constant__ NormOut out)
 {
     constexpr int W = DAT_THREADS / 32;
-    __shared__ double s_sum[SUMSQ_WORKERS][W];
-    __shared__ bool s_last;
+    __shared__ double s_sum[SUMSQ_JOBS][W];
+    __shared__ uint32_t s_last;                   // bit k: the layer of the CTA's tile k is complete
     cudaTriggerProgrammaticLaunchCompletion();    // a step's next phase may set itself up; it waits for this one's end
-    const int64_t tile = blockIdx.x;
-    const int w0 = blockIdx.y * per_cta, w1 = min(w0 + per_cta, M);
+    const int64_t t0 = TILES ? (int64_t)blockIdx.x * tiles_per_cta : (int64_t)blockIdx.x;
+    const int nt = TILES ? (int)min((int64_t)tiles_per_cta, n_tiles - t0) : 1;
+    const int w0 = blockIdx.y * per_cta, w1 = min(w0 + per_cta, M), nw = w1 - w0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const TileRange r = dat_tile_range(tiles, tile);
-    const bool keep = tile >= keep_from;          // read again first thing by the call that follows (which walks back)
-    if (r.begin >= r.lo && r.begin + DAT_TILE <= r.hi) sumsq_rows<NW, true>(gp, r, w0, w1, keep, s_sum);
-    else sumsq_rows<NW, false>(gp, r, w0, w1, keep, s_sum);
+    TileRange r;                                  // of the last tile, behind the loop
+#pragma unroll 1
+    for (int k = 0; k < nt; ++k) {                // (no barrier in between: the warps run apart and keep loads in flight)
+        r = dat_tile_range(tiles, t0 + k);
+        const bool keep = t0 + k >= keep_from;    // read again first thing by the call that follows (which walks back)
+        if (r.begin >= r.lo && r.begin + DAT_TILE <= r.hi) sumsq_rows<NW, true>(gp, r, w0, w1, keep, s_sum + k * nw);
+        else sumsq_rows<NW, false>(gp, r, w0, w1, keep, s_sum + k * nw);
+    }
     __syncthreads();
-    for (int i = threadIdx.x; i < w1 - w0; i += DAT_THREADS) {
-        double s = 0.0;
+    if (warp == 0) {                              // (at most 32 sums: the partials are warp 0's)
+        if (lane < nt * nw) {
+            double s = 0.0;
 #pragma unroll
-        for (int w = 0; w < W; ++w) s += s_sum[i][w];
-        partials[tile * M + w0 + i] = s;
-    }
-    const int64_t T = dat_layer_tiles(r);
-    if (warp == 0) {                              // (at most 32 workers: the partials are warp 0's)
+            for (int x = 0; x < W; ++x) s += s_sum[lane][x];
+            partials[(t0 + lane / nw) * M + w0 + lane % nw] = s;
+        }
         __syncwarp();
-        if (lane == 0) s_last = dat_count_in(out.count + r.layer, (uint32_t)(T * gridDim.y));
+        if (lane == 0) {
+            uint32_t last = 0;
+            TileRange x = r;
+            dat_fence();
+            for (int i = nt - 1;;) {              // from the last tile on; tiles of one layer are counted in together
+                const uint32_t n = (uint32_t)min((int64_t)(i + 1), t0 + i - x.first + 1);
+                if (atomicAdd(out.count + x.layer, n) == (uint32_t)(dat_layer_tiles(x) * gridDim.y) - n) last |= 1u << i;
+                i -= (int)n;
+                if (i < 0) break;
+                x = dat_tile_range(tiles, t0 + i);
+            }
+            if (last) dat_fence();
+            s_last = last;
+        }
     }
     __syncthreads();
-    if (s_last) sumsq_finish(r.layer, r.first, r.first + T, tiles.h, M, partials, out);
+    for (uint32_t last = s_last; last; last &= last - 1) {
+        const int i = __ffs(last) - 1;
+        const TileRange x = i == nt - 1 ? r : dat_tile_range(tiles, t0 + i);
+        sumsq_finish(x.layer, x.first, x.first + dat_layer_tiles(x), tiles.h, M, partials, out);
+        __syncthreads();
+    }
 }
 
 static TileSource plan_tiles(const dat_plan_t *plan) { return TileSource{plan->d_tiles, plan->d_offsets, plan->d_tile_base, (int)plan->h}; }
@@ -161,13 +188,19 @@ static TileSource plan_tiles(const dat_plan_t *plan) { return TileSource{plan->d
 static int sumsq_go(dat_plan_t *plan, const GradPtrs &gp, int M, const NormOut &o, cudaStream_t s)
 {
     // several workers in a CTA (fewer arrivals at the layer's counter, a longer stream per CTA) as long as the CTAs
-    // still fill the GPU
-    int per_cta = 1;
-    while (per_cta < SUMSQ_WORKERS && per_cta < M && plan->n_tiles * ((M + 2 * per_cta - 1) / (2 * per_cta)) >= 8 * plan->sm_count) per_cta *= 2;
-    dim3 grid((unsigned)plan->n_tiles, (unsigned)((M + per_cta - 1) / per_cta));
+    // still fill the GPU, then several tiles
+    int per_cta = 1, tiles_per_cta = 1;
+    auto ctas = [&](int workers, int n) { return (plan->n_tiles + n - 1) / n * ((M + workers - 1) / workers); };
+    while (per_cta < SUMSQ_JOBS && per_cta < M && ctas(2 * per_cta, 1) >= 8 * plan->sm_count) per_cta *= 2;
+    if (per_cta >= M)
+        while (2 * tiles_per_cta * per_cta <= SUMSQ_JOBS && ctas(per_cta, 2 * tiles_per_cta) >= 8 * plan->sm_count) tiles_per_cta *= 2;
+    dim3 grid((unsigned)((plan->n_tiles + tiles_per_cta - 1) / tiles_per_cta), (unsigned)((M + per_cta - 1) / per_cta));
     const int64_t keep_from = plan->n_tiles - SUMSQ_KEEP_BYTES / (4 * DAT_TILE * M);
-    if (per_cta == 1) k_sumsq<1><<<grid, DAT_THREADS, 0, s>>>(gp, plan_tiles(plan), M, per_cta, keep_from, plan->d_partials, o);
-    else k_sumsq<2><<<grid, DAT_THREADS, 0, s>>>(gp, plan_tiles(plan), M, per_cta, keep_from, plan->d_partials, o);
+#define DAT_SUMSQ(NW, T) k_sumsq<NW, T><<<grid, DAT_THREADS, 0, s>>>(gp, plan_tiles(plan), M, per_cta, tiles_per_cta, plan->n_tiles, keep_from, plan->d_partials, o)
+    if (tiles_per_cta > 1) { if (per_cta == 1) DAT_SUMSQ(1, true); else DAT_SUMSQ(2, true); }
+    else if (per_cta == 1) DAT_SUMSQ(1, false);
+    else DAT_SUMSQ(2, false);
+#undef DAT_SUMSQ
     DAT_LAUNCHED(plan);
     return DAT_OK;
 }
