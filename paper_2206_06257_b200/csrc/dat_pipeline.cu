@@ -893,6 +893,7 @@ static std::vector<PipeItem> p_items(const dat_plan_t *plan, const std::vector<i
         return pp;
     };
     std::vector<PipeItem> items;
+    items.reserve(2 * (size_t)(tb[l1] - tb[l0]) + 4096);
     auto at = [&](int64_t slot) -> PipeItem & {
         if ((int64_t)items.size() <= slot) items.resize((size_t)slot + 1, none);
         return items[(size_t)slot];
@@ -959,6 +960,7 @@ int dat_pipe_build(dat_plan_t *plan)
         auto take = [&](size_t bytes) { size_t o = off; off = p_align(off + bytes); return o; };
         const size_t o_items = take(items.size() * sizeof(PipeItem)), o_items2 = take(items2.size() * sizeof(PipeItem));
         std::vector<PipePart> parts;
+        parts.reserve((size_t)nt);
         for (int l = 0; l < h; ++l)
             for (int64_t t = 0; t < tb[l + 1] - tb[l]; ++t)
                 parts.push_back(PipePart{plan->offsets[l], plan->offsets[l + 1], (int32_t)tb[l], (int32_t)(tb[l + 1] - tb[l]), l, (int32_t)t});
@@ -979,7 +981,7 @@ int dat_pipe_build(dat_plan_t *plan)
         g->d_partN = (double *)(g->mem + o_pn);
         g->d_partQ = (double *)(g->mem + o_pq);
         g->d_sync = (uint32_t *)(g->mem + o_sync);
-        e = cudaMemset(g->mem, 0, off);
+        e = cudaMemset(g->mem + o_pn, 0, off - o_pn);
         if (e == cudaSuccess) e = cudaMemcpy(g->d_items, items.data(), items.size() * sizeof(PipeItem), cudaMemcpyHostToDevice);
         if (e == cudaSuccess && !items2.empty())
             e = cudaMemcpy(g->d_items2, items2.data(), items2.size() * sizeof(PipeItem), cudaMemcpyHostToDevice);

@@ -1,4 +1,5 @@
 // Plan object, argument validation, status word and the host-buffer entry point.
+#include <algorithm>
 #include <cmath>
 #include <new>
 
@@ -166,35 +167,35 @@ extern "C" int dat_plan_create(dat_plan_t **out, int64_t num_layers, const int64
     p->level_bytes = (int64_t)align_up((size_t)((p->d * eff_bits + 7) / 8), 16);
     p->sign_bytes = (bits == 32) ? 0 : (int64_t)align_up((size_t)((p->d + 7) / 8), 16);
 
-    // per-layer tiles, and the layer of every flat piece's first element
-    std::vector<int32_t> flat_layer;
-    std::vector<TileDesc> tiles;
-    try {
-        tiles.resize((size_t)nt);
-        for (int64_t l = 0; l < num_layers; ++l)
-            for (int64_t t = p->tile_base[l]; t < p->tile_base[l + 1]; ++t)
-                tiles[(size_t)t] = TileDesc{p->offsets[l], p->offsets[l + 1], (p->offsets[l] & ~(int64_t)7) + (t - p->tile_base[l]) * DAT_TILE,
-                                            (int32_t)l, (int32_t)p->tile_base[l]};
-        const int64_t pieces = (p->d + DAT_FLAT - 1) / DAT_FLAT;
-        flat_layer.resize((size_t)pieces + 1);
-        int64_t l = 0;
-        for (int64_t t = 0; t < pieces; ++t) {
-            while (p->offsets[l + 1] <= t * DAT_FLAT) ++l;
-            flat_layer[t] = (int32_t)l;
-        }
-        flat_layer[pieces] = (int32_t)(num_layers - 1);
-    } catch (...) { delete p; return DAT_ERR_NOMEM; }
-
     // carve the workspace
     const size_t h1 = (size_t)num_layers + 1, h = (size_t)num_layers;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
-    const size_t o_off = take(h1 * 8), o_tb = take(h1 * 8), o_fl = take(flat_layer.size() * 4), o_td = take(tiles.size() * sizeof(TileDesc)), o_ct = take(h * 4);
+    const int64_t pieces = (p->d + DAT_FLAT - 1) / DAT_FLAT;
+    const size_t o_off = take(h1 * 8), o_tb = take(h1 * 8), o_fl = take(((size_t)pieces + 1) * 4), o_td = take((size_t)nt * sizeof(TileDesc)), o_ct = take(h * 4);
     const size_t o_part = take((size_t)nt * (size_t)(num_workers > 2 ? num_workers : 2) * 8);
     const size_t o_wn = take((size_t)num_workers * h * 4);
     const size_t o_sc = take(h * 4), o_qm = take((size_t)num_workers * h * 4), o_dq = take(h * 4), o_sa = take(h * 4);
     const size_t o_nr = take(2 * h * 4), o_st = take(256);
     p->ws_bytes = off;
+
+    // the tables, laid out as on the device (one copy): layers, per-layer tiles, the layer of every flat piece's first element
+    std::vector<char> tables;
+    try { tables.resize(o_ct); } catch (...) { delete p; return DAT_ERR_NOMEM; }
+    std::copy(p->offsets.begin(), p->offsets.end(), (int64_t *)(tables.data() + o_off));
+    std::copy(p->tile_base.begin(), p->tile_base.end(), (int64_t *)(tables.data() + o_tb));
+    TileDesc *tile = (TileDesc *)(tables.data() + o_td);
+    for (int64_t l = 0; l < num_layers; ++l)
+        for (int64_t t = p->tile_base[l]; t < p->tile_base[l + 1]; ++t)
+            *tile++ = TileDesc{p->offsets[l], p->offsets[l + 1], (p->offsets[l] & ~(int64_t)7) + (t - p->tile_base[l]) * DAT_TILE, (int32_t)l,
+                               (int32_t)p->tile_base[l]};
+    int32_t *flat_layer = (int32_t *)(tables.data() + o_fl);
+    for (int64_t t = 0, l = 0; t < pieces; ++t) {
+        while (p->offsets[l + 1] <= t * DAT_FLAT) ++l;
+        flat_layer[t] = (int32_t)l;
+    }
+    flat_layer[pieces] = (int32_t)(num_layers - 1);
+
     e = cudaMalloc((void **)&p->ws, p->ws_bytes);
     if (e != cudaSuccess) { delete p; (void)cudaGetLastError(); return DAT_ERR_NOMEM; }
     p->d_offsets = (int64_t *)(p->ws + o_off);
@@ -210,11 +211,8 @@ extern "C" int dat_plan_create(dat_plan_t **out, int64_t num_layers, const int64
     p->d_step_a = (float *)(p->ws + o_sa);
     p->d_norms = (float *)(p->ws + o_nr);
     p->d_status = (uint32_t *)(p->ws + o_st);
-    e = cudaMemset(p->ws, 0, p->ws_bytes);
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_offsets, p->offsets.data(), h1 * 8, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_tiles, tiles.data(), tiles.size() * sizeof(TileDesc), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_flat_layer, flat_layer.data(), flat_layer.size() * 4, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_tile_base, p->tile_base.data(), h1 * 8, cudaMemcpyHostToDevice);
+    e = cudaMemset(p->ws + o_ct, 0, p->ws_bytes - o_ct);
+    if (e == cudaSuccess) e = cudaMemcpy(p->ws, tables.data(), tables.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         cudaFree(p->ws);
         delete p;
