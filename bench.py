@@ -418,7 +418,8 @@ def run_gpu(args):
         second_read = int(4 * cfg.M * sizes[4 * cfg.M * sizes > l2_bytes].sum()) if not unfused and cfg.bits != 32 else 0
         per_step = launches // K
         traffic, traffic_src = ncu_traffic(args.path, cfg)
-        kernel_name = {"step": "dat_step (k_step_pipelined)", "pipelined": "dat_step_pipelined (k_step_pipelined)",
+        form = "k_step_pipelined" if per_step == 1 else "a launch per phase"
+        kernel_name = {"step": "dat_step (%s)" % form, "pipelined": "dat_step_pipelined (k_step_pipelined)",
                        "passes": "dat_step_passes"}.get(args.path, args.path)
         kernel_name += ": %d launch%s per step, the whole step timed" % (per_step, "" if per_step == 1 else "es")
         sm_mhz = clocks.get("sm_mhz") or 0
@@ -536,7 +537,7 @@ def main():
     ap.add_argument("--impl", default="dat", choices=["dat", "reference"])
     ap.add_argument("--path", default="step",
                     choices=["step", "step_per_worker", "step_lamb", "step_two_sided", "pipelined", "passes", "unfused", "unfused_per_worker", "unfused_two_sided", "unfused_lamb"],
-                    help="step: dat_step (the headline: one pipelined launch); pipelined: the same by its own name; "
+                    help="step: dat_step (the headline: one pipelined launch, or one per phase for small workloads); pipelined: the one launch by its own name; "
                          "step_per_worker: dat_step on a plan with one quantizer norm per worker; step_lamb: dat_step_lamb; step_two_sided: dat_step_two_sided (Step 10 in the same launch); "
                          "passes: dat_step_passes, three streaming passes; unfused: dat_quantize + dat_aggregate + dat_lalr_step; "
                          "unfused_per_worker: the same with one quantizer norm per worker; unfused_two_sided: with "

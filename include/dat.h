@@ -318,8 +318,9 @@ int dat_lalr_step_static(int64_t num_layers, const int64_t *layer_offsets, float
  * dat_step -- Steps 7, 9 and 12 of Algorithm A1 in one call: the result equals
  * dat_quantize -> dat_aggregate -> dat_lalr_step (or dat_average -> dat_lalr_step when b = 32),
  * but codes, code sums and g_hat are never written to device memory.  One kernel launch
- * (dat_step_pipelined) for problems that fill the GPU, one launch per phase (dat_step_passes) for smaller ones and
- * for a single worker; nothing is allocated and nothing synchronises: every table the launches
+ * (dat_step_pipelined) for problems that fill the GPU, one launch per phase (dat_step_passes) below four tiles of 4096
+ * elements per SM; with b < 32 also below nine (two-sided steps: with eight workers and more) and, for a single worker,
+ * at any size.  Nothing is allocated and nothing synchronises: every table the launches
  * need was built by dat_plan_create.
  *   theta, mom        device fp32[d], updated in place.
  *   grads             host array of M device pointers, fp32[d] each, read-only.
@@ -359,7 +360,7 @@ int dat_step_pipelined(dat_plan_t *plan, float *theta, float *mom, const float *
 
 /* dat_step_lamb -- dat_step with LAMB (Algorithm A2) as the outer-minimisation oracle instead of the momentum
  * direction: Steps 7 and 9 as in dat_step, then m', v', the bias-corrected direction and the layer-wise update
- * exactly as dat_lamb_step computes them from g_hat -- in the same single launch, g_hat never stored.
+ * exactly as dat_lamb_step computes them from g_hat -- in the same launch or launches, g_hat never stored.
  *   var   device fp32[d], the second moment, updated in place;  t >= 1 the iteration count;  hp as in dat_lamb_step.
  * Other arguments, the bounded wait and its status bit as in dat_step.
  * Errors: ARG (null pointer, t < 1, beta outside (0,1)), ALIGN, CUDA. */
@@ -370,9 +371,9 @@ int dat_step_lamb(dat_plan_t *plan, float *theta, float *mom, float *var, const 
 /* dat_step_two_sided -- dat_step with two-sided quantisation (Algorithm A1 Step 10, the parameter-server
  * setting): after Steps 7 and 9 the server quantizes the aggregate itself, g_hat <- Q(g_hat), with its own
  * norm nu^_l = ||g_hat_l||_2 per layer and the levels of Eq. xi drawn on the random stream of index M (the
- * first one no worker uses) -- what dat_requantize computes -- and Step 12 uses the receiver's value.  All in
- * the same single launch: a fourth stream of tiles runs between the Q and the U tiles, waiting (bounded, as
- * in dat_step) for the layer's nu^_l.  Neither the workers' nor the server's packed message is written.
+ * first one no worker uses) -- what dat_requantize computes -- and Step 12 uses the receiver's value.  In the
+ * one launch a fourth stream of tiles runs between the Q and the U tiles, waiting (bounded, as
+ * in dat_step) for the layer's nu^_l; by phases it is a fourth launch.  Neither the workers' nor the server's packed message is written.
  *   g_hat               device fp32[d], caller-owned, 16-byte aligned: workspace (the aggregate is stored
  *                       here between the two phases) and output: on return the receiver's value
  *                       nu^_l * sign * level / S of every element.

@@ -280,14 +280,6 @@ __device__ __forceinline__ uint32_t dat_level_u1(float g, float qmul, float S1_f
     return dat_level_bits_u1(g, qmul, S1_f, u1) & 0x007FFFFFu;
 }
 
-// sum += sign(g) * level, from the bits of dat_level_bits: with sm = 0 or -1 (all ones) for
-// g's sign bit, (level ^ sm) - sm is level or -level.  (-0.0 has level 0, so its sign is moot.)
-__device__ __forceinline__ int dat_add_signed_level(int sum, float g, uint32_t level_bits)
-{
-    const int sm = (int)__float_as_uint(g) >> 31;
-    return sum + (int)((level_bits & 0x007FFFFFu) ^ (uint32_t)sm) - sm;
-}
-
 // Largest l in [0, h) with table[l] <= x (table[0] <= x < table[h] assumed).
 __device__ __forceinline__ int dat_find(const int64_t *__restrict__ table, int h, int64_t x)
 {

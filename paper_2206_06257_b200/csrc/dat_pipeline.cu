@@ -1041,16 +1041,22 @@ cudaError_t dat_pipe_reset(dat_plan_t *plan, cudaStream_t s)
     return cudaMemsetAsync(g->d_sync, 0, g->sync_bytes, s);
 }
 
-// Which form a step takes.  One launch per phase wins where the GPU is not full: the one launch keeps its streams 256 and
-// 512 items apart, so a small problem runs through waves of nearly empty CTAs (us, one launch / phases, B200):
-//   tiny MLP (61 tiles) M = 4: 22.9 / 18.2    300 thousand elements, M = 8: 38.3 / 24.3, M = 64 in 200 layers: 265 / 121
-//   1 million (290 tiles), M = 8: 50.1 / 37.3, b = 32: 22.1 / 17.5; LAMB 60.3 / 43.4; two-sided 58.7 / 46.0
-// Up to nine tiles per SM it still does, the two-sided step's four launches with few workers excepted:
-//   3 million (800 tiles), M = 16: 119 / 108   4 million, M = 3: 59.1 / 51.1, LAMB M = 8: 107 / 95   5 million, M = 16: 176 / 165
-//   3 million, M = 3, two-sided: 63.9 / 66.1
-// Beyond that the overlap of the streams wins: 8 million (2000 tiles), M = 4: 103 / 102, 60 million, M = 4: 536 / 585, ResNet-50,
-// M = 8: 312 / 381.  With one worker there is little to overlap (a gradient is read twice and the update's vectors four
-// times): 60 million, 413 / 365; LAMB 607 / 531; two-sided 538 / 511.
+// Which form a step takes.  The one launch keeps its streams 256 and 512 items apart, so a small problem runs through waves
+// of nearly empty CTAs; the phases have a launch's set-up and last wave each.  Both forms of the momentum step, b = 8, in us
+// (one launch / phases; 30 to 60 layers):
+//   elements, tiles per SM   M = 1        2          4          6           8           16          32
+//   2.2 million, 3.8      26 / 29    29 / 33    36 / 39    43 / 45     52 / 52     98 / 79    190 / 135
+//   3.6 million, 6.1      31 / 31    35 / 37    45 / 47    58 / 59     71 / 71    128 / 115   241 / 197
+//   5.2 million, 8.8      41 / 38    47 / 45    64 / 62    83 / 81    101 / 99    182 / 157   336 / 270
+//   8.0 million, 13.5     60 / 53    66 / 68    88 / 91   111 / 115   134 / 140   229 / 237   422 / 423
+//   16 million, 26.7     122 / 105  135 / 126  177 / 168  219 / 213   258 / 257   438 / 434   804 / 798
+//   60 million           409 / 359  453 / 438; ResNet-50, M = 8: 312 / 381;  tiny MLP (61 tiles), M = 4: 23 / 18
+// So: phases below a wave's size are worth 5 to 40 us with many workers or few elements and cost up to 4 with few workers
+// and 3 million; one worker gains at every size from seven tiles per SM on; above that size the two differ by less than 10 %
+// either way until the streams' overlap wins (the large models).
+// The two-sided step has a fourth launch: 2.2 to 3.6 million elements, M = 2 and 4, 36 / 42, 55 / 61, M = 8, 62 / 64, 83 / 86,
+// M = 16, 110 / 91, 140 / 130; at 4.5 to 8 million, M = 2 to 8, within 4 % of each other.  b = 32 (no
+// norms): 1 million, M = 8, 22 / 18, 2.2 million, M = 1 to 8, 17 to 25 / 19 to 25, M = 8: 2.8 million 28 / 34, 16 million 153 / 159.
 #define P_PHASES_WAVE 4                           // tiles per SM: one wave of a phase's CTAs
 #define P_PHASES_MOST 9
 static bool p_phases(const dat_plan_t *plan, bool two)
