@@ -88,7 +88,7 @@ struct PipeSchedule {
     double *d_partQ = nullptr;                    // 2 per half tile
     uint32_t *d_sync = nullptr;                   // [0] ticket, [1] abort epoch, then cntN[h], cntQ[h], readyN[h], readyQ[h], cntR[h], readyR[h]
     size_t sync_bytes = 0;
-    int64_t n_tiles = 0;
+    int64_t n_tiles = 0, largest = 0;             // elements of the largest layer
     std::vector<int64_t> tile_base;               // h + 1
     std::vector<PipeGroup> groups;                // built by the first dat_step_host that goes in groups
     PipeItem *d_group_items = nullptr;
@@ -411,6 +411,36 @@ __device__ __noinline__ float4 p_rows_per_worker_slow4(const PArgs &a, const flo
     }
     return make_float4(acc[0], acc[1], acc[2], acc[3]);
 }
+// A ragged group by its whole warp (see qu_rows_ragged4): a lane draws a worker's levels, every lane forms the ordered
+// sums from the lanes' levels.
+template <bool RNG16>
+__device__ __noinline__ float4 p_rows_per_worker_ragged4(const PArgs &a, const float2 *s_fac, int64_t e0, int64_t lo, int64_t hi)
+{
+    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    for (int i0 = 0; i0 < a.M; i0 += 32) {
+        const int i = i0 + (threadIdx.x & 31), n = min(32, a.M - i0);
+        int lev[4] = {0, 0, 0, 0};
+        if (i < a.M) dat_signed_levels4<RNG16>(a.gp.p[i], (uint32_t)i, a.keys, s_fac[i].x, a.S_f + 1.0f, e0, lo, hi, lev);
+        __syncwarp();
+        for (int k = 0; k < n; ++k) {
+            const float nu = s_fac[i0 + k].y;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[j] = __fmaf_rn(nu, (float)__shfl_sync(0xFFFFFFFFu, lev[j], k), acc[j]);
+        }
+    }
+    return make_float4(acc[0], acc[1], acc[2], acc[3]);
+}
+// The group's sums for its own thread, in shared memory (a layer's first or last group, drawn before the others).
+template <bool RNG16, int MODE>
+__device__ __forceinline__ void p_ragged(const PArgs &a, const QuConst &qc, const float2 *s_fac, int64_t e0, int64_t lo, int64_t hi, float *s_out)
+{
+#pragma unroll 1
+    for (int p = 0; p < 2; ++p) {
+        const float4 x = MODE == P_MODE_PER_WORKER ? p_rows_per_worker_ragged4<RNG16>(a, s_fac, e0 + 4 * p, lo, hi)
+                                                   : qu_rows_ragged4<RNG16>(a.gp, a.keys, qc.t, qc.two_b, a.M, e0 + 4 * p, lo, hi);
+        if ((threadIdx.x & 31) == 0) { s_out[4 * p] = x.x; s_out[4 * p + 1] = x.y; s_out[4 * p + 2] = x.z; s_out[4 * p + 3] = x.w; }
+    }
+}
 template <bool RNG16, int UNROLL>
 __device__ __forceinline__ void p_rows_per_worker(const PArgs &a, const QuConst &qc, const float2 *s_fac, bool fast, int64_t e0, int64_t lo, int64_t hi, float acc[8])
 {
@@ -477,7 +507,8 @@ __device__ __forceinline__ void p_direction(const PArgs &a, int64_t e0, int64_t 
 // warp in scratch[2w], scratch[2w + 1].  TWO (Algorithm A1 Step 10 follows): stops at g_hat, which is
 // stored, and leaves the tile's sum of g_hat^2 per warp in scratch[2w]. ----------------------------
 // G: groups of eight per thread, from the tile's piece `piece` on (G = 2: the whole tile, piece 0; G = 1: half a tile).
-template <bool RNG16, int MODE, int OPT, bool TWO, int G>
+// ENDS: the groups at the layer's two ends by whole warps.
+template <bool RNG16, int MODE, int OPT, bool TWO, int G, bool ENDS = (MODE != P_MODE_IDENTITY)>
 __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt, int piece, double *scratch, float2 *s_fac)
 {
     const int M = a.M, layer = pt.layer;
@@ -497,6 +528,14 @@ __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt,
     }
     double ss_theta = 0.0, ss_u = 0.0;
     const int64_t begin = p_tile_begin(pt) + (int64_t)piece * (8 * DAT_P_THREADS);
+    __shared__ float s_ends[ENDS ? 2 : 1][8];
+    if (ENDS && !plain && begin < hi) {
+        const int64_t last = min(begin + 8 * (G * DAT_P_THREADS - 1), (hi - 1) & ~(int64_t)7);
+        if ((threadIdx.x >> 5) == 0 && (begin < lo || begin + 8 > hi)) p_ragged<RNG16, MODE>(a, qc, s_fac, begin, lo, hi, s_ends[0]);
+        if ((threadIdx.x >> 5) == (unsigned)((last - begin) / 256) % (DAT_P_THREADS / 32) && last > begin && last + 8 > hi)
+            p_ragged<RNG16, MODE>(a, qc, s_fac, last, lo, hi, s_ends[ENDS]);
+        __syncwarp();                              // (read by a lane of the warp that drew it)
+    }
 #pragma unroll 1
     for (int k = 0; k < G; ++k) {
         const int64_t e0 = begin + 8 * (int64_t)(k * DAT_P_THREADS + threadIdx.x);
@@ -513,6 +552,9 @@ __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt,
 #pragma unroll
                 for (int j = 0; j < 8; ++j) acc[j] += v[j];
             }
+        } else if (ENDS && !full && !plain) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[j] = s_ends[e0 != begin][j];
         } else if (MODE == P_MODE_PER_WORKER) p_rows_per_worker<RNG16, G == 1 ? 4 : 1>(a, qc, s_fac, full && !plain, e0, lo, hi, acc);
         else if (full && !plain) qu_rows<RNG16, G == 1 ? 4 : 2>(a.gp, a.keys, a.workers, qc, M, e0, acc);       // nearly always
         else qu_rows_slow<RNG16, G == 1 ? 4 : 1>(a.gp, a.keys, qc, M, e0, lo, hi, acc);
@@ -755,7 +797,9 @@ k_step_pipelined(const __grid_constant__ PArgs a)
     __syncthreads();                               // (A)
     if (s_ctl[0]) p_norm_finish<MODE>(a, pn, s_norm);
     bool alive = (s_ctl[1] != 0);
-    if (alive && pq.layer >= 0) p_part_quant<RNG16, MODE, OPT, TWO, DAT_P_GROUPS>(a, pq, 0, s_unit, s_fac);
+    // (the groups at a layer's ends by their own lanes: the wait is hidden here, and the code beside the long loop is not --
+    // with whole warps ResNet-50 takes 336 us instead of 330, 1 billion parameters 13.9 ms instead of 13.7)
+    if (alive && pq.layer >= 0) p_part_quant<RNG16, MODE, OPT, TWO, DAT_P_GROUPS, false>(a, pq, 0, s_unit, s_fac);
     __syncthreads();
     if (TWO) {
         // Step 10: the tile's sum of g_hat^2 counted in; the layer's last tile publishes the server's norm;
@@ -945,6 +989,7 @@ int dat_pipe_build(dat_plan_t *plan)
         int64_t nt = 0;
         for (int l = 0; l < h; ++l) {
             tb[l] = nt;
+            g->largest = std::max(g->largest, plan->offsets[l + 1] - plan->offsets[l]);
             nt += (plan->offsets[l + 1] - (plan->offsets[l] & ~(int64_t)7) + DAT_P_TILE - 1) / DAT_P_TILE;
         }
         tb[h] = nt;
@@ -1042,29 +1087,31 @@ cudaError_t dat_pipe_reset(dat_plan_t *plan, cudaStream_t s)
 }
 
 // Which form a step takes.  The one launch keeps its streams 256 and 512 items apart, so a small problem runs through waves
-// of nearly empty CTAs; the phases have a launch's set-up and last wave each.  Both forms of the momentum step, b = 8, in us
-// (one launch / phases; 30 to 60 layers):
-//   elements, tiles per SM   M = 1        2          4          6           8           16          32
-//   2.2 million, 3.8      26 / 29    29 / 33    36 / 39    43 / 45     52 / 52     98 / 79    190 / 135
-//   3.6 million, 6.1      31 / 31    35 / 37    45 / 47    58 / 59     71 / 71    128 / 115   241 / 197
-//   5.2 million, 8.8      41 / 38    47 / 45    64 / 62    83 / 81    101 / 99    182 / 157   336 / 270
-//   8.0 million, 13.5     60 / 53    66 / 68    88 / 91   111 / 115   134 / 140   229 / 237   422 / 423
-//   16 million, 26.7     122 / 105  135 / 126  177 / 168  219 / 213   258 / 257   438 / 434   804 / 798
-//   60 million           409 / 359  453 / 438; ResNet-50, M = 8: 312 / 381;  tiny MLP (61 tiles), M = 4: 23 / 18
-// So: phases below a wave's size are worth 5 to 40 us with many workers or few elements and cost up to 4 with few workers
-// and 3 million; one worker gains at every size from seven tiles per SM on; above that size the two differ by less than 10 %
-// either way until the streams' overlap wins (the large models).
-// The two-sided step has a fourth launch: 2.2 to 3.6 million elements, M = 2 and 4, 36 / 42, 55 / 61, M = 8, 62 / 64, 83 / 86,
-// M = 16, 110 / 91, 140 / 130; at 4.5 to 8 million, M = 2 to 8, within 4 % of each other.  b = 32 (no
-// norms): 1 million, M = 8, 22 / 18, 2.2 million, M = 1 to 8, 17 to 25 / 19 to 25, M = 8: 2.8 million 28 / 34, 16 million 153 / 159.
+// of nearly empty CTAs; the phases have a launch's set-up and last wave each.  And the streams of the largest layer, which
+// come last, overlap with nothing: a model that is one third one layer does better by phases at every size.  Both forms of
+// the momentum step, b = 8, in us (one launch / phases; 50 to 60 odd layers, the largest 0.33 of the elements):
+//   elements, tiles per SM    M = 1        2          4          6           8           16          32
+//   2.2 million, 3.8      29 / 31    33 / 34    43 / 41    53 / 46     63 / 52    106 / 74    190 / 119
+//   3.6 million, 6.1      37 / 35    41 / 39    54 / 49    67 / 58     79 / 72    132 / 110   239 / 174
+//   5.2 million, 8.8      48 / 45    53 / 51    68 / 64    83 / 79     99 / 98    166 / 147   305 / 240
+//   8.0 million, 13.5     69 / 60    75 / 69   100 / 89   119 / 109   139 / 130   231 / 207   422 / 367
+//   16 million, 26.7     124 / 108  137 / 125  178 / 164  218 / 198   258 / 237   438 / 391   803 / 706
+// The largest 0.17: 24 million 162 / 152, 178 / 177, 233 / 235, 284 / 288, 337 / 345, 593 / 577; 48 million 315 / 288 to
+// 686 / 672.  0.21 (ResNet-18): M = 1, 6, 16: 72 / 76, 123 / 139, 242 / 276.  0.09 (ResNet-50): M = 1, 2, 8: 146 / 152,
+// 161 / 178, 309 / 358.  Two-sided, 0.33: 3.6 million, M = 1 to 16, 49 / 46, 52 / 52, 65 / 62, 78 / 72, 90 / 87, 143 / 126, 5.2 million
+// 60 / 59 to 111 / 116, 8 to 16 million 87 / 80 to 470 / 429; ResNet-18, M = 6, 145 / 166; 3 million, M = 3, the
+// largest 0.23: 63.5 / 65.6.
+// b = 32 (no norms): 1 million, M = 8, 22 / 18, 2.2 million, M = 1 to 8, 17 to 25 / 19 to 25, M = 8: 2.8 million 28 / 34, 16 million 153 / 159.
 #define P_PHASES_WAVE 4                           // tiles per SM: one wave of a phase's CTAs
 #define P_PHASES_MOST 9
+#define P_PHASES_SHARE 0.27                       // of the elements, in the largest layer
 static bool p_phases(const dat_plan_t *plan, bool two)
 {
     const int64_t n = plan->pipe->n_tiles, sm = plan->sm_count;
     if (n <= P_PHASES_WAVE * sm) return true;
     if (plan->bits == 32) return false;
-    return plan->M == 1 || (n <= P_PHASES_MOST * sm && (!two || plan->M >= 8));
+    if (plan->M == 1 && !two) return true;        // (60 million elements: 409 / 359)
+    return (n <= P_PHASES_MOST * sm && (!two || plan->M >= 8)) || (double)plan->pipe->largest >= P_PHASES_SHARE * (double)plan->d;
 }
 // Half a tile per CTA: in one wave, and with many workers (a long loop per CTA, so that a last wave of whole tiles costs
 // much: 2.5 million elements, 617 tiles, M = 32: 185 / 156 us; 4 million, M = 3: 51.1 / 53.5).
