@@ -320,7 +320,8 @@ int dat_lalr_step_static(int64_t num_layers, const int64_t *layer_offsets, float
  * but codes, code sums and g_hat are never written to device memory.  One kernel launch
  * (dat_step_pipelined) for problems that fill the GPU, one launch per phase (dat_step_passes) up to four tiles of 4096
  * elements per SM; with b < 32 also up to nine (two-sided steps: with eight workers and more), where one layer has more than 0.27 of the elements, and (one-sided) for a
- * single worker at any size.  Nothing is allocated and nothing synchronises: every table the launches
+ * single worker at any size.  With b < 32 and at most three pieces of 2048 elements per SM it is one (cooperative) launch
+ * whose CTAs keep a piece each through all phases and wait, bounded, for its layer.  Nothing is allocated and nothing synchronises: every table the launches
  * need was built by dat_plan_create.
  *   theta, mom        device fp32[d], updated in place.
  *   grads             host array of M device pointers, fp32[d] each, read-only.
@@ -406,12 +407,13 @@ int dat_step_passes(dat_plan_t *plan, float *theta, float *mom, const float *con
  * `wait_cycles` SM clock cycles (0 restores the default) and, if `layer` >= 0, marks that layer's norm
  * as never completing for the next call (its tile counter is pre-set on the host side of the stream so
  * that the count cannot be reached): work items that need the layer give up after the limit and the
- * call ends with DAT_STATUS_TIMEOUT.  Only the one launch waits, so the plan's steps take that form until a call with
+ * call ends with DAT_STATUS_TIMEOUT.  Only the forms of one launch wait; the plan's steps take the general one until a call with
  * (0, -1) gives it back to the rule by size.  Nothing else uses this.  Errors: ARG, CUDA. */
 int dat_plan_test_stall(dat_plan_t *plan, int64_t wait_cycles, int64_t layer, void *stream);
 
 /* dat_plan_test_form -- TEST HOOK: the form of the plan's dat_step, dat_step_lamb and two-sided steps whatever their size:
- * 1 the one launch, 2 a launch per phase, 0 by the rule again.  Nothing else uses this.  Errors: ARG. */
+ * 1 the one launch, 2 a launch per phase, 3 one launch whose CTAs keep their pieces (ARG where the problem has more than
+ * three pieces of 2048 elements per SM), 0 by the rule again.  Nothing else uses this.  Errors: ARG. */
 int dat_plan_test_form(dat_plan_t *plan, int form);
 
 /* dat_step_host -- dat_step for callers whose data lives in HOST memory: copies theta, mom and

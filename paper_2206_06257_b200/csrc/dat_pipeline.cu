@@ -55,7 +55,7 @@
 #endif
 #define DAT_P_WAIT_CYCLES (4000000000ll)          // about two seconds
 
-enum { P_BY_RULE = 0, P_ONE_LAUNCH = 1, P_PHASES = 2 };     // which form a step takes (see p_phases)
+enum { P_BY_RULE = 0, P_ONE_LAUNCH = 1, P_PHASES = 2, P_RESIDENT = 3 };     // which form a step takes (see p_resident, p_phases)
 enum { P_MODE_SHARED = 0, P_MODE_PER_WORKER = 1, P_MODE_IDENTITY = 2 };
 enum { P_OPT_MOMENTUM = 0, P_OPT_LAMB = 1 };     // the descent direction u of Eq. 3: heavy-ball momentum, or Algorithm A2
 
@@ -80,11 +80,13 @@ struct PipeSchedule {
     PipeItem *d_items = nullptr;                  // the three streams N, Q, U
     int64_t n_items = 0;
     PipePart *d_parts = nullptr;                  // n_tiles: every tile once, in slot order (the phases)
+    PipePart *d_pieces = nullptr;                 // the half tiles that hold elements, numbered as such (tb, T, tile); small problems only
+    int64_t n_pieces = 0;
     PipeItem *d_items2 = nullptr;                 // the four streams N, Q, R, U of the two-sided step
     int64_t n_items2 = 0;
     double *d_partR = nullptr;                    // 1 per half tile
     float *d_server = nullptr;                    // 2h: S / nu^_l and nu^_l / S
-    double *d_partN = nullptr;                    // n_tiles * M
+    double *d_partN = nullptr;                    // n_tiles * M (with pieces twice that)
     double *d_partQ = nullptr;                    // 2 per half tile
     uint32_t *d_sync = nullptr;                   // [0] ticket, [1] abort epoch, then cntN[h], cntQ[h], readyN[h], readyQ[h], cntR[h], readyR[h]
     size_t sync_bytes = 0;
@@ -169,12 +171,13 @@ __device__ __forceinline__ void p_st8(float *p, bool wide, int64_t e0, int64_t l
 // One thread: waits until `word` carries this call's epoch.  Bounded: when the limit runs out the status
 // word gets DAT_STATUS_TIMEOUT and the call's abort word is set, which ends every other wait at once.
 // Returns false if the part that needs the word must be skipped.
+template <int SLEEP = 128>
 __device__ __forceinline__ bool p_poll(const PArgs &a, const uint32_t *word)
 {
     if (p_ld_acquire(word) == a.epoch) return true;
     const long long t0 = clock64();
     for (;;) {
-        __nanosleep(128);
+        __nanosleep(SLEEP);
         if (p_ld_acquire(word) == a.epoch) return true;
         if (p_ld_acquire(a.abort_epoch) == a.epoch) return false;
         if (clock64() - t0 > a.wait_cycles) {
@@ -658,14 +661,25 @@ __device__ __forceinline__ void p_part_requant(const PArgs &a, const PipePart &p
     }
 }
 
-// Two-sided step, one thread after the barrier that follows the Q part: the tile's sum of g_hat^2 (warps in
-// index order), counted in.  Returns whether this was the layer's last tile.
-__device__ __forceinline__ bool p_server_publish(const PArgs &a, const PipePart &pt, const double *scratch)
+// One thread: a part's sums from its warps', in index order -- the even places, and both into the part's slot.
+__device__ __forceinline__ double p_warps_sum(const double *scratch)
 {
     double x = 0.0;
 #pragma unroll
     for (int w = 0; w < DAT_P_THREADS / 32; ++w) x += scratch[2 * w];
-    a.partR[(int64_t)pt.tb + pt.tile] = x;
+    return x;
+}
+__device__ __forceinline__ void p_quant_sums(const PArgs &a, int64_t slot, const double *scratch)
+{
+    a.partQ[2 * slot] = p_warps_sum(scratch);
+    a.partQ[2 * slot + 1] = p_warps_sum(scratch + 1);
+}
+
+// Two-sided step, one thread after the barrier that follows the Q part: the tile's sum of g_hat^2 (warps in
+// index order), counted in.  Returns whether this was the layer's last tile.
+__device__ __forceinline__ bool p_server_publish(const PArgs &a, const PipePart &pt, const double *scratch)
+{
+    a.partR[(int64_t)pt.tb + pt.tile] = p_warps_sum(scratch);
     return dat_count_in(a.cntR + pt.layer, (uint32_t)pt.T);
 }
 
@@ -700,11 +714,7 @@ __device__ __forceinline__ void p_server_finish(const PArgs &a, const PipePart &
 // counted in.  Returns whether this was the layer's last tile.
 __device__ __forceinline__ bool p_quant_publish(const PArgs &a, const PipePart &pt, const double *scratch)
 {
-    double x = 0.0, y = 0.0;
-#pragma unroll
-    for (int w = 0; w < DAT_P_THREADS / 32; ++w) { x += scratch[2 * w]; y += scratch[2 * w + 1]; }
-    a.partQ[2 * ((int64_t)pt.tb + pt.tile)] = x;
-    a.partQ[2 * ((int64_t)pt.tb + pt.tile) + 1] = y;
+    p_quant_sums(a, (int64_t)pt.tb + pt.tile, scratch);
     return dat_count_in(a.cntQ + pt.layer, (uint32_t)pt.T);      // releases m' (and v', or g_hat) of the whole CTA too
 }
 
@@ -905,6 +915,8 @@ k_phase_update(const __grid_constant__ PArgs a)
     p_part_update<OPT, G>(a, pt, cta % PIECES);
 }
 
+#include "dat_resident.cuh"
+
 // ---- host: the item list -----------------------------------------------------------------------------
 void dat_pipe_destroy(dat_plan_t *plan)
 {
@@ -1010,7 +1022,19 @@ int dat_pipe_build(dat_plan_t *plan)
             for (int64_t t = 0; t < tb[l + 1] - tb[l]; ++t)
                 parts.push_back(PipePart{plan->offsets[l], plan->offsets[l + 1], (int32_t)tb[l], (int32_t)(tb[l + 1] - tb[l]), l, (int32_t)t});
         const size_t o_parts = take(parts.size() * sizeof(PipePart));
-        const size_t o_pn = take((size_t)nt * (size_t)M * 8), o_pq = take((size_t)nt * 32), o_pr = take((size_t)nt * 16);
+        std::vector<PipePart> pieces;
+        if (nt <= (int64_t)R_CTAS * plan->sm_count) {
+            pieces.reserve((size_t)(2 * nt));
+            for (int l = 0; l < h; ++l) {
+                const int64_t lo = plan->offsets[l], hi = plan->offsets[l + 1], n = (hi - (lo & ~(int64_t)7) + R_PIECE - 1) / R_PIECE;
+                const int32_t first = (int32_t)pieces.size();
+                for (int64_t t = 0; t < n; ++t) pieces.push_back(PipePart{lo, hi, first, (int32_t)n, l, (int32_t)t});
+            }
+        }
+        if ((int64_t)pieces.size() > (int64_t)R_CTAS * plan->sm_count) pieces.clear();
+        g->n_pieces = (int64_t)pieces.size();
+        const size_t o_pieces = take(pieces.size() * sizeof(PipePart));
+        const size_t o_pn = take((size_t)nt * (size_t)M * (pieces.empty() ? 8 : 16)), o_pq = take((size_t)nt * 32), o_pr = take((size_t)nt * 16);
         const size_t o_server = take(2 * (size_t)h * 4);
         g->sync_bytes = (2 + 6 * (size_t)h) * 4;
         const size_t o_sync = take(g->sync_bytes);
@@ -1023,6 +1047,7 @@ int dat_pipe_build(dat_plan_t *plan)
         g->d_partR = (double *)(g->mem + o_pr);
         g->d_server = (float *)(g->mem + o_server);
         g->d_parts = (PipePart *)(g->mem + o_parts);
+        g->d_pieces = (PipePart *)(g->mem + o_pieces);
         g->d_partN = (double *)(g->mem + o_pn);
         g->d_partQ = (double *)(g->mem + o_pq);
         g->d_sync = (uint32_t *)(g->mem + o_sync);
@@ -1031,6 +1056,8 @@ int dat_pipe_build(dat_plan_t *plan)
         if (e == cudaSuccess && !items2.empty())
             e = cudaMemcpy(g->d_items2, items2.data(), items2.size() * sizeof(PipeItem), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(g->d_parts, parts.data(), parts.size() * sizeof(PipePart), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess && !pieces.empty())
+            e = cudaMemcpy(g->d_pieces, pieces.data(), pieces.size() * sizeof(PipePart), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) return dat_cuda_fail(plan, e);
     } catch (...) {
         return DAT_ERR_NOMEM;
@@ -1113,12 +1140,42 @@ static bool p_phases(const dat_plan_t *plan, bool two)
     if (plan->M == 1 && !two) return true;        // (60 million elements: 409 / 359)
     return (n <= P_PHASES_MOST * sm && (!two || plan->M >= 8)) || (double)plan->pipe->largest >= P_PHASES_SHARE * (double)plan->d;
 }
+// The resident form: one piece of 2048 elements per CTA, all CTAs on the chip at once (up to 0.9 million elements).  Phases /
+// resident in us, 30 odd layers:
+//   elements       M = 1          4            8           16          48         two-sided: M = 4     16
+//   20 thousand  18.4 / 16.5  16.5 / 16.5  18.6 / 18.6  20.7 / 20.7  35.2 / 37.2      22.7 / 20.6  25.8 / 24.7
+//   150          16.6 / 16.5  18.6 / 18.3  19.8 / 19.0  25.6 / 22.8  48.5 / 43.5      22.7 / 20.6  30.8 / 25.9
+//   300          18.2 / 16.5  19.9 / 17.5  22.7 / 19.5  29.4 / 24.8  55.8 / 49.4      24.7 / 22.8  35.4 / 28.9
+//   790          20.5 / 19.0  22.7 / 20.5  28.8 / 24.7  39.0 / 32.9  75.9 / 72.2      30.8 / 26.2  45.6 / 38.0
+// 300 thousand in 150 layers, M = 6: 25.1 / 23.0, per-worker norms 24.6 / 22.6, LAMB 24.8 / 22.7.  With several pieces per CTA it
+// loses to the phases (1 million, M = 32: 70 / 85).  b = 32, two phases without norms, gains nothing (12.4 / 12.8).
+static bool p_resident(const dat_plan_t *plan) { return plan->pipe->n_pieces > 0 && plan->bits != 32; }
+
+
 // Half a tile per CTA: in one wave, and with many workers (a long loop per CTA, so that a last wave of whole tiles costs
 // much: 2.5 million elements, 617 tiles, M = 32: 185 / 156 us; 4 million, M = 3: 51.1 / 53.5).
 static bool p_halves(const dat_plan_t *plan)
 {
     const int64_t n = plan->pipe->n_tiles, sm = plan->sm_count;
     return n <= P_PHASES_WAVE * sm || (n <= P_PHASES_MOST * sm && plan->M >= 8);
+}
+
+// A launch whose CTAs are all resident at once.  False: the device (as this process sees it) does not hold so many.
+template <class K>
+static bool p_launch_resident(K kernel, unsigned grid, cudaStream_t s, const PArgs &a)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(DAT_P_THREADS);
+    cfg.stream = s;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeCooperative;
+    attr.val.cooperative = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kernel, a) == cudaSuccess) return true;
+    (void)cudaGetLastError();
+    return false;
 }
 
 // A launch that may be set up while the one before it ends (its kernel waits for that end itself).
@@ -1217,8 +1274,31 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
     a.n_tiles = g->n_tiles;
     cudaStream_t s = (cudaStream_t)stream;
     const bool rng16 = (plan->rng_bits == 16);
-    const int form = group ? P_ONE_LAUNCH : how == P_BY_RULE ? g->form : how;
-    const bool phases = form == P_PHASES || (form == P_BY_RULE && p_phases(plan, two));
+    int form = group ? P_ONE_LAUNCH : how == P_BY_RULE ? g->form : how;
+    if (form == P_BY_RULE) form = p_resident(plan) ? P_RESIDENT : p_phases(plan, two) ? P_PHASES : P_ONE_LAUNCH;
+    if (form == P_RESIDENT) {
+        a.parts = g->d_pieces;
+        const unsigned ctas = (unsigned)g->n_pieces;
+        bool done = false;
+#define P_RES(R, MODE, TWO)                                                                                         \
+    done = lamb ? p_launch_resident(k_step_resident<R, MODE, P_OPT_LAMB, TWO>, ctas, s, a)                          \
+                : p_launch_resident(k_step_resident<R, MODE, P_OPT_MOMENTUM, TWO>, ctas, s, a)
+#define P_RES_TWO(R, MODE) do { if (two) P_RES(R, MODE, true); else P_RES(R, MODE, false); } while (0)
+        if (identity) P_RES(true, P_MODE_IDENTITY, false);
+        else if (per_worker && rng16) P_RES_TWO(true, P_MODE_PER_WORKER);
+        else if (per_worker) P_RES_TWO(false, P_MODE_PER_WORKER);
+        else if (rng16) P_RES_TWO(true, P_MODE_SHARED);
+        else P_RES_TWO(false, P_MODE_SHARED);
+#undef P_RES_TWO
+#undef P_RES
+        if (done) {
+            DAT_LAUNCHED(plan);
+            return DAT_OK;
+        }
+        a.parts = g->d_parts;                      // fewer SMs than the device has (a partition): the launch per phase
+        form = P_PHASES;
+    }
+    const bool phases = form == P_PHASES;
     const bool halves = phases && p_halves(plan);
     const unsigned grid = phases ? (unsigned)g->n_tiles * (halves ? 2u : 1u) : a.n_items;
     if (phases && !identity) {
@@ -1347,7 +1427,7 @@ extern "C" int dat_plan_test_form(dat_plan_t *plan, int form)
 {
     int rc = dat_check_plan(plan);
     if (rc != DAT_OK) return rc;
-    if (!plan->pipe || (form != P_BY_RULE && form != P_ONE_LAUNCH && form != P_PHASES)) return DAT_ERR_ARG;
+    if (!plan->pipe || form < P_BY_RULE || form > P_RESIDENT || (form == P_RESIDENT && !plan->pipe->n_pieces)) return DAT_ERR_ARG;
     plan->pipe->form = form;
     return DAT_OK;
 }
