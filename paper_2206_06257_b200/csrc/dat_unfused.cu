@@ -14,6 +14,34 @@
 #define SUMSQ_KEEP_BYTES (64ll << 20)             // of the last tiles' gradients, that stay in L2
 #define SUMSQ_JOBS 8                              // sums (of a tile and a worker) of a CTA, at most (a warp's partials: <= 32)
 
+// The separate calls follow one another on a stream: a kernel that is launched by dat_launch_after may be set up while the one
+// before it ends, and waits for that end (dat_after_previous) before it touches memory that a kernel writes.  It lets the next
+// one start only then, so a launch never overlaps with more than the launch before it -- whatever that was: after a kernel
+// that does not take part it starts when that one has ended.
+__device__ __forceinline__ void dat_after_previous()
+{
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
+}
+template <class K, class... ARGS>
+static cudaError_t dat_launch_after(K kernel, dim3 grid, cudaStream_t s, const ARGS &...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(DAT_THREADS);
+    cfg.stream = s;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    // (recorded into a graph, whose nodes before may be no kernels, a launch waits for them as any other does)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool known = cudaStreamIsCapturing(s, &cap) == cudaSuccess;
+    if (!known) (void)cudaGetLastError();
+    cfg.numAttrs = (known && cap == cudaStreamCaptureStatusNone) ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 struct NormOut {
     float S_f;
     float *worker_norms, *scales, *qmul;
@@ -426,7 +454,7 @@ k_quantize(const __grid_constant__ QuantArgs<N> all)
         dat_ld8<EV_FIRST>(ahead, true, v[0]);
         dat_ld8<EV_FIRST>(ahead + 256, true, v[1]);
     }
-    cudaGridDependencySynchronize();                         // (the norms, where k_sumsq runs just before)
+    dat_after_previous();                                    // (the norms, where k_sumsq runs just before)
     const int l0 = __ldg(a.flat_layer + e_piece / DAT_FLAT);
     const float t = quant_mul(a.qs, (a.per_worker ? (int64_t)worker * a.h : 0) + l0);
     if (whole && __ldg(a.off + l0 + 1) >= e_piece + 256 * a.groups && dat_scaled_factor(t, (float)(1u << BITS)) &&
@@ -763,6 +791,7 @@ __global__ void __launch_bounds__(DAT_THREADS, 4)
 k_aggregate(const __grid_constant__ SRC src, int M, const int64_t *__restrict__ off, const int32_t *__restrict__ flat_layer, int64_t d,
             const float *__restrict__ scales, float SM_f, bool wide, int32_t *__restrict__ code_sum, float *__restrict__ g_hat)
 {
+    dat_after_previous();
     const int64_t e0 = 16 * ((int64_t)blockIdx.x * DAT_THREADS + threadIdx.x);
     if (e0 >= d) return;
     const bool tail = BITS == 16 && e0 + 8 >= d;
@@ -780,7 +809,7 @@ k_aggregate(const __grid_constant__ SRC src, int M, const int64_t *__restrict__ 
     const int l0 = __ldg(flat_layer + piece), nl = __ldg(flat_layer + piece + 1) - l0 + 1;
     int l = l0 + ((nl > 1) ? dat_find(off + l0, nl, e0) : 0);
     int64_t l_hi = __ldg(off + l + 1);
-    float nu = __ldg(scales + l), f = (nu == 0.0f) ? 0.0f : nu / SM_f;
+    float nu = __ldcg(scales + l), f = (nu == 0.0f) ? 0.0f : nu / SM_f;
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
         const int64_t e = e0 + 8 * p;
@@ -791,7 +820,7 @@ k_aggregate(const __grid_constant__ SRC src, int M, const int64_t *__restrict__ 
             while (e + j >= l_hi && e + j < d) {
                 ++l;
                 l_hi = __ldg(off + l + 1);
-                nu = __ldg(scales + l);
+                nu = __ldcg(scales + l);
                 f = (nu == 0.0f) ? 0.0f : nu / SM_f;
             }
             out[j] = (float)sum[8 * p + j] * f;
@@ -821,6 +850,7 @@ __global__ void __launch_bounds__(DAT_THREADS)
 k_aggregate_per_worker(const __grid_constant__ SRC src, int M, const int64_t *__restrict__ off, const int32_t *__restrict__ flat_layer, int h,
                        int64_t d, const float *__restrict__ scales, float SM_f, float *__restrict__ g_hat)
 {
+    dat_after_previous();
     const int64_t e0 = 8 * ((int64_t)blockIdx.x * DAT_THREADS + threadIdx.x);
     if (e0 >= d) return;
     int lidx[8];
@@ -848,13 +878,13 @@ k_aggregate_per_worker(const __grid_constant__ SRC src, int M, const int64_t *__
         dat_unpack8<BITS>(src.lv(i), e0, lev);
         const uint32_t sg = src.sg(i)[e0 >> 3];
         const float *__restrict__ nu_i = scales + (int64_t)i * h;
-        const float nu0 = __ldg(nu_i + lidx[0]);
+        const float nu0 = __ldcg(nu_i + lidx[0]);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             // (float)level without the conversion unit: 2^23 + level is exact, the sign bit goes on afterwards
             const float mag = __uint_as_float(0x4B000000u | lev[j]) - 8388608.0f;
             const float code = __uint_as_float(__float_as_uint(mag) | (((sg >> j) & 1u) << 31));
-            const float nu = one_layer ? nu0 : __ldg(nu_i + lidx[j]);
+            const float nu = one_layer ? nu0 : __ldcg(nu_i + lidx[j]);
             acc[j] = __fmaf_rn(nu, code, acc[j]);
         }
     }
@@ -911,7 +941,8 @@ static int aggregate_launch(dat_plan_t *plan, const SRC &src, const float *scale
     if (plan->scale_mode == DAT_SCALE_PER_WORKER) {
         if (code_sum) return DAT_ERR_ARG;        // differently scaled codes have no integer sum
 #define DAT_APW(B)                                                                                                  \
-    k_aggregate_per_worker<B, SRC><<<grid, DAT_THREADS, 0, s>>>(src, plan->M, plan->d_offsets, plan->d_flat_layer, h, plan->d, scales, SM_f, g_hat)
+    DAT_CUDA(plan, dat_launch_after(k_aggregate_per_worker<B, SRC>, dim3(grid), s, src, plan->M, (const int64_t *)plan->d_offsets,       \
+                                    (const int32_t *)plan->d_flat_layer, h, plan->d, scales, SM_f, g_hat))
         switch (plan->bits) {
         case 1: DAT_APW(1); break;
         case 2: DAT_APW(2); break;
@@ -925,8 +956,8 @@ static int aggregate_launch(dat_plan_t *plan, const SRC &src, const float *scale
     }
     const unsigned grid16 = (unsigned)((plan->d + DAT_THREADS * 16 - 1) / (DAT_THREADS * 16));
 #define DAT_A(B)                                                                                                                 \
-    k_aggregate<B, SRC><<<grid16, DAT_THREADS, 0, s>>>(src, plan->M, plan->d_offsets, plan->d_flat_layer, plan->d, scales, SM_f, \
-                                                       dat_aligned32_host(g_hat), code_sum, g_hat)
+    DAT_CUDA(plan, dat_launch_after(k_aggregate<B, SRC>, dim3(grid16), s, src, plan->M, (const int64_t *)plan->d_offsets,                 \
+                                    (const int32_t *)plan->d_flat_layer, plan->d, scales, SM_f, dat_aligned32_host(g_hat), code_sum, g_hat))
     switch (plan->bits) {
     case 1: DAT_A(1); break;
     case 2: DAT_A(2); break;
@@ -1090,6 +1121,7 @@ k_update_pass1(const __grid_constant__ UpdateArgs a)
     __shared__ double scratch[DAT_THREADS / 32];
     __shared__ bool s_last;
     const int64_t tile = (int64_t)gridDim.x - 1 - blockIdx.x;
+    dat_after_previous();
     const TileRange r = dat_tile_range(a.tiles, tile);
     double ss_theta = 0.0, ss_u = 0.0;
 #pragma unroll 1
@@ -1130,8 +1162,9 @@ template <int OPT>
 __global__ void __launch_bounds__(DAT_THREADS, UPDATE_CTAS)
 k_update_pass2(const __grid_constant__ UpdateArgs a)
 {
+    dat_after_previous();
     const TileRange r = dat_tile_range(a.tiles, blockIdx.x);
-    const float na = -__ldg(a.step_a + r.layer);
+    const float na = -__ldcg(a.step_a + r.layer);        // (no __ldg: written by a kernel that this one may have been started under)
 #pragma unroll
     for (int it = 0; it < DAT_TILE / 8 / DAT_THREADS; ++it) {
         const int64_t e0 = r.begin + 8 * (int64_t)(it * DAT_THREADS + threadIdx.x);
@@ -1195,9 +1228,9 @@ extern "C" int dat_lalr_step(dat_plan_t *plan, float *theta, float *mom, const f
     UpdateArgs a = update_args(plan, theta, mom, nullptr, g_hat, hp->lr, hp->c_l, hp->c_u, layer_norms_out);
     a.mu = hp->momentum;
     a.wd = hp->weight_decay;
-    k_update_pass1<OPT_MOMENTUM><<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(a);
+    DAT_CUDA(plan, dat_launch_after(k_update_pass1<OPT_MOMENTUM>, dim3((unsigned)plan->n_tiles), s, a));
     DAT_LAUNCHED(plan);
-    k_update_pass2<OPT_MOMENTUM><<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(a);
+    DAT_CUDA(plan, dat_launch_after(k_update_pass2<OPT_MOMENTUM>, dim3((unsigned)plan->n_tiles), s, a));
     DAT_LAUNCHED(plan);
     return DAT_OK;
 }
@@ -1215,9 +1248,9 @@ extern "C" int dat_lamb_step(dat_plan_t *plan, float *theta, float *mom, float *
     cudaStream_t s = (cudaStream_t)stream;
     UpdateArgs a = update_args(plan, theta, mom, var, g_hat, hp->lr, hp->c_l, hp->c_u, layer_norms_out);
     a.lamb = dat_lamb_const(hp, t);
-    k_update_pass1<OPT_LAMB><<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(a);
+    DAT_CUDA(plan, dat_launch_after(k_update_pass1<OPT_LAMB>, dim3((unsigned)plan->n_tiles), s, a));
     DAT_LAUNCHED(plan);
-    k_update_pass2<OPT_LAMB><<<(unsigned)plan->n_tiles, DAT_THREADS, 0, s>>>(a);
+    DAT_CUDA(plan, dat_launch_after(k_update_pass2<OPT_LAMB>, dim3((unsigned)plan->n_tiles), s, a));
     DAT_LAUNCHED(plan);
     return DAT_OK;
 }
@@ -1305,7 +1338,7 @@ extern "C" int dat_lalr_step_static(int64_t num_layers, const int64_t *layer_off
     a.count = sc->count;
     a.status = &sc->status;
     k_update_pass1<OPT_MOMENTUM><<<(unsigned)nt, DAT_THREADS, 0, s>>>(a);
-    k_update_pass2<OPT_MOMENTUM><<<(unsigned)nt, DAT_THREADS, 0, s>>>(a);
+    (void)dat_launch_after(k_update_pass2<OPT_MOMENTUM>, dim3((unsigned)nt), s, a);
     if (cudaGetLastError() != cudaSuccess) return DAT_ERR_CUDA;
     return DAT_OK;
 }
