@@ -108,8 +108,15 @@ def _array_type(ctype, n):
     return ctype * n
 
 
+def _c_array(ctype, xs):
+    """xs as a C array; an array made before passes as it is."""
+    return xs if isinstance(xs, C.Array) else _array_type(ctype, len(xs))(*xs)
+
+
 def _ptr_array(xs):
-    return _array_type(C.c_void_p, len(xs))(*[_ptr(x) for x in xs])
+    if isinstance(xs, C.Array):
+        return xs
+    return _array_type(C.c_void_p, len(xs))(*[x if type(x) is int else _ptr(x) for x in xs])
 
 
 def _stream(stream):
@@ -166,7 +173,7 @@ def dat_quantize(plan, grads, seed, step, levels, signs, scales, scales_in=None,
 def dat_quantize_ranges(plans, first_layer, padded, grads, seed, step, norms, levels, signs, stream=None):
     """One entry per range in plans, first_layer, padded, levels, signs; grads: the M whole vectors."""
     n = len(plans)
-    _ok(_lib.dat_quantize_ranges(n, _ptr_array(plans), _array_type(_i64, n)(*first_layer), _array_type(C.c_int32, n)(*padded), _ptr_array(grads),
+    _ok(_lib.dat_quantize_ranges(n, _ptr_array(plans), _c_array(_i64, first_layer), _c_array(C.c_int32, padded), _ptr_array(grads),
                                  int(seed), int(step), _ptr(norms), _ptr_array(levels), _ptr_array(signs), _stream(stream)), "dat_quantize_ranges")
 
 
@@ -250,7 +257,7 @@ def dat_plan_test_stall(plan, wait_cycles, layer=-1, stream=None):
 
 
 def dat_plan_test_form(plan, form):
-    """Test hook: 1 one launch, 2 a launch per phase, 0 by the rule."""
+    """Test hook: 1 one launch, 2 a launch per phase, 3 one launch whose CTAs keep their pieces, 0 by the rule."""
     _ok(_lib.dat_plan_test_form(plan, int(form)), "dat_plan_test_form")
 
 

@@ -23,6 +23,8 @@ the CUDA library through the C ABI (dat_worker_norms, dat_quantize with caller-s
 dat_aggregate, dat_lalr_step on plans that cover one range each, with dat_plan_set_origin giving the
 range's place in the global random streams), so the result is the one the unsharded dat_step gives.
 """
+import ctypes as C
+
 import numpy as np
 import torch
 import torch.distributed as dist
@@ -63,6 +65,7 @@ class RangeLayout:
         local = offs[l0:l1 + 1] - self.a8
         self.offsets = np.concatenate([[0], local]).astype(np.int64) if self.pad else local.astype(np.int64)
         self.n = self.b - self.a8                     # elements of the sub-problem (pad included)
+        self.key = (l0, l1)
         self.h = self.offsets.size - 1
 
     def scales(self, nu):
@@ -222,15 +225,15 @@ class CudaOps:
         self.h = self.offsets.size - 1
         self.bits, self.rng_bits = bits, rng_bits
         self.plan_norms = api.dat_plan_create(self.offsets, M_loc, bits, rng_bits=rng_bits)
-        self.plans_q, self.plans_agg, self.messages = {}, {}, {}
+        self.plans_q, self.plans_agg, self.messages, self.sizes = {}, {}, {}, {}
 
     def close(self):
         for p in [self.plan_norms] + list(self.plans_q.values()) + list(self.plans_agg.values()):
             self.api.dat_plan_destroy(p)
-        self.plans_q, self.plans_agg, self.messages, self.plan_norms = {}, {}, {}, None
+        self.plans_q, self.plans_agg, self.messages, self.sizes, self.plan_norms = {}, {}, {}, {}, None
 
     def _plan(self, table, rg, workers, worker_base):
-        key = (rg.l0, rg.l1)
+        key = rg.key
         if key not in table:
             p = self.api.dat_plan_create(rg.offsets, workers, self.bits, rng_bits=self.rng_bits)
             self.api.dat_plan_set_origin(p, rg.a8, worker_base)
@@ -238,8 +241,9 @@ class CudaOps:
         return table[key]
 
     def plane_bytes(self, rg):
-        lb, sb, _, _ = self.api.dat_plan_sizes(self._plan(self.plans_agg, rg, self.M, 0))
-        return lb, sb
+        if rg.key not in self.sizes:
+            self.sizes[rg.key] = self.api.dat_plan_sizes(self._plan(self.plans_agg, rg, self.M, 0))[:2]
+        return self.sizes[rg.key]
 
     def worker_norms(self, grads_local):
         out = torch.empty(self.M_loc * self.h, dtype=torch.float32, device=grads_local[0].device)
@@ -258,7 +262,7 @@ class CudaOps:
 
     def _messages(self, ranges):
         """Plans, layer origins and plane sizes of a rank's messages to the owners of `ranges`."""
-        key = tuple((rg.l0, rg.l1) for rg in ranges)
+        key = tuple([rg.key for rg in ranges])
         if key not in self.messages:
             plans = [self._plan(self.plans_q, rg, self.M_loc, self.rank * self.M_loc) for rg in ranges]
             sizes = []
@@ -266,7 +270,9 @@ class CudaOps:
                 lb, sb, _, _ = self.api.dat_plan_sizes(p)
                 sizes += [self.M_loc * lb, self.M_loc * sb]             # (multiples of 16 bytes)
             at = np.concatenate([[0], np.cumsum(sizes)]).tolist()
-            self.messages[key] = (plans, [rg.l0 for rg in ranges], [int(rg.pad > 0) for rg in ranges], sizes, at)
+            n = len(ranges)                                             # (as C arrays: they are the same in every step)
+            self.messages[key] = ((C.c_void_p * n)(*plans), (C.c_int64 * n)(*[rg.l0 for rg in ranges]),
+                                  (C.c_int32 * n)(*[int(rg.pad > 0) for rg in ranges]), sizes, at)
         return self.messages[key]
 
     def quantize_ranges(self, ranges, grads_local, nu, seed, step, out=None):
