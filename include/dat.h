@@ -319,7 +319,7 @@ int dat_lalr_step_static(int64_t num_layers, const int64_t *layer_offsets, float
  * dat_quantize -> dat_aggregate -> dat_lalr_step (or dat_average -> dat_lalr_step when b = 32),
  * but codes, code sums and g_hat are never written to device memory.  One kernel launch
  * (dat_step_pipelined) for problems that fill the GPU, one launch per phase (dat_step_passes) up to four tiles of 4096
- * elements per SM; with b < 32 also up to nine (two-sided steps: with eight workers and more), where one layer has more than 0.27 of the elements, and (one-sided) for a
+ * elements per SM; with b < 32 also up to nine, where one layer has more than 0.27 of the elements, and (one-sided) for a
  * single worker at any size.  With b < 32 and at most three pieces of 2048 elements per SM it is one (cooperative) launch
  * whose CTAs keep a piece each through all phases and wait, bounded, for its layer.  Nothing is allocated and nothing synchronises: every table the launches
  * need was built by dat_plan_create.

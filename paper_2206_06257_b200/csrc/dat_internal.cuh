@@ -314,10 +314,10 @@ __device__ __forceinline__ void dat_fence() { asm volatile("fence.acq_rel.gpu;" 
 
 // One thread, the CTA's part of a count being complete: counts it in; returns whether it was the last of `total`
 // (what the others released before counting is then visible to this CTA's threads after their next barrier).
-__device__ __forceinline__ bool dat_count_in(uint32_t *count, uint32_t total)
+__device__ __forceinline__ bool dat_count_in(uint32_t *count, uint32_t total, uint32_t n = 1u)
 {
     dat_fence();
-    const bool last = atomicAdd(count, 1u) == total - 1u;
+    const bool last = atomicAdd(count, n) == total - n;
     if (last) dat_fence();
     return last;
 }

@@ -115,7 +115,7 @@ struct PArgs {
     int32_t *code_sum;
     long long wait_cycles;
     float S_f, SM_f, M_f, mu, wd, lr, c_l, c_u;
-    uint32_t epoch, n_items;
+    uint32_t epoch, n_items, n_whole;             // n_whole: of a phase's tiles, those that a CTA takes whole
     int M, h;
     bool wide;                                    // every bulk buffer starts on a 32-byte boundary
     int64_t d, n_tiles;
@@ -509,10 +509,11 @@ __device__ __forceinline__ void p_direction(const PArgs &a, int64_t e0, int64_t 
 // (Eq. 3, pass 1) of one tile; codes, sums and g_hat stay in registers.  Leaves the tile's two sums per
 // warp in scratch[2w], scratch[2w + 1].  TWO (Algorithm A1 Step 10 follows): stops at g_hat, which is
 // stored, and leaves the tile's sum of g_hat^2 per warp in scratch[2w]. ----------------------------
-// G: groups of eight per thread, from the tile's piece `piece` on (G = 2: the whole tile, piece 0; G = 1: half a tile).
+// G: groups of eight per thread, from the tile's piece `piece` on (G = 2: the whole tile, piece 0; G = 1: half a tile; with
+// G = 2 a call may ask for one group: half a tile too).
 // ENDS: the groups at the layer's two ends by whole warps.
 template <bool RNG16, int MODE, int OPT, bool TWO, int G, bool ENDS = (MODE != P_MODE_IDENTITY)>
-__device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt, int piece, double *scratch, float2 *s_fac)
+__device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt, int piece, double *scratch, float2 *s_fac, int groups = G)
 {
     const int M = a.M, layer = pt.layer;
     const int64_t lo = pt.lo, hi = pt.hi;
@@ -533,14 +534,14 @@ __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt,
     const int64_t begin = p_tile_begin(pt) + (int64_t)piece * (8 * DAT_P_THREADS);
     __shared__ float s_ends[ENDS ? 2 : 1][8];
     if (ENDS && !plain && begin < hi) {
-        const int64_t last = min(begin + 8 * (G * DAT_P_THREADS - 1), (hi - 1) & ~(int64_t)7);
+        const int64_t last = min(begin + 8 * (groups * DAT_P_THREADS - 1), (hi - 1) & ~(int64_t)7);
         if ((threadIdx.x >> 5) == 0 && (begin < lo || begin + 8 > hi)) p_ragged<RNG16, MODE>(a, qc, s_fac, begin, lo, hi, s_ends[0]);
         if ((threadIdx.x >> 5) == (unsigned)((last - begin) / 256) % (DAT_P_THREADS / 32) && last > begin && last + 8 > hi)
             p_ragged<RNG16, MODE>(a, qc, s_fac, last, lo, hi, s_ends[ENDS]);
         __syncwarp();                              // (read by a lane of the warp that drew it)
     }
 #pragma unroll 1
-    for (int k = 0; k < G; ++k) {
+    for (int k = 0; k < groups; ++k) {
         const int64_t e0 = begin + 8 * (int64_t)(k * DAT_P_THREADS + threadIdx.x);
         if (e0 >= hi) continue;
         const bool full = (e0 >= lo && e0 + 8 <= hi);
@@ -624,7 +625,7 @@ __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt,
 // drawn on the random stream of index M (the first one no worker uses), then m' and the layer sums as in
 // the Q part of the one-sided step. ------------------------------------------------------------------
 template <bool RNG16, int OPT, int G>
-__device__ __forceinline__ void p_part_requant(const PArgs &a, const PipePart &pt, int piece, double *scratch)
+__device__ __forceinline__ void p_part_requant(const PArgs &a, const PipePart &pt, int piece, double *scratch, int groups = G)
 {
     const int64_t lo = pt.lo, hi = pt.hi;
     const float t = __ldcg(a.qmul2 + pt.layer), f = __ldcg(a.dq2 + pt.layer);
@@ -632,7 +633,7 @@ __device__ __forceinline__ void p_part_requant(const PArgs &a, const PipePart &p
     double ss_theta = 0.0, ss_u = 0.0;
     const int64_t begin = p_tile_begin(pt) + (int64_t)piece * (8 * DAT_P_THREADS);
 #pragma unroll 1
-    for (int k = 0; k < G; ++k) {
+    for (int k = 0; k < groups; ++k) {
         const int64_t e0 = begin + 8 * (int64_t)(k * DAT_P_THREADS + threadIdx.x);
         if (e0 >= hi) continue;
         float v[8];
@@ -720,7 +721,7 @@ __device__ __forceinline__ bool p_quant_publish(const PArgs &a, const PipePart &
 
 // ---- U: theta' = theta - a_l m' (Eq. 3, pass 2) of one tile ---------------------------------------
 template <int OPT, int G>
-__device__ __forceinline__ void p_part_update(const PArgs &a, const PipePart &pt, int piece)
+__device__ __forceinline__ void p_part_update(const PArgs &a, const PipePart &pt, int piece, int groups = G)
 {
     const int64_t lo = pt.lo, hi = pt.hi;
     const float na = -__ldcg(a.step_a + pt.layer);
@@ -728,7 +729,7 @@ __device__ __forceinline__ void p_part_update(const PArgs &a, const PipePart &pt
 #pragma unroll
     for (int k = 0; k < G; ++k) {
         const int64_t e0 = begin + 8 * (int64_t)(k * DAT_P_THREADS + threadIdx.x);
-        if (e0 >= hi) continue;
+        if (e0 >= hi || k >= groups) continue;
         float th[8], m[8];
         if (OPT == P_OPT_LAMB) {
             // the direction once more from the stored moments: the same fp32 operations give the same bits
@@ -849,70 +850,102 @@ __device__ __forceinline__ PipePart p_part_of(const PArgs &a, uint32_t tile)
     reinterpret_cast<uint4 *>(&pt)[1] = __ldg(src + 1);
     return pt;
 }
-// The part as the partial sums see it: pieces of tiles, each with a slot of its own.
+// What a CTA of a phase does: `groups` halves of a tile from `piece` on.  A phase's CTAs take whole tiles as long as those
+// fill waves; the tiles of a last wave that is at most half full go by halves (a.n_whole whole ones), in half the time (see
+// p_whole).
+struct PhaseShare {
+    PipePart pt, slot;                             // the tile; the first half as the partial sums see it, a slot per half tile
+    int piece, groups;
+};
 template <int G>
-__device__ __forceinline__ PipePart p_piece_of(const PipePart &pt, int piece)
+__device__ __forceinline__ PhaseShare p_share(const PArgs &a, uint32_t cta, bool back)
 {
-    constexpr int PIECES = DAT_P_GROUPS / G;
-    PipePart x = pt;
-    x.tb *= PIECES;
-    x.T *= PIECES;
-    x.tile = x.tile * PIECES + piece;
+    uint32_t tile, half = 0;
+    int groups = G;
+    if (G == 1) {
+        tile = cta / 2;
+        half = cta & 1;
+    } else if (cta < a.n_whole) {
+        tile = cta;
+    } else {
+        tile = a.n_whole + (cta - a.n_whole) / 2;
+        half = (cta - a.n_whole) & 1;
+        groups = 1;
+    }
+    if (back) tile = (uint32_t)a.n_tiles - 1u - tile;
+    PhaseShare x;
+    x.pt = p_part_of(a, tile);
+    x.slot = x.pt;
+    x.slot.tb *= 2;
+    x.slot.T *= 2;
+    x.slot.tile = 2 * x.slot.tile + (int)half;
+    x.piece = (int)half;
+    x.groups = groups;
     return x;
 }
+// One thread: the share's sums (of a whole tile in its first half's slot, 0 in the other), counted in by halves.  Returns
+// whether it was the layer's last.
+template <bool TWO>
+__device__ __forceinline__ bool p_share_publish(const PArgs &a, const PhaseShare &x, const double *scratch)
+{
+    const int64_t slot = (int64_t)x.slot.tb + x.slot.tile;
+    if (TWO) {
+        a.partR[slot] = p_warps_sum(scratch);
+        if (x.groups == 2) a.partR[slot + 1] = 0.0;
+    } else {
+        p_quant_sums(a, slot, scratch);
+        if (x.groups == 2) a.partQ[2 * slot + 2] = a.partQ[2 * slot + 3] = 0.0;
+    }
+    return dat_count_in((TWO ? a.cntR : a.cntQ) + x.pt.layer, (uint32_t)x.slot.T, (uint32_t)x.groups);
+}
 
-// G = 2: a tile per CTA.  G = 1: half a tile (see p_halves): twice the CTAs, and four workers' loads in flight
+// G = 2: whole tiles (see p_share).  G = 1: half a tile (see p_halves): twice the CTAs, and four workers' loads in flight
 // per thread, which then has the registers (300 thousand elements, M = 64: 166 us with G = 2, 121 with G = 1).
 template <bool RNG16, int MODE, int OPT, bool TWO, int G>
 __global__ void __launch_bounds__(DAT_P_THREADS, G == 1 ? 3 : DAT_P_MINB)
 k_phase_quant(const __grid_constant__ PArgs a)
 {
-    constexpr int PIECES = DAT_P_GROUPS / G;
     __shared__ double s_red[2 * (DAT_P_THREADS / 32)];
     __shared__ float2 s_fac[MODE == P_MODE_PER_WORKER ? DAT_MAX_WORKERS : 1];
     __shared__ bool s_last;
-    const uint32_t cta = gridDim.x - 1u - blockIdx.x;
-    const PipePart pt = p_part_of(a, cta / PIECES), pp = p_piece_of<G>(pt, cta % PIECES);
+    const PhaseShare x = p_share<G>(a, blockIdx.x, true);
     cudaTriggerProgrammaticLaunchCompletion();
     cudaGridDependencySynchronize();
-    if (!P_CHECK(a, p_part_valid(a, pt))) return;
-    p_part_quant<RNG16, MODE, OPT, TWO, G>(a, pt, cta % PIECES, s_red, s_fac);
+    if (!P_CHECK(a, p_part_valid(a, x.pt))) return;
+    p_part_quant<RNG16, MODE, OPT, TWO, G>(a, x.pt, x.piece, s_red, s_fac, x.groups);
     __syncthreads();
-    if (threadIdx.x == 0) s_last = TWO ? p_server_publish(a, pp, s_red) : p_quant_publish(a, pp, s_red);
+    if (threadIdx.x == 0) s_last = p_share_publish<TWO>(a, x, s_red);
     __syncthreads();
     if (!s_last) return;
-    if (TWO) p_server_finish(a, pp, s_red);
-    else p_quant_finish(a, pp, s_red);
+    if (TWO) p_server_finish(a, x.slot, s_red);
+    else p_quant_finish(a, x.slot, s_red);
 }
 
 template <bool RNG16, int OPT, int G>
 __global__ void __launch_bounds__(DAT_P_THREADS, DAT_P_MINB)
 k_phase_requant(const __grid_constant__ PArgs a)
 {
-    constexpr int PIECES = DAT_P_GROUPS / G;
     __shared__ double s_red[2 * (DAT_P_THREADS / 32)];
     __shared__ bool s_last;
-    const PipePart pt = p_part_of(a, blockIdx.x / PIECES), pp = p_piece_of<G>(pt, blockIdx.x % PIECES);
+    const PhaseShare x = p_share<G>(a, blockIdx.x, false);
     cudaTriggerProgrammaticLaunchCompletion();
     cudaGridDependencySynchronize();
-    if (!P_CHECK(a, p_part_valid(a, pt))) return;
-    p_part_requant<RNG16, OPT, G>(a, pt, blockIdx.x % PIECES, s_red);
+    if (!P_CHECK(a, p_part_valid(a, x.pt))) return;
+    p_part_requant<RNG16, OPT, G>(a, x.pt, x.piece, s_red, x.groups);
     __syncthreads();
-    if (threadIdx.x == 0) s_last = p_quant_publish(a, pp, s_red);
+    if (threadIdx.x == 0) s_last = p_share_publish<false>(a, x, s_red);
     __syncthreads();
-    if (s_last) p_quant_finish(a, pp, s_red);
+    if (s_last) p_quant_finish(a, x.slot, s_red);
 }
 
 template <int OPT, bool BACK, int G>
 __global__ void __launch_bounds__(DAT_P_THREADS, DAT_P_MINB)
 k_phase_update(const __grid_constant__ PArgs a)
 {
-    constexpr int PIECES = DAT_P_GROUPS / G;
-    const uint32_t cta = BACK ? gridDim.x - 1u - blockIdx.x : blockIdx.x;
-    const PipePart pt = p_part_of(a, cta / PIECES);
+    const PhaseShare x = p_share<G>(a, blockIdx.x, BACK);
     cudaGridDependencySynchronize();
-    if (!P_CHECK(a, p_part_valid(a, pt))) return;
-    p_part_update<OPT, G>(a, pt, cta % PIECES);
+    if (!P_CHECK(a, p_part_valid(a, x.pt))) return;
+    p_part_update<OPT, G>(a, x.pt, x.piece, x.groups);
 }
 
 #include "dat_resident.cuh"
@@ -1126,8 +1159,8 @@ cudaError_t dat_pipe_reset(dat_plan_t *plan, cudaStream_t s)
 // The largest 0.17: 24 million 162 / 152, 178 / 177, 233 / 235, 284 / 288, 337 / 345, 593 / 577; 48 million 315 / 288 to
 // 686 / 672.  0.21 (ResNet-18): M = 1, 6, 16: 72 / 76, 123 / 139, 242 / 276.  0.09 (ResNet-50): M = 1, 2, 8: 146 / 152,
 // 161 / 178, 309 / 358.  Two-sided, 0.33: 3.6 million, M = 1 to 16, 49 / 46, 52 / 52, 65 / 62, 78 / 72, 90 / 87, 143 / 126, 5.2 million
-// 60 / 59 to 111 / 116, 8 to 16 million 87 / 80 to 470 / 429; ResNet-18, M = 6, 145 / 166; 3 million, M = 3, the
-// largest 0.23: 63.5 / 65.6.
+// 62 / 58, 67 / 66, 85 / 80, 103 / 94 (M = 1, 2, 4, 6), 111 / 116 (M = 8), 8 to 16 million 87 / 80 to 470 / 429; ResNet-18, M = 6, 145 / 166; 3 million, M = 3, the
+// largest 0.23: 63.4 / 61.6.
 // b = 32 (no norms): 1 million, M = 8, 22 / 18, 2.2 million, M = 1 to 8, 17 to 25 / 19 to 25, M = 8: 2.8 million 28 / 34, 16 million 153 / 159.
 #define P_PHASES_WAVE 4                           // tiles per SM: one wave of a phase's CTAs
 #define P_PHASES_MOST 9
@@ -1138,7 +1171,7 @@ static bool p_phases(const dat_plan_t *plan, bool two)
     if (n <= P_PHASES_WAVE * sm) return true;
     if (plan->bits == 32) return false;
     if (plan->M == 1 && !two) return true;        // (60 million elements: 409 / 359)
-    return (n <= P_PHASES_MOST * sm && (!two || plan->M >= 8)) || (double)plan->pipe->largest >= P_PHASES_SHARE * (double)plan->d;
+    return n <= P_PHASES_MOST * sm || (double)plan->pipe->largest >= P_PHASES_SHARE * (double)plan->d;
 }
 // The resident form: one piece of 2048 elements per CTA, all CTAs on the chip at once (up to 0.9 million elements).  Phases /
 // resident in us, 30 odd layers:
@@ -1158,6 +1191,15 @@ static bool p_halves(const dat_plan_t *plan)
 {
     const int64_t n = plan->pipe->n_tiles, sm = plan->sm_count;
     return n <= P_PHASES_WAVE * sm || (n <= P_PHASES_MOST * sm && plan->M >= 8);
+}
+
+// The tiles that a phase's CTAs take whole, where not all go by halves: full waves of them, if the rest fits half a wave.
+// All whole / the rest by halves, in us, 592 CTAs a wave: 2.5 million elements in 40 odd layers, M = 1, 4, 6: 29.8 / 29.0, 41.0 / 39.8,
+// 47.6 / 45.8, LAMB 47.5 / 43.2, 54.9 / 50.8, 61.9 / 56.5, two-sided 39.6 / 38.9, 51.8 / 49.5, 58.3 / 56.0; 5.2 million, LAMB, M = 4, 86.5 / 83.4.
+static uint32_t p_whole(const dat_plan_t *plan)
+{
+    const int64_t n = plan->pipe->n_tiles, wave = DAT_P_MINB * (int64_t)plan->sm_count, rest = n % wave;
+    return (uint32_t)(2 * rest <= wave ? n - rest : n);
 }
 
 // A launch whose CTAs are all resident at once.  False: the device (as this process sees it) does not hold so many.
@@ -1300,7 +1342,8 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
     }
     const bool phases = form == P_PHASES;
     const bool halves = phases && p_halves(plan);
-    const unsigned grid = phases ? (unsigned)g->n_tiles * (halves ? 2u : 1u) : a.n_items;
+    a.n_whole = phases && !halves ? p_whole(plan) : 0u;
+    const unsigned grid = phases ? 2u * (unsigned)g->n_tiles - a.n_whole : a.n_items;
     if (phases && !identity) {
         rc = dat_norm_phase(plan, a.gp, a.scales_out, s);
         if (rc != DAT_OK) return rc;
