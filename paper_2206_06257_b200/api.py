@@ -108,13 +108,14 @@ def _array_type(ctype, n):
     return ctype * n
 
 
-def _c_array(ctype, xs):
-    """xs as a C array; an array made before passes as it is."""
-    return xs if isinstance(xs, C.Array) else _array_type(ctype, len(xs))(*xs)
+def _c_array(ctype, n, xs):
+    """xs as a C array of n; one made before, of just this type and length, passes as it is."""
+    t = _array_type(ctype, n)
+    return xs if type(xs) is t else t(*xs)
 
 
 def _ptr_array(xs):
-    if isinstance(xs, C.Array):
+    if isinstance(xs, C.Array) and xs._type_ is C.c_void_p:
         return xs
     return _array_type(C.c_void_p, len(xs))(*[x if type(x) is int else _ptr(x) for x in xs])
 
@@ -173,7 +174,7 @@ def dat_quantize(plan, grads, seed, step, levels, signs, scales, scales_in=None,
 def dat_quantize_ranges(plans, first_layer, padded, grads, seed, step, norms, levels, signs, stream=None):
     """One entry per range in plans, first_layer, padded, levels, signs; grads: the M whole vectors."""
     n = len(plans)
-    _ok(_lib.dat_quantize_ranges(n, _ptr_array(plans), _c_array(_i64, first_layer), _c_array(C.c_int32, padded), _ptr_array(grads),
+    _ok(_lib.dat_quantize_ranges(n, _ptr_array(plans), _c_array(_i64, n, first_layer), _c_array(C.c_int32, n, padded), _ptr_array(grads),
                                  int(seed), int(step), _ptr(norms), _ptr_array(levels), _ptr_array(signs), _stream(stream)), "dat_quantize_ranges")
 
 
