@@ -80,7 +80,7 @@ struct PipeSchedule {
     PipeItem *d_items = nullptr;                  // the three streams N, Q, U
     int64_t n_items = 0;
     PipePart *d_parts = nullptr;                  // n_tiles: every tile once, in slot order (the phases)
-    PipePart *d_pieces = nullptr;                 // the half tiles that hold elements, numbered as such (tb, T, tile); small problems only
+    PipePart *d_pieces = nullptr;                 // the half tiles that hold elements, numbered as such (tb, T, tile); small problems with b < 32 only
     int64_t n_pieces = 0;
     PipeItem *d_items2 = nullptr;                 // the four streams N, Q, R, U of the two-sided step
     int64_t n_items2 = 0;
@@ -1056,7 +1056,7 @@ int dat_pipe_build(dat_plan_t *plan)
                 parts.push_back(PipePart{plan->offsets[l], plan->offsets[l + 1], (int32_t)tb[l], (int32_t)(tb[l + 1] - tb[l]), l, (int32_t)t});
         const size_t o_parts = take(parts.size() * sizeof(PipePart));
         std::vector<PipePart> pieces;
-        if (nt <= (int64_t)R_CTAS * plan->sm_count) {
+        if (!identity && nt <= (int64_t)R_CTAS * plan->sm_count) {
             pieces.reserve((size_t)(2 * nt));
             for (int l = 0; l < h; ++l) {
                 const int64_t lo = plan->offsets[l], hi = plan->offsets[l + 1], n = (hi - (lo & ~(int64_t)7) + R_PIECE - 1) / R_PIECE;
@@ -1182,8 +1182,7 @@ static bool p_phases(const dat_plan_t *plan, bool two)
 //   790          20.5 / 19.0  22.7 / 20.5  28.8 / 24.7  39.0 / 32.9  75.9 / 72.2      30.8 / 26.2  45.6 / 38.0
 // 300 thousand in 150 layers, M = 6: 25.1 / 23.0, per-worker norms 24.6 / 22.6, LAMB 24.8 / 22.7.  With several pieces per CTA it
 // loses to the phases (1 million, M = 32: 70 / 85).  b = 32, two phases without norms, gains nothing (12.4 / 12.8).
-static bool p_resident(const dat_plan_t *plan) { return plan->pipe->n_pieces > 0 && plan->bits != 32; }
-
+static bool p_resident(const dat_plan_t *plan) { return plan->pipe->n_pieces > 0; }
 
 // Half a tile per CTA: in one wave, and with many workers (a long loop per CTA, so that a last wave of whole tiles costs
 // much: 2.5 million elements, 617 tiles, M = 32: 185 / 156 us; 4 million, M = 3: 51.1 / 53.5).
@@ -1326,8 +1325,7 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
     done = lamb ? p_launch_resident(k_step_resident<R, MODE, P_OPT_LAMB, TWO>, ctas, s, a)                          \
                 : p_launch_resident(k_step_resident<R, MODE, P_OPT_MOMENTUM, TWO>, ctas, s, a)
 #define P_RES_TWO(R, MODE) do { if (two) P_RES(R, MODE, true); else P_RES(R, MODE, false); } while (0)
-        if (identity) P_RES(true, P_MODE_IDENTITY, false);
-        else if (per_worker && rng16) P_RES_TWO(true, P_MODE_PER_WORKER);
+        if (per_worker && rng16) P_RES_TWO(true, P_MODE_PER_WORKER);
         else if (per_worker) P_RES_TWO(false, P_MODE_PER_WORKER);
         else if (rng16) P_RES_TWO(true, P_MODE_SHARED);
         else P_RES_TWO(false, P_MODE_SHARED);

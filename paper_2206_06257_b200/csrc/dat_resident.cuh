@@ -91,22 +91,20 @@ k_step_resident(const __grid_constant__ PArgs a)
         return s_go;
     };
 
-    if (MODE != P_MODE_IDENTITY) {
-        if (e0 < pc.hi) {                          // what the next phase reads beside the gradients
-            asm volatile("prefetch.global.L2 [%0];" :: "l"(a.theta + e0));
-            asm volatile("prefetch.global.L2 [%0];" :: "l"(a.mom + e0));
-            if (OPT == P_OPT_LAMB) asm volatile("prefetch.global.L2 [%0];" :: "l"(a.var + e0));
-        }
-        for (int u = threadIdx.x; u < 2 * M; u += DAT_P_THREADS) s_unit[u] = 0.0;
-        __syncthreads();
-        r_norm_sums(a, pc, begin, s_unit);
-        __syncthreads();
-        if (warp == 0) {
-            for (int i = threadIdx.x; i < M; i += 32) a.partN[slot * M + i] = s_unit[2 * i] + s_unit[2 * i + 1];
-            __syncwarp();
-        }
-        if (!phase_end(a.cntN, a.readyN, [&] { p_norm_finish<MODE>(a, pc, s_norm); })) return;
+    if (e0 < pc.hi) {                          // what the next phase reads beside the gradients
+        asm volatile("prefetch.global.L2 [%0];" :: "l"(a.theta + e0));
+        asm volatile("prefetch.global.L2 [%0];" :: "l"(a.mom + e0));
+        if (OPT == P_OPT_LAMB) asm volatile("prefetch.global.L2 [%0];" :: "l"(a.var + e0));
     }
+    for (int u = threadIdx.x; u < 2 * M; u += DAT_P_THREADS) s_unit[u] = 0.0;
+    __syncthreads();
+    r_norm_sums(a, pc, begin, s_unit);
+    __syncthreads();
+    if (warp == 0) {
+        for (int i = threadIdx.x; i < M; i += 32) a.partN[slot * M + i] = s_unit[2 * i] + s_unit[2 * i + 1];
+        __syncwarp();
+    }
+    if (!phase_end(a.cntN, a.readyN, [&] { p_norm_finish<MODE>(a, pc, s_norm); })) return;
     p_part_quant<RNG16, MODE, OPT, TWO, 1>(a, pt, half, s_red, s_fac);
     __syncthreads();
     if (TWO) {

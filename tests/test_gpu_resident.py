@@ -16,14 +16,15 @@ RESIDENT, PHASES = 3, 2
 def resident(api, monkeypatch):  # noqa: F811
     create = api.dat_plan_create
 
-    def create_with_form(*args, **kw):
-        plan = create(*args, **kw)
-        api.dat_plan_test_form(plan, RESIDENT)
+    def create_with_form(offs, M, bits, **kw):
+        plan = create(offs, M, bits, **kw)
+        if bits != 32:                               # (the form is for steps with norms)
+            api.dat_plan_test_form(plan, RESIDENT)
         return plan
     monkeypatch.setattr(api, "dat_plan_create", create_with_form)
 
 
-@pytest.mark.parametrize("bits", [1, 8, 16, 32])
+@pytest.mark.parametrize("bits", [1, 8, 16])
 def test_ragged(api, oracle, resident, bits, rng_bits):  # noqa: F811
     parity.test_fused_parity_ragged(api, oracle, bits, rng_bits)
 
@@ -38,7 +39,7 @@ def test_extreme_scales(api, oracle, resident, bits, rng_bits):  # noqa: F811
     parity.test_fused_parity_extreme_scales(api, oracle, bits, rng_bits)
 
 
-@pytest.mark.parametrize("mode", ["shared", "per_worker", "b32"])
+@pytest.mark.parametrize("mode", ["shared", "per_worker"])
 def test_lamb(api, oracle, resident, mode):  # noqa: F811
     parity.test_step_lamb_parity_three_steps(api, oracle, mode)
 
@@ -109,9 +110,10 @@ def test_up_to_the_most_pieces_equals_the_phases(api, pieces, kind):  # noqa: F8
             assert_close_per_layer(b[k], a[k], offs, name)
 
 
-def test_a_larger_problem_has_no_resident_form(api):  # noqa: F811
+@pytest.mark.parametrize("bits", [8, 32])
+def test_a_larger_problem_and_one_without_norms_have_no_resident_form(api, bits):  # noqa: F811
     n = 3 * torch.cuda.get_device_properties(0).multi_processor_count
-    with GpuPlan(api, np.array([0, 2048 * n + 1], dtype=np.int64), 2, 8) as P:
+    with GpuPlan(api, np.array([0, 2048 * n + 1 if bits != 32 else 31], dtype=np.int64), 2, bits) as P:
         with pytest.raises(api.DatError) as e:
             api.dat_plan_test_form(P.plan, RESIDENT)
         assert e.value.code == api.DAT_ERR_ARG
