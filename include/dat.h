@@ -320,7 +320,7 @@ int dat_lalr_step_static(int64_t num_layers, const int64_t *layer_offsets, float
  * but codes, code sums and g_hat are never written to device memory.  One kernel launch
  * (dat_step_pipelined) for problems that fill the GPU, one launch per phase (dat_step_passes) up to four tiles of 4096
  * elements per SM; with b < 32 also up to nine, where one layer has more than 0.27 of the elements, and (one-sided) for a
- * single worker at any size.  With b < 32 and at most three pieces of 2048 elements per SM it is one (cooperative) launch
+ * single worker at any size.  With b < 32 and at most three pieces of 2048 elements per SM it is one launch
  * whose CTAs keep a piece each through all phases and wait, bounded, for its layer.  Nothing is allocated and nothing synchronises: every table the launches
  * need was built by dat_plan_create.
  *   theta, mom        device fp32[d], updated in place.
@@ -330,8 +330,10 @@ int dat_lalr_step_static(int64_t num_layers, const int64_t *layer_offsets, float
  *   code_sum_out      device int32[d] or NULL (checking aid; ignored when b = 32).
  *   layer_norms_out   device fp32[2h] or NULL.
  *   scales_out        device fp32[h] or NULL: nu_l (not written when b = 32).
- * Inside the launch a work item may have to wait for a layer's norm that another item is still
- * producing; that wait is bounded (about two seconds).  If it ever runs out, the call returns as
+ * Inside the one launch a work item may have to wait for a layer's norm that another item is still
+ * producing (and in the form whose CTAs keep their pieces, a piece for its layer); that wait is bounded (about two
+ * seconds).  It is only ever for CTAs that run: kernels of other streams that hold SMs for longer delay a step, and do
+ * not make it give up.  If a wait ever runs out, the call returns as
  * usual, DAT_STATUS_TIMEOUT is set in the status word, and the outputs of that call -- and of
  * later calls on the plan -- are undefined until dat_get_status has been called, which reports the
  * bit and restores the plan's counters.
@@ -413,7 +415,8 @@ int dat_plan_test_stall(dat_plan_t *plan, int64_t wait_cycles, int64_t layer, vo
 
 /* dat_plan_test_form -- TEST HOOK: the form of the plan's dat_step, dat_step_lamb and two-sided steps whatever their size:
  * 1 the one launch, 2 a launch per phase, 3 one launch whose CTAs keep their pieces (ARG where b = 32 or the problem has more
- * than three pieces of 2048 elements per SM), 0 by the rule again.  Nothing else uses this.  Errors: ARG. */
+ * than three pieces of 2048 elements per SM), 4 the same with a CTA per layer, which takes the layer's other pieces as
+ * running CTAs do where the others cannot start, 0 by the rule again.  Nothing else uses this.  Errors: ARG. */
 int dat_plan_test_form(dat_plan_t *plan, int form);
 
 /* dat_step_host -- dat_step for callers whose data lives in HOST memory: copies theta, mom and

@@ -258,7 +258,7 @@ def dat_plan_test_stall(plan, wait_cycles, layer=-1, stream=None):
 
 
 def dat_plan_test_form(plan, form):
-    """Test hook: 1 one launch, 2 a launch per phase, 3 one launch whose CTAs keep their pieces, 0 by the rule."""
+    """Test hook: 1 one launch, 2 a launch per phase, 3 one launch whose CTAs keep their pieces, 4 the same with a CTA per layer, 0 by the rule."""
     _ok(_lib.dat_plan_test_form(plan, int(form)), "dat_plan_test_form")
 
 

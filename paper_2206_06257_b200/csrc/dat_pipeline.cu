@@ -55,7 +55,8 @@
 #endif
 #define DAT_P_WAIT_CYCLES (4000000000ll)          // about two seconds
 
-enum { P_BY_RULE = 0, P_ONE_LAUNCH = 1, P_PHASES = 2, P_RESIDENT = 3 };     // which form a step takes (see p_resident, p_phases)
+// which form a step takes (see p_resident, p_phases); the last one for tests: the resident form as if most of its CTAs were late
+enum { P_BY_RULE = 0, P_ONE_LAUNCH = 1, P_PHASES = 2, P_RESIDENT = 3, P_RESIDENT_LATE = 4 };
 enum { P_MODE_SHARED = 0, P_MODE_PER_WORKER = 1, P_MODE_IDENTITY = 2 };
 enum { P_OPT_MOMENTUM = 0, P_OPT_LAMB = 1 };     // the descent direction u of Eq. 3: heavy-ball momentum, or Algorithm A2
 
@@ -80,7 +81,8 @@ struct PipeSchedule {
     PipeItem *d_items = nullptr;                  // the three streams N, Q, U
     int64_t n_items = 0;
     PipePart *d_parts = nullptr;                  // n_tiles: every tile once, in slot order (the phases)
-    PipePart *d_pieces = nullptr;                 // the half tiles that hold elements, numbered as such (tb, T, tile); small problems with b < 32 only
+    PipePart *d_pieces = nullptr;                 // the half tiles that hold elements, numbered as such (tb, T, tile), then each layer's
+                                                  // first once more; small problems with b < 32 only
     int64_t n_pieces = 0;
     PipeItem *d_items2 = nullptr;                 // the four streams N, Q, R, U of the two-sided step
     int64_t n_items2 = 0;
@@ -88,7 +90,8 @@ struct PipeSchedule {
     float *d_server = nullptr;                    // 2h: S / nu^_l and nu^_l / S
     double *d_partN = nullptr;                    // n_tiles * M (with pieces twice that)
     double *d_partQ = nullptr;                    // 2 per half tile
-    uint32_t *d_sync = nullptr;                   // [0] ticket, [1] abort epoch, then cntN[h], cntQ[h], readyN[h], readyQ[h], cntR[h], readyR[h]
+    uint32_t *d_sync = nullptr;                   // [0] ticket, [1] abort epoch, then cntN[h], cntQ[h], readyN[h], readyQ[h], cntR[h], readyR[h] and
+                                                  // claim[n_pieces], the epoch of the call in which a piece was last taken
     size_t sync_bytes = 0;
     int64_t n_tiles = 0, largest = 0;             // elements of the largest layer
     std::vector<int64_t> tile_base;               // h + 1
@@ -108,7 +111,7 @@ struct PArgs {
     float *theta, *mom, *var;                     // var: second moment (LAMB only)
     LambConst lamb;
     double *partN, *partQ, *partR;
-    uint32_t *ticket, *abort_epoch, *cntN, *cntQ, *readyN, *readyQ, *cntR, *readyR, *status;
+    uint32_t *ticket, *abort_epoch, *cntN, *cntQ, *readyN, *readyQ, *cntR, *readyR, *claim, *status;
     float *worker_norms, *scales, *qmul, *dq, *step_a;
     float *ghat, *qmul2, *dq2;                    // two-sided: g_hat / the receiver's value (d), the server's factors (h each)
     float *norms_out, *scales_out, *server_scales_out;
@@ -1056,20 +1059,25 @@ int dat_pipe_build(dat_plan_t *plan)
                 parts.push_back(PipePart{plan->offsets[l], plan->offsets[l + 1], (int32_t)tb[l], (int32_t)(tb[l + 1] - tb[l]), l, (int32_t)t});
         const size_t o_parts = take(parts.size() * sizeof(PipePart));
         std::vector<PipePart> pieces;
-        if (!identity && nt <= (int64_t)R_CTAS * plan->sm_count) {
-            pieces.reserve((size_t)(2 * nt));
+        const int64_t most = std::min<int64_t>(R_MOST, (int64_t)R_CTAS * plan->sm_count);
+        if (!identity && nt <= most) {
+            pieces.reserve((size_t)(2 * nt + h));
             for (int l = 0; l < h; ++l) {
                 const int64_t lo = plan->offsets[l], hi = plan->offsets[l + 1], n = (hi - (lo & ~(int64_t)7) + R_PIECE - 1) / R_PIECE;
                 const int32_t first = (int32_t)pieces.size();
                 for (int64_t t = 0; t < n; ++t) pieces.push_back(PipePart{lo, hi, first, (int32_t)n, l, (int32_t)t});
             }
         }
-        if ((int64_t)pieces.size() > (int64_t)R_CTAS * plan->sm_count) pieces.clear();
+        if ((int64_t)pieces.size() > most) pieces.clear();
         g->n_pieces = (int64_t)pieces.size();
+        for (int64_t k = 0; k < g->n_pieces; ++k) {
+            const PipePart piece = pieces[(size_t)k];
+            if (piece.tile == 0) pieces.push_back(piece);
+        }
         const size_t o_pieces = take(pieces.size() * sizeof(PipePart));
         const size_t o_pn = take((size_t)nt * (size_t)M * (pieces.empty() ? 8 : 16)), o_pq = take((size_t)nt * 32), o_pr = take((size_t)nt * 16);
         const size_t o_server = take(2 * (size_t)h * 4);
-        g->sync_bytes = (2 + 6 * (size_t)h) * 4;
+        g->sync_bytes = (2 + 6 * (size_t)h + (size_t)g->n_pieces) * 4;
         const size_t o_sync = take(g->sync_bytes);
         g->mem_bytes = off;
         cudaError_t e;
@@ -1201,24 +1209,6 @@ static uint32_t p_whole(const dat_plan_t *plan)
     return (uint32_t)(2 * rest <= wave ? n - rest : n);
 }
 
-// A launch whose CTAs are all resident at once.  False: the device (as this process sees it) does not hold so many.
-template <class K>
-static bool p_launch_resident(K kernel, unsigned grid, cudaStream_t s, const PArgs &a)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(DAT_P_THREADS);
-    cfg.stream = s;
-    cudaLaunchAttribute attr = {};
-    attr.id = cudaLaunchAttributeCooperative;
-    attr.val.cooperative = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, kernel, a) == cudaSuccess) return true;
-    (void)cudaGetLastError();
-    return false;
-}
-
 // A launch that may be set up while the one before it ends (its kernel waits for that end itself).
 template <class K>
 static cudaError_t p_launch_after(K kernel, unsigned grid, cudaStream_t s, const PArgs &a)
@@ -1284,6 +1274,7 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
     a.readyQ = a.readyN + h;
     a.cntR = a.readyQ + h;
     a.readyR = a.cntR + h;
+    a.claim = a.readyR + h;
     a.ghat = g_hat;
     a.qmul2 = g->d_server;
     a.dq2 = g->d_server + h;
@@ -1317,26 +1308,24 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
     const bool rng16 = (plan->rng_bits == 16);
     int form = group ? P_ONE_LAUNCH : how == P_BY_RULE ? g->form : how;
     if (form == P_BY_RULE) form = p_resident(plan) ? P_RESIDENT : p_phases(plan, two) ? P_PHASES : P_ONE_LAUNCH;
-    if (form == P_RESIDENT) {
-        a.parts = g->d_pieces;
-        const unsigned ctas = (unsigned)g->n_pieces;
-        bool done = false;
-#define P_RES(R, MODE, TWO)                                                                                         \
-    done = lamb ? p_launch_resident(k_step_resident<R, MODE, P_OPT_LAMB, TWO>, ctas, s, a)                          \
-                : p_launch_resident(k_step_resident<R, MODE, P_OPT_MOMENTUM, TWO>, ctas, s, a)
-#define P_RES_TWO(R, MODE) do { if (two) P_RES(R, MODE, true); else P_RES(R, MODE, false); } while (0)
-        if (per_worker && rng16) P_RES_TWO(true, P_MODE_PER_WORKER);
-        else if (per_worker) P_RES_TWO(false, P_MODE_PER_WORKER);
-        else if (rng16) P_RES_TWO(true, P_MODE_SHARED);
-        else P_RES_TWO(false, P_MODE_SHARED);
-#undef P_RES_TWO
+    if (form == P_RESIDENT || form == P_RESIDENT_LATE) {
+        a.parts = form == P_RESIDENT ? g->d_pieces : g->d_pieces + g->n_pieces;
+        const unsigned ctas = form == P_RESIDENT ? (unsigned)g->n_pieces : (unsigned)plan->h;
+#define P_RES(R, MODE, OPT, TWO) k_step_resident<R, MODE, OPT, TWO><<<ctas, DAT_P_THREADS, 0, s>>>(a)
+#define P_RES_OPT(R, MODE)                                                                                          \
+    do {                                                                                                            \
+        if (two) { if (lamb) P_RES(R, MODE, P_OPT_LAMB, true); else P_RES(R, MODE, P_OPT_MOMENTUM, true); }         \
+        else if (lamb) P_RES(R, MODE, P_OPT_LAMB, false);                                                           \
+        else P_RES(R, MODE, P_OPT_MOMENTUM, false);                                                                 \
+    } while (0)
+        if (per_worker && rng16) P_RES_OPT(true, P_MODE_PER_WORKER);
+        else if (per_worker) P_RES_OPT(false, P_MODE_PER_WORKER);
+        else if (rng16) P_RES_OPT(true, P_MODE_SHARED);
+        else P_RES_OPT(false, P_MODE_SHARED);
+#undef P_RES_OPT
 #undef P_RES
-        if (done) {
-            DAT_LAUNCHED(plan);
-            return DAT_OK;
-        }
-        a.parts = g->d_parts;                      // fewer SMs than the device has (a partition): the launch per phase
-        form = P_PHASES;
+        DAT_LAUNCHED(plan);
+        return DAT_OK;
     }
     const bool phases = form == P_PHASES;
     const bool halves = phases && p_halves(plan);
@@ -1468,7 +1457,7 @@ extern "C" int dat_plan_test_form(dat_plan_t *plan, int form)
 {
     int rc = dat_check_plan(plan);
     if (rc != DAT_OK) return rc;
-    if (!plan->pipe || form < P_BY_RULE || form > P_RESIDENT || (form == P_RESIDENT && !plan->pipe->n_pieces)) return DAT_ERR_ARG;
+    if (!plan->pipe || form < P_BY_RULE || form > P_RESIDENT_LATE || (form >= P_RESIDENT && !plan->pipe->n_pieces)) return DAT_ERR_ARG;
     plan->pipe->form = form;
     return DAT_OK;
 }
@@ -1481,7 +1470,7 @@ extern "C" int dat_plan_test_stall(dat_plan_t *plan, int64_t wait_cycles, int64_
     PipeSchedule *g = plan->pipe;
     if (!g || !g->mem || wait_cycles < 0 || layer >= plan->h) return DAT_ERR_ARG;
     g->wait_cycles = wait_cycles ? (long long)wait_cycles : DAT_P_WAIT_CYCLES;
-    g->form = (wait_cycles || layer >= 0) ? P_ONE_LAUNCH : P_BY_RULE;        // only the one launch waits
+    g->form = (wait_cycles || layer >= 0) ? P_ONE_LAUNCH : P_BY_RULE;        // (the phases, which the rule may choose, do not wait)
     if (layer >= 0) {
         // a count that the layer's tiles cannot bring to T - 1: nobody becomes the layer's last tile
         static const uint32_t far = 0x40000000u;
