@@ -789,7 +789,7 @@ __device__ __forceinline__ void agg_add4(const AggWords<BITS> w[4], int sum[16])
 template <int BITS, class SRC>
 __global__ void __launch_bounds__(DAT_THREADS, 4)
 k_aggregate(const __grid_constant__ SRC src, int M, const int64_t *__restrict__ off, const int32_t *__restrict__ flat_layer, int64_t d,
-            const float *__restrict__ scales, float SM_f, bool wide, int32_t *__restrict__ code_sum, float *__restrict__ g_hat)
+            const float *scales, float SM_f, bool wide, int32_t *__restrict__ code_sum, float *__restrict__ g_hat)
 {
     dat_after_previous();
     const int64_t e0 = 16 * ((int64_t)blockIdx.x * DAT_THREADS + threadIdx.x);
@@ -809,7 +809,7 @@ k_aggregate(const __grid_constant__ SRC src, int M, const int64_t *__restrict__ 
     const int l0 = __ldg(flat_layer + piece), nl = __ldg(flat_layer + piece + 1) - l0 + 1;
     int l = l0 + ((nl > 1) ? dat_find(off + l0, nl, e0) : 0);
     int64_t l_hi = __ldg(off + l + 1);
-    float nu = __ldcg(scales + l), f = (nu == 0.0f) ? 0.0f : nu / SM_f;
+    float nu = scales[l], f = (nu == 0.0f) ? 0.0f : nu / SM_f;
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
         const int64_t e = e0 + 8 * p;
@@ -820,7 +820,7 @@ k_aggregate(const __grid_constant__ SRC src, int M, const int64_t *__restrict__ 
             while (e + j >= l_hi && e + j < d) {
                 ++l;
                 l_hi = __ldg(off + l + 1);
-                nu = __ldcg(scales + l);
+                nu = scales[l];
                 f = (nu == 0.0f) ? 0.0f : nu / SM_f;
             }
             out[j] = (float)sum[8 * p + j] * f;
@@ -844,14 +844,18 @@ k_aggregate(const __grid_constant__ SRC src, int M, const int64_t *__restrict__ 
 
 // The same with one norm per worker (Eq. grad_agg as written): no integer sum exists;
 // g_hat = (sum_i nu_{i,l} * signed level_i) / (S*M), accumulated in fp32 with one fused
-// multiply-add per worker, in ascending worker order.
+// multiply-add per worker, in ascending worker order.  The norms are read by plain loads: not by __ldg, for a kernel that this
+// one may have been started under writes them, and not past L1 (500 thousand elements, M = 40, b = 8: 60 us; 13 with plain loads
+// of one norm per worker, four workers at a time, where a warp lies in one layer).  Six CTAs per SM: with few workers a thread
+// has little in flight (60 million elements, b = 4, M = 1: 185 us with four, 163 with five, 148; M = 16: 419, 415, 418).
 template <int BITS, class SRC>
-__global__ void __launch_bounds__(DAT_THREADS)
+__global__ void __launch_bounds__(DAT_THREADS, 6)
 k_aggregate_per_worker(const __grid_constant__ SRC src, int M, const int64_t *__restrict__ off, const int32_t *__restrict__ flat_layer, int h,
-                       int64_t d, const float *__restrict__ scales, float SM_f, float *__restrict__ g_hat)
+                       int64_t d, const float *scales, float SM_f, float *__restrict__ g_hat)
 {
     dat_after_previous();
     const int64_t e0 = 8 * ((int64_t)blockIdx.x * DAT_THREADS + threadIdx.x);
+    const unsigned live = __ballot_sync(0xFFFFFFFFu, e0 < d);
     if (e0 >= d) return;
     int lidx[8];
     {
@@ -868,24 +872,35 @@ k_aggregate_per_worker(const __grid_constant__ SRC src, int M, const int64_t *__
             lidx[j] = l;
         }
     }
-    const bool one_layer = (lidx[0] == lidx[7]);
     float acc[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) acc[j] = 0.0f;
-#pragma unroll 1
-    for (int i = 0; i < M; ++i) {
+    auto add = [&](int i, auto &&nu) {
         uint32_t lev[8];
         dat_unpack8<BITS>(src.lv(i), e0, lev);
         const uint32_t sg = src.sg(i)[e0 >> 3];
-        const float *__restrict__ nu_i = scales + (int64_t)i * h;
-        const float nu0 = __ldcg(nu_i + lidx[0]);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             // (float)level without the conversion unit: 2^23 + level is exact, the sign bit goes on afterwards
             const float mag = __uint_as_float(0x4B000000u | lev[j]) - 8388608.0f;
             const float code = __uint_as_float(__float_as_uint(mag) | (((sg >> j) & 1u) << 31));
-            const float nu = one_layer ? nu0 : __ldcg(nu_i + lidx[j]);
-            acc[j] = __fmaf_rn(nu, code, acc[j]);
+            acc[j] = __fmaf_rn(nu(j), code, acc[j]);
+        }
+    };
+    // (one way for the whole warp: as two ways, a warp at a layer's end goes through the workers twice)
+    if (!__any_sync(live, lidx[0] != lidx[7])) {
+#pragma unroll 4
+        for (int i = 0; i < M; ++i) {
+            const float nu = scales[(int64_t)i * h + lidx[0]];
+            add(i, [&](int) { return nu; });
+        }
+    } else {
+#pragma unroll 1
+        for (int i = 0; i < M; ++i) {
+            float nu[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) nu[j] = scales[(int64_t)i * h + lidx[j]];
+            add(i, [&](int j) { return nu[j]; });
         }
     }
     float out[8];
