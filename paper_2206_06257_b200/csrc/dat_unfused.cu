@@ -454,7 +454,10 @@ k_quantize(const __grid_constant__ QuantArgs<N> all)
         dat_ld8<EV_FIRST>(ahead, true, v[0]);
         dat_ld8<EV_FIRST>(ahead + 256, true, v[1]);
     }
-    dat_after_previous();                                    // (the norms, where k_sumsq runs just before)
+    // (the norms, where k_sumsq runs just before.  The next launch may not start under this one: its CTAs would take the
+    // places of the last ones here -- dat_quantize of 20 thousand elements, M = 16: 16.1 us instead of 15.0; dat_quantize,
+    // dat_aggregate and dat_lalr_step of 500 thousand, M = 40, b = 8: 73.8 instead of 70.9)
+    cudaGridDependencySynchronize();
     const int l0 = __ldg(a.flat_layer + e_piece / DAT_FLAT);
     const float t = quant_mul(a.qs, (a.per_worker ? (int64_t)worker * a.h : 0) + l0);
     if (whole && __ldg(a.off + l0 + 1) >= e_piece + 256 * a.groups && dat_scaled_factor(t, (float)(1u << BITS)) &&
