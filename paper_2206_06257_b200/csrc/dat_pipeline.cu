@@ -514,7 +514,10 @@ __device__ __forceinline__ void p_direction(const PArgs &a, int64_t e0, int64_t 
 // stored, and leaves the tile's sum of g_hat^2 per warp in scratch[2w]. ----------------------------
 // G: groups of eight per thread, from the tile's piece `piece` on (G = 2: the whole tile, piece 0; G = 1: half a tile; with
 // G = 2 a call may ask for one group: half a tile too).
-// ENDS: the groups at the layer's two ends by whole warps.
+// ENDS: the groups at the layer's two ends by whole warps, with P_ENDS_FROM workers and more: one or two are drawn sooner by the
+// group's own lane than handed out (own lane / warp, by phases: 1.5 million elements in 300 layers, M = 1, 26.1 / 27.2 us,
+// M = 2, 30.8 / 32.6, M = 3, 34.5 / 34.9, M = 4, 39.3 / 38.1, M = 5, 43.9 / 41.3).
+#define P_ENDS_FROM 3
 template <bool RNG16, int MODE, int OPT, bool TWO, int G, bool ENDS = (MODE != P_MODE_IDENTITY)>
 __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt, int piece, double *scratch, float2 *s_fac, int groups = G)
 {
@@ -536,7 +539,8 @@ __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt,
     double ss_theta = 0.0, ss_u = 0.0;
     const int64_t begin = p_tile_begin(pt) + (int64_t)piece * (8 * DAT_P_THREADS);
     __shared__ float s_ends[ENDS ? 2 : 1][8];
-    if (ENDS && !plain && begin < hi) {
+    const bool ends = ENDS && !plain && M >= P_ENDS_FROM;
+    if (ends && begin < hi) {
         const int64_t last = min(begin + 8 * (groups * DAT_P_THREADS - 1), (hi - 1) & ~(int64_t)7);
         if ((threadIdx.x >> 5) == 0 && (begin < lo || begin + 8 > hi)) p_ragged<RNG16, MODE>(a, qc, s_fac, begin, lo, hi, s_ends[0]);
         if ((threadIdx.x >> 5) == (unsigned)((last - begin) / 256) % (DAT_P_THREADS / 32) && last > begin && last + 8 > hi)
@@ -559,7 +563,7 @@ __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt,
 #pragma unroll
                 for (int j = 0; j < 8; ++j) acc[j] += v[j];
             }
-        } else if (ENDS && !full && !plain) {
+        } else if (ends && !full) {
 #pragma unroll
             for (int j = 0; j < 8; ++j) acc[j] = s_ends[e0 != begin][j];
         } else if (MODE == P_MODE_PER_WORKER) p_rows_per_worker<RNG16, G == 1 ? 4 : 1>(a, qc, s_fac, full && !plain, e0, lo, hi, acc);

@@ -1,5 +1,5 @@
 """GPU: groups of eight at a layer's ends, which a warp draws together with a worker per lane, at the worker counts around one
-and two rounds of lanes, against the oracle's integers (given the GPU's norm bits: code sums and m' bit for bit)."""
+and two rounds of lanes (with one and two workers by the group's own lane), against the oracle's integers (given the GPU's norm bits: code sums and m' bit for bit)."""
 import numpy as np
 import pytest
 import torch
@@ -14,7 +14,7 @@ SIZES = [3, 8, 13, 2049, 5, 4095, 1, 8191]       # ends in one group, in two, on
 
 @pytest.mark.parametrize("form", [1, 2])
 @pytest.mark.parametrize("mode", ["shared", "per_worker"])
-@pytest.mark.parametrize("M", [1, 31, 32, 33, 64])
+@pytest.mark.parametrize("M", [1, 2, 3, 31, 32, 33, 64])
 def test_ragged_groups(api, oracle, M, mode, form, rng_bits):  # noqa: F811
     sm = oracle.SCALE_PER_WORKER if mode == "per_worker" else oracle.SCALE_SHARED_MAX
     offs, grads, theta, mom = _random_problem(300 + M, SIZES, M)
