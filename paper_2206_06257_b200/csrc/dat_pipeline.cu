@@ -364,13 +364,27 @@ __device__ __forceinline__ void p_norm_finish(const PArgs &a, const PipePart &pt
 
 // ---- the layer's step length from the partial sums of theta^2 and m'^2 (Eq. 3), by the CTA that counted
 // in the layer's last Q tile (every thread) ----------------------------------------------------------
+// U: sums in flight per thread and quantity (the order of the additions is the same).
+template <int U = 1>
 __device__ __forceinline__ void p_quant_finish(const PArgs &a, const PipePart &pt, double *scratch)
 {
     const int layer = pt.layer;
     const int64_t tb = pt.tb;
     const uint32_t T = (uint32_t)pt.T;
     double x = 0.0, y = 0.0;
-    for (uint32_t t = threadIdx.x; t < T; t += DAT_P_THREADS) {
+    uint32_t t = threadIdx.x;
+    if (U > 1)
+        for (; t + (U - 1) * DAT_P_THREADS < T; t += U * DAT_P_THREADS) {
+            double vx[U], vy[U];
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                vx[k] = __ldcg(a.partQ + 2 * (tb + t + k * DAT_P_THREADS));
+                vy[k] = __ldcg(a.partQ + 2 * (tb + t + k * DAT_P_THREADS) + 1);
+            }
+#pragma unroll
+            for (int k = 0; k < U; ++k) { x += vx[k]; y += vy[k]; }
+        }
+    for (; t < T; t += DAT_P_THREADS) {
         x += __ldcg(a.partQ + 2 * (tb + t));
         y += __ldcg(a.partQ + 2 * (tb + t) + 1);
     }
@@ -693,13 +707,23 @@ __device__ __forceinline__ bool p_server_publish(const PArgs &a, const PipePart 
 
 // The CTA that counted in the layer's last Q tile of a two-sided step (every thread): the server's norm
 // nu^_l = ||g_hat_l||_2 from the tiles' sums in index order, and its two factors, published with the epoch.
+template <int U = 1>
 __device__ __forceinline__ void p_server_finish(const PArgs &a, const PipePart &pt, double *scratch)
 {
     const int layer = pt.layer;
     const int64_t tb = pt.tb;
     const uint32_t T = (uint32_t)pt.T;
     double x = 0.0;
-    for (uint32_t t = threadIdx.x; t < T; t += DAT_P_THREADS) x += __ldcg(a.partR + tb + t);
+    uint32_t t = threadIdx.x;
+    if (U > 1)
+        for (; t + (U - 1) * DAT_P_THREADS < T; t += U * DAT_P_THREADS) {
+            double v[U];
+#pragma unroll
+            for (int k = 0; k < U; ++k) v[k] = __ldcg(a.partR + tb + t + k * DAT_P_THREADS);
+#pragma unroll
+            for (int k = 0; k < U; ++k) x += v[k];
+        }
+    for (; t < T; t += DAT_P_THREADS) x += __ldcg(a.partR + tb + t);
     x = dat_warp_sum(x);
     __syncthreads();
     if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = x;
@@ -906,6 +930,10 @@ __device__ __forceinline__ bool p_share_publish(const PArgs &a, const PhaseShare
     return dat_count_in((TWO ? a.cntR : a.cntQ) + x.pt.layer, (uint32_t)x.slot.T, (uint32_t)x.groups);
 }
 
+// A phase ends with the largest layer's last CTA, which adds a slot per half tile: eight in flight per thread (60 million
+// elements in one layer, M = 1: 395 -> 387 us, two-sided 550 -> 531).
+#define P_FINISH 8
+
 // G = 2: whole tiles (see p_share).  G = 1: half a tile (see p_halves): twice the CTAs, and four workers' loads in flight
 // per thread, which then has the registers (300 thousand elements, M = 64: 166 us with G = 2, 121 with G = 1).
 template <bool RNG16, int MODE, int OPT, bool TWO, int G>
@@ -924,8 +952,8 @@ k_phase_quant(const __grid_constant__ PArgs a)
     if (threadIdx.x == 0) s_last = p_share_publish<TWO>(a, x, s_red);
     __syncthreads();
     if (!s_last) return;
-    if (TWO) p_server_finish(a, x.slot, s_red);
-    else p_quant_finish(a, x.slot, s_red);
+    if (TWO) p_server_finish<P_FINISH>(a, x.slot, s_red);
+    else p_quant_finish<P_FINISH>(a, x.slot, s_red);
 }
 
 template <bool RNG16, int OPT, int G>
@@ -942,7 +970,7 @@ k_phase_requant(const __grid_constant__ PArgs a)
     __syncthreads();
     if (threadIdx.x == 0) s_last = p_share_publish<false>(a, x, s_red);
     __syncthreads();
-    if (s_last) p_quant_finish(a, x.slot, s_red);
+    if (s_last) p_quant_finish<P_FINISH>(a, x.slot, s_red);
 }
 
 template <int OPT, bool BACK, int G>
