@@ -530,7 +530,8 @@ __device__ __forceinline__ void p_direction(const PArgs &a, int64_t e0, int64_t 
 // G = 2 a call may ask for one group: half a tile too).
 // ENDS: the groups at the layer's two ends by whole warps, with P_ENDS_FROM workers and more: one or two are drawn sooner by the
 // group's own lane than handed out (own lane / warp, by phases: 1.5 million elements in 300 layers, M = 1, 26.1 / 27.2 us,
-// M = 2, 30.8 / 32.6, M = 3, 34.5 / 34.9, M = 4, 39.3 / 38.1, M = 5, 43.9 / 41.3).
+// M = 2, 30.8 / 32.6, M = 3, 34.5 / 34.9, M = 4, 39.3 / 38.1, M = 5, 43.9 / 41.3); with whole tiles by a kernel without the warps'
+// code, which has 64 registers (16 million elements, M = 1, 108.3 / 106.7 us, two-sided 149.6 / 147.0, M = 2, 168.3 / 165.3).
 #define P_ENDS_FROM 3
 template <bool RNG16, int MODE, int OPT, bool TWO, int G, bool ENDS = (MODE != P_MODE_IDENTITY)>
 __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt, int piece, double *scratch, float2 *s_fac, int groups = G)
@@ -553,7 +554,7 @@ __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt,
     double ss_theta = 0.0, ss_u = 0.0;
     const int64_t begin = p_tile_begin(pt) + (int64_t)piece * (8 * DAT_P_THREADS);
     __shared__ float s_ends[ENDS ? 2 : 1][8];
-    const bool ends = ENDS && !plain && M >= P_ENDS_FROM;
+    const bool ends = ENDS && !plain && (G == 2 || M >= P_ENDS_FROM);        // (G = 2: a kernel of its own without them)
     if (ends && begin < hi) {
         const int64_t last = min(begin + 8 * (groups * DAT_P_THREADS - 1), (hi - 1) & ~(int64_t)7);
         if ((threadIdx.x >> 5) == 0 && (begin < lo || begin + 8 > hi)) p_ragged<RNG16, MODE>(a, qc, s_fac, begin, lo, hi, s_ends[0]);
@@ -936,7 +937,7 @@ __device__ __forceinline__ bool p_share_publish(const PArgs &a, const PhaseShare
 
 // G = 2: whole tiles (see p_share).  G = 1: half a tile (see p_halves): twice the CTAs, and four workers' loads in flight
 // per thread, which then has the registers (300 thousand elements, M = 64: 166 us with G = 2, 121 with G = 1).
-template <bool RNG16, int MODE, int OPT, bool TWO, int G>
+template <bool RNG16, int MODE, int OPT, bool TWO, int G, bool ENDS>
 __global__ void __launch_bounds__(DAT_P_THREADS, G == 1 ? 3 : DAT_P_MINB)
 k_phase_quant(const __grid_constant__ PArgs a)
 {
@@ -947,7 +948,7 @@ k_phase_quant(const __grid_constant__ PArgs a)
     cudaTriggerProgrammaticLaunchCompletion();
     cudaGridDependencySynchronize();
     if (!P_CHECK(a, p_part_valid(a, x.pt))) return;
-    p_part_quant<RNG16, MODE, OPT, TWO, G>(a, x.pt, x.piece, s_red, s_fac, x.groups);
+    p_part_quant<RNG16, MODE, OPT, TWO, G, ENDS>(a, x.pt, x.piece, s_red, s_fac, x.groups);
     __syncthreads();
     if (threadIdx.x == 0) s_last = p_share_publish<TWO>(a, x, s_red);
     __syncthreads();
@@ -1367,10 +1368,10 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
         rc = dat_norm_phase(plan, a.gp, a.scales_out, s);
         if (rc != DAT_OK) return rc;
     }
-#define P_PHASES_GO(R, MODE, OPT, TWO, G)                                                                           \
+#define P_PHASES_GO(R, MODE, OPT, TWO, G, ENDS)                                                                     \
     do {                                                                                                            \
-        if (MODE == P_MODE_IDENTITY) k_phase_quant<R, MODE, OPT, TWO, G><<<grid, DAT_P_THREADS, 0, s>>>(a);         \
-        else DAT_CUDA(plan, p_launch_after(k_phase_quant<R, MODE, OPT, TWO, G>, grid, s, a));                       \
+        if (MODE == P_MODE_IDENTITY) k_phase_quant<R, MODE, OPT, TWO, G, ENDS><<<grid, DAT_P_THREADS, 0, s>>>(a);   \
+        else DAT_CUDA(plan, p_launch_after(k_phase_quant<R, MODE, OPT, TWO, G, ENDS>, grid, s, a));                 \
         DAT_LAUNCHED(plan);                                                                                         \
         if (TWO) {                                                                                                  \
             DAT_CUDA(plan, p_launch_after(k_phase_requant<R, OPT, G>, grid, s, a));                                 \
@@ -1381,8 +1382,9 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
 #define P_GO(R, MODE, OPT, TWO)                                                                                     \
     do {                                                                                                            \
         if (!phases) k_step_pipelined<R, MODE, OPT, TWO><<<grid, DAT_P_THREADS, 0, s>>>(a);                         \
-        else if (halves) P_PHASES_GO(R, MODE, OPT, TWO, 1);                                                         \
-        else P_PHASES_GO(R, MODE, OPT, TWO, 2);                                                                     \
+        else if (halves) P_PHASES_GO(R, MODE, OPT, TWO, 1, MODE != P_MODE_IDENTITY);                                \
+        else if (plan->M >= P_ENDS_FROM) P_PHASES_GO(R, MODE, OPT, TWO, 2, MODE != P_MODE_IDENTITY);                \
+        else P_PHASES_GO(R, MODE, OPT, TWO, 2, false);                                                              \
     } while (0)
 #define P_GO_OPT(R, MODE)                                                                                           \
     do {                                                                                                            \
