@@ -931,9 +931,10 @@ __device__ __forceinline__ bool p_share_publish(const PArgs &a, const PhaseShare
     return dat_count_in((TWO ? a.cntR : a.cntQ) + x.pt.layer, (uint32_t)x.slot.T, (uint32_t)x.groups);
 }
 
-// A phase ends with the largest layer's last CTA, which adds a slot per half tile: eight in flight per thread (60 million
-// elements in one layer, M = 1: 395 -> 387 us, two-sided 550 -> 531).
-#define P_FINISH 8
+// A phase ends with the largest layer's last CTA, which adds a slot per half tile: four in flight per thread (60 million
+// elements in one layer, M = 1: 395 -> 387 us, two-sided 550 -> 531; eight are no better there, and 8 million, one layer half of
+// them, two-sided, M = 4, take 116.1 instead of 113.6).
+#define P_FINISH 4
 
 // G = 2: whole tiles (see p_share).  G = 1: half a tile (see p_halves): twice the CTAs, and four workers' loads in flight
 // per thread, which then has the registers (300 thousand elements, M = 64: 166 us with G = 2, 121 with G = 1).
@@ -1187,42 +1188,45 @@ cudaError_t dat_pipe_reset(dat_plan_t *plan, cudaStream_t s)
     return cudaMemsetAsync(g->d_sync, 0, g->sync_bytes, s);
 }
 
-// Which form a step takes.  The one launch keeps its streams 256 and 512 items apart, so a small problem runs through waves
-// of nearly empty CTAs; the phases have a launch's set-up and last wave each.  And the streams of the largest layer, which
-// come last, overlap with nothing: a model that is one third one layer does better by phases at every size.  Both forms of
-// the momentum step, b = 8, in us (one launch / phases; 50 to 60 odd layers, the largest 0.33 of the elements):
-//   elements, tiles per SM    M = 1        2          4          6           8           16          32
-//   2.2 million, 3.8      29 / 31    33 / 34    43 / 41    53 / 46     63 / 52    106 / 74    190 / 119
-//   3.6 million, 6.1      37 / 35    41 / 39    54 / 49    67 / 58     79 / 72    132 / 110   239 / 174
-//   5.2 million, 8.8      48 / 45    53 / 51    68 / 64    83 / 79     99 / 98    166 / 147   305 / 240
-//   8.0 million, 13.5     69 / 60    75 / 69   100 / 89   119 / 109   139 / 130   231 / 207   422 / 367
-//   16 million, 26.7     124 / 108  137 / 125  178 / 164  218 / 198   258 / 237   438 / 391   803 / 706
-// The largest 0.17: 24 million 162 / 152, 178 / 177, 233 / 235, 284 / 288, 337 / 345, 593 / 577; 48 million 315 / 288 to
-// 686 / 672.  0.21 (ResNet-18): M = 1, 6, 16: 72 / 76, 123 / 139, 242 / 276.  0.09 (ResNet-50): M = 1, 2, 8: 146 / 152,
-// 161 / 178, 309 / 358.  Two-sided, 0.33: 3.6 million, M = 1 to 16, 49 / 46, 52 / 52, 65 / 62, 78 / 72, 90 / 87, 143 / 126, 5.2 million
-// 62 / 58, 67 / 66, 85 / 80, 103 / 94 (M = 1, 2, 4, 6), 111 / 116 (M = 8), 8 to 16 million 87 / 80 to 470 / 429; ResNet-18, M = 6, 145 / 166; 3 million, M = 3, the
-// largest 0.23: 63.4 / 61.6.
-// b = 32 (no norms): 1 million, M = 8, 22 / 18, 2.2 million, M = 1 to 8, 17 to 25 / 19 to 25, M = 8: 2.8 million 28 / 34, 16 million 153 / 159.
+// Which form a step takes (both sides measured over sizes, shares and workers; the figures here are us of the momentum step,
+// b = 8, where nothing else is said).
+//
+// The one launch keeps its streams 256 and 512 items apart, so a small problem runs through waves of nearly empty CTAs; the
+// phases have a launch's set-up and last wave each.  And the streams of the largest layer, which come last, overlap with
+// nothing: where one layer has a good part of the elements the phases win at every measured size (one launch / phases; the
+// largest 0.28 of 10 million elements, M = 2, 94 / 83, M = 8, 178 / 158, of 30 million 232 / 216, 463 / 433; LAMB two-sided,
+// M = 3, 163 / 156, 430 / 419; 0.3 of 100 million 737 / 695, 1463 / 1447; a smaller share than 0.27 may gain too, but ResNet-18,
+// 0.21, M = 6, 123 / 139, and ResNet-50, 0.09, M = 8, 309 / 358, do not).  Two-sided momentum steps of more than 24 tiles per SM
+// have less to gain below 16 workers: the largest 0.28 of 30 million, M = 4, 359 / 365, 0.33: 360 / 370, 0.4: 375 / 371.
+// One worker: by phases (60 million elements: 409 / 359), but two-sided momentum steps of more than 14 tiles per SM only where
+// a layer is large (30 million, the largest 0.06: 235 / 256, 0.15: 247 / 257, 0.2: 256 / 259; LAMB 330 / 335, 342 / 337, 351 / 337).
+// b = 32 has no norms: 1 million, M = 8, 22 / 18, but 2.8 million 28 / 34, 16 million 153 / 159.
 #define P_PHASES_WAVE 4                           // tiles per SM: one wave of a phase's CTAs
 #define P_PHASES_MOST 9
 #define P_PHASES_SHARE 0.27                       // of the elements, in the largest layer
-static bool p_phases(const dat_plan_t *plan, bool two)
+#define P_TWO_LARGE 24                            // tiles per SM
+#define P_TWO_SHARE 0.38
+#define P_TWO_LARGE_1 14                          // with one worker
+#define P_TWO_SHARE_1 0.16
+static bool p_phases(const dat_plan_t *plan, bool two, bool lamb)
 {
     const int64_t n = plan->pipe->n_tiles, sm = plan->sm_count;
     if (n <= P_PHASES_WAVE * sm) return true;
     if (plan->bits == 32) return false;
-    if (plan->M == 1 && !two) return true;        // (60 million elements: 409 / 359)
-    return n <= P_PHASES_MOST * sm || (double)plan->pipe->largest >= P_PHASES_SHARE * (double)plan->d;
+    if (n <= P_PHASES_MOST * sm) return true;
+    const double share = (double)plan->pipe->largest / (double)plan->d;
+    const bool two_large = two && !lamb && n > (plan->M == 1 ? P_TWO_LARGE_1 : P_TWO_LARGE) * sm;
+    if (plan->M == 1) return !two_large || share >= P_TWO_SHARE_1;
+    return share >= (two_large && plan->M < 16 ? P_TWO_SHARE : P_PHASES_SHARE);
 }
-// The resident form: one piece of 2048 elements per CTA, all CTAs on the chip at once (up to 0.9 million elements).  Phases /
-// resident in us, 30 odd layers:
-//   elements       M = 1          4            8           16          48         two-sided: M = 4     16
-//   20 thousand  18.4 / 16.5  16.5 / 16.5  18.6 / 18.6  20.7 / 20.7  35.2 / 37.2      22.7 / 20.6  25.8 / 24.7
-//   150          16.6 / 16.5  18.6 / 18.3  19.8 / 19.0  25.6 / 22.8  48.5 / 43.5      22.7 / 20.6  30.8 / 25.9
-//   300          18.2 / 16.5  19.9 / 17.5  22.7 / 19.5  29.4 / 24.8  55.8 / 49.4      24.7 / 22.8  35.4 / 28.9
-//   790          20.5 / 19.0  22.7 / 20.5  28.8 / 24.7  39.0 / 32.9  75.9 / 72.2      30.8 / 26.2  45.6 / 38.0
-// 300 thousand in 150 layers, M = 6: 25.1 / 23.0, per-worker norms 24.6 / 22.6, LAMB 24.8 / 22.7.  With several pieces per CTA it
-// loses to the phases (1 million, M = 32: 70 / 85).  b = 32, two phases without norms, gains nothing (12.4 / 12.8).
+
+// The resident form: one piece of 2048 elements per CTA, up to 0.9 million elements.  Phases / resident in us, 40 odd layers:
+//   elements       M = 1          4            8           16          64         two-sided: M = 4     16
+//   20 thousand  16.4 / 16.4  18.5 / 16.7  18.5 / 18.5  21.6 / 22.6  47.2 / 47.3      22.8 / 21.0  26.6 / 26.7
+//   150          16.4 / 16.4  18.5 / 17.1  20.5 / 18.5  26.9 / 22.6  62.1 / 51.5      23.6 / 21.7  31.8 / 26.8
+//   300          16.4 / 17.8  18.5 / 18.8  22.1 / 20.2  29.8 / 24.7  70.6 / 63.0      23.9 / 23.3  35.2 / 29.9
+//   850          20.4 / 20.6  24.6 / 21.1  29.3 / 23.7  39.2 / 33.0  95.1 / 94.7      30.8 / 26.8  47.1 / 39.5
+// With several pieces per CTA it loses to the phases (1 million, M = 32: 70 / 85).  b = 32, two phases without norms, gains nothing.
 static bool p_resident(const dat_plan_t *plan) { return plan->pipe->n_pieces > 0; }
 
 // Half a tile per CTA: in one wave, and with many workers (a long loop per CTA, so that a last wave of whole tiles costs
@@ -1340,7 +1344,7 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
     cudaStream_t s = (cudaStream_t)stream;
     const bool rng16 = (plan->rng_bits == 16);
     int form = group ? P_ONE_LAUNCH : how == P_BY_RULE ? g->form : how;
-    if (form == P_BY_RULE) form = p_resident(plan) ? P_RESIDENT : p_phases(plan, two) ? P_PHASES : P_ONE_LAUNCH;
+    if (form == P_BY_RULE) form = p_resident(plan) ? P_RESIDENT : p_phases(plan, two, lamb != nullptr) ? P_PHASES : P_ONE_LAUNCH;
     if (form == P_RESIDENT || form == P_RESIDENT_LATE) {
         a.parts = form == P_RESIDENT ? g->d_pieces : g->d_pieces + g->n_pieces;
         const unsigned ctas = form == P_RESIDENT ? (unsigned)g->n_pieces : (unsigned)plan->h;
