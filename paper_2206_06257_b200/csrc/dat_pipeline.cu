@@ -1227,7 +1227,23 @@ static bool p_phases(const dat_plan_t *plan, bool two, bool lamb)
 //   300          16.4 / 17.8  18.5 / 18.8  22.1 / 20.2  29.8 / 24.7  70.6 / 63.0      23.9 / 23.3  35.2 / 29.9
 //   850          20.4 / 20.6  24.6 / 21.1  29.3 / 23.7  39.2 / 33.0  95.1 / 94.7      30.8 / 26.8  47.1 / 39.5
 // With several pieces per CTA it loses to the phases (1 million, M = 32: 70 / 85).  b = 32, two phases without norms, gains nothing.
-static bool p_resident(const dat_plan_t *plan) { return plan->pipe->n_pieces > 0; }
+//
+// Not where a few CTAs would read many workers' gradients one after the other, which the phases' norms spread over the chip (20
+// thousand elements in one layer, M = 16, 17.4 / 18.5, M = 64, 30.9 / 41.2; two-sided M = 64, 35.3 / 45.3, but M = 16, 22.5 / 20.6
+// at 5 thousand); nor with so many workers on nearly all places (850 thousand in one layer, M = 64: 92.7 / 99.4); nor where one
+// or two workers have hardly anything to read and most pieces end a layer (150 layers, 20 to 300 thousand elements, M = 1, 16.4 /
+// 18.5 to 16.6 / 20.3, LAMB 20.5 / 22.1 to 21.3 / 22.7, two-sided 21.8 / 23.5 to 22.6 / 24.9); nor for the momentum step of two
+// workers on up to half of the chip (150 thousand in 40 layers 16.4 / 17.3, 300 thousand 16.6 / 17.9).
+static bool p_resident(const dat_plan_t *plan, bool two, bool lamb)
+{
+    const int64_t n = plan->pipe->n_pieces;
+    const int M = plan->M;
+    if (n == 0) return false;
+    if (M >= (two ? 32 : 16) && n <= 48) return false;
+    if (M >= 48 && n > 400) return false;
+    if (M <= 2 && n >= 100 && n <= 2 * plan->h) return false;
+    return !(M == 2 && !two && !lamb && n > 48 && n < 250);
+}
 
 // Half a tile per CTA: in one wave, and with many workers (a long loop per CTA, so that a last wave of whole tiles costs
 // much: 2.5 million elements, 617 tiles, M = 32: 185 / 156 us; 4 million, M = 3: 51.1 / 53.5).
@@ -1344,7 +1360,7 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
     cudaStream_t s = (cudaStream_t)stream;
     const bool rng16 = (plan->rng_bits == 16);
     int form = group ? P_ONE_LAUNCH : how == P_BY_RULE ? g->form : how;
-    if (form == P_BY_RULE) form = p_resident(plan) ? P_RESIDENT : p_phases(plan, two, lamb != nullptr) ? P_PHASES : P_ONE_LAUNCH;
+    if (form == P_BY_RULE) form = p_resident(plan, two, lamb != nullptr) ? P_RESIDENT : p_phases(plan, two, lamb != nullptr) ? P_PHASES : P_ONE_LAUNCH;
     if (form == P_RESIDENT || form == P_RESIDENT_LATE) {
         a.parts = form == P_RESIDENT ? g->d_pieces : g->d_pieces + g->n_pieces;
         const unsigned ctas = form == P_RESIDENT ? (unsigned)g->n_pieces : (unsigned)plan->h;

@@ -39,3 +39,16 @@ def test_large_layers_and_few_workers(api, kind, M, tiles, share, launches):  # 
     n = tiles * torch.cuda.get_device_properties(0).multi_processor_count - 40
     big, rest = int(4096 * n * share), 4096 * n - int(4096 * n * share)
     assert _launches(api, [rest // 25 + 8 * (k % 3) for k in range(25)] + [big], M, kind) == launches
+
+
+@pytest.mark.parametrize("kind,M,layers,pieces,launches", [
+    ("step", 16, 1, 48, 3), ("step", 16, 1, 49, 1), ("step", 15, 1, 48, 1), ("lamb", 16, 3, 48, 3), ("two", 16, 1, 48, 1), ("two", 32, 1, 48, 4),
+    ("two", 32, 1, 49, 1), ("step", 48, 2, 400, 1), ("step", 48, 2, 401, 3), ("step", 47, 2, 401, 1), ("step", 1, 50, 99, 1), ("step", 1, 50, 100, 3),
+    ("step", 1, 50, 101, 1), ("lamb_two", 2, 100, 200, 4), ("lamb_two", 2, 100, 201, 1), ("step", 3, 100, 200, 1), ("step", 2, 3, 48, 1),
+    ("step", 2, 3, 49, 3), ("step", 2, 3, 249, 3), ("step", 2, 3, 250, 1), ("lamb", 2, 3, 100, 1), ("two", 2, 3, 100, 1)])
+def test_small_steps(api, kind, M, layers, pieces, launches):  # noqa: F811
+    """pieces: of 2048 elements, spread over the layers (each of whole pieces)."""
+    if pieces > 3 * torch.cuda.get_device_properties(0).multi_processor_count:
+        pytest.skip("the device holds fewer")
+    sizes = [2048 * (pieces // layers + (k < pieces % layers)) for k in range(layers)]
+    assert _launches(api, sizes, M, kind) == launches
