@@ -528,12 +528,14 @@ __device__ __forceinline__ void p_direction(const PArgs &a, int64_t e0, int64_t 
 // stored, and leaves the tile's sum of g_hat^2 per warp in scratch[2w]. ----------------------------
 // G: groups of eight per thread, from the tile's piece `piece` on (G = 2: the whole tile, piece 0; G = 1: half a tile; with
 // G = 2 a call may ask for one group: half a tile too).
-// ENDS: the groups at the layer's two ends by whole warps, with P_ENDS_FROM workers and more: one or two are drawn sooner by the
-// group's own lane than handed out (own lane / warp, by phases: 1.5 million elements in 300 layers, M = 1, 26.1 / 27.2 us,
-// M = 2, 30.8 / 32.6, M = 3, 34.5 / 34.9, M = 4, 39.3 / 38.1, M = 5, 43.9 / 41.3); with whole tiles by a kernel without the warps'
-// code, which has 64 registers (16 million elements, M = 1, 108.3 / 106.7 us, two-sided 149.6 / 147.0, M = 2, 168.3 / 165.3).
+// ENDS: the groups at the layer's two ends by whole warps.  One or two workers are drawn sooner by the group's own lane than
+// handed out (own lane / warp, by phases: 1.5 million elements in 300 layers, M = 1, 26.1 / 27.2 us, M = 2, 30.8 / 32.6, M = 3,
+// 34.5 / 34.9, M = 4, 39.3 / 38.1, M = 5, 43.9 / 41.3): half tiles leave it to the number, whole tiles have a kernel without the
+// warps' code, beside which 64 registers are tight (16 million elements, M = 1, 108.3 / 106.7 us, two-sided 149.6 / 147.0, M = 2,
+// 168.3 / 165.3), and the resident form always does it (there both take the same: 300 thousand in 150 layers, M = 1, 20.6 / 20.3).
+enum { P_ENDS_NONE = 0, P_ENDS_ALL = 1, P_ENDS_BY_M = 2 };
 #define P_ENDS_FROM 3
-template <bool RNG16, int MODE, int OPT, bool TWO, int G, bool ENDS = (MODE != P_MODE_IDENTITY)>
+template <bool RNG16, int MODE, int OPT, bool TWO, int G, int ENDS>
 __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt, int piece, double *scratch, float2 *s_fac, int groups = G)
 {
     const int M = a.M, layer = pt.layer;
@@ -554,12 +556,12 @@ __device__ __forceinline__ void p_part_quant(const PArgs &a, const PipePart &pt,
     double ss_theta = 0.0, ss_u = 0.0;
     const int64_t begin = p_tile_begin(pt) + (int64_t)piece * (8 * DAT_P_THREADS);
     __shared__ float s_ends[ENDS ? 2 : 1][8];
-    const bool ends = ENDS && !plain && (G == 2 || M >= P_ENDS_FROM);        // (G = 2: a kernel of its own without them)
+    const bool ends = ENDS != P_ENDS_NONE && !plain && (ENDS == P_ENDS_ALL || M >= P_ENDS_FROM);
     if (ends && begin < hi) {
         const int64_t last = min(begin + 8 * (groups * DAT_P_THREADS - 1), (hi - 1) & ~(int64_t)7);
         if ((threadIdx.x >> 5) == 0 && (begin < lo || begin + 8 > hi)) p_ragged<RNG16, MODE>(a, qc, s_fac, begin, lo, hi, s_ends[0]);
         if ((threadIdx.x >> 5) == (unsigned)((last - begin) / 256) % (DAT_P_THREADS / 32) && last > begin && last + 8 > hi)
-            p_ragged<RNG16, MODE>(a, qc, s_fac, last, lo, hi, s_ends[ENDS]);
+            p_ragged<RNG16, MODE>(a, qc, s_fac, last, lo, hi, s_ends[ENDS ? 1 : 0]);
         __syncwarp();                              // (read by a lane of the warp that drew it)
     }
 #pragma unroll 1
@@ -842,7 +844,7 @@ k_step_pipelined(const __grid_constant__ PArgs a)
     bool alive = (s_ctl[1] != 0);
     // (the groups at a layer's ends by their own lanes: the wait is hidden here, and the code beside the long loop is not --
     // with whole warps ResNet-50 takes 336 us instead of 330, 1 billion parameters 13.9 ms instead of 13.7)
-    if (alive && pq.layer >= 0) p_part_quant<RNG16, MODE, OPT, TWO, DAT_P_GROUPS, false>(a, pq, 0, s_unit, s_fac);
+    if (alive && pq.layer >= 0) p_part_quant<RNG16, MODE, OPT, TWO, DAT_P_GROUPS, P_ENDS_NONE>(a, pq, 0, s_unit, s_fac);
     __syncthreads();
     if (TWO) {
         // Step 10: the tile's sum of g_hat^2 counted in; the layer's last tile publishes the server's norm;
@@ -938,7 +940,7 @@ __device__ __forceinline__ bool p_share_publish(const PArgs &a, const PhaseShare
 
 // G = 2: whole tiles (see p_share).  G = 1: half a tile (see p_halves): twice the CTAs, and four workers' loads in flight
 // per thread, which then has the registers (300 thousand elements, M = 64: 166 us with G = 2, 121 with G = 1).
-template <bool RNG16, int MODE, int OPT, bool TWO, int G, bool ENDS>
+template <bool RNG16, int MODE, int OPT, bool TWO, int G, int ENDS>
 __global__ void __launch_bounds__(DAT_P_THREADS, G == 1 ? 3 : DAT_P_MINB)
 k_phase_quant(const __grid_constant__ PArgs a)
 {
@@ -1402,9 +1404,9 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
 #define P_GO(R, MODE, OPT, TWO)                                                                                     \
     do {                                                                                                            \
         if (!phases) k_step_pipelined<R, MODE, OPT, TWO><<<grid, DAT_P_THREADS, 0, s>>>(a);                         \
-        else if (halves) P_PHASES_GO(R, MODE, OPT, TWO, 1, MODE != P_MODE_IDENTITY);                                \
-        else if (plan->M >= P_ENDS_FROM) P_PHASES_GO(R, MODE, OPT, TWO, 2, MODE != P_MODE_IDENTITY);                \
-        else P_PHASES_GO(R, MODE, OPT, TWO, 2, false);                                                              \
+        else if (halves) P_PHASES_GO(R, MODE, OPT, TWO, 1, MODE != P_MODE_IDENTITY ? P_ENDS_BY_M : P_ENDS_NONE);    \
+        else if (plan->M >= P_ENDS_FROM) P_PHASES_GO(R, MODE, OPT, TWO, 2, MODE != P_MODE_IDENTITY ? P_ENDS_ALL : P_ENDS_NONE); \
+        else P_PHASES_GO(R, MODE, OPT, TWO, 2, P_ENDS_NONE);                                                        \
     } while (0)
 #define P_GO_OPT(R, MODE)                                                                                           \
     do {                                                                                                            \

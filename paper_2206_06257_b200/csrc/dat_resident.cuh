@@ -156,7 +156,7 @@ __device__ __forceinline__ void r_late(const PArgs &a, const PipePart &pc, doubl
 #pragma unroll 1
         for (int k = 0; k < n; ++k) {
             const int tile = s_own[k];
-            if (!TWO || server) p_part_quant<RNG16, MODE, OPT, TWO, 1>(a, r_tile(pc, tile), tile & 1, s_red, s_fac);
+            if (!TWO || server) p_part_quant<RNG16, MODE, OPT, TWO, 1, P_ENDS_ALL>(a, r_tile(pc, tile), tile & 1, s_red, s_fac);
             else p_part_requant<RNG16, OPT, 1>(a, r_tile(pc, tile), tile & 1, s_red);
             __syncthreads();
             if (threadIdx.x == 0) {
@@ -233,7 +233,7 @@ k_step_resident(const __grid_constant__ PArgs a)
         return;
     }
 
-    p_part_quant<RNG16, MODE, OPT, TWO, 1>(a, r_tile(pc, pc.tile), pc.tile & 1, s_red, s_fac);
+    p_part_quant<RNG16, MODE, OPT, TWO, 1, P_ENDS_ALL>(a, r_tile(pc, pc.tile), pc.tile & 1, s_red, s_fac);
     __syncthreads();
     if (TWO) {
         if (threadIdx.x == 0) a.partR[slot] = p_warps_sum(s_red);
