@@ -1,5 +1,5 @@
-"""GPU: the two forms of a step -- one launch, and one launch per phase for small problems -- on both sides of the line
-between them, against the separate calls (dat_quantize, dat_aggregate / dat_average, dat_requantize, dat_lalr_step,
+"""GPU: the three forms of a step -- one launch, one launch per phase, and one whose CTAs keep their pieces -- as the rule
+chooses them by size, workers and the largest layer, against the separate calls (dat_quantize, dat_aggregate / dat_average, dat_requantize, dat_lalr_step,
 dat_lamb_step) on the same inputs.  The quantizer norms and the layers' norms are sums of the same numbers in other orders
 (at most one unit in the last place apart); where the bits of the quantizer norms agree, codes and moments have to be the
 same, and theta within 1e-5 relative of rounding through the layers' norms.
@@ -15,14 +15,18 @@ pytestmark = pytest.mark.gpu
 HP = (0.1, 0.9, 5e-4, 0.0, 10.0)
 LAMB_HP = (0.1, 0.9, 0.999, 1e-6, 1e-4, 0.0, 10.0)
 TILE = 4096
-# tiles on a 148-SM GPU: one wave of half tiles; above one wave (phases; two-sided and b = 32 in one launch, M >= 8 by half
-# tiles); above nine per SM (one launch), where one worker still goes by phases
-SIZES = {"small": [1, 7, 2047, 2049, 4097], "below": [9, 600 * TILE - 3, 4095], "above": [9, 1340 * TILE + 5, 33]}
+# tiles on a 148-SM GPU: a few pieces (kept by their CTAs; many workers and b = 32 by phases); above one wave (phases, M >= 8 by
+# half tiles; b = 32 in one launch); above nine tiles per SM in one layer (phases; b = 32 in one launch), and in eight equal ones
+# (one launch; one worker by phases)
+SIZES = {"small": [1, 7, 2047, 2049, 4097], "below": [9, 600 * TILE - 3, 4095], "above": [9, 1340 * TILE + 5, 33],
+         "spread": [9, 33] + [170 * TILE + k for k in (-3, 0, 5, 1, 8, -7, 2, 11)]}
 
 
 @pytest.mark.parametrize("kind", ["step", "lamb", "two_sided"])
 @pytest.mark.parametrize("where,M,bits,rng_bits,per_worker", [("small", 5, 8, 16, False), ("below", 3, 4, 23, False), ("below", 9, 8, 16, False), ("below", 2, 32, 16, False), ("above", 3, 8, 16, False),
                                                               ("above", 2, 4, 16, True), ("below", 2, 2, 23, True), ("above", 1, 8, 16, False),
+                                                              ("spread", 3, 8, 16, False), ("spread", 2, 4, 16, True), ("spread", 9, 1, 23, False),
+                                                              ("spread", 2, 16, 23, True), ("spread", 1, 8, 16, False), ("spread", 2, 32, 16, False),
                                                               ("small", 64, 1, 16, True), ("above", 2, 32, 16, False), ("small", 3, 32, 16, False)])
 def test_step_forms_equal_separate_calls(kind, where, M, bits, rng_bits, per_worker):
     from paper_2206_06257_b200 import api
