@@ -414,8 +414,8 @@ int dat_step_passes(dat_plan_t *plan, float *theta, float *mom, const float *con
 int dat_plan_test_stall(dat_plan_t *plan, int64_t wait_cycles, int64_t layer, void *stream);
 
 /* dat_plan_test_form -- TEST HOOK: the form of the plan's dat_step, dat_step_lamb and two-sided steps whatever their size:
- * 1 the one launch, 2 a launch per phase, 3 one launch whose CTAs keep their pieces (ARG where b = 32 or the problem has more
- * than three pieces of 2048 elements per SM), 4 the same with a CTA per layer, which takes the layer's other pieces as
+ * 1 the one launch, 2 a launch per phase, 3 one launch whose CTAs keep their pieces (ARG where the problem has more than
+ * three pieces of 2048 elements per SM; a plan of b = 32 has no such form and takes 2), 4 the same with a CTA per layer, which takes the layer's other pieces as
  * running CTAs do where the others cannot start, 0 by the rule again.  Nothing else uses this.  Errors: ARG. */
 int dat_plan_test_form(dat_plan_t *plan, int form);
 

@@ -1513,7 +1513,9 @@ extern "C" int dat_plan_test_form(dat_plan_t *plan, int form)
 {
     int rc = dat_check_plan(plan);
     if (rc != DAT_OK) return rc;
-    if (!plan->pipe || form < P_BY_RULE || form > P_RESIDENT_LATE || (form >= P_RESIDENT && !plan->pipe->n_pieces)) return DAT_ERR_ARG;
+    if (!plan->pipe || form < P_BY_RULE || form > P_RESIDENT_LATE) return DAT_ERR_ARG;
+    if (form >= P_RESIDENT && plan->bits == 32) form = P_PHASES;            // (no norms to wait for: no resident form)
+    if (form >= P_RESIDENT && !plan->pipe->n_pieces) return DAT_ERR_ARG;
     plan->pipe->form = form;
     return DAT_OK;
 }

@@ -1,6 +1,5 @@
-"""GPU: the oracle's parity cases of the step calls in the resident form (one launch whose CTAs keep their pieces) -- as it is,
-and with one CTA per layer, which takes all the layer's pieces as the running CTAs do where the others cannot start --, its
-largest problems against the form of a launch per phase, and steps of several plans at once."""
+"""GPU: the oracle's parity cases of the step calls in the resident form (one launch whose CTAs keep their pieces), and its
+largest problems against the form of a launch per phase."""
 import numpy as np
 import pytest
 import torch
@@ -10,22 +9,21 @@ from helpers import GpuPlan, assert_close_per_layer, np_of, ulp_diff
 from test_gpu_parity import api  # noqa: F401  (fixture)
 
 pytestmark = pytest.mark.gpu
-RESIDENT, LATE, PHASES = 3, 4, 2
+RESIDENT, PHASES = 3, 2
 
 
-@pytest.fixture(params=[RESIDENT, LATE], ids=["all", "late"])
-def resident(request, api, monkeypatch):  # noqa: F811
+@pytest.fixture
+def resident(api, monkeypatch):  # noqa: F811
     create = api.dat_plan_create
 
-    def create_with_form(offs, M, bits, **kw):
-        plan = create(offs, M, bits, **kw)
-        if bits != 32:                               # (the form is for steps with norms)
-            api.dat_plan_test_form(plan, request.param)
+    def create_with_form(*args, **kw):
+        plan = create(*args, **kw)
+        api.dat_plan_test_form(plan, RESIDENT)
         return plan
     monkeypatch.setattr(api, "dat_plan_create", create_with_form)
 
 
-@pytest.mark.parametrize("bits", [1, 8, 16])
+@pytest.mark.parametrize("bits", [1, 8, 16, 32])
 def test_ragged(api, oracle, resident, bits, rng_bits):  # noqa: F811
     parity.test_fused_parity_ragged(api, oracle, bits, rng_bits)
 
@@ -40,7 +38,7 @@ def test_extreme_scales(api, oracle, resident, bits, rng_bits):  # noqa: F811
     parity.test_fused_parity_extreme_scales(api, oracle, bits, rng_bits)
 
 
-@pytest.mark.parametrize("mode", ["shared", "per_worker"])
+@pytest.mark.parametrize("mode", ["shared", "per_worker", "b32"])
 def test_lamb(api, oracle, resident, mode):  # noqa: F811
     parity.test_step_lamb_parity_three_steps(api, oracle, mode)
 
@@ -59,14 +57,13 @@ def test_zero_layers_nonfinite_inputs_margins_and_capture(api, oracle, resident)
     parity.test_step_refuses_stream_capture(api)
 
 
-@pytest.mark.parametrize("form", [RESIDENT, LATE])
-def test_a_wait_that_runs_out_is_reported_and_the_plan_recovers(api, oracle, form):  # noqa: F811
+def test_a_wait_that_runs_out_is_reported_and_the_plan_recovers(api, oracle):  # noqa: F811
     """A layer whose norm never completes: the status says so, and the next step is the oracle's again."""
     offs, grads, theta, mom = parity._random_problem(5, [4096, 9000, 70], 3)
     with GpuPlan(api, offs, 3, 8) as P:
         th, mo, g = torch.from_numpy(theta).cuda(), torch.from_numpy(mom).cuda(), [torch.from_numpy(x).cuda() for x in grads]
         api.dat_plan_test_stall(P.plan, 2_000_000, 1)
-        api.dat_plan_test_form(P.plan, form)
+        api.dat_plan_test_form(P.plan, RESIDENT)
         api.dat_step(P.plan, th, mo, g, 3, 5, parity.HP)
         assert api.dat_get_status(P.plan) & api.DAT_STATUS_TIMEOUT
         th, mo, sc = torch.from_numpy(theta).cuda(), torch.from_numpy(mom).cuda(), torch.zeros(P.h, device="cuda")
@@ -90,7 +87,7 @@ def test_up_to_the_most_pieces_equals_the_phases(api, pieces, kind):  # noqa: F8
     rnd = lambda s: torch.randn(d, generator=gen, device="cuda") * s  # noqa: E731
     theta, mom, var, grads = rnd(0.05), rnd(1e-3), rnd(1e-3).square(), [rnd(1e-2) for _ in range(M)]
     out = {}
-    for form in (PHASES, RESIDENT, LATE):
+    for form in (PHASES, RESIDENT):
         with GpuPlan(api, offs, M, 8) as P:
             api.dat_plan_test_form(P.plan, form)
             th, mo, va, gh, sc = theta.clone(), mom.clone(), var.clone(), torch.zeros_like(theta), torch.zeros(P.h, device="cuda")
@@ -102,50 +99,19 @@ def test_up_to_the_most_pieces_equals_the_phases(api, pieces, kind):  # noqa: F8
                 api.dat_step_two_sided(P.plan, th, mo, grads, 7, 3, parity.HP, gh, None, None, sc)
             assert P.status() == 0
             out[form] = [np_of(x) for x in (th, mo, va, gh, sc)]
-    for x, y in zip(out[RESIDENT], out[LATE]):           # the sums are the same, whoever forms them
-        assert np.array_equal(x, y)
     a, b = out[PHASES], out[RESIDENT]
     assert ulp_diff(a[4], b[4]).max() <= 1
-    for l in range(len(offs) - 1):
-        s = slice(int(offs[l]), int(offs[l + 1]))
-        if a[4][l] == b[4][l]:
-            if kind != "two_sided":                          # (the server's norm is a sum in another order too)
-                assert np.array_equal(a[1][s], b[1][s]) and np.array_equal(a[2][s], b[2][s])
-            for k, name in enumerate(("theta", "momentum", "var", "g_hat")):
-                assert_close_per_layer(b[k][s], a[k][s], [0, s.stop - s.start], name)
+    same = np.array_equal(a[4], b[4])
+    if same and kind != "two_sided":
+        assert np.array_equal(a[1], b[1]) and np.array_equal(a[2], b[2])
+    for k, name in enumerate(("theta", "momentum", "var", "g_hat")):
+        if same:
+            assert_close_per_layer(b[k], a[k], offs, name)
 
 
-@pytest.mark.parametrize("bits", [8, 32])
-def test_a_larger_problem_and_one_without_norms_have_no_resident_form(api, bits):  # noqa: F811
+def test_a_larger_problem_has_no_resident_form(api):  # noqa: F811
     n = 3 * torch.cuda.get_device_properties(0).multi_processor_count
-    with GpuPlan(api, np.array([0, 2048 * n + 1 if bits != 32 else 31], dtype=np.int64), 2, bits) as P:
+    with GpuPlan(api, np.array([0, 2048 * n + 1], dtype=np.int64), 2, 8) as P:
         with pytest.raises(api.DatError) as e:
             api.dat_plan_test_form(P.plan, RESIDENT)
         assert e.value.code == api.DAT_ERR_ARG
-
-
-def test_steps_of_several_plans_at_once(api):  # noqa: F811
-    """Each problem alone takes the whole chip; on six streams at once every step ends, with the same bits as alone."""
-    n, steps, M = 3 * torch.cuda.get_device_properties(0).multi_processor_count, 8, 2
-    offs = np.concatenate([[0], np.cumsum([2048 * (n // 2) - 5, 40, 2048 * (n - n // 2 - 4)])]).astype(np.int64)
-    d = int(offs[-1])
-    gen = torch.Generator(device="cuda").manual_seed(n)
-    rnd = lambda s: torch.randn(d, generator=gen, device="cuda") * s  # noqa: E731
-    theta, mom, grads = rnd(0.05), rnd(1e-3), [rnd(1e-2) for _ in range(M)]
-    out = []
-    for streams in ([torch.cuda.current_stream()], [torch.cuda.Stream() for _ in range(6)]):
-        plans = [GpuPlan(api, offs, M, 8) for _ in streams]
-        states = [(theta.clone(), mom.clone()) for _ in streams]
-        torch.cuda.synchronize()
-        for P in plans:
-            api.dat_plan_test_form(P.plan, RESIDENT)
-        for t in range(steps):
-            for P, (th, mo), s in zip(plans, states, streams):
-                api.dat_step(P.plan, th, mo, grads, 7, t, parity.HP, stream=s)
-        torch.cuda.synchronize()
-        for P, (th, mo) in zip(plans, states):
-            assert P.status() == 0
-            out.append((np_of(th), np_of(mo)))
-            P.close()
-    for th, mo in out[1:]:
-        assert np.array_equal(th, out[0][0]) and np.array_equal(mo, out[0][1])
