@@ -318,11 +318,12 @@ int dat_lalr_step_static(int64_t num_layers, const int64_t *layer_offsets, float
  * dat_step -- Steps 7, 9 and 12 of Algorithm A1 in one call: the result equals
  * dat_quantize -> dat_aggregate -> dat_lalr_step (or dat_average -> dat_lalr_step when b = 32),
  * but codes, code sums and g_hat are never written to device memory.  One kernel launch
- * (dat_step_pipelined) for problems that fill the GPU, one launch per phase (dat_step_passes) up to four tiles of 4096
- * elements per SM; with b < 32 also up to nine, where one layer has more than 0.27 of the elements, and (one-sided) for a
- * single worker at any size.  With b < 32 and at most three pieces of 2048 elements per SM it is one launch
- * whose CTAs keep a piece each through all phases and wait, bounded, for its layer.  Nothing is allocated and nothing synchronises: every table the launches
- * need was built by dat_plan_create.
+ * (dat_step_pipelined) for problems that fill the GPU; with b < 32 and at most three pieces of 2048 elements per SM mostly one
+ * launch whose CTAs keep a piece each through all phases and wait, bounded, for its layer; otherwise one launch per phase
+ * (dat_step_passes) for problems of up to four tiles of 4096 elements per SM, with b < 32 of up to nine, and with b < 32, at any
+ * size, where one layer has 0.27 or more of the elements or there is a single worker (two-sided momentum steps of many tiles per SM: only
+ * where a layer is larger).  The results are the same up to the norms' last place.  Nothing is allocated and nothing synchronises:
+ * every table the launches need was built by dat_plan_create.
  *   theta, mom        device fp32[d], updated in place.
  *   grads             host array of M device pointers, fp32[d] each, read-only.
  *   seed, step        as in dat_quantize.
@@ -398,7 +399,7 @@ int dat_step_lamb_two_sided(dat_plan_t *plan, float *theta, float *mom, float *v
 /* dat_step_passes -- the same step as dat_step, with the same arguments and the same results bit for
  * bit up to the norms' last place, as one launch per phase: quantizer norms; then levels, signed sum over the
  * workers, g_hat, m' and the layer sums in one pass that keeps codes, sums and g_hat in registers; then the theta
- * update.  What dat_step does for small problems, whatever the size.  For plans with b < 32 and the shared scale
+ * update.  One of the forms that dat_step takes, here whatever the size.  For plans with b < 32 and the shared scale
  * (DAT_ERR_UNSUPPORTED otherwise).  The call can be recorded into a CUDA graph; a replay repeats the recorded seed and
  * step. */
 int dat_step_passes(dat_plan_t *plan, float *theta, float *mom, const float *const *grads,

@@ -1,5 +1,6 @@
 // dat_step_pipelined: Steps 7, 9 and 12 of Algorithm A1 in ONE launch of ordinary (non-persistent)
-// CTAs (and, further down, the same parts as one launch per phase, which small problems take: see p_phases).  Codes, integer sums and g_hat never reach memory; the gradients are read twice (for the norm, then
+// CTAs (and, further down, the two other forms of a step: one launch per phase, and one launch whose CTAs keep their
+// pieces; see p_phases and p_resident).  Codes, integer sums and g_hat never reach memory; the gradients are read twice (for the norm, then
 // for the levels), the second time from L2 only where a layer is small enough to still be there.
 //
 // The quantizer norm of a layer (Eq. rand_q) must be known before the first level of that layer
@@ -1444,7 +1445,7 @@ extern "C" int dat_step_pipelined(dat_plan_t *plan, float *theta, float *mom, co
                     layer_norms_out, scales_out, stream, nullptr, nullptr, nullptr, P_ONE_LAUNCH);
 }
 
-// dat_step: Steps 7, 9 and 12 in the form that p_phases chooses.
+// dat_step: Steps 7, 9 and 12 in the form that p_resident and p_phases choose.
 extern "C" int dat_step(dat_plan_t *plan, float *theta, float *mom, const float *const *grads,
                         uint64_t seed, uint64_t step, const dat_hparams_t *hp,
                         int32_t *code_sum_out, float *layer_norms_out, float *scales_out, void *stream)
