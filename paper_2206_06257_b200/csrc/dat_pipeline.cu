@@ -1256,13 +1256,16 @@ static bool p_halves(const dat_plan_t *plan)
     return n <= P_PHASES_WAVE * sm || (n <= P_PHASES_MOST * sm && plan->M >= 8);
 }
 
-// The tiles that a phase's CTAs take whole, where not all go by halves: full waves of them, if the rest fits half a wave.
+// The tiles that a phase's CTAs take whole, where not all go by halves: full waves of them, if the rest fits 0.4 of a wave, of LAMB
+// steps half a wave.
 // All whole / the rest by halves, in us, 592 CTAs a wave: 2.5 million elements in 40 odd layers, M = 1, 4, 6: 29.8 / 29.0, 41.0 / 39.8,
-// 47.6 / 45.8, LAMB 47.5 / 43.2, 54.9 / 50.8, 61.9 / 56.5, two-sided 39.6 / 38.9, 51.8 / 49.5, 58.3 / 56.0; 5.2 million, LAMB, M = 4, 86.5 / 83.4.
-static uint32_t p_whole(const dat_plan_t *plan)
+// 47.6 / 45.8, LAMB 47.5 / 43.2, 54.9 / 50.8, 61.9 / 56.5, two-sided 39.6 / 38.9, 51.8 / 49.5, 58.3 / 56.0; 5.2 million, LAMB, M = 4, 86.5 / 83.4.  A rest of 0.3 of a wave, M = 1, 4, 6: 27.5 / 26.7, 42.1 / 41.0,
+// 51.0 / 48.8; 0.4: 28.8 / 28.5, 43.3 / 43.1, 52.9 / 51.7, two-sided 41.0 / 40.5, 56.0 / 55.5, 66.0 / 65.0; but 0.5: 29.9 / 30.7, 45.5 / 45.6, 55.2 / 55.0,
+// two-sided 41.7 / 42.0, 58.8 / 59.3, 69.0 / 68.4; LAMB 45.2 / 43.6, 61.1 / 59.4, 70.3 / 67.9.
+static uint32_t p_whole(const dat_plan_t *plan, bool lamb)
 {
     const int64_t n = plan->pipe->n_tiles, wave = DAT_P_MINB * (int64_t)plan->sm_count, rest = n % wave;
-    return (uint32_t)(2 * rest <= wave ? n - rest : n);
+    return (uint32_t)((lamb ? 2 * rest <= wave : 5 * rest <= 2 * wave) ? n - rest : n);
 }
 
 // A launch that may be set up while the one before it ends (its kernel waits for that end itself).
@@ -1385,7 +1388,7 @@ static int p_launch(dat_plan_t *plan, float *theta, float *mom, float *var, cons
     }
     const bool phases = form == P_PHASES;
     const bool halves = phases && p_halves(plan);
-    a.n_whole = phases && !halves ? p_whole(plan) : 0u;
+    a.n_whole = phases && !halves ? p_whole(plan, lamb != nullptr) : 0u;
     const unsigned grid = phases ? 2u * (unsigned)g->n_tiles - a.n_whole : a.n_items;
     if (phases && !identity) {
         rc = dat_norm_phase(plan, a.gp, a.scales_out, s);

@@ -31,12 +31,12 @@ def _offs(tiles):
 
 
 # tiles beyond one wave of CTAs (at one wave all go by halves)
-@pytest.mark.parametrize("rest", ["1", "half", "half + 1", "wave - 1", "wave", "wave + 1"])
+@pytest.mark.parametrize("rest", ["1", "0.4", "0.4 + 1", "half", "half + 1", "wave - 1", "wave", "wave + 1"])
 @pytest.mark.parametrize("kind", ["step", "lamb", "two_sided"])
 @pytest.mark.parametrize("M,rng_bits,per_worker", [(2, 16, False), (3, 23, True)])
 def test_last_wave_by_half_tiles(api, kind, rest, M, rng_bits, per_worker):  # noqa: F811
     wave = _wave()
-    offs = _offs(wave + {"1": 1, "half": wave // 2, "half + 1": wave // 2 + 1, "wave - 1": wave - 1, "wave": wave, "wave + 1": wave + 1}[rest])
+    offs = _offs(wave + {"1": 1, "0.4": 2 * wave // 5, "0.4 + 1": 2 * wave // 5 + 1, "half": wave // 2, "half + 1": wave // 2 + 1, "wave - 1": wave - 1, "wave": wave, "wave + 1": wave + 1}[rest])
     d = int(offs[-1])
     gen = torch.Generator(device="cuda").manual_seed(d)
     rnd = lambda s: torch.randn(d, generator=gen, device="cuda") * s  # noqa: E731
